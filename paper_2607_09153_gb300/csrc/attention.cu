@@ -39,6 +39,7 @@
 #include <cuda_bf16.h>
 
 #include <algorithm>
+#include <cstring>
 #include <climits>
 #include <unordered_map>
 #include <vector>
@@ -1010,7 +1011,9 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
     total_refs += np[b];
   }
   // ---- 1. runs
-  std::vector<uint8_t> is_shared(static_cast<size_t>(n) * max_blocks, 0);
+  std::vector<uint8_t> in_group_dense;   // by page id (or, sparse, in_group): scored with a group
+  std::unordered_map<int32_t, char> in_group;
+  bool grouped = false;
   std::vector<Run> runs;
   if (share && total_refs > 0) {
     // Every full page's referencing candidates, in increasing candidate order.  Page ids up to a few
@@ -1032,17 +1035,22 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
     std::unordered_map<int32_t, std::vector<int32_t>> refs;           // sparse
     bool any_dup = false;
     if (dense) {
+      // counts first: a call whose pages are all private (the common ragged batch) needs no lists
       ref_off.assign(static_cast<size_t>(max_page) + 2, 0);
-      for (int b = 0; b < n; ++b)
-        for (int j = 0, nfull = sl[b] / 16; j < nfull; ++j) ++ref_off[bt[static_cast<int64_t>(b) * max_blocks + j] + 1];
-      for (size_t pg = 1; pg < ref_off.size(); ++pg) {
-        any_dup = any_dup || ref_off[pg] > 1;
-        ref_off[pg] += ref_off[pg - 1];
+      int32_t most = 0;
+      for (int b = 0; b < n; ++b) {
+        const int32_t* row = bt + static_cast<int64_t>(b) * max_blocks;
+        for (int j = 0, nfull = sl[b] / 16; j < nfull; ++j) most = std::max(most, ++ref_off[row[j] + 1]);
       }
-      ref_list.resize(static_cast<size_t>(full_refs));
-      std::vector<int32_t> fill(ref_off.begin(), ref_off.end() - 1);
-      for (int b = 0; b < n; ++b)
-        for (int j = 0, nfull = sl[b] / 16; j < nfull; ++j) ref_list[fill[bt[static_cast<int64_t>(b) * max_blocks + j]]++] = b;
+      any_dup = most > 1;
+      if (any_dup) {
+        for (size_t pg = 1; pg < ref_off.size(); ++pg) ref_off[pg] += ref_off[pg - 1];
+        ref_list.resize(static_cast<size_t>(full_refs));
+        std::vector<int32_t> fill(ref_off.begin(), ref_off.end() - 1);
+        for (int b = 0; b < n; ++b)
+          for (int j = 0, nfull = sl[b] / 16; j < nfull; ++j)
+            ref_list[fill[bt[static_cast<int64_t>(b) * max_blocks + j]]++] = b;
+      }
     } else {
       refs.reserve(static_cast<size_t>(total_refs));
       for (int b = 0; b < n; ++b) {
@@ -1057,25 +1065,31 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
     if (any_dup) {
       std::vector<std::vector<int32_t>> group_cands, group_pages;
       std::unordered_map<uint64_t, int> gidx;
-      std::vector<uint8_t> in_group_dense(dense ? static_cast<size_t>(max_page) + 1 : 0, 0);
-      std::unordered_map<int32_t, char> in_group;
+      if (dense) in_group_dense.assign(static_cast<size_t>(max_page) + 1, 0);
+      int last = -1;   // the group of the page before: neighbours in a pool often share one
       // a page referenced (in full) by the candidates c[0 .. len), in increasing order
       auto consider = [&](int32_t page, const int32_t* c, size_t len) {
         if (len < 2) return;
         for (size_t i = 1; i < len; ++i)
           if (c[i] == c[i - 1]) return;   // a candidate listing the page twice keeps it private
-        const uint64_t h = hash_list(c, static_cast<int>(len));
-        auto itg = gidx.find(h);
-        int gi;
-        if (itg != gidx.end()) {
-          const std::vector<int32_t>& g = group_cands[itg->second];
-          if (g.size() != len || !std::equal(g.begin(), g.end(), c)) return;   // hash collision: private
-          gi = itg->second;
-        } else {
-          gi = static_cast<int>(group_cands.size());
-          gidx.emplace(h, gi);
-          group_cands.emplace_back(c, c + len);
-          group_pages.emplace_back();
+        auto same = [&](int gi) {
+          const std::vector<int32_t>& g = group_cands[gi];
+          return g.size() == len && std::memcmp(g.data(), c, len * sizeof(int32_t)) == 0;
+        };
+        int gi = last;
+        if (gi < 0 || !same(gi)) {
+          const uint64_t h = hash_list(c, static_cast<int>(len));
+          auto itg = gidx.find(h);
+          if (itg != gidx.end()) {
+            if (!same(itg->second)) return;   // hash collision: private
+            gi = itg->second;
+          } else {
+            gi = static_cast<int>(group_cands.size());
+            gidx.emplace(h, gi);
+            group_cands.emplace_back(c, c + len);
+            group_pages.emplace_back();
+          }
+          last = gi;
         }
         group_pages[gi].push_back(page);
         if (dense)
@@ -1089,13 +1103,7 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
       } else {
         for (auto& kv : refs) consider(kv.first, kv.second.data(), kv.second.size());
       }
-      for (int b = 0; b < n; ++b) {
-        const int nfull = sl[b] / 16;
-        for (int j = 0; j < nfull; ++j) {
-          const int32_t pg = bt[static_cast<int64_t>(b) * max_blocks + j];
-          if (dense ? in_group_dense[pg] != 0 : in_group.count(pg) != 0) is_shared[static_cast<size_t>(b) * max_blocks + j] = 1;
-        }
-      }
+      grouped = !group_cands.empty();
       for (auto& pgs : group_pages) std::sort(pgs.begin(), pgs.end());   // deterministic contents
       std::vector<int> order(group_cands.size());   // deterministic group order
       for (size_t i = 0; i < order.size(); ++i) order[i] = static_cast<int>(i);
@@ -1169,11 +1177,19 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
     r.n_cands = 1;
     r.page_off = static_cast<int>(w.pages.size());
     r.last_valid = 16;
-    for (int j = 0; j < np[b]; ++j)
-      if (!is_shared[static_cast<size_t>(b) * max_blocks + j]) {
-        w.pages.push_back(bt[static_cast<int64_t>(b) * max_blocks + j]);
-        if (j == np[b] - 1) r.last_valid = sl[b] - 16 * (np[b] - 1);
+    const int32_t* row = bt + static_cast<int64_t>(b) * max_blocks;
+    if (!grouped) {
+      w.pages.insert(w.pages.end(), row, row + np[b]);
+      if (np[b] > 0) r.last_valid = sl[b] - 16 * (np[b] - 1);
+    } else {
+      const int nfull = sl[b] / 16;   // a last page in part is the candidate's own
+      for (int j = 0; j < nfull; ++j)
+        if (in_group_dense.empty() ? in_group.count(row[j]) == 0 : in_group_dense[row[j]] == 0) w.pages.push_back(row[j]);
+      if (np[b] > nfull) {
+        w.pages.push_back(row[nfull]);
+        r.last_valid = sl[b] - 16 * nfull;
       }
+    }
     r.n_pages = static_cast<int>(w.pages.size()) - r.page_off;
     if (r.n_pages == 0) continue;   // an empty cache, or every page shared
     r.cost = kPrivateCost;

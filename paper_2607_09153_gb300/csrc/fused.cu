@@ -4,15 +4,19 @@
 // that feeds a tensor-core contraction is stored as a bf16 (hi, lo) pair,
 // hi = bf16(x), lo = bf16(x - hi), so no bf16 rounding of the activation
 // itself enters the result.
-//   rope_table   cos/sin of p * base^(-2i/hd) at p = L_b (fp64 angles)
-//   embed_norm   h = e_v ; per-tile sums of squares of h ; x = h ⊙ g (the
+//   call_begin   the call's tables from pinned host memory into the device
+//                tables (and, for the attention entry point, q as hi/lo)
+//   prologue     cos/sin of p * base^(-2i/hd) at p = L_b (fp64 angles);
+//                h = e_v ; per-tile sums of squares of h ; x = h ⊙ g (the
 //                RMSNorm's per-candidate factor 1/sqrt(mean(h^2) + eps) is
 //                applied by the QKV epilogue, as between all projections)
 //   head         x = RMSNorm(h) * g_final with mean(h^2) from the per-tile
 //                sums of squares the last residual epilogue wrote (summed in
-//                tile order: deterministic);
+//                a fixed order: deterministic);
 //                P(+) = 1/(1 + exp(w_minus.x - w_plus.x)) (Eq. score, App. B.2)
 #include <cuda_bf16.h>
+
+#include <algorithm>
 
 #include "kernels.h"
 #include "ptx.cuh"
@@ -27,96 +31,159 @@ __device__ __forceinline__ void store_hilo(HiLo o, int64_t i, float x) {
   o.lo[i] = __float2bfloat16_rn(x - __bfloat162float(hi));
 }
 
-// Sum over the block; every thread gets the total.  `red` has >= 32 floats.
-__device__ __forceinline__ float block_sum(float v, float* red) {
+// Four consecutive activations as 8-byte hi and lo stores.
+__device__ __forceinline__ void store_hilo4(HiLo o, int64_t i, float4 x) {
+  const __nv_bfloat162 h0 = __floats2bfloat162_rn(x.x, x.y), h1 = __floats2bfloat162_rn(x.z, x.w);
+  const float2 f0 = __bfloat1622float2(h0), f1 = __bfloat1622float2(h1);
+  const __nv_bfloat162 l0 = __floats2bfloat162_rn(x.x - f0.x, x.y - f0.y);
+  const __nv_bfloat162 l1 = __floats2bfloat162_rn(x.z - f1.x, x.w - f1.y);
+  uint2 hi, lo;
+  hi.x = *reinterpret_cast<const uint32_t*>(&h0);
+  hi.y = *reinterpret_cast<const uint32_t*>(&h1);
+  lo.x = *reinterpret_cast<const uint32_t*>(&l0);
+  lo.y = *reinterpret_cast<const uint32_t*>(&l1);
+  *reinterpret_cast<uint2*>(o.hi + i) = hi;
+  *reinterpret_cast<uint2*>(o.lo + i) = lo;
+}
+
+// Four consecutive bf16 (8-byte aligned) as fp32.
+__device__ __forceinline__ float4 load_bf16x4(const __nv_bfloat16* p) {
+  const uint2 r = *reinterpret_cast<const uint2*>(p);
+  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r.x));
+  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r.y));
+  return make_float4(a.x, a.y, b.x, b.y);
+}
+
+// The call's tables, read by the GPU from the pinned staging buffer (one launch instead of a copy per
+// table: seven to nine small copies took ~2 us each on the stream, ahead of every call), and for the
+// attention entry point the query as a bf16 pair.  Measured per call with calls queued back to back:
+// 2 layers of d 256 with 4 candidates 74 -> 55 us (with prologue_kernel in place of two launches and
+// the head's own store instead of a copy), the attention entry point with 37 ragged candidates 99 -> 71
+// us and with 24 candidates behind a prefix 81 -> 56 us (with the planner's counts first).  CTAs below pull_ctas copy the parts' 16-byte quads,
+// four loads in flight per thread (the host link's latency bounds it); the others split.
+__global__ void __launch_bounds__(128) call_begin_kernel(const __grid_constant__ TableParts parts, const uint4* src,
+                                                         uint4* dst, int pull_ctas, const float4* __restrict__ q,
+                                                         int64_t q_quads, HiLo out) {
+  if (static_cast<int>(blockIdx.x) < pull_ctas) {
+    const uint32_t total = parts.end[parts.n - 1], stride = static_cast<uint32_t>(pull_ctas) * blockDim.x;
+    for (uint32_t i0 = blockIdx.x * blockDim.x + threadIdx.x; i0 < total; i0 += 4 * stride) {
+      uint4 v[4];
+      uint32_t at[4];
 #pragma unroll
-  for (int off = 16; off > 0; off >>= 1) v += __shfl_xor_sync(0xffffffffu, v, off);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31, nw = (blockDim.x + 31) >> 5;
-  __syncthreads();
-  if (l == 0) red[w] = v;
-  __syncthreads();
-  float t = 0.f;
-  for (int i = 0; i < nw; ++i) t += red[i];
-  return t;
-}
-
-// 1/sqrt(mean(h^2) + eps) of candidate b from the per-tile sums of squares,
-// summed in tile order by one thread and broadcast through shared memory.
-__device__ __forceinline__ float row_rscale(const float* __restrict__ sumsq, int m_tiles, int n_cand, int b, int d,
-                                            float eps, float* slot) {
-  if (threadIdx.x == 0) {
-    float s = 0.f;
-    for (int t = 0; t < m_tiles; ++t) s += sumsq[static_cast<int64_t>(t) * n_cand + b];
-    *slot = 1.0f / sqrtf(s / d + eps);
+      for (int k = 0; k < 4; ++k) {
+        const uint32_t i = i0 + k * stride;
+        if (i >= total) continue;
+        int p = 0;
+        while (i >= parts.end[p]) ++p;
+        at[k] = parts.off[p] + (i - (p ? parts.end[p - 1] : 0u));
+        v[k] = __ldcv(src + at[k]);   // host memory that the next call rewrites
+      }
+#pragma unroll
+      for (int k = 0; k < 4; ++k)
+        if (i0 + k * stride < total) dst[at[k]] = v[k];
+    }
+    return;
   }
-  __syncthreads();
-  return *slot;
+  const int64_t stride = static_cast<int64_t>(gridDim.x - pull_ctas) * blockDim.x;
+  for (int64_t i = static_cast<int64_t>(blockIdx.x - pull_ctas) * blockDim.x + threadIdx.x; i < q_quads; i += stride)
+    store_hilo4(out, 4 * i, q[i]);
 }
 
-__global__ void rope_table_kernel(const int32_t* __restrict__ seq_lens, int hd, double base, int depth,
-                                  float2* __restrict__ tab, unsigned long long* ts) {
-  trace_begin(ts);
-  grid_dep_launch();
-  grid_dep_wait();
-  const int b = blockIdx.x, i = threadIdx.x;
-  if (i < hd / 2) {
-    // row b is verify token b % depth of its candidate: position L + b % depth
-    const double ang = static_cast<double>(seq_lens[b] + b % depth) * pow(base, -2.0 * i / hd);
-    tab[b * (hd / 2) + i] = make_float2(static_cast<float>(cos(ang)), static_cast<float>(sin(ang)));
-  }
-  trace_end(ts);
-}
-
-// One CTA per candidate: h = e_v, its per-tile sums of squares, and x.
-__global__ void embed_norm_kernel(const __nv_bfloat16* __restrict__ e_v, const __nv_bfloat16* __restrict__ gain,
-                                  int d, int n_cand, float* __restrict__ h, float* __restrict__ sumsq, HiLo x,
-                                  unsigned long long* ts) {
+// One CTA of 256 threads per row: its rotation (row b is verify token b % depth of its candidate, at
+// position L + b % depth), h = e_v with its per-tile sums of squares as the residual epilogue writes
+// them, and x.  Latency only; the rotation's fp64 sine and cosine are its longest chain, so the powers
+// base^(-2i/hd) come from a table laid down with the context.
+__global__ void __launch_bounds__(256) prologue_kernel(const int32_t* __restrict__ seq_lens,
+                                                       const double* __restrict__ inv_freq, int half, int depth,
+                                                       float2* __restrict__ rope, const __nv_bfloat16* __restrict__ e_v,
+                                                       const __nv_bfloat16* __restrict__ gain, int d, int n_rows,
+                                                       float* __restrict__ h, float* __restrict__ sumsq, HiLo x,
+                                                       unsigned long long* ts) {
   trace_begin(ts);
   grid_dep_launch();
   grid_dep_wait();
   const int b = blockIdx.x;
-  // per-tile sums of squares of h, as the residual GEMM epilogue writes them
-  const int m_tiles = (d + 127) / 128;
-  if (threadIdx.x < m_tiles) {
-    float t = 0.f;
-    for (int c = threadIdx.x * 128; c < min(d, threadIdx.x * 128 + 128); ++c) {
-      const float v = __bfloat162float(e_v[c]);
-      t += v * v;
-    }
-    sumsq[static_cast<int64_t>(threadIdx.x) * n_cand + b] = t;
+  const int64_t row = static_cast<int64_t>(b) * d;
+  for (int c = 4 * threadIdx.x; c < d; c += 4 * blockDim.x) {   // d % 64 == 0
+    const float4 v = load_bf16x4(e_v + c), g = load_bf16x4(gain + c);
+    *reinterpret_cast<float4*>(h + row + c) = v;
+    store_hilo4(x, row + c, make_float4(v.x * g.x, v.y * g.y, v.z * g.z, v.w * g.w));
   }
-  // h = e_v, and the QKV projection's input h ⊙ g before the RMSNorm's
-  // per-candidate factor, which its epilogue applies from the tile sums
-  for (int c = threadIdx.x; c < d; c += blockDim.x) {
-    const float v = __bfloat162float(e_v[c]);
-    h[static_cast<int64_t>(b) * d + c] = v;
-    store_hilo(x, static_cast<int64_t>(b) * d + c, v * __bfloat162float(gain[c]));
+  // the rotation on the first warps, the sums on the last ones first
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
+  if (static_cast<int>(threadIdx.x) < half) {
+    const double ang = static_cast<double>(seq_lens[b] + b % depth) * inv_freq[threadIdx.x];
+    double sn, cs;
+    sincos(ang, &sn, &cs);
+    rope[b * half + threadIdx.x] = make_float2(static_cast<float>(cs), static_cast<float>(sn));
+  }
+  const int m_tiles = (d + 127) / 128;
+  for (int t = nw - 1 - warp; t < m_tiles; t += nw) {
+    const int c = t * 128 + 4 * lane;
+    float s = 0.f;
+    if (c < d) {
+      const float4 v = load_bf16x4(e_v + c);
+      s = (v.x * v.x + v.y * v.y) + (v.z * v.z + v.w * v.w);
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) s += __shfl_xor_sync(0xffffffffu, s, off);
+    if (lane == 0) sumsq[static_cast<int64_t>(t) * n_rows + b] = s;
   }
   trace_end(ts);
 }
 
-// One CTA per candidate: the reward of its last row (its last verify token; one row per candidate
-// except in a depth-k readout).
-__global__ void head_kernel(const float* __restrict__ h, const float* __restrict__ sumsq, int m_tiles, int n_rows,
-                            int depth, int d, float eps, const __nv_bfloat16* __restrict__ gain,
-                            const __nv_bfloat16* __restrict__ w_plus, const __nv_bfloat16* __restrict__ w_minus,
-                            float* __restrict__ rewards, unsigned long long* ts) {
+// One CTA of 256 threads per candidate: the reward of its last row (its last verify token; one row per
+// candidate except in a depth-k readout), also stored at *out_slot when that is set (the caller's
+// buffer of an asynchronous call).  The RMSNorm factor is common to both logits, so the logits' sums
+// and the sum of the tiles' squares meet in one reduction.
+__global__ void __launch_bounds__(256) head_kernel(const float* __restrict__ h, const float* __restrict__ sumsq,
+                                                   int m_tiles, int n_rows, int depth, int d, float eps,
+                                                   const __nv_bfloat16* __restrict__ gain,
+                                                   const __nv_bfloat16* __restrict__ w_plus,
+                                                   const __nv_bfloat16* __restrict__ w_minus,
+                                                   float* __restrict__ rewards, float* const* out_slot,
+                                                   unsigned long long* ts) {
   trace_begin(ts);
-  __shared__ float red[32];
-  __shared__ float slot;
+  __shared__ float red[8][3];
   grid_dep_launch();
   grid_dep_wait();
   const int b = blockIdx.x, row = b * depth + depth - 1;
-  const float r = row_rscale(sumsq, m_tiles, n_rows, row, d, eps, &slot);
-  float zp = 0.f, zm = 0.f;
-  for (int c = threadIdx.x; c < d; c += blockDim.x) {
-    const float xf = h[static_cast<int64_t>(row) * d + c] * r * __bfloat162float(gain[c]);
-    zp += xf * __bfloat162float(w_plus[c]);
-    zm += xf * __bfloat162float(w_minus[c]);
+  float zp = 0.f, zm = 0.f, ss = 0.f;
+  for (int t = threadIdx.x; t < m_tiles; t += blockDim.x) ss += sumsq[static_cast<int64_t>(t) * n_rows + row];
+  for (int c = 4 * threadIdx.x; c < d; c += 4 * blockDim.x) {
+    const float4 hv = *reinterpret_cast<const float4*>(h + static_cast<int64_t>(row) * d + c);
+    const float4 g = load_bf16x4(gain + c), p = load_bf16x4(w_plus + c), m = load_bf16x4(w_minus + c);
+    const float4 x = make_float4(hv.x * g.x, hv.y * g.y, hv.z * g.z, hv.w * g.w);
+    zp += (x.x * p.x + x.y * p.y) + (x.z * p.z + x.w * p.w);
+    zm += (x.x * m.x + x.y * m.y) + (x.z * m.z + x.w * m.w);
   }
-  zp = block_sum(zp, red);
-  zm = block_sum(zm, red);
-  if (threadIdx.x == 0) rewards[b] = 1.0f / (1.0f + expf(zm - zp));
+#pragma unroll
+  for (int off = 16; off > 0; off >>= 1) {
+    zp += __shfl_xor_sync(0xffffffffu, zp, off);
+    zm += __shfl_xor_sync(0xffffffffu, zm, off);
+    ss += __shfl_xor_sync(0xffffffffu, ss, off);
+  }
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+  if (lane == 0) {
+    red[warp][0] = zp;
+    red[warp][1] = zm;
+    red[warp][2] = ss;
+  }
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    zp = zm = ss = 0.f;
+#pragma unroll
+    for (int w = 0; w < 8; ++w) {
+      zp += red[w][0];
+      zm += red[w][1];
+      ss += red[w][2];
+    }
+    const float r = 1.0f / sqrtf(ss / d + eps);
+    const float p = 1.0f / (1.0f + expf(zm * r - zp * r));
+    rewards[b] = p;
+    float* out = *out_slot;
+    if (out) out[b] = p;
+  }
   trace_end(ts);
 }
 
@@ -141,28 +208,35 @@ cudaLaunchConfig_t make_cfg(dim3 grid, dim3 block, cudaStream_t st, cudaLaunchAt
 
 }  // namespace
 
-cudaError_t launch_rope_table(const int32_t* seq_lens, int n_rows, int hd, double base, int depth, float2* table,
-                              cudaStream_t stream, bool pdl, unsigned long long* ts) {
-  cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = make_cfg(dim3(n_rows), dim3(64), stream, attr, pdl);
-  return cudaLaunchKernelEx(&cfg, rope_table_kernel, seq_lens, hd, base, depth, table, ts);
+cudaError_t launch_call_begin(const TableParts& parts, const int32_t* staging, int32_t* tables, const float* q,
+                              int64_t count, HiLo out, cudaStream_t stream) {
+  if (parts.n < 1 || parts.n > kMaxTableParts || (count & 3)) return cudaErrorInvalidValue;
+  // 64 CTAs hold the host link's bandwidth (as the cache copy does)
+  const int pull = static_cast<int>(std::min<uint32_t>(64, (parts.end[parts.n - 1] + 511) / 512));
+  const int64_t split = std::min<int64_t>(152 * 8, (count / 4 + 127) / 128);
+  call_begin_kernel<<<static_cast<unsigned>(pull + split), 128, 0, stream>>>(
+      parts, reinterpret_cast<const uint4*>(staging), reinterpret_cast<uint4*>(tables), pull,
+      reinterpret_cast<const float4*>(q), count / 4, out);
+  return cudaGetLastError();
 }
 
-cudaError_t launch_embed_norm(const ModelDims& m, const __nv_bfloat16* e_v, const __nv_bfloat16* gain, int n_cand,
-                              float* h, float* sumsq, HiLo x, cudaStream_t stream, bool pdl,
-                              unsigned long long* ts) {
+cudaError_t launch_prologue(const ModelDims& m, const int32_t* seq_lens, const double* inv_freq, int depth,
+                            float2* rope, const __nv_bfloat16* e_v, const __nv_bfloat16* gain, int n_rows, float* h,
+                            float* sumsq, HiLo x, cudaStream_t stream, bool pdl, unsigned long long* ts) {
   cudaLaunchAttribute attr[1];
-  cudaLaunchConfig_t cfg = make_cfg(dim3(n_cand), dim3(256), stream, attr, pdl);
-  return cudaLaunchKernelEx(&cfg, embed_norm_kernel, e_v, gain, m.d, n_cand, h, sumsq, x, ts);
+  cudaLaunchConfig_t cfg = make_cfg(dim3(n_rows), dim3(256), stream, attr, pdl);
+  return cudaLaunchKernelEx(&cfg, prologue_kernel, seq_lens, inv_freq, m.hd / 2, depth, rope, e_v, gain, m.d, n_rows,
+                            h, sumsq, x, ts);
 }
 
 cudaError_t launch_head(const ModelDims& m, const float* h, const float* sumsq, int m_tiles, int n_rows, int depth,
                         const __nv_bfloat16* gain, const __nv_bfloat16* w_plus, const __nv_bfloat16* w_minus,
-                        float* rewards, cudaStream_t stream, bool pdl, unsigned long long* ts) {
+                        float* rewards, float* const* out_slot, cudaStream_t stream, bool pdl,
+                        unsigned long long* ts) {
   cudaLaunchAttribute attr[1];
   cudaLaunchConfig_t cfg = make_cfg(dim3(n_rows / depth), dim3(256), stream, attr, pdl);
   return cudaLaunchKernelEx(&cfg, head_kernel, h, sumsq, m_tiles, n_rows, depth, m.d, m.eps, gain, w_plus, w_minus,
-                            rewards, ts);
+                            rewards, out_slot, ts);
 }
 
 __global__ void wait_probe_kernel(const int* flag, int* err, unsigned long long limit_ns) {

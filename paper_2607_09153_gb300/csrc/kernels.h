@@ -225,22 +225,35 @@ struct ModelDims {
   int d, n_q, n_kv, hd, ff, qkv_rows;
   float eps;
 };
-// rows b: verify token b % depth of candidate b / depth, at position seq_lens[b] + b % depth
-cudaError_t launch_rope_table(const int32_t* seq_lens, int n_rows, int hd, double base, int depth, float2* table,
-                              cudaStream_t stream, bool pdl, unsigned long long* ts = nullptr);
 // Activations handed to a projection are stored as a bf16 (hi, lo) pair.
 struct HiLo {
   __nv_bfloat16* hi;
   __nv_bfloat16* lo;
 };
-cudaError_t launch_embed_norm(const ModelDims& m, const __nv_bfloat16* e_v, const __nv_bfloat16* gain,
-                              int n_cand, float* h, float* sumsq, HiLo x, cudaStream_t stream, bool pdl,
-                              unsigned long long* ts = nullptr);
+// Parts of a call's tables to copy from the staging buffer to the same place in the device tables:
+// part p holds end[p] - end[p - 1] quads (16 bytes) from quad off[p] on.
+constexpr int kMaxTableParts = 12;
+struct TableParts {
+  int n = 0;
+  uint32_t off[kMaxTableParts];
+  uint32_t end[kMaxTableParts];
+};
+// staging: pinned host memory, 16-byte aligned like tables; count > 0: also q (count values, 16-byte
+// aligned, count % 4 == 0) as a bf16 pair
+cudaError_t launch_call_begin(const TableParts& parts, const int32_t* staging, int32_t* tables, const float* q,
+                              int64_t count, HiLo out, cudaStream_t stream);
+// rows b: verify token b % depth of candidate b / depth, at position seq_lens[b] + b % depth;
+// inv_freq[i] = base^(-2i/hd), i < hd / 2
+cudaError_t launch_prologue(const ModelDims& m, const int32_t* seq_lens, const double* inv_freq, int depth,
+                            float2* rope, const __nv_bfloat16* e_v, const __nv_bfloat16* gain, int n_rows, float* h,
+                            float* sumsq, HiLo x, cudaStream_t stream, bool pdl, unsigned long long* ts = nullptr);
 // rewards = P(+) from the final RMSNorm of h and the two head rows
-// rewards[b] from row b depth + depth - 1 (each candidate's last verify token)
+// rewards[b] from row b depth + depth - 1 (each candidate's last verify token), also to *out_slot (a
+// device word) when that is not null
 cudaError_t launch_head(const ModelDims& m, const float* h, const float* sumsq, int m_tiles, int n_rows, int depth,
                         const __nv_bfloat16* gain, const __nv_bfloat16* w_plus, const __nv_bfloat16* w_minus,
-                        float* rewards, cudaStream_t stream, bool pdl, unsigned long long* ts = nullptr);
+                        float* rewards, float* const* out_slot, cudaStream_t stream, bool pdl,
+                        unsigned long long* ts = nullptr);
 cudaError_t launch_split_hilo(const float* in, int64_t count, HiLo out, cudaStream_t stream);
 // ---------------------------------------------------------------- backward pass (KV Steering, grad.cu)
 constexpr int kMaxGroup = 16;   // query heads per kv head

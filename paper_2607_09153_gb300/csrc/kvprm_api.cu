@@ -133,11 +133,12 @@ struct kvprm_ctx {
   float *apart_o = nullptr, *apart_ml = nullptr;   // [slot_cap][group][hd], [slot_cap][group][2]
   size_t slot_cap = 0;
   float2* rope = nullptr;
+  double* inv_freq = nullptr;   // [hd / 2] rope_base^(-2i/hd)
   int32_t* tables_d = nullptr;   // [Bmax] seq_lens, [Bmax][max_blocks] block table, then the attention work
   // attention work list: host plan of the current call and fixed offsets (ints) in tables_d / staging
   kvprm::AttnWorkHost work_host;
   size_t off_segs = 0, off_cta = 0, off_pages = 0, off_cands = 0, off_slots = 0, off_base = 0, off_nslots = 0,
-         off_tc_cta = 0;
+         off_tc_cta = 0, off_out = 0;
   size_t tables_ints = 0;
   size_t cap_segs = 0, cap_pages = 0, cap_cands = 0;
   int share_mode = 3;   // sharing of pages referenced by several candidates (build_attn_work)
@@ -299,6 +300,7 @@ void free_ctx(kvprm_ctx* c) {
   cudaFree(c->apart_o);
   cudaFree(c->apart_ml);
   cudaFree(c->rope);
+  cudaFree(c->inv_freq);
   cudaFree(c->tables_d);
   cudaFree(c->rewards_d);
   cudaFree(c->err_d);
@@ -347,6 +349,20 @@ void free_ctx(kvprm_ctx* c) {
   if (c->pool_free) cudaEventDestroy(c->pool_free);
 
   delete c;
+}
+
+// Whether all of [p, p + bytes) is memory of the context's device (first and last byte checked), 4-byte aligned.
+bool on_device(const kvprm_ctx* ctx, const void* p, size_t bytes) {
+  if (reinterpret_cast<uintptr_t>(p) & 3u) return false;
+  for (const uint8_t* q : {static_cast<const uint8_t*>(p), static_cast<const uint8_t*>(p) + bytes - 1}) {
+    cudaPointerAttributes a{};
+    if (cudaPointerGetAttributes(&a, q) != cudaSuccess) {
+      cudaGetLastError();
+      return false;
+    }
+    if (a.type != cudaMemoryTypeDevice || a.device != ctx->device) return false;
+  }
+  return true;
 }
 
 // ---------------------------------------------------------------- per-call checks and plan
@@ -398,8 +414,11 @@ int plan_work(kvprm_ctx* ctx, const int32_t* bt, const int32_t* sl, int32_t n, b
   return KVPRM_OK;
 }
 
-// Copy the tables and the planned work into pinned staging and then to the device.
-int upload_tables(kvprm_ctx* ctx, const int32_t* bt, const int32_t* sl, int32_t n, cudaStream_t st) {
+// Put the tables, the planned work and the address of the caller's reward buffer (or null) into the
+// pinned staging buffer and enqueue the kernel that pulls them to the device; q_count > 0: that launch
+// also splits the caller's query into ctx->qhi / qlo.
+int upload_tables(kvprm_ctx* ctx, const int32_t* bt, const int32_t* sl, int32_t n, cudaStream_t st,
+                  float* rewards_out = nullptr, const float* q = nullptr, int64_t q_count = 0) {
   const int Bmax = ctx->cfg.max_candidates, mb = ctx->cfg.max_blocks_per_seq;
   if (ctx->staging_pending) {
     CK(cudaEventSynchronize(ctx->staging_ev), "cudaEventSynchronize(staging)");
@@ -415,6 +434,7 @@ int upload_tables(kvprm_ctx* ctx, const int32_t* bt, const int32_t* sl, int32_t 
     const void* src;
     size_t ints;
   } parts[] = {
+      {0, nullptr, static_cast<size_t>(Bmax) + static_cast<size_t>(n) * mb},   // already in place
       {ctx->off_segs, w.segs.data(), w.segs.size() * kSegInts},
       {ctx->off_cta, w.cta_seg.data(), w.cta_seg.size()},
       {ctx->off_pages, w.pages.data(), w.pages.size()},
@@ -423,15 +443,19 @@ int upload_tables(kvprm_ctx* ctx, const int32_t* bt, const int32_t* sl, int32_t 
       {ctx->off_base, w.slot_base.data(), w.slot_base.size()},
       {ctx->off_nslots, w.nslots.data(), w.nslots.size()},
       {ctx->off_tc_cta, w.tc_cta.data(), w.tc_cta.size()},
+      {ctx->off_out, &rewards_out, sizeof(rewards_out) / sizeof(int32_t)},
   };
-  for (const Part& p : parts)
-    if (p.ints) std::memcpy(S + p.off, p.src, sizeof(int32_t) * p.ints);
-  auto up = [&](size_t off, size_t ints) -> cudaError_t {
-    if (ints == 0) return cudaSuccess;
-    return cudaMemcpyAsync(ctx->tables_d + off, S + off, ints * sizeof(int32_t), cudaMemcpyHostToDevice, st);
-  };
-  CK(up(0, static_cast<size_t>(Bmax) + static_cast<size_t>(n) * mb), "cudaMemcpyAsync(tables)");
-  for (const Part& p : parts) CK(up(p.off, p.ints), "cudaMemcpyAsync(attention work)");
+  // every part starts at a multiple of eight ints, so a part rounded up to whole quads ends before the next
+  kvprm::TableParts tp;
+  uint32_t quads = 0;
+  for (const Part& p : parts) {
+    if (!p.ints) continue;
+    if (p.src) std::memcpy(S + p.off, p.src, sizeof(int32_t) * p.ints);
+    quads += static_cast<uint32_t>((p.ints + 3) / 4);
+    tp.off[tp.n] = static_cast<uint32_t>(p.off / 4);
+    tp.end[tp.n++] = quads;
+  }
+  CK(kvprm::launch_call_begin(tp, S, ctx->tables_d, q, q_count, kvprm::HiLo{ctx->qhi, ctx->qlo}, st), "call_begin");
   CK(cudaEventRecord(ctx->staging_ev, st), "cudaEventRecord(staging)");
   ctx->staging_pending = true;
   return KVPRM_OK;
@@ -695,10 +719,9 @@ int enqueue_forward(kvprm_ctx* ctx, const CallPlan& P, Enq& E, const FwdSaves* s
     CK(cudaMemsetAsync(ctx->trace_d, 0xFF, sizeof(unsigned long long) * kvprm::kTraceStride * ctx->trace_cap, st),
        "trace reset");
   LAUNCH(KVPRM_PROF_FUSED,
-         kvprm::launch_rope_table(sl, n, m.hd, ctx->cfg.rope_base, ctx->depth, ctx->rope, st, false, TS), "rope");
-  LAUNCH(KVPRM_PROF_FUSED,
-         kvprm::launch_embed_norm(m, ctx->embed, ctx->attn_norm[0], n, ctx->h, ctx->sumsq, X, st, pdl, TS),
-         "embed_norm");
+         kvprm::launch_prologue(m, sl, ctx->inv_freq, ctx->depth, ctx->rope, ctx->embed, ctx->attn_norm[0], n, ctx->h,
+                                ctx->sumsq, X, st, false, TS),
+         "prologue");
   for (int l = 0; l < NL; ++l) {
     kvprm::GemmLowRank lr_qkv, lr_o, lr_gu, lr_down;
     int arc;
@@ -770,7 +793,8 @@ int enqueue_forward(kvprm_ctx* ctx, const CallPlan& P, Enq& E, const FwdSaves* s
     if (l + 1 == NL) {
       LAUNCH(KVPRM_PROF_FUSED,
              kvprm::launch_head(m, ctx->h, ctx->sumsq, ctx->d_tiles, n, ctx->depth, ctx->final_norm, ctx->w_plus,
-                                ctx->w_minus, ctx->rewards_d, st, pdl, TS),
+                                ctx->w_minus, ctx->rewards_d,
+                                reinterpret_cast<float* const*>(ctx->tables_d + ctx->off_out), st, pdl, TS),
              "reward_head");
     }
     if (ctx->debug_flags & 4) {
@@ -898,11 +922,13 @@ int enqueue_pool_copy(kvprm_ctx* ctx, cudaStream_t st) {
   return KVPRM_OK;
 }
 
-// Score into ctx->rewards_d on stream `st` (stream-ordered).  With `prepared` set, the call is
+// Score into ctx->rewards_d, and into device buffer rewards_out when that is set, on stream `st`
+// (stream-ordered).  With `prepared` set, the call is
 // planned and its tables uploaded (stream-ordered on `st`), and its plan returned there instead of
 // enqueueing the forward (the gradient call enqueues the forward together with the backward).
 int score_device(kvprm_ctx* ctx, const void* kv_pages, int64_t n_pages, const int32_t* bt, const int32_t* sl, int32_t n,
-                 cudaStream_t st, const FwdSaves* sv = nullptr, CallPlan* prepared = nullptr) {
+                 cudaStream_t st, const FwdSaves* sv = nullptr, CallPlan* prepared = nullptr,
+                 float* rewards_out = nullptr) {
   int max_pages = 0;
   int rc = validate_tables(ctx, n_pages, bt, sl, n, &max_pages);
   if (rc) return rc;
@@ -943,7 +969,7 @@ int score_device(kvprm_ctx* ctx, const void* kv_pages, int64_t n_pages, const in
   const CallPlan P = make_plan(ctx, n, max_pages);
   if ((rc = ensure_x_maps(ctx, P.n_pad))) return rc;
   if ((rc = ensure_t_maps(ctx, P.n_pad))) return rc;
-  if ((rc = upload_tables(ctx, bt, sl, n, st))) return rc;
+  if ((rc = upload_tables(ctx, bt, sl, n, st, rewards_out))) return rc;
   if (ctx->layer_waits && (rc = enqueue_pool_copy(ctx, st))) return rc;
   ctx->last_n = n;
   ctx->last_stream = st;
@@ -1435,6 +1461,13 @@ int kvprm_create(const kvprm_config* cfg, const kvprm_weights* w, kvprm_ctx** ou
   CREATE_CK(dalloc(ctx, &ctx->apart_ml, ctx->slot_cap * group * 2, "attn stats"));
   CREATE_CK(dalloc(ctx, &ctx->rope, static_cast<size_t>(Bmax) * (m.hd / 2), "rope table"));
   {
+    double f[64];
+    for (int i = 0; i < m.hd / 2; ++i) f[i] = std::pow(static_cast<double>(c.rope_base), -2.0 * i / m.hd);
+    CREATE_CK(dalloc(ctx, &ctx->inv_freq, static_cast<size_t>(m.hd / 2), "rotary frequencies"));
+    CREATE_CK(cu(cudaMemcpy(ctx->inv_freq, f, sizeof(double) * (m.hd / 2), cudaMemcpyHostToDevice),
+                 "cudaMemcpy(rotary frequencies)"));
+  }
+  {
     const size_t tbl = static_cast<size_t>(Bmax) * (1 + c.max_blocks_per_seq);
     auto al8 = [](size_t x) { return (x + 7) & ~static_cast<size_t>(7); };
     // private runs need at most Bmax * n_kv + n_ctas segments, Bmax * max_blocks
@@ -1451,7 +1484,8 @@ int kvprm_create(const kvprm_config* cfg, const kvprm_weights* w, kvprm_ctx** ou
     ctx->off_base = al8(ctx->off_slots + ctx->slot_cap);
     ctx->off_nslots = al8(ctx->off_base + bkv);
     ctx->off_tc_cta = al8(ctx->off_nslots + bkv);
-    ctx->tables_ints = al8(ctx->off_tc_cta + ctx->num_sms + 1);
+    ctx->off_out = al8(ctx->off_tc_cta + ctx->num_sms + 1);
+    ctx->tables_ints = al8(ctx->off_out + 2);
   }
   CREATE_CK(dalloc(ctx, &ctx->tables_d, ctx->tables_ints, "tables and attention work"));
   CREATE_CK(dalloc(ctx, &ctx->rewards_d, static_cast<size_t>(Bmax), "rewards"));
@@ -1592,8 +1626,11 @@ int kvprm_score_async(kvprm_ctx* ctx, const void* kv_pages, int64_t n_pages, con
   if (!ctx) return KVPRM_EINVAL;
   if (n > 0 && !d_rewards) return fail(ctx, KVPRM_EINVAL, "d_rewards is NULL");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
-  int rc = score_device(ctx, kv_pages, n_pages, block_table, seq_lens, n, st);
-  if (rc || n == 0) return rc;
+  // memory of this device takes the rewards from the head kernel itself, anything else by a copy
+  const bool direct = n > 0 && on_device(ctx, d_rewards, sizeof(float) * static_cast<size_t>(n));
+  int rc = score_device(ctx, kv_pages, n_pages, block_table, seq_lens, n, st, nullptr, nullptr,
+                        direct ? d_rewards : nullptr);
+  if (rc || n == 0 || direct) return rc;
   CK(cudaMemcpyAsync(d_rewards, ctx->rewards_d, sizeof(float) * n, cudaMemcpyDeviceToDevice, st),
      "cudaMemcpyAsync(d_rewards)");
   return KVPRM_OK;
@@ -1677,21 +1714,25 @@ int kvprm_attention(kvprm_ctx* ctx, const void* kv_layer, int64_t n_pages, const
   }
   if ((rc = ensure_pool_map(ctx, pool, pages, 1))) return rc;
   if ((rc = plan_work(ctx, block_table, seq_lens, n, true))) return rc;
-  if ((rc = upload_tables(ctx, block_table, seq_lens, n, st))) return rc;
+  Enq E{ctx, st, false, ctx->profile, &ctx->live_marks};
+  {
+    cudaEvent_t evb = nullptr;
+    if ((rc = E.begin(KVPRM_PROF_FUSED, &evb))) return rc;
+    if ((rc = upload_tables(ctx, block_table, seq_lens, n, st, nullptr, static_cast<const float*>(q),
+                            static_cast<int64_t>(n) * ctx->md.n_q * ctx->md.hd)))
+      return rc;
+    if ((rc = E.end(evb))) return rc;
+  }
   AttnShape as = ctx->as;
   as.layer_pages = pages;
-  Enq E{ctx, st, false, ctx->profile, &ctx->live_marks};
-  LAUNCH(KVPRM_PROF_FUSED,
-         kvprm::launch_split_hilo(static_cast<const float*>(q), static_cast<int64_t>(n) * ctx->md.n_q * ctx->md.hd, Q,
-                                  st),
-         "split_hilo");
   const kvprm::AttnMerge mg{static_cast<const float*>(q), static_cast<const float*>(k_self),
                             static_cast<const float*>(v_self), ctx->ohi, ctx->olo, out, nullptr};
   const kvprm::AttnWork wk = device_work(ctx);
   if ((rc = enqueue_attention(ctx, E, as, wk, 0, Q, mg, false))) return rc;
   if (wk.fuse_cs == 0)
     LAUNCH(KVPRM_PROF_COMBINE,
-           kvprm::launch_attn_combine(as, wk, n, ctx->apart_o, ctx->apart_ml, mg, st, false, TS,
+           kvprm::launch_attn_combine(as, wk, n, ctx->apart_o, ctx->apart_ml, mg, st,
+                                      ctx->use_pdl && !ctx->profile && !ctx->work_host.tc_concurrent, TS,
                                       (ctx->debug_flags & 64) != 0),
            "attn_combine");
   ctx->last_n = n;

@@ -87,10 +87,10 @@ def lib() -> ctypes.CDLL:
         L.kvprm_destroy.restype = None
         L.kvprm_last_error.argtypes = [vp]
         L.kvprm_last_error.restype = ctypes.c_char_p
-        L.kvprm_score.argtypes = [vp, vp, i64, i32p, i32p, i32, f32p, vp]
-        L.kvprm_score_async.argtypes = [vp, vp, i64, i32p, i32p, i32, vp, vp]
-        L.kvprm_score_host.argtypes = [vp, vp, i64, i32p, i32p, i32, f32p, vp]
-        L.kvprm_attention.argtypes = [vp, vp, i64, i32p, i32p, i32, vp, vp, vp, vp, vp]
+        L.kvprm_score.argtypes = [vp, vp, i64, vp, vp, i32, f32p, vp]
+        L.kvprm_score_async.argtypes = [vp, vp, i64, vp, vp, i32, vp, vp]
+        L.kvprm_score_host.argtypes = [vp, vp, i64, vp, vp, i32, f32p, vp]
+        L.kvprm_attention.argtypes = [vp, vp, i64, vp, vp, i32, vp, vp, vp, vp, vp]
         L.kvprm_projection.argtypes = [vp, vp, i32, i32, vp, i32, vp, vp]
         L.kvprm_set_lora.argtypes = [vp, i32, ctypes.c_float, ctypes.POINTER(KvprmLora)]
         L.kvprm_set_readout_depth.argtypes = [vp, i32]
@@ -103,8 +103,8 @@ def lib() -> ctypes.CDLL:
         L.kvprm_resolve.argtypes = [vp, i32, i64p]
         L.kvprm_check_device.argtypes = [vp]
         L.kvprm_debug_set_alloc_limit.argtypes = [i64]
-        L.kvprm_score_grad.argtypes = [vp, vp, i64, i32p, i32p, i32, vp, f32p, vp]
-        L.kvprm_steer.argtypes = [vp, vp, i64, i32p, i32p, i32, ctypes.c_float, i32, f32p, f32p, vp]
+        L.kvprm_score_grad.argtypes = [vp, vp, i64, vp, vp, i32, vp, f32p, vp]
+        L.kvprm_steer.argtypes = [vp, vp, i64, vp, vp, i32, ctypes.c_float, i32, f32p, f32p, vp]
         L.kvprm_debug_inject_error.argtypes = [vp, i32]
         L.kvprm_debug_wait_probe.argtypes = [vp, i32, vp]
         L.kvprm_set_profile.argtypes = [vp, ctypes.c_int]
@@ -132,6 +132,11 @@ def _i32(a) -> np.ndarray:
     return np.ascontiguousarray(a, dtype=np.int32)
 
 
+def _a(a: np.ndarray) -> int:
+    """Address of an array, for the tables of a call (a typed ctypes pointer takes three times as long)."""
+    return a.ctypes.data
+
+
 def _p(a: np.ndarray, t):
     return a.ctypes.data_as(ctypes.POINTER(t))
 
@@ -152,7 +157,7 @@ def kvprm_destroy(ctx) -> None:
 def kvprm_score(ctx, kv_pages_ptr: int, n_pages: int, block_table, seq_lens, n: int, stream_ptr: int = 0) -> np.ndarray:
     bt, sl = _i32(block_table), _i32(seq_lens)
     out = np.zeros(n, np.float32)
-    _check(ctx, lib().kvprm_score(ctx, kv_pages_ptr, n_pages, _p(bt, ctypes.c_int32), _p(sl, ctypes.c_int32), n,
+    _check(ctx, lib().kvprm_score(ctx, kv_pages_ptr, n_pages, _a(bt), _a(sl), n,
                                   _p(out, ctypes.c_float), stream_ptr))
     return out
 
@@ -160,7 +165,7 @@ def kvprm_score(ctx, kv_pages_ptr: int, n_pages: int, block_table, seq_lens, n: 
 def kvprm_score_async(ctx, kv_pages_ptr: int, n_pages: int, block_table, seq_lens, n: int, d_rewards_ptr: int,
                       stream_ptr: int = 0) -> None:
     bt, sl = _i32(block_table), _i32(seq_lens)
-    _check(ctx, lib().kvprm_score_async(ctx, kv_pages_ptr, n_pages, _p(bt, ctypes.c_int32), _p(sl, ctypes.c_int32),
+    _check(ctx, lib().kvprm_score_async(ctx, kv_pages_ptr, n_pages, _a(bt), _a(sl),
                                         n, d_rewards_ptr, stream_ptr))
 
 
@@ -169,7 +174,7 @@ def kvprm_score_host(ctx, h_kv_pages_ptr: int, n_pages: int, block_table, seq_le
     bt, sl = _i32(block_table), _i32(seq_lens)
     if out is None:
         out = np.zeros(n, np.float32)
-    _check(ctx, lib().kvprm_score_host(ctx, h_kv_pages_ptr, n_pages, _p(bt, ctypes.c_int32), _p(sl, ctypes.c_int32),
+    _check(ctx, lib().kvprm_score_host(ctx, h_kv_pages_ptr, n_pages, _a(bt), _a(sl),
                                        n, _p(out, ctypes.c_float), stream_ptr))
     return out
 
@@ -180,7 +185,7 @@ def kvprm_score_grad(ctx, kv_pages_ptr: int, n_pages: int, block_table, seq_lens
     (the pool's layout); returns P(+) [n]."""
     bt, sl = _i32(block_table), _i32(seq_lens)
     out = np.zeros(n, np.float32)
-    _check(ctx, lib().kvprm_score_grad(ctx, kv_pages_ptr, n_pages, _p(bt, ctypes.c_int32), _p(sl, ctypes.c_int32), n,
+    _check(ctx, lib().kvprm_score_grad(ctx, kv_pages_ptr, n_pages, _a(bt), _a(sl), n,
                                        d_grad_ptr, _p(out, ctypes.c_float), stream_ptr))
     return out
 
@@ -191,7 +196,7 @@ def kvprm_steer(ctx, kv_pages_ptr: int, n_pages: int, block_table, seq_lens, n: 
     bt, sl = _i32(block_table), _i32(seq_lens)
     p0 = np.zeros(n, np.float32)
     p1 = np.zeros(n, np.float32)
-    _check(ctx, lib().kvprm_steer(ctx, kv_pages_ptr, n_pages, _p(bt, ctypes.c_int32), _p(sl, ctypes.c_int32), n,
+    _check(ctx, lib().kvprm_steer(ctx, kv_pages_ptr, n_pages, _a(bt), _a(sl), n,
                                   float(eta), int(steps), _p(p0, ctypes.c_float), _p(p1, ctypes.c_float), stream_ptr))
     return p0, p1
 
@@ -199,7 +204,7 @@ def kvprm_steer(ctx, kv_pages_ptr: int, n_pages: int, block_table, seq_lens, n: 
 def kvprm_attention(ctx, kv_layer_ptr: int, n_pages: int, block_table, seq_lens, n: int, q_ptr: int, k_self_ptr: int,
                     v_self_ptr: int, out_ptr: int, stream_ptr: int = 0) -> None:
     bt, sl = _i32(block_table), _i32(seq_lens)
-    _check(ctx, lib().kvprm_attention(ctx, kv_layer_ptr, n_pages, _p(bt, ctypes.c_int32), _p(sl, ctypes.c_int32), n,
+    _check(ctx, lib().kvprm_attention(ctx, kv_layer_ptr, n_pages, _a(bt), _a(sl), n,
                                       q_ptr, k_self_ptr, v_self_ptr, out_ptr, stream_ptr))
 
 

@@ -1,0 +1,38 @@
+"""The call's tables on their way to the device (one kernel reading pinned host memory) and the
+rewards on their way out: odd table sizes (parts that end inside a 16-byte quad, empty parts, more
+than one launch round of quads), two calls in flight that share the staging buffer, and the
+caller's device buffer written by the head kernel instead of a copy."""
+import numpy as np
+import pytest
+
+import kvsynth as ks
+from tests.gpu_util import make_scorer, require_gpu
+
+pytestmark = pytest.mark.gpu
+
+
+@pytest.mark.parametrize("lens", [[0], [1], [16, 17, 0], [5, 300, 31, 64, 129], [40] * 33,
+                                  list(range(1, 4097, 97))])
+def test_tables_and_rewards(lens):
+    torch = require_gpu()
+    import paper_2607_09153_gb300 as kp
+    w = ks.distinct("setup", ks.ARCH_TINY, 60 + len(lens), lens)
+    dev = ks.DeviceInputs(w, ks.Tables.make())
+    n = len(lens)
+    sc = make_scorer(dev, n + 3, w.max_blocks)
+    bt, sl = np.asarray(w.block_table), np.asarray(w.seq_lens)
+    want = [sc.score(dev.pool, bt, sl), sc.score(dev.pool, bt[::-1], sl[::-1])]
+    # both orders in flight at once, each into its own buffer (at an address that is no multiple of 16)
+    out = [torch.full((n + 1,), -1.0, dtype=torch.float32, device="cuda")[1:] for _ in range(2)]
+    for _ in range(3):
+        sc.score_async(dev.pool, bt, sl, out[0])
+        sc.score_async(dev.pool, np.ascontiguousarray(bt[::-1]), np.ascontiguousarray(sl[::-1]), out[1])
+    torch.cuda.synchronize()
+    for o, r in zip(out, want):
+        assert np.array_equal(o.cpu().numpy(), r)
+    assert np.allclose(want[0], want[1][::-1], rtol=0, atol=1e-6)
+    for i in range(n):   # the last call's tables on the device: reversed order
+        b = n - 1 - i
+        j = np.arange(sl[b])
+        assert np.array_equal(kp.kvprm_resolve(sc.ctx, i, int(sl[b])), bt[b, j // 16].astype(np.int64) * 16 + j % 16)
+    sc.close()
