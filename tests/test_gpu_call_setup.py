@@ -6,7 +6,7 @@ import numpy as np
 import pytest
 
 import kvsynth as ks
-from tests.gpu_util import make_scorer, require_gpu
+from tests.gpu_util import P_PLUS_ATOL, make_scorer, require_gpu
 
 pytestmark = pytest.mark.gpu
 
@@ -30,7 +30,8 @@ def test_tables_and_rewards(lens):
     torch.cuda.synchronize()
     for o, r in zip(out, want):
         assert np.array_equal(o.cpu().numpy(), r)
-    assert np.allclose(want[0], want[1][::-1], rtol=0, atol=1e-6)
+    # the two orders are scheduled differently: the same up to fp32 rounding order
+    assert np.abs(want[0] - want[1][::-1]).max() <= P_PLUS_ATOL
     for i in range(n):   # the last call's tables on the device: reversed order
         b = n - 1 - i
         j = np.arange(sl[b])
