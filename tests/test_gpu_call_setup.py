@@ -37,3 +37,29 @@ def test_tables_and_rewards(lens):
         j = np.arange(sl[b])
         assert np.array_equal(kp.kvprm_resolve(sc.ctx, i, int(sl[b])), bt[b, j // 16].astype(np.int64) * 16 + j % 16)
     sc.close()
+
+
+@pytest.mark.parametrize("shift", [1, 2, 3, 4])
+def test_vectors_at_any_address(shift):
+    # embedding, gains and head rows that start anywhere (2-byte aligned views) score as aligned ones do
+    torch = require_gpu()
+    w = ks.distinct("shift", ks.ARCH_TINY, 90, [33, 128, 5])
+    t = ks.Tables.make(0.2)
+    dev = ks.DeviceInputs(w, t)
+    sc = make_scorer(dev, 3, w.max_blocks)
+    want = sc.score(dev.pool, w.block_table, w.seq_lens)
+    sc.close()
+
+    def moved(v):
+        buf = torch.zeros(v.numel() + 8, dtype=v.dtype, device="cuda")
+        buf[shift:shift + v.numel()] = v.reshape(-1)
+        return buf[shift:shift + v.numel()]
+
+    for k in (ks.EMBED, ks.FINAL_NORM, ks.W_PLUS, ks.W_MINUS):
+        dev.top[k] = moved(dev.top[k])
+    for layer in dev.layers:
+        for k in (ks.ATTN_NORM, ks.MLP_NORM):
+            layer[k] = moved(layer[k])
+    sc = make_scorer(dev, 3, w.max_blocks)
+    assert np.array_equal(sc.score(dev.pool, w.block_table, w.seq_lens), want)
+    sc.close()
