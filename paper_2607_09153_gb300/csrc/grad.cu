@@ -7,7 +7,8 @@
 //   rms_back        dh = dres + r g dy - h r^3 (sum_i g_i dy_i h_i) / d,  r = (mean h^2 + eps)^-1/2
 //   silu_back       du = da t SiLU'(u),  dt = da SiLU(u)
 //   attn_back_pre   per (candidate, kv head): D_h = do_h . o_h and the self entry's terms
-//   attn_back_pages per run of cached pages: w_j = exp(q.K_j / sqrt(hd) - lse), ds_j = w_j (do.V_j - D),
+//   attn_back_tc / attn_back_pages (G > 8)  per cached token:
+//                   w_j = exp(q.K_j / sqrt(hd) - lse), ds_j = w_j (do.V_j - D),
 //                   dK_j = sum_h ds_j q_h / sqrt(hd), dV_j = sum_h w_j do_h, dq_h += ds_j K_j / sqrt(hd)
 //   rope_back       the rotation by the negative angle, and [dq; dk; dv] as the next GEMM's input
 //   zero_pages      clears the gradient of pages several candidates read (they are accumulated)
@@ -16,6 +17,10 @@
 // (hi, lo) pair like the forward's activations.
 #include <cuda_bf16.h>
 
+#include <algorithm>
+#include <functional>
+#include <map>
+#include <queue>
 #include <utility>
 
 #include "kernels.h"
@@ -26,6 +31,7 @@ namespace kvprm {
 namespace {
 
 typedef __nv_bfloat16 bf16;
+constexpr float kLog2eBack = 1.4426950408889634f;
 
 __device__ __forceinline__ void put_hilo(bf16* hi, bf16* lo, int64_t i, float x) {
   const bf16 h = __float2bfloat16_rn(x);
@@ -142,11 +148,14 @@ __global__ void silu_back_kernel(const float* __restrict__ da, const float* __re
 // One CTA of 128 threads per (row b, kv head g): D_h = do_h . o_h for the G query heads, and the
 // verify token's own entry: w_s = exp(q_h . k_s / sqrt(hd) - lse_h), ds_s = w_s (do_h . v_s - D_h),
 // dk_s = sum_h ds_s q_h / sqrt(hd), dv_s = sum_h w_s do_h, dq_h = ds_s k_s / sqrt(hd) (the pages add on).
-__global__ void attn_back_pre_kernel(const float* __restrict__ q, const float* __restrict__ ks,
-                                     const float* __restrict__ vs, const float* __restrict__ o,
-                                     const float* __restrict__ dout, const float* __restrict__ lse, int n_q, int n_kv,
-                                     int hd, float* __restrict__ D, float* __restrict__ dq, float* __restrict__ dks,
-                                     float* __restrict__ dvs) {
+// With ops set (G <= 8) also the tensor-core backward's operands of this (b, g): q, then dO, each as a
+// hi and a lo block of 8 rows (heads past G: zeros) in the 128-byte swizzle, [q, dO][hi, lo]
+// [HD / 64][8 rows][128 B], and meta [8] = (lse, D) (heads past G: lse = inf, so that their weight is 0).
+__global__ void __launch_bounds__(128) attn_back_pre_kernel(
+    const float* __restrict__ q, const float* __restrict__ ks, const float* __restrict__ vs, const float* __restrict__ o,
+    const float* __restrict__ dout, const float* __restrict__ lse, int n_q, int n_kv, int hd, float* __restrict__ D,
+    float* __restrict__ dq, float* __restrict__ dks, float* __restrict__ dvs, uint8_t* __restrict__ ops,
+    float2* __restrict__ meta) {
   __shared__ float s_w[kMaxGroup], s_ds[kMaxGroup];
   grid_dep_launch();
   grid_dep_wait();
@@ -154,8 +163,9 @@ __global__ void attn_back_pre_kernel(const float* __restrict__ q, const float* _
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const float scale = rsqrtf(static_cast<float>(hd));
   const int64_t hk = (static_cast<int64_t>(b) * n_kv + g) * hd;
+  const int64_t row0 = static_cast<int64_t>(b) * n_q + static_cast<int64_t>(g) * G;
   for (int r = warp; r < G; r += blockDim.x >> 5) {
-    const int64_t hq = (static_cast<int64_t>(b) * n_q + g * G + r) * hd;
+    const int64_t hq = (row0 + r) * hd;
     float dd = 0.f, sq = 0.f, dp = 0.f;
     for (int e = lane; e < hd; e += 32) {
       dd += dout[hq + e] * o[hq + e];
@@ -169,18 +179,46 @@ __global__ void attn_back_pre_kernel(const float* __restrict__ q, const float* _
       dp += __shfl_xor_sync(0xffffffffu, dp, off);
     }
     if (lane == 0) {
-      const int64_t row = static_cast<int64_t>(b) * n_q + g * G + r;
-      const float w = expf(sq * scale - lse[row]);
-      D[row] = dd;
+      const float ls = lse[row0 + r];
+      const float w = expf(sq * scale - ls);
+      D[row0 + r] = dd;
       s_w[r] = w;
       s_ds[r] = w * (dp - dd);
+      if (ops) meta[static_cast<int64_t>(blockIdx.x) * 8 + r] = make_float2(ls, dd);
+    }
+  }
+  if (ops) {
+    if (static_cast<int>(threadIdx.x) >= G && threadIdx.x < 8)
+      meta[static_cast<int64_t>(blockIdx.x) * 8 + threadIdx.x] = make_float2(INFINITY, 0.f);
+    // 8 consecutive elements (one 16-byte chunk of the hi and of the lo row) per step
+    const int per_row = hd / 8, block = (hd / 64) * 1024;
+    uint8_t* dst = ops + static_cast<int64_t>(blockIdx.x) * 4 * block;
+    for (int i = threadIdx.x; i < 2 * 8 * per_row; i += blockDim.x) {
+      const int which = i / (8 * per_row), r = (i / per_row) & 7, c = i % per_row;
+      uint32_t hi[4] = {0u, 0u, 0u, 0u}, lo[4] = {0u, 0u, 0u, 0u};
+      if (r < G) {
+        const float4* src = reinterpret_cast<const float4*>((which ? dout : q) + (row0 + r) * hd + c * 8);
+        const float4 x0 = src[0], x1 = src[1];
+        const float x[8] = {x0.x, x0.y, x0.z, x0.w, x1.x, x1.y, x1.z, x1.w};
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+          const __nv_bfloat162 h2 = __floats2bfloat162_rn(x[2 * e], x[2 * e + 1]);
+          const float2 hf = __bfloat1622float2(h2);
+          const __nv_bfloat162 l2 = __floats2bfloat162_rn(x[2 * e] - hf.x, x[2 * e + 1] - hf.y);
+          hi[e] = *reinterpret_cast<const uint32_t*>(&h2);
+          lo[e] = *reinterpret_cast<const uint32_t*>(&l2);
+        }
+      }
+      uint8_t* at = dst + which * 2 * block + (c >> 3) * 1024 + r * 128 + (((c & 7) ^ r) << 4);
+      *reinterpret_cast<uint4*>(at) = make_uint4(hi[0], hi[1], hi[2], hi[3]);
+      *reinterpret_cast<uint4*>(at + block) = make_uint4(lo[0], lo[1], lo[2], lo[3]);
     }
   }
   __syncthreads();
   for (int e = threadIdx.x; e < hd; e += blockDim.x) {
     float ak = 0.f, av = 0.f;
     for (int r = 0; r < G; ++r) {
-      const int64_t hq = (static_cast<int64_t>(b) * n_q + g * G + r) * hd;
+      const int64_t hq = (row0 + r) * hd;
       ak += s_ds[r] * q[hq + e];
       av += s_w[r] * dout[hq + e];
       dq[hq + e] = s_ds[r] * ks[hk + e] * scale;
@@ -372,254 +410,463 @@ __global__ void __launch_bounds__(128) attn_back_pages_kernel(
 }
 
 // ---------------------------------------------------------------- attention backward on the tensor cores
-// The same unit of work (candidate b, kv head g, up to kBackUnitPages pages) for G <= 8 query heads
-// per kv head.  Thread 0 loads the unit's pages with the forward's tensor map (one 128-byte-swizzled
-// box per page: K then V), so each page's keys and values are addressed exactly as in the forward.
-// Each warp takes pages w, w + 4 and per page of 16 tokens computes, with mma.m16n8k16 (bf16 in,
-// fp32 accumulate) -- every fp32 operand entering as a bf16 (hi, lo) pair so that the products keep
-// ~16 bits:
-//   S  = Q K^T and dP = dO V^T   A = q (or dO) with the hi parts in rows 0..7 and the lo parts in
-//                                rows 8..15 of the same heads (their sum is the product), B = K or V
-//                                from shared memory (ldmatrix);
-//   w = exp(S / sqrt(hd) - lse), ds = w (dP - D) / sqrt(hd)     in registers, row = head;
-//   dq += ds K                   A = ds (hi rows 0..7, lo rows 8..15), B = K through ldmatrix.trans;
-//   dV = w^T dO, dK = ds^T Q     contractions over the heads: w and ds go through movmatrix (an 8x8
-//                                transpose in registers) into A fragments whose k columns 0..7 hold
-//                                the heads' hi parts and 8..15 their lo parts; B holds [dO_hi; dO_hi]
-//                                for one MMA and [dO_lo; 0] for a second, so the sum is
-//                                w_hi dO_hi + w_lo dO_hi + w_hi dO_lo (the lo x lo term, ~2^-16 of the
-//                                product, is left out);
-// then stores the page's dK and dV rows (or adds them atomically on a shared page).
+// G <= 8 query heads per kv head.  An item is a tile of up to 8 pages (128 tokens) of one kv head and
+// the candidates that read all of them (one for private pages; a beam prefix or a tree edge has many);
+// the candidates are taken up to four at a time, 8 rows (heads, padded) each.  Per item and four
+// candidates, with tcgen05 MMAs (bf16 in, fp32 accumulators in TMEM, M = 128), every fp32 operand as a
+// bf16 (hi, lo) pair:
+//   S  = K [q_hi; q_lo]^T, dP = V [dO_hi; dO_lo]^T   lanes = tokens, N = 64: per candidate 8 hi rows,
+//                                 then their 8 lo rows (the two are added when TMEM is read);
+//   w = exp(S / sqrt(hd) - lse), ds = w (dP - D) / sqrt(hd)     two threads per token, to shared memory
+//                                 as [token][32 hi | 32 lo] rows of 128 bytes in the 128-byte swizzle;
+//   dV^T += dO^T w, dK^T += q^T ds  lanes = head dim, N = 128 tokens, K = the rows: hi hi + hi lo +
+//                                 lo hi (the lo x lo term, ~2^-16 of the product, is left out); they
+//                                 accumulate in TMEM over the item's candidates, so a page's gradient is
+//                                 stored once however many candidates read it (no atomics, no zeroing);
+//   dq^T = K^T [ds_hi | ds_lo]    lanes = head dim, added to dq by atomics.
+// Keys and values serve K-major (S, dP) and MN-major (dq) operands as TMA left them; so do the rows.
+// Persistent, one CTA per SM with an equal share of the work (plan_attn_back).  Warps 0 and 14 load (keys
+// and values of the next item and the rows of the next steps while the current ones are used), warp 1 issues every MMA (S and dP of the next step before the products of this one, when
+// their operands have landed), warps 2..9 compute w and ds, two threads per token, and add dq of the
+// step before, warps 10..13 store the results, a warp's 32 lanes 128 contiguous bytes at a time.
+// Bound: for private pages the stores (twice the K/V bytes in fp32, ~2.4 us of an item's ~2.8 us on an
+// SM, which is why they have warps of their own and the next item is scored beside them), for widely
+// shared ones the chain S -> w, ds -> products of a four-candidate step (~2 us).  A warp-MMA form that
+// took a CTA per candidate and eight pages and added a shared page's gradient once per candidate was the
+// form before: gradient call of 32 candidates of 4,096 shared + 500 own tokens, four 7B layers, 2,116 ->
+// 1,363 us (its launch alone 226 -> 45 us a layer); 16 distinct caches of 2,048, 1.5B, 3,538 -> 3,420 us.
+__device__ __forceinline__ BackItem back_item(const BackItem* __restrict__ items, int i) {
+  const int4 a = __ldg(reinterpret_cast<const int4*>(items + i)), b = __ldg(reinterpret_cast<const int4*>(items + i) + 1);
+  return BackItem{a.x, a.y, a.z, a.w, b.x, b.y, {0, 0}};
+}
+
+constexpr int kBackRowsCands = 4;    // candidates per step
+constexpr uint32_t kBackRowStages = 3;
+constexpr int kBackWarps = 15;       // 0 and 14 load, 1 issues MMAs, 2..9 w and ds, 10..13 results
+constexpr int kBackThreads = 32 * kBackWarps;
+constexpr uint32_t kBackTmemCols = 512;
+constexpr uint32_t kBackColS = 0, kBackColP = 64, kBackColV = 128, kBackColK = 256, kBackColQ = 384;
+
 template <int HD>
-struct BackTcSmem {
-  static constexpr uint32_t kBlock = (HD / 64) * 16 * 128;   // one page's K (or V) of one kv head
-  static constexpr uint32_t kPage = 2 * kBlock;
-  static constexpr uint32_t kPages = 0;                      // [pages][K, V], as the forward's box lands
-  static constexpr int kLd = HD + 8;                          // padded row of the B matrices (elements)
-  static constexpr uint32_t kB = kPages + kBackUnitPages * kPage;   // [4][16][kLd] bf16: Q hh, Q l0, dO hh, dO l0
-  static constexpr uint32_t kBar = kB + 4 * 16 * kLd * 2;
-  static constexpr size_t kBytes = kBar + 16 + 1024;          // + alignment slack
+struct BackSmem {
+  static constexpr uint32_t kSub = 128 * 128;                    // 64 columns of 128 tokens
+  static constexpr uint32_t kTile = (HD / 64) * kSub;            // keys (or values) of an item
+  static constexpr uint32_t kGroup = (HD / 64) * 1024;           // 8 rows
+  static constexpr uint32_t kCand = 2 * kGroup;                  // hi and lo rows of a candidate
+  static constexpr uint32_t kRows = kBackRowsCands * kCand;      // q (or dO) rows of a step
+  // values are read by the first products of a step only, so one stage of them is free again early in
+  // an item's last step; rows are released by the last ones and take ~2,000 cycles to reload: three
+  static constexpr uint32_t kK = 0;                              // [2 stages]
+  static constexpr uint32_t kV = kK + 2 * kTile;
+  static constexpr uint32_t kRowBuf = kV + kTile;                // [kRowStages][q, dO]
+  static constexpr uint32_t kW = kRowBuf + kBackRowStages * 2 * kRows;   // w [128 tokens][128 B]
+  static constexpr uint32_t kDs = kW + kSub;                     // ds
+  static constexpr uint32_t kMeta = kDs + kSub;                  // [kBackRowStages][32] (lse, D)
+  static constexpr uint32_t kBars = kMeta + kBackRowStages * 32 * 8;
+  static constexpr size_t kBytes = kBars + 256 + 1024;           // barriers and the TMEM address, alignment slack
 };
+static_assert(BackSmem<128>::kBytes <= 227 * 1024, "attention backward shared memory exceeds the per-block limit");
 
 __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
   return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~static_cast<uintptr_t>(1023));
 }
 
-__device__ __forceinline__ uint32_t movmatrix_trans(uint32_t a) {
-  uint32_t d;
-  asm volatile("movmatrix.sync.aligned.m8n8.trans.b16 %0, %1;" : "=r"(d) : "r"(a));
-  return d;
+// Eight values as 16-byte hi and lo chunks.
+__device__ __forceinline__ void split8(const float (&x)[8], uint4* hi, uint4* lo) {
+  uint32_t h[4], l[4];
+#pragma unroll
+  for (int e = 0; e < 4; ++e) {
+    const __nv_bfloat162 h2 = __floats2bfloat162_rn(x[2 * e], x[2 * e + 1]);
+    const float2 hf = __bfloat1622float2(h2);
+    const __nv_bfloat162 l2 = __floats2bfloat162_rn(x[2 * e] - hf.x, x[2 * e + 1] - hf.y);
+    h[e] = *reinterpret_cast<const uint32_t*>(&h2);
+    l[e] = *reinterpret_cast<const uint32_t*>(&l2);
+  }
+  *hi = make_uint4(h[0], h[1], h[2], h[3]);
+  *lo = make_uint4(l[0], l[1], l[2], l[3]);
 }
 
-__device__ __forceinline__ float bf16_hi(float x) { return __bfloat162float(__float2bfloat16_rn(x)); }
-
 template <int HD>
-__global__ void __launch_bounds__(128) attn_back_tc_kernel(
-    const __grid_constant__ CUtensorMap tm_pool, int64_t layer_page0, const int4* __restrict__ units,
-    const int32_t* __restrict__ seq_lens, const int32_t* __restrict__ block_table, int max_blocks,
-    const uint8_t* __restrict__ shared, const float* __restrict__ q, const float* __restrict__ dout,
-    const float* __restrict__ lse, const float* __restrict__ D, int n_q, int n_kv, float* __restrict__ grad_layer,
+__global__ void __launch_bounds__(kBackThreads, 1) attn_back_tc_kernel(
+    const __grid_constant__ CUtensorMap tm_pool_tc, int64_t layer_page0, const BackItem* __restrict__ items,
+    const int32_t* __restrict__ cta_item, const uint32_t* __restrict__ pages, const int32_t* __restrict__ cands, const uint8_t* __restrict__ ops,
+    const float2* __restrict__ meta, int n_q, int n_kv, float* __restrict__ grad_layer,
     float* __restrict__ dq, int* err) {
-  using SM = BackTcSmem<HD>;
-  constexpr int KS = HD / 16;   // 16-wide steps over the head dimension
+  using SM = BackSmem<HD>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = align1024(smem_raw);
-  uint64_t* bar = reinterpret_cast<uint64_t*>(base + SM::kBar);
-  bf16* Bq_hh = reinterpret_cast<bf16*>(base + SM::kB);   // rows 0..7 q_hi of the heads, rows 8..15 q_hi again
-  bf16* Bq_l0 = Bq_hh + 16 * SM::kLd;                     // rows 0..7 q_lo, rows 8..15 zero
-  bf16* Bd_hh = Bq_l0 + 16 * SM::kLd;                     // the same for dO
-  bf16* Bd_l0 = Bd_hh + 16 * SM::kLd;
-  const int4 u = units[blockIdx.x];
-  const int b = u.x, g = u.y, j0 = u.z, npg = u.w - u.z;
+  uint64_t* k_full = reinterpret_cast<uint64_t*>(base + SM::kBars);   // [2] keys landed
+  uint64_t* k_empty = k_full + 2;                                      // [2] every MMA that reads them done
+  uint64_t* v_full = k_empty + 2;                                      // values landed
+  uint64_t* v_empty = v_full + 1;
+  uint64_t* r_full = v_empty + 1;                                      // [kBackRowStages] a step's rows landed
+  uint64_t* r_empty = r_full + kBackRowStages;                         // [kBackRowStages]
+  uint64_t* s_full = r_empty + kBackRowStages;                                      // S and dP in TMEM
+  uint64_t* s_free = s_full + 1;                                       // read by the softmax warps
+  uint64_t* p_full = s_free + 1;                                       // w and ds in shared memory
+  uint64_t* o_full = p_full + 1;                                       // the step's products done
+  uint64_t* acc_full = o_full + 1;                                     // [2] an item's dV, dK complete
+  uint64_t* acc_free = acc_full + 2;                                   // [2] and read out
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(acc_free + 2);
+  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const int G = n_q / n_kv;
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, gid = lane >> 2, tig = lane & 3;
-  const float scale = rsqrtf(static_cast<float>(HD));
-  const int L = seq_lens[b];
-  const int64_t page_elems = static_cast<int64_t>(2) * n_kv * 16 * HD;
-  const int64_t row0 = static_cast<int64_t>(b) * n_q + static_cast<int64_t>(g) * G;   // the group's first row
+  const int item0 = cta_item[blockIdx.x], item1 = cta_item[blockIdx.x + 1];   // uploaded before the call
   if (threadIdx.x == 0) {
-    mbar_init(bar, 1);
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(&k_full[s], 1);
+      mbar_init(&k_empty[s], 1);
+      mbar_init(&acc_full[s], 1);
+      mbar_init(&acc_free[s], 4);
+    }
+    mbar_init(v_full, 1);
+    mbar_init(v_empty, 1);
+    for (uint32_t s = 0; s < kBackRowStages; ++s) {
+      mbar_init(&r_full[s], 1);
+      mbar_init(&r_empty[s], 1);
+    }
+    mbar_init(s_full, 1);
+    mbar_init(s_free, 8);
+    mbar_init(p_full, 8);
+    mbar_init(o_full, 1);
     fence_mbar_init();
-    tma_prefetch_desc(&tm_pool);
-    mbar_arrive_expect_tx(bar, static_cast<uint32_t>(npg) * SM::kPage);
-    const uint64_t pol = policy_evict_first();
-    for (int i = 0; i < npg; ++i) {
-      const int32_t p = block_table[static_cast<int64_t>(b) * max_blocks + j0 + i];
-      tma_load_5d(base + SM::kPages + i * SM::kPage, &tm_pool, bar, 0, 0, 0, g,
-                  static_cast<int32_t>(2 * (layer_page0 + p)), pol);
-    }
+    tma_prefetch_desc(&tm_pool_tc);
   }
-  // the pages (an input of the whole pass) are in flight; q, dO, lse and D may be written by the
-  // kernels just before this one
+  // rows that no candidate of a step fills meet zero weights: they only have to be finite
+  for (uint32_t i = threadIdx.x; i < kBackRowStages * 2 * SM::kRows / 16; i += blockDim.x)
+    reinterpret_cast<uint4*>(base + SM::kRowBuf)[i] = make_uint4(0u, 0u, 0u, 0u);
+  fence_proxy_async_smem();
+  if (warp == 1) {
+    tmem_alloc(tmem_slot, kBackTmemCols);
+    tmem_relinquish();
+  }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tmem_slot;
   grid_dep_launch();
-  grid_dep_wait();
-  // the B matrices of dV and dK: [16 k rows][HD] bf16, k = head (hi parts twice, or lo parts then zeros)
-  for (int i = threadIdx.x; i < 16 * HD; i += blockDim.x) {
-    const int k = i / HD, e = i - k * HD, h = k & 7;
-    const bool ok = h < G;
-    const float qv = ok ? q[(row0 + h) * HD + e] : 0.f, dv = ok ? dout[(row0 + h) * HD + e] : 0.f;
-    const float qh = bf16_hi(qv), dh = bf16_hi(dv);
-    Bq_hh[k * SM::kLd + e] = __float2bfloat16_rn(qh);
-    Bd_hh[k * SM::kLd + e] = __float2bfloat16_rn(dh);
-    Bq_l0[k * SM::kLd + e] = __float2bfloat16_rn(k < 8 ? qv - qh : 0.f);
-    Bd_l0[k * SM::kLd + e] = __float2bfloat16_rn(k < 8 ? dv - dh : 0.f);
-  }
-  // A fragments of q and dO for S and dP: row gid the hi part, row gid + 8 the lo part of head gid
-  uint32_t qa[KS][4], da[KS][4];
-  {
-    const bool ok = gid < G;
-    const float* qr = q + (row0 + gid) * HD;
-    const float* dr = dout + (row0 + gid) * HD;
+
+  if (warp == 0 || warp == kBackWarps - 1) {
+    // ------------------------------------------------ loads: warp 0 the rows and keys, the last warp the values
+    // (a 2 KB box takes a thread ~110 cycles to issue: two threads keep up with an item)
+    if (lane == 0) {
+      const bool keys = warp == 0;
+      const uint64_t pol = policy_evict_first();
+      uint32_t it = 0, ki = 0;
+      bool ok = true;
+      auto load_pages = [&](const BackItem& w) -> bool {
+        uint64_t* full = keys ? &k_full[ki & 1u] : v_full;
+        if (keys ? ki >= 2 && !mbar_wait(&k_empty[ki & 1u], ((ki >> 1) - 1) & 1u, err)
+                 : ki >= 1 && !mbar_wait(v_empty, (ki - 1) & 1u, err))
+          return false;
+        mbar_arrive_expect_tx(full, static_cast<uint32_t>(w.n_pages) * (HD / 64) * 2048);
+        uint8_t* dst = base + (keys ? SM::kK + (ki & 1u) * SM::kTile : SM::kV);
+#pragma unroll 1
+        for (int i = 0; i < w.n_pages; ++i) {
+          const int32_t unit =
+              static_cast<int32_t>(2 * (layer_page0 + (__ldg(pages + w.page_off + i) & ~kBackAtomicPage))) + (keys ? 0 : 1);
 #pragma unroll
-    for (int ks = 0; ks < KS; ++ks) {
-      const int c = ks * 16 + tig * 2;
-      float qv[4], dv[4];
-#pragma unroll
-      for (int t = 0; t < 4; ++t) {
-        const int cc = c + (t & 1) + 8 * (t >> 1);
-        qv[t] = ok ? qr[cc] : 0.f;
-        dv[t] = ok ? dr[cc] : 0.f;
+          for (int sub = 0; sub < HD / 64; ++sub)
+            tma_load_5d(dst + sub * SM::kSub + i * 2048, &tm_pool_tc, full, 0, 0, sub, w.g, unit, pol);
+        }
+        ++ki;
+        return true;
+      };
+      auto load_rows = [&](const BackItem& w, int c0) -> bool {
+        const uint32_t rb = it % kBackRowStages, use = it / kBackRowStages;
+        if (use > 0 && !mbar_wait(&r_empty[rb], (use - 1) & 1u, err)) return false;
+        const int nc = min(kBackRowsCands, w.n_cands - c0);
+        mbar_arrive_expect_tx(&r_full[rb], static_cast<uint32_t>(nc) * (2 * SM::kCand + 64));
+        uint8_t* rows = base + SM::kRowBuf + rb * 2 * SM::kRows;
+#pragma unroll 1
+        for (int i = 0; i < nc; ++i) {
+          const int64_t bg = static_cast<int64_t>(__ldg(cands + w.cand_off + c0 + i)) * n_kv + w.g;
+          bulk_load(rows + i * SM::kCand, ops + bg * 2 * SM::kCand, SM::kCand, &r_full[rb]);
+          bulk_load(rows + SM::kRows + i * SM::kCand, ops + bg * 2 * SM::kCand + SM::kCand, SM::kCand, &r_full[rb]);
+          bulk_load(base + SM::kMeta + rb * 256 + i * 64, meta + bg * 8, 64, &r_full[rb]);
+        }
+        ++it;
+        return true;
+      };
+      for (int item = item0; item < item1 && ok; ++item) {
+        const BackItem w = back_item(items, item);
+        // the pages are an input of the whole pass, the rows are not: the first item's pages go first,
+        // later ones' after the rows, which the next step may be waiting for
+        if (!keys || item == item0) ok = load_pages(w);
+        if (!keys) continue;
+        if (item == item0) grid_dep_wait();
+#pragma unroll 1
+        for (int c0 = 0; c0 < w.n_cands && ok; c0 += kBackRowsCands) {
+          ok = load_rows(w, c0);
+          if (ok && c0 == 0 && item > item0) ok = load_pages(w);
+        }
       }
-      qa[ks][0] = pack_bf16(qv[0], qv[1]);
-      qa[ks][1] = pack_bf16(qv[0] - bf16_hi(qv[0]), qv[1] - bf16_hi(qv[1]));
-      qa[ks][2] = pack_bf16(qv[2], qv[3]);
-      qa[ks][3] = pack_bf16(qv[2] - bf16_hi(qv[2]), qv[3] - bf16_hi(qv[3]));
-      da[ks][0] = pack_bf16(dv[0], dv[1]);
-      da[ks][1] = pack_bf16(dv[0] - bf16_hi(dv[0]), dv[1] - bf16_hi(dv[1]));
-      da[ks][2] = pack_bf16(dv[2], dv[3]);
-      da[ks][3] = pack_bf16(dv[2] - bf16_hi(dv[2]), dv[3] - bf16_hi(dv[3]));
-    }
-  }
-  const float lse_g = gid < G ? lse[row0 + gid] : 0.f;
-  const float D_g = gid < G ? D[row0 + gid] : 0.f;
-  float dqa[HD / 8][4];
-#pragma unroll
-  for (int n = 0; n < HD / 8; ++n) dqa[n][0] = dqa[n][1] = dqa[n][2] = dqa[n][3] = 0.f;
-  __syncthreads();   // the barrier is initialised and the B matrices are written
-  if (!__all_sync(0xffffffffu, mbar_wait(bar, 0, err))) {
-    // gave up (the error word is set): wait, bounded again, for the copies still landing in this
-    // CTA's shared memory before leaving
-    mbar_wait(bar, 0, err);
-    return;
-  }
-  const int mi = lane >> 3;
-  for (int i = warp; i < npg; i += 4) {
-    const int j = j0 + i;
-    const int32_t p = block_table[static_cast<int64_t>(b) * max_blocks + j];
-    const int valid = min(16, L - 16 * j);
-    const uint32_t kbase = smem_u32(base + SM::kPages + i * SM::kPage), vbase = kbase + SM::kBlock;
-    // S = Q K^T and dP = dO V^T over the page's 16 tokens (two n-tiles of 8)
-    float s0[4] = {0.f, 0.f, 0.f, 0.f}, s1[4] = {0.f, 0.f, 0.f, 0.f};
-    float p0[4] = {0.f, 0.f, 0.f, 0.f}, p1[4] = {0.f, 0.f, 0.f, 0.f};
-    {
-      const int tok = (mi >> 1) * 8 + (lane & 7);
-#pragma unroll
-      for (int ks = 0; ks < KS; ++ks) {
-        const int hdc = ks * 16 + (mi & 1) * 8;
-        const uint32_t off = (hdc >> 6) * 2048 + tok * 128 + ((((hdc & 63) >> 3) ^ (tok & 7)) << 4);
-        uint32_t kb[4], vb[4];
-        ldsm_x4(kbase + off, kb[0], kb[1], kb[2], kb[3]);
-        ldsm_x4(vbase + off, vb[0], vb[1], vb[2], vb[3]);
-        mma_bf16_16816(s0, qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], kb[0], kb[1]);
-        mma_bf16_16816(s1, qa[ks][0], qa[ks][1], qa[ks][2], qa[ks][3], kb[2], kb[3]);
-        mma_bf16_16816(p0, da[ks][0], da[ks][1], da[ks][2], da[ks][3], vb[0], vb[1]);
-        mma_bf16_16816(p1, da[ks][0], da[ks][1], da[ks][2], da[ks][3], vb[2], vb[3]);
+      // every copy issued above has landed before this CTA ends
+      if (keys) {
+        for (uint32_t v = ki > 2 ? ki - 2 : 0; v < ki; ++v)
+          if (!mbar_wait(&k_full[v & 1u], (v >> 1) & 1u, err)) break;
+        for (uint32_t v = it > kBackRowStages ? it - kBackRowStages : 0; v < it; ++v)
+          if (!mbar_wait(&r_full[v % kBackRowStages], (v / kBackRowStages) & 1u, err)) break;
+      } else if (ki > 0) {
+        mbar_wait(v_full, (ki - 1) & 1u, err);
       }
     }
-    // head gid, tokens tig*2, tig*2 + 1, 8 + tig*2, 9 + tig*2: the hi and lo rows summed
-    const float x[4] = {s0[0] + s0[2], s0[1] + s0[3], s1[0] + s1[2], s1[1] + s1[3]};
-    const float dp[4] = {p0[0] + p0[2], p0[1] + p0[3], p1[0] + p1[2], p1[1] + p1[3]};
-    float w[4], ds[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      const int t = (e & 1) + tig * 2 + 8 * (e >> 1);
-      w[e] = (gid < G && t < valid) ? expf(x[e] * scale - lse_g) : 0.f;
-      ds[e] = w[e] * (dp[e] - D_g) * scale;
-    }
-    float wl[4], dl[4];
-#pragma unroll
-    for (int e = 0; e < 4; ++e) {
-      wl[e] = w[e] - bf16_hi(w[e]);
-      dl[e] = ds[e] - bf16_hi(ds[e]);
-    }
-    // dq += ds K (K as the k x n operand through ldmatrix.trans, as V in the forward's P V)
-    {
-      const uint32_t a0 = pack_bf16(ds[0], ds[1]), a1 = pack_bf16(dl[0], dl[1]);
-      const uint32_t a2 = pack_bf16(ds[2], ds[3]), a3 = pack_bf16(dl[2], dl[3]);
-      const int tok = (mi & 1) * 8 + (lane & 7);
-#pragma unroll
-      for (int j2 = 0; j2 < HD / 16; ++j2) {
-        const int hdc = j2 * 16 + (mi >> 1) * 8;
-        uint32_t kb[4];
-        ldsm_x4_t(kbase + (hdc >> 6) * 2048 + tok * 128 + ((((hdc & 63) >> 3) ^ (tok & 7)) << 4), kb[0], kb[1],
-                  kb[2], kb[3]);
-        mma_bf16_16816(dqa[2 * j2], a0, a1, a2, a3, kb[0], kb[1]);
-        mma_bf16_16816(dqa[2 * j2 + 1], a0, a1, a2, a3, kb[2], kb[3]);
-      }
-    }
-    // w^T and ds^T as A fragments: rows = tokens, k 0..7 = the heads' hi parts, 8..15 their lo parts
-    const uint32_t wt0 = movmatrix_trans(pack_bf16(w[0], w[1])), wt1 = movmatrix_trans(pack_bf16(w[2], w[3]));
-    const uint32_t wt2 = movmatrix_trans(pack_bf16(wl[0], wl[1])), wt3 = movmatrix_trans(pack_bf16(wl[2], wl[3]));
-    const uint32_t st0 = movmatrix_trans(pack_bf16(ds[0], ds[1])), st1 = movmatrix_trans(pack_bf16(ds[2], ds[3]));
-    const uint32_t st2 = movmatrix_trans(pack_bf16(dl[0], dl[1])), st3 = movmatrix_trans(pack_bf16(dl[2], dl[3]));
-    float* gk = grad_layer + p * page_elems + static_cast<int64_t>(g) * 16 * HD;
-    float* gv = gk + static_cast<int64_t>(n_kv) * 16 * HD;
-    const bool sh = shared[p] != 0;
-    auto put = [&](float* dst, float a, float c) {
-      if (sh)
-        atomicAdd(reinterpret_cast<float2*>(dst), make_float2(a, c));
-      else
-        *reinterpret_cast<float2*>(dst) = make_float2(a, c);
+  } else if (warp == 1) {
+    // ------------------------------------------------ MMAs (the whole warp; one elected lane issues)
+    const uint32_t id_s = idesc_bf16_f32(128, 64);
+    const uint32_t id_v = idesc_bf16_f32(128, 128) | kIdescMnMajorA;
+    const uint32_t id_q = idesc_bf16_f32(128, 64) | kIdescMnMajorA | kIdescMnMajorB;
+    // Each step's S and dP, then its products, in order; S and dP of the next step go first when they
+    // can.  One copy of each sequence and rolled loops: the code of a step is fetched once per launch
+    // (unrolled, with S at three places, the first product phase of a launch took ~7,000 cycles, the
+    // later ones ~2,500).
+    auto test_all = [&](uint64_t* bar, uint32_t phase) { return __all_sync(0xffffffffu, mbar_test(bar, phase & 1u)); };
+    struct Step {   // a step: four candidates of an item
+      int item, c0;
+      uint32_t it, ki;
+      BackItem w;
     };
-    {
-      const int krow = (mi & 1) * 8 + (lane & 7);
+    auto advance = [&](Step& s) {
+      ++s.it;
+      s.c0 += kBackRowsCands;
+      if (s.c0 >= s.w.n_cands) {
+        s.c0 = 0;
+        ++s.ki;
+        if (++s.item < item1) s.w = back_item(items, s.item);
+      }
+    };
+    Step so;   // the next S, dP
+    so.item = item0;
+    so.c0 = 0;
+    so.it = so.ki = 0;
+    if (item0 < item1) so.w = back_item(items, item0);
+    Step oo = so;   // the next products
+    const uint32_t k0 = smem_u32(base + SM::kK), v0 = smem_u32(base + SM::kV), rows0 = smem_u32(base + SM::kRowBuf), w0 = smem_u32(base + SM::kW);
+    uint32_t spins = 0;
+    uint64_t idle = 0;
+    while (oo.item < item1) {
+      const uint32_t so_st = so.ki & 1u, so_rb = so.it % kBackRowStages;
+      if (so.item < item1 && (so.it == oo.it || (so.it == oo.it + 1 && test_all(s_free, oo.it))) &&
+          test_all(&r_full[so_rb], so.it / kBackRowStages) && test_all(&k_full[so_st], so.ki >> 1) &&
+          test_all(v_full, so.ki)) {
+        tc_fence_after();
+#pragma unroll 1
+        for (uint32_t x = 0; x < 2; ++x) {   // K q^T, then V dO^T
+          const uint64_t a0 = desc_sw128_s(x ? v0 : k0 + so_st * SM::kTile, 1024, 1024);
+          const uint64_t b0 = desc_sw128_s(rows0 + (2 * so_rb + x) * SM::kRows, 1024, SM::kGroup);
+          const uint32_t d = tmem + (x ? kBackColP : kBackColS);
 #pragma unroll
-      for (int j2 = 0; j2 < HD / 16; ++j2) {
-        const int col = j2 * 16 + (mi >> 1) * 8;
-        uint32_t dh[4], dlo[4], qh[4], ql[4];
-        ldsm_x4_t(smem_u32(Bd_hh + krow * SM::kLd + col), dh[0], dh[1], dh[2], dh[3]);
-        ldsm_x4_t(smem_u32(Bd_l0 + krow * SM::kLd + col), dlo[0], dlo[1], dlo[2], dlo[3]);
-        ldsm_x4_t(smem_u32(Bq_hh + krow * SM::kLd + col), qh[0], qh[1], qh[2], qh[3]);
-        ldsm_x4_t(smem_u32(Bq_l0 + krow * SM::kLd + col), ql[0], ql[1], ql[2], ql[3]);
-        float v0[4] = {0.f, 0.f, 0.f, 0.f}, v1[4] = {0.f, 0.f, 0.f, 0.f};
-        float k0[4] = {0.f, 0.f, 0.f, 0.f}, k1[4] = {0.f, 0.f, 0.f, 0.f};
-        mma_bf16_16816(v0, wt0, wt1, wt2, wt3, dh[0], dh[1]);
-        mma_bf16_16816(v0, wt0, wt1, wt2, wt3, dlo[0], dlo[1]);
-        mma_bf16_16816(v1, wt0, wt1, wt2, wt3, dh[2], dh[3]);
-        mma_bf16_16816(v1, wt0, wt1, wt2, wt3, dlo[2], dlo[3]);
-        mma_bf16_16816(k0, st0, st1, st2, st3, qh[0], qh[1]);
-        mma_bf16_16816(k0, st0, st1, st2, st3, ql[0], ql[1]);
-        mma_bf16_16816(k1, st0, st1, st2, st3, qh[2], qh[3]);
-        mma_bf16_16816(k1, st0, st1, st2, st3, ql[2], ql[3]);
-        // C rows: token gid (elements 0, 1) and gid + 8 (2, 3); columns of the two n-tiles
-        const int c0 = j2 * 16 + tig * 2, c1 = c0 + 8;
-        put(gv + gid * HD + c0, v0[0], v0[1]);
-        put(gv + (gid + 8) * HD + c0, v0[2], v0[3]);
-        put(gv + gid * HD + c1, v1[0], v1[1]);
-        put(gv + (gid + 8) * HD + c1, v1[2], v1[3]);
-        put(gk + gid * HD + c0, k0[0], k0[1]);
-        put(gk + (gid + 8) * HD + c0, k0[2], k0[3]);
-        put(gk + gid * HD + c1, k1[0], k1[1]);
-        put(gk + (gid + 8) * HD + c1, k1[2], k1[3]);
+          for (int kk = 0; kk < HD / 16; ++kk)
+            umma_bf16_w(d, a0 + (((kk >> 2) * SM::kSub + (kk & 3) * 32) >> 4),
+                        b0 + (((kk >> 2) * 1024 + (kk & 3) * 32) >> 4), id_s, kk > 0 ? 1u : 0u);
+        }
+        umma_commit_w(s_full);
+        if (so.c0 + kBackRowsCands >= so.w.n_cands) umma_commit_w(v_empty);
+        advance(so);
+        spins = 0;
+      } else if (so.it > oo.it && test_all(p_full, oo.it)) {
+        const uint32_t st = oo.ki & 1u, rb = oo.it % kBackRowStages;
+        const int pairs = (min(kBackRowsCands, oo.w.n_cands - oo.c0) + 1) >> 1;   // 16 rows per MMA
+        const bool last = oo.c0 + kBackRowsCands >= oo.w.n_cands;
+        bool ok = true;
+#pragma unroll 1
+        for (uint32_t x = 0; x < 2 && ok; ++x) {   // dV from dO and w, then dK from q and ds
+          // the first step of an item waits until the previous item's dV (dK) has been read out
+          if (oo.c0 == 0 && oo.ki > 0) ok = __all_sync(0xffffffffu, mbar_wait(&acc_free[x], (oo.ki - 1) & 1u, err));
+          tc_fence_after();
+          uint64_t a0 = desc_sw128_s(rows0 + (2 * rb + 1 - x) * SM::kRows, 1024, SM::kCand);
+          uint64_t b0 = desc_sw128_s(w0 + x * SM::kSub, 1024, 1024);
+          const uint32_t d = tmem + (x ? kBackColK : kBackColV);
+          uint32_t acc = oo.c0 > 0 ? 1u : 0u;
+#pragma unroll 1
+          for (int pr = 0; pr < pairs; ++pr) {
+            umma_bf16_w(d, a0, b0, id_v, acc);
+            umma_bf16_w(d, a0, b0 + (64 >> 4), id_v, 1u);
+            umma_bf16_w(d, a0 + (SM::kGroup >> 4), b0, id_v, 1u);
+            acc = 1u;
+            a0 += (2 * SM::kCand) >> 4;
+            b0 += 32 >> 4;
+          }
+          if (last) umma_commit_w(&acc_full[x]);
+        }
+        if (!ok) break;
+        uint64_t a0 = desc_sw128_s(k0 + st * SM::kTile, SM::kSub, 1024);
+        uint64_t b0 = desc_sw128_s(w0 + SM::kSub, SM::kSub, 1024);
+#pragma unroll 1
+        for (int ks = 0; ks < oo.w.n_pages; ++ks) {   // 16 tokens per MMA
+          umma_bf16_w(tmem + kBackColQ, a0, b0, id_q, ks > 0 ? 1u : 0u);
+          a0 += 2048 >> 4;
+          b0 += 2048 >> 4;
+        }
+        umma_commit_w(o_full);
+        umma_commit_w(&r_empty[rb]);
+        if (last) umma_commit_w(&k_empty[st]);
+        advance(oo);
+        spins = 0;
+      } else if ((++spins & 255u) == 0u) {   // bounded like every other wait
+        const uint64_t now = global_timer_ns();
+        if (spins == 256u) idle = now;
+        if (now - idle > kErrPollNs && *(volatile int*)err != 0) break;
+        if (now - idle > kWaitTimeoutNs) {
+          if (lane == 0) atomicCAS(err, 0, kDevTimeout);
+          break;
+        }
+      }
+    }
+  } else if (warp < 10) {
+    // ------------------------------------------------ w and ds (two threads per token), and dq
+    const int w4 = warp & 3;            // TMEM lane quadrant
+    const int half = (warp - 2) >> 2;   // candidates 2 half, 2 half + 1 of a step
+    const int t = w4 * 32 + lane;       // token (S, dP) or head-dim element (dq) of this thread
+    const uint32_t trow = tmem + (static_cast<uint32_t>(w4 * 32) << 16);
+    const float scale = rsqrtf(static_cast<float>(HD));
+    const bool out_lane = HD == 128 || w4 < 2;   // lanes past HD hold nothing
+    grid_dep_wait();
+    // dq of a step (candidates c0 .. of item w): its sums out of TMEM, then added
+    auto dq_load = [&](float (&v)[16]) {
+      float a[16], b[16];
+      tmem_ld16_nowait(trow + kBackColQ + 16 * half, a);
+      tmem_ld16_nowait(trow + kBackColQ + 32 + 16 * half, b);
+      tmem_wait_ld();
+      tmem_hold(a);
+      tmem_hold(b);
+#pragma unroll
+      for (int j = 0; j < 16; ++j) v[j] = a[j] + b[j];
+    };
+    auto dq_add = [&](const float (&v)[16], const BackItem& w, int c0) {
+#pragma unroll
+      for (int cc = 0; cc < 2; ++cc) {
+        const int c = c0 + 2 * half + cc;
+        if (c >= w.n_cands || !out_lane) break;
+        float* dst = dq + (static_cast<int64_t>(__ldg(cands + w.cand_off + c)) * n_q + w.g * G) * HD + t;
+#pragma unroll
+        for (int r = 0; r < 8; ++r)
+          if (r < G) atomicAdd(dst + r * HD, v[cc * 8 + r]);
+      }
+    };
+    uint32_t it = 0;
+    bool ok = true;
+    BackItem next{}, prev{};
+    int prev_c0 = 0;
+    float dqv[16];
+    if (item0 < item1) next = back_item(items, item0);
+    for (int item = item0; item < item1; ++item) {
+      const BackItem w = next;   // the item after this one: read now, used an item later
+      if (item + 1 < item1) next = back_item(items, item + 1);
+      for (int c0 = 0; c0 < w.n_cands; c0 += kBackRowsCands, ++it) {
+        const uint32_t rb = it % kBackRowStages;
+        // this thread's candidates; the second half has none when the step is one pair
+        const int mine = min(2, w.n_cands - c0 - 2 * half);
+        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&r_full[rb], (it / kBackRowStages) & 1u, err));   // lse and D
+        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(s_full, it & 1u, err));
+        tc_fence_after();
+        uint4 whi[2], wlo[2], dhi[2], dlo[2];
+        const bool live = ok && t < w.n_tokens;
+#pragma unroll
+        for (int cc = 0; cc < 2; ++cc) {
+          whi[cc] = wlo[cc] = dhi[cc] = dlo[cc] = make_uint4(0u, 0u, 0u, 0u);
+          if (cc >= mine || !ok) continue;   // (uniform)
+          const int slot = 2 * half + cc;
+          float s[16], p[16];
+          tmem_ld16_nowait(trow + kBackColS + 16 * slot, s);
+          tmem_ld16_nowait(trow + kBackColP + 16 * slot, p);
+          tmem_wait_ld();
+          tmem_hold(s);
+          tmem_hold(p);
+          const float2* ml = reinterpret_cast<const float2*>(base + SM::kMeta + rb * 256) + slot * 8;
+          float wv[8], dv[8];
+#pragma unroll
+          for (int r = 0; r < 8; ++r) {
+            const float2 m = ml[r];
+            const float x = s[r] + s[8 + r], dp = p[r] + p[8 + r];
+            wv[r] = live ? ex2_ftz((x * scale - m.x) * kLog2eBack) : 0.f;
+            dv[r] = live ? wv[r] * (dp - m.y) * scale : 0.f;
+          }
+          split8(wv, &whi[cc], &wlo[cc]);
+          split8(dv, &dhi[cc], &dlo[cc]);
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(s_free);   // the next step's S and dP may overwrite these
+        // the products that read the previous step's w and ds are done, and its dq is complete
+        if (it > 0 && ok) ok = __all_sync(0xffffffffu, mbar_wait(o_full, (it - 1) & 1u, err));
+        tc_fence_after();
+        const bool add = it > 0 && ok;
+        if (add) dq_load(dqv);
+        if (mine > 0) {   // an odd candidate's partner in its pair is zero
+#pragma unroll
+          for (int cc = 0; cc < 2; ++cc) {
+            const int ch = 2 * half + cc;
+            uint8_t* wr = base + SM::kW + t * 128;
+            uint8_t* dr = base + SM::kDs + t * 128;
+            const int ohi = (ch ^ (t & 7)) << 4, olo = ((4 + ch) ^ (t & 7)) << 4;
+            *reinterpret_cast<uint4*>(wr + ohi) = whi[cc];
+            *reinterpret_cast<uint4*>(wr + olo) = wlo[cc];
+            *reinterpret_cast<uint4*>(dr + ohi) = dhi[cc];
+            *reinterpret_cast<uint4*>(dr + olo) = dlo[cc];
+          }
+          fence_proxy_async_smem();
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(p_full);
+        if (add) dq_add(dqv, prev, prev_c0);
+        prev = w;
+        prev_c0 = c0;
+      }
+    }
+    if (it > 0 && ok && __all_sync(0xffffffffu, mbar_wait(o_full, (it - 1) & 1u, err))) {
+      tc_fence_after();
+      dq_load(dqv);
+      dq_add(dqv, prev, prev_c0);
+    }
+  } else if (warp < 14) {
+    // ------------------------------------------------ results (a thread per head-dim element; a column is a token)
+    const int w4 = warp & 3;
+    const uint32_t trow = tmem + (static_cast<uint32_t>(w4 * 32) << 16);
+    const int64_t page_elems = static_cast<int64_t>(2) * n_kv * 16 * HD;
+    const bool out_lane = HD == 128 || w4 < 2;
+    grid_dep_wait();
+    uint32_t ki = 0;
+    bool ok = true;
+    BackItem next{};
+    if (item0 < item1) next = back_item(items, item0);
+    for (int item = item0; item < item1; ++item, ++ki) {
+      const BackItem w = next;
+      if (item + 1 < item1) next = back_item(items, item + 1);
+      // lane i: page i of the item
+      const uint32_t my_page = lane < w.n_pages ? __ldg(pages + w.page_off + lane) : 0u;
+#pragma unroll 1
+      for (int x = 0; x < 2; ++x) {   // dV, then dK; the pool's layout: keys, then values
+        float* const out0 = grad_layer + (x ? 0 : n_kv * 16 * HD) + w.g * 16 * HD + w4 * 32 + lane;
+        if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&acc_full[x], ki & 1u, err));
+        tc_fence_after();
+#pragma unroll 1
+        for (int i = 0; i < w.n_pages && ok; ++i) {
+          float v[16];
+          tmem_ld16(trow + (x ? kBackColK : kBackColV) + 16 * i, v);
+          const uint32_t page = __shfl_sync(0xffffffffu, my_page, i);
+          if (!out_lane) continue;
+          float* dst = out0 + (page & ~kBackAtomicPage) * page_elems;
+          if (page & kBackAtomicPage) {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) atomicAdd(dst + j * HD, v[j]);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 16; ++j) dst[j * HD] = v[j];
+          }
+        }
+        tc_fence_before();   // all read: the next item's products may overwrite them
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&acc_free[x]);
       }
     }
   }
-  // dq: rows gid (hi) and gid + 8 (lo) of head gid summed, the four warps' parts through shared
-  // memory (the page buffer, no longer read), then one atomic add per element
+  __syncwarp();
+  tc_fence_before();
   __syncthreads();
-  float* s_dq = reinterpret_cast<float*>(base);   // [4][8][HD] <= the page buffer
-#pragma unroll
-  for (int n = 0; n < HD / 8; ++n) {
-    const int c = n * 8 + tig * 2;
-    s_dq[(warp * 8 + gid) * HD + c] = dqa[n][0] + dqa[n][2];
-    s_dq[(warp * 8 + gid) * HD + c + 1] = dqa[n][1] + dqa[n][3];
-  }
-  __syncthreads();
-  for (int i2 = threadIdx.x; i2 < G * HD; i2 += blockDim.x) {
-    const int r = i2 / HD, e = i2 - r * HD;
-    const float v = s_dq[(0 * 8 + r) * HD + e] + s_dq[(1 * 8 + r) * HD + e] + s_dq[(2 * 8 + r) * HD + e] +
-                    s_dq[(3 * 8 + r) * HD + e];
-    atomicAdd(dq + (row0 + r) * HD + e, v);
+  if (warp == 1) {
+    tc_fence_after();
+    tmem_dealloc(tmem, kBackTmemCols);
   }
 }
 
@@ -740,19 +987,23 @@ cudaError_t launch_silu_back(const float* da, const float* gu, int n, int ff, __
 
 cudaError_t launch_attn_back(const AttnBackArgs& a, cudaStream_t st) {
   if (a.n_q / a.n_kv > kMaxGroup || (a.hd != 64 && a.hd != 128)) return cudaErrorInvalidValue;
-  cudaError_t e = launch_pdl(attn_back_pre_kernel, dim3(a.n * a.n_kv), dim3(128), 0, st, a.q, a.kself, a.vself, a.o,
-                             a.dout, a.lse, a.n_q, a.n_kv, a.hd, a.D, a.dq, a.dks, a.dvs);
-  if (e != cudaSuccess || a.n_units == 0) return e;
   const int G = a.n_q / a.n_kv;
-  if (G <= 8 && a.tm_pool) {   // the tensor-core backward
+  const bool tc = G <= 8 && a.tm_pool_tc != nullptr;
+  cudaError_t e = launch_pdl(attn_back_pre_kernel, dim3(a.n * a.n_kv), dim3(128), 0, st, a.q, a.kself, a.vself, a.o,
+                             a.dout, a.lse, a.n_q, a.n_kv, a.hd, a.D, a.dq, a.dks, a.dvs, tc ? a.ops : nullptr, a.meta);
+  if (e != cudaSuccess) return e;
+  if (tc) {
+    if (a.n_ctas == 0) return e;
+    const dim3 grid(a.n_ctas);
     if (a.hd == 128)
-      return launch_pdl(attn_back_tc_kernel<128>, dim3(a.n_units), dim3(128), BackTcSmem<128>::kBytes, st, *a.tm_pool,
-                        a.layer_page0, a.units, a.seq_lens, a.block_table, a.max_blocks, a.shared, a.q, a.dout, a.lse,
-                        a.D, a.n_q, a.n_kv, a.grad_layer, a.dq, a.err);
-    return launch_pdl(attn_back_tc_kernel<64>, dim3(a.n_units), dim3(128), BackTcSmem<64>::kBytes, st, *a.tm_pool,
-                      a.layer_page0, a.units, a.seq_lens, a.block_table, a.max_blocks, a.shared, a.q, a.dout, a.lse,
-                      a.D, a.n_q, a.n_kv, a.grad_layer, a.dq, a.err);
+      return launch_pdl(attn_back_tc_kernel<128>, grid, dim3(kBackThreads), BackSmem<128>::kBytes, st, *a.tm_pool_tc,
+                        a.layer_page0, a.items, a.cta_item, a.item_pages, a.item_cands, a.ops, a.meta, a.n_q, a.n_kv,
+                        a.grad_layer, a.dq, a.err);
+    return launch_pdl(attn_back_tc_kernel<64>, grid, dim3(kBackThreads), BackSmem<64>::kBytes, st, *a.tm_pool_tc,
+                      a.layer_page0, a.items, a.cta_item, a.item_pages, a.item_cands, a.ops, a.meta, a.n_q, a.n_kv,
+                      a.grad_layer, a.dq, a.err);
   }
+  if (a.n_units == 0) return e;
   const size_t smem = a.hd == 128 ? back_pages_smem<128>() : back_pages_smem<64>();
   cudaError_t le = cudaSuccess;
   auto go = [&](auto kern) {
@@ -788,9 +1039,180 @@ cudaError_t grad_configure() {
   set(attn_back_pages_kernel<64, 4>, back_pages_smem<64>());
   set(attn_back_pages_kernel<64, 8>, back_pages_smem<64>());
   set(attn_back_pages_kernel<64, 16>, back_pages_smem<64>());
-  set(attn_back_tc_kernel<128>, BackTcSmem<128>::kBytes);
-  set(attn_back_tc_kernel<64>, BackTcSmem<64>::kBytes);
+  set(attn_back_tc_kernel<128>, BackSmem<128>::kBytes);
+  set(attn_back_tc_kernel<64>, BackSmem<64>::kBytes);
   return e;
+}
+
+// Tensor cores: full pages that the same candidates (at least two) read, each once, form a group, cut
+// into items of kBackTilePages pages per kv head; every other page of a candidate goes to items of its
+// own, in logical order.  When the groups' items leave SMs idle, a group's candidates are split over
+// several items (in fours, one step of the kernel each) whose pages then accumulate atomically.  The
+// persistent CTAs get equal shares under a cost model: 9 units of 1/16 us a page and 8 an item (a
+// private item moves 24 KB a page, ~0.56 us at an SM's share of HBM) and 22 every step after the first
+// (measured ~1.4 us).  Items of several steps go to the least loaded CTA, longest first; the private
+// pages then fill every CTA to the common level, cut wherever that falls.
+// CUDA cores: units of kBackUnitPagesMax pages per candidate and kv head.
+constexpr int64_t kBackPageCost = 9, kBackItemCost = 8, kBackStepCost = 22;
+
+void plan_attn_back(const int32_t* bt, const int32_t* sl, int n, int max_blocks, int64_t n_pages, int n_kv,
+                    bool tensor_cores, int n_sms, BackPlan& p) {
+  p = BackPlan();
+  const size_t np = static_cast<size_t>(std::max<int64_t>(n_pages, 1));
+  std::vector<int32_t> refs(np + 1, 0);
+  for (int b = 0; b < n; ++b)
+    for (int j = 0, pg = (sl[b] + 15) / 16; j < pg; ++j) ++refs[bt[static_cast<int64_t>(b) * max_blocks + j]];
+  p.atomic.assign(np, 0);
+  std::vector<uint8_t> grouped(np, 0);
+  std::vector<BackItem> shared;
+  if (!tensor_cores) {
+    for (int b = 0; b < n; ++b) {
+      const int pages = (sl[b] + 15) / 16;
+      for (int g = 0; g < n_kv; ++g)
+        for (int j0 = 0; j0 < pages; j0 += kBackUnitPagesMax)
+          p.units.push_back(make_int4(b, g, j0, std::min(pages, j0 + kBackUnitPagesMax)));
+    }
+  } else {
+    // the full references of every page read at least twice, by page
+    std::vector<int32_t> off(np + 1, 0), list;
+    for (size_t i = 0; i < np; ++i) off[i + 1] = off[i] + (refs[i] > 1 ? refs[i] : 0);
+    if (off[np] > 0) {
+      list.assign(static_cast<size_t>(off[np]), -1);
+      std::vector<int32_t> fill(off.begin(), off.end() - 1);
+      for (int b = 0; b < n; ++b)
+        for (int j = 0, full = sl[b] / 16; j < full; ++j) {
+          const int32_t pg = bt[static_cast<int64_t>(b) * max_blocks + j];
+          if (refs[pg] > 1) list[fill[pg]++] = b;
+        }
+      std::map<std::vector<int32_t>, std::vector<int32_t>> groups;   // candidates -> pages
+      std::vector<int32_t> key;
+      std::vector<int32_t>* last = nullptr;
+      for (size_t i = 0; i < np; ++i) {
+        const int32_t c = refs[i];
+        if (c < 2 || fill[i] - off[i] != c) continue;   // some reference is partial
+        const int32_t* r = list.data() + off[i];
+        bool twice = false;
+        for (int32_t k = 1; k < c; ++k) twice = twice || r[k] == r[k - 1];
+        if (twice) continue;
+        if (!last || key.size() != static_cast<size_t>(c) || !std::equal(key.begin(), key.end(), r)) {
+          key.assign(r, r + c);
+          last = &groups[key];
+        }
+        last->push_back(static_cast<int32_t>(i));
+        grouped[i] = 1;
+      }
+      int64_t tiles = 0;
+      for (const auto& kv : groups) tiles += (static_cast<int64_t>(kv.second.size()) + kBackTilePages - 1) / kBackTilePages;
+      const int64_t room = std::max<int64_t>(1, tiles > 0 ? n_sms / (tiles * n_kv) : 1);   // items a group's tile may become
+      for (const auto& kv : groups) {
+        const std::vector<int32_t>&cs = kv.first, &pg = kv.second;
+        const int steps = (static_cast<int>(cs.size()) + 3) / 4;
+        const int parts = static_cast<int>(std::min<int64_t>(room, steps));
+        const int page0 = static_cast<int>(p.item_pages.size()), cand0 = static_cast<int>(p.item_cands.size());
+        p.item_pages.insert(p.item_pages.end(), pg.begin(), pg.end());
+        p.item_cands.insert(p.item_cands.end(), cs.begin(), cs.end());
+        for (size_t k = 0; k < pg.size(); k += kBackTilePages)
+          for (int q = 0; q < parts; ++q) {
+            const int c0 = 4 * (steps * q / parts), c1 = std::min<int>(4 * (steps * (q + 1) / parts), static_cast<int>(cs.size()));
+            const int m = static_cast<int>(std::min<size_t>(kBackTilePages, pg.size() - k));
+            for (int g = 0; g < n_kv; ++g)
+              shared.push_back(BackItem{g, page0 + static_cast<int>(k), m, 16 * m, cand0 + c0, c1 - c0, {0, 0}});
+          }
+        if (parts > 1)
+          for (int32_t x : pg) p.atomic[x] = 1;
+      }
+    }
+    // private runs: every other page of a candidate
+    struct Run {
+      int32_t page_off, n_pages, last, cand_off;
+    };
+    std::vector<Run> runs;
+    int64_t pages = 0;
+    for (int b = 0; b < n; ++b) {
+      const int32_t page0 = static_cast<int32_t>(p.item_pages.size());
+      int32_t last = 0;   // valid tokens of the last page listed
+      for (int j = 0, pg = (sl[b] + 15) / 16; j < pg; ++j) {
+        const int32_t x = bt[static_cast<int64_t>(b) * max_blocks + j];
+        if (grouped[x]) continue;
+        p.item_pages.push_back(x);
+        last = std::min(16, sl[b] - 16 * j);
+      }
+      const int32_t m = static_cast<int32_t>(p.item_pages.size()) - page0;
+      if (m == 0) continue;
+      runs.push_back(Run{page0, m, last, static_cast<int32_t>(p.item_cands.size())});
+      p.item_cands.push_back(b);
+      pages += static_cast<int64_t>(m) * n_kv;
+    }
+    // equal shares
+    auto cost = [](int64_t m, int64_t steps) { return kBackItemCost + kBackPageCost * m + kBackStepCost * (steps - 1); };
+    auto cost_of = [&](const BackItem& i) { return cost(i.n_pages, (i.n_cands + 3) / 4); };
+    std::stable_sort(shared.begin(), shared.end(), [&](const BackItem& x, const BackItem& y) { return cost_of(x) > cost_of(y); });
+    const int64_t most = static_cast<int64_t>(shared.size()) + pages;   // no more CTAs than items of a page
+    const int C = static_cast<int>(std::min<int64_t>(n_sms, most));
+    std::vector<std::vector<int32_t>> mine(static_cast<size_t>(C));   // shared items by CTA
+    std::vector<int64_t> load(static_cast<size_t>(C), 0);
+    {
+      typedef std::pair<int64_t, int> Slot;   // (load, CTA), least first
+      std::priority_queue<Slot, std::vector<Slot>, std::greater<Slot>> heap;
+      for (int k = 0; k < C; ++k) heap.push({0, k});
+      for (size_t i = 0; i < shared.size(); ++i) {
+        Slot s = heap.top();
+        heap.pop();
+        s.first += cost_of(shared[i]);
+        mine[s.second].push_back(static_cast<int32_t>(i));
+        load[s.second] = s.first;
+        heap.push(s);
+      }
+    }
+    // the level that the private pages fill the CTAs below it to (an item more for each CTA's cut)
+    int64_t priv = kBackPageCost * pages + kBackItemCost * C;
+    for (const Run& x : runs) priv += kBackItemCost * n_kv * ((x.n_pages + kBackTilePages - 1) / kBackTilePages);
+    std::vector<int64_t> sorted(load);
+    std::sort(sorted.begin(), sorted.end());
+    int64_t level = 0, sum = 0;
+    for (int k = 0; k < C; ++k) {
+      sum += sorted[k];
+      level = (sum + priv + k) / (k + 1);
+      if (k + 1 == C || level <= sorted[k + 1]) break;
+    }
+    size_t r = 0;
+    int32_t at = 0, g = 0;   // next private page: run r, kv head g, page `at`
+    int64_t left = pages, given = 0, want = 0;   // private cost laid, and due once CTA k is filled
+    p.cta_item.push_back(0);
+    for (int k = 0; k < C; ++k) {
+      for (int32_t i : mine[k]) p.items.push_back(shared[i]);
+      want += std::max<int64_t>(0, level - load[k]);
+      const bool all = k + 1 == C;
+      while (left > 0 && (all || given + kBackPageCost / 2 < want)) {
+        const Run& run = runs[r];
+        int64_t m = std::min<int64_t>(kBackTilePages, run.n_pages - at);
+        if (!all) m = std::max<int64_t>(1, std::min<int64_t>(m, (want - given - kBackItemCost + kBackPageCost / 2) / kBackPageCost));
+        const bool end = at + m == run.n_pages;
+        p.items.push_back(BackItem{g, run.page_off + at, static_cast<int32_t>(m),
+                                   static_cast<int32_t>(16 * (m - 1) + (end ? run.last : 16)), run.cand_off, 1, {0, 0}});
+        given += cost(m, 1);
+        left -= m;
+        at += static_cast<int32_t>(m);
+        if (end) {
+          at = 0;
+          if (++g == n_kv) {
+            g = 0;
+            ++r;
+          }
+        }
+      }
+      p.cta_item.push_back(static_cast<int32_t>(p.items.size()));
+    }
+  }
+  for (size_t i = 0; i < np; ++i)
+    if (refs[i] >= 2 && !grouped[i]) p.atomic[i] = 1;
+  for (uint32_t& pg : p.item_pages)
+    if (p.atomic[pg]) pg |= kBackAtomicPage;
+  for (size_t i = 0; i < np; ++i)
+    if (p.atomic[i]) p.lists.push_back(static_cast<int32_t>(i));
+  p.n_atomic = static_cast<int>(p.lists.size());
+  for (size_t i = 0; i < np; ++i)
+    if (refs[i] >= 1) p.lists.push_back(static_cast<int32_t>(i));
 }
 
 cudaError_t launch_rope_back(const float* dq, const float* dks, const float* dvs, const float2* rope, int n, int n_q,

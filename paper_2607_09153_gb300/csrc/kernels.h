@@ -268,27 +268,62 @@ cudaError_t launch_rms_back(const float* h, const __nv_bfloat16* h_bf16, const _
                             __nv_bfloat16* o_lo, cudaStream_t st);
 cudaError_t launch_silu_back(const float* da, const float* gu, int n, int ff, __nv_bfloat16* o_hi,
                              __nv_bfloat16* o_lo, cudaStream_t st);
-// The attention read-out's backward of one layer.  units: int4 {b, g, j0, j1} (candidate b's logical
-// pages j0 .. j1 - 1 of kv head g); shared[page] != 0 for pages several candidates read (their
-// gradient accumulates atomically and must be zeroed first).
+// An item of the tensor-core attention backward: up to kBackTilePages pages of one kv head and the
+// candidates that read all of them.
+struct BackItem {
+  int32_t g;
+  int32_t page_off, n_pages;   // in the page list (entries with kBackAtomicPage set accumulate atomically)
+  int32_t n_tokens;            // valid tokens (only the last page may be partial)
+  int32_t cand_off, n_cands;   // in the candidate list
+  int32_t pad[2];
+};
+constexpr int kBackTilePages = 8;
+constexpr uint32_t kBackAtomicPage = 0x80000000u;
+// Host schedule of the backward: items for the tensor-core form (group <= 8), CTA k's being
+// items[cta_item[k]] .. items[cta_item[k + 1] - 1], or units {b, g, j0, j1}
+// (candidate b's logical pages j0 .. j1 - 1 of kv head g) for the CUDA-core form; atomic[page] != 0 for
+// pages whose gradient several items or units add to (they accumulate atomically and must be zeroed
+// first).
+struct BackPlan {
+  std::vector<BackItem> items;
+  std::vector<uint32_t> item_pages;
+  std::vector<int32_t> item_cands, cta_item;
+  std::vector<int4> units;
+  std::vector<uint8_t> atomic;      // [n_pages]
+  std::vector<int32_t> lists;       // the atomic pages, then every referenced page
+  int n_atomic = 0;
+};
+void plan_attn_back(const int32_t* bt, const int32_t* sl, int n, int max_blocks, int64_t n_pages, int n_kv,
+                    bool tensor_cores, int n_sms, BackPlan& p);
+// The attention read-out's backward of one layer.
 struct AttnBackArgs {
   int n, n_q, n_kv, hd;
   const float *q, *kself, *vself, *o, *dout, *lse;   // forward saves [n][...] and d(out) [n][n_q hd]
   float *D, *dq, *dks, *dvs;                         // [n][n_q], [n][n_q hd], [n][n_kv hd] x 2
+  // tensor-core form: the plan (BackPlan), the rows' operand blocks and (lse, D) [n][n_kv][8] (workspace),
+  // the pool's 2 KB-box map (or NULL: the CUDA-core form) and this layer's first page unit
+  const BackItem* items;
+  const int32_t* cta_item;
+  int n_ctas;
+  const uint32_t* item_pages;
+  const int32_t* item_cands;
+  uint8_t* ops;
+  float2* meta;
+  const CUtensorMap* tm_pool_tc = nullptr;
+  int64_t layer_page0 = 0;
+  // CUDA-core form
   const int4* units;
   int n_units;
   const int32_t* seq_lens;
   const int32_t* block_table;
   int max_blocks;
   const __nv_bfloat16* pool_layer;                   // [n_pages][2][n_kv][16][hd]
-  const uint8_t* shared;
-  float* grad_layer;                                 // same layout, fp32
+  const uint8_t* shared;                             // BackPlan::atomic
+  float* grad_layer;                                 // pool layout, fp32
   int* err;                                          // device error word (a bounded wait that gave up)
-  // the pool's tensor map (the forward's, one box per page) and this layer's first page unit; with
-  // group <= 8 the backward then runs on the tensor cores, else (or when NULL) on the CUDA cores
-  const CUtensorMap* tm_pool = nullptr;
-  int64_t layer_page0 = 0;
 };
+// bytes of AttnBackArgs::ops for n rows
+inline size_t attn_back_ops_bytes(size_t n, int n_kv, int hd) { return n * n_kv * 4 * (hd / 64) * 1024; }
 // units hold at most this many pages (the pages kernel stages them all in shared memory)
 constexpr int kBackUnitPagesMax = 8;
 cudaError_t grad_configure();

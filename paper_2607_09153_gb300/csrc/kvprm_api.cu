@@ -78,12 +78,19 @@ struct GradState {
   __nv_bfloat16 *ghi = nullptr, *glo = nullptr;   // a gradient as the next product's bf16 hi/lo input
   int tm_npad = -1;
   CUtensorMap tm_d_hi{}, tm_d_lo{}, tm_gu_hi{}, tm_gu_lo{}, tm_qkv_hi{}, tm_qkv_lo{};
-  // per call: work units of the attention backward, shared-page flags and page lists
+  uint8_t* ops = nullptr;    // tensor-core attention backward: the rows' operand blocks, their (lse, D)
+  float2* meta = nullptr;
+  // per call: the attention backward's schedule, atomic-page flags and page lists (BackPlan)
+  kvprm::BackPlan plan;
   int4* units = nullptr;
   size_t units_cap = 0;
+  kvprm::BackItem* items = nullptr;
+  uint32_t* item_pages = nullptr;
+  int32_t *item_cands = nullptr, *cta_item = nullptr;
+  size_t items_cap = 0, item_pages_cap = 0, item_cands_cap = 0, cta_item_cap = 0;
   uint8_t* shared = nullptr;
   size_t shared_cap = 0;
-  int32_t* lists = nullptr;   // [shared pages][all referenced pages]
+  int32_t* lists = nullptr;   // [atomic pages][all referenced pages]
   size_t lists_cap = 0;
   int n_shared = 0, n_ref = 0;   // of the last call
   float* grad_own = nullptr;   // kvprm_steer's gradient buffer
@@ -320,7 +327,13 @@ void free_ctx(kvprm_ctx* c) {
     cudaFree(g.dh);
     cudaFree(g.ghi);
     cudaFree(g.glo);
+    cudaFree(g.ops);
+    cudaFree(g.meta);
     cudaFree(g.units);
+    cudaFree(g.items);
+    cudaFree(g.item_pages);
+    cudaFree(g.item_cands);
+    cudaFree(g.cta_item);
     cudaFree(g.shared);
     cudaFree(g.lists);
     cudaFree(g.grad_own);
@@ -1066,38 +1079,39 @@ int ensure_grad(kvprm_ctx* ctx, cudaStream_t st) {
   const size_t Bm = static_cast<size_t>(ctx->cfg.max_candidates);
   const size_t nqh = static_cast<size_t>(m.n_q) * m.hd, nkh = static_cast<size_t>(m.n_kv) * m.hd;
   int rc;
-  // saves: one allocation carved per array
-  const size_t per_layer = Bm * (nqh + 2 * nkh + nqh + m.n_q + 2 * static_cast<size_t>(m.d) + 2 * static_cast<size_t>(m.ff));
+  // saves: one allocation carved per array, each array at a multiple of 64 floats (the kernels move 16
+  // bytes at a time; n_q per candidate is the one size that need not be a multiple of four)
+  auto al64 = [](size_t x) { return (x + 63) / 64 * 64; };
+  const size_t save_elems[8] = {Bm * nqh, Bm * nkh, Bm * nkh, Bm * nqh, Bm * m.n_q, Bm * m.d, Bm * m.d,
+                                Bm * 2 * static_cast<size_t>(m.ff)};
+  size_t save_total = 0;
+  for (size_t e : save_elems) save_total += al64(e * NL);
   float* base = nullptr;
-  if ((rc = dalloc(ctx, &base, per_layer * NL, "backward saves"))) return rc;
+  if ((rc = dalloc(ctx, &base, save_total, "backward saves"))) return rc;
   FwdSaves& sv = g.sv;
   float* p = base;
-  auto take = [&](size_t per) {
-    float* r = p;
-    p += per * NL;
-    return r;
-  };
-  sv.q = take(Bm * nqh);
-  sv.k = take(Bm * nkh);
-  sv.v = take(Bm * nkh);
-  sv.o = take(Bm * nqh);
-  sv.lse = take(Bm * m.n_q);
-  sv.hmid = take(Bm * m.d);
-  sv.hout = take(Bm * m.d);
-  sv.gu = take(Bm * 2 * static_cast<size_t>(m.ff));
+  float** const save_ptr[8] = {&sv.q, &sv.k, &sv.v, &sv.o, &sv.lse, &sv.hmid, &sv.hout, &sv.gu};
+  for (int i = 0; i < 8; ++i) {
+    *save_ptr[i] = p;
+    p += al64(save_elems[i] * NL);
+  }
   // backward buffers
   const size_t wmax = std::max<size_t>(std::max<size_t>(m.ff, m.d), nqh);
   const size_t gmax = std::max<size_t>(std::max<size_t>(2 * static_cast<size_t>(m.ff), m.qkv_rows), m.d);
   float* bb = nullptr;
-  if ((rc = dalloc(ctx, &bb, Bm * (m.d + wmax + m.n_q + nqh + 2 * nkh), "backward buffers"))) return rc;
+  if ((rc = dalloc(ctx, &bb, Bm * (m.d + wmax + nqh + 2 * nkh) + al64(Bm * m.n_q), "backward buffers"))) return rc;
   g.dh = bb;
   g.tmp = g.dh + Bm * m.d;
   g.D = g.tmp + Bm * wmax;
-  g.dq = g.D + Bm * m.n_q;
+  g.dq = g.D + al64(Bm * m.n_q);
   g.dks = g.dq + Bm * nqh;
   g.dvs = g.dks + Bm * nkh;
   if ((rc = dalloc(ctx, &g.ghi, static_cast<size_t>(ctx->npad_max) * gmax, "backward hi"))) return rc;
   if ((rc = dalloc(ctx, &g.glo, static_cast<size_t>(ctx->npad_max) * gmax, "backward lo"))) return rc;
+  if (m.n_q / m.n_kv <= 8 && !ctx->grad_cuda_cores) {
+    if ((rc = dalloc(ctx, &g.ops, kvprm::attn_back_ops_bytes(Bm, m.n_kv, m.hd), "backward operands"))) return rc;
+    if ((rc = dalloc(ctx, &g.meta, Bm * m.n_kv * 8, "backward row statistics"))) return rc;
+  }
   // transposed weights: W [out][in] -> W^T [in][out], from the borrowed weights' tensor-map bases
   g.tm_qkv.resize(NL);
   g.tm_o.resize(NL);
@@ -1175,36 +1189,24 @@ int score_grad_device(kvprm_ctx* ctx, const void* kv_pages, int64_t n_pages, con
   const int NL = ctx->cfg.n_layers, mb = ctx->cfg.max_blocks_per_seq;
   const int np = (n + 15) / 16 * 16;
   if ((rc = ensure_grad_maps(ctx, np))) return rc;
-  // host plan: work units (candidate, kv head, <= 8 pages) and the pages several candidates read
-  std::vector<int4> units;
-  std::vector<uint8_t> refs(static_cast<size_t>(n_pages > 0 ? n_pages : 1), 0);
-  constexpr int kUnitPages = kvprm::kBackUnitPagesMax;
-  for (int b = 0; b < n; ++b) {
-    const int pages = (sl[b] + 15) / 16;
-    for (int j = 0; j < pages; ++j) {
-      uint8_t& r = refs[bt[static_cast<int64_t>(b) * mb + j]];
-      if (r < 2) ++r;
-    }
-    for (int gg = 0; gg < m.n_kv; ++gg)
-      for (int j0 = 0; j0 < pages; j0 += kUnitPages) units.push_back(make_int4(b, gg, j0, std::min(pages, j0 + kUnitPages)));
-  }
-  std::vector<int32_t> lists;   // shared pages, then every referenced page
-  for (int64_t p = 0; p < n_pages; ++p)
-    if (refs[p] >= 2) lists.push_back(static_cast<int32_t>(p));
-  const int n_shared = static_cast<int>(lists.size());
-  for (int64_t p = 0; p < n_pages; ++p)
-    if (refs[p] >= 1) lists.push_back(static_cast<int32_t>(p));
-  for (auto& r : refs) r = r >= 2 ? 1 : 0;
-  if ((rc = grow(ctx, &g.units, &g.units_cap, std::max<size_t>(units.size(), 1), "backward units"))) return rc;
-  if ((rc = grow(ctx, &g.shared, &g.shared_cap, refs.size(), "shared-page flags"))) return rc;
-  if ((rc = grow(ctx, &g.lists, &g.lists_cap, std::max<size_t>(lists.size(), 1), "page lists"))) return rc;
-  if (!units.empty())
-    CK(cudaMemcpyAsync(g.units, units.data(), sizeof(int4) * units.size(), cudaMemcpyHostToDevice, st), "units");
-  CK(cudaMemcpyAsync(g.shared, refs.data(), refs.size(), cudaMemcpyHostToDevice, st), "shared flags");
-  if (!lists.empty())
-    CK(cudaMemcpyAsync(g.lists, lists.data(), sizeof(int32_t) * lists.size(), cudaMemcpyHostToDevice, st), "lists");
+  kvprm::BackPlan& bp = g.plan;
+  kvprm::plan_attn_back(bt, sl, n, mb, n_pages, m.n_kv, g.ops != nullptr, ctx->num_sms, bp);
+  const int n_shared = bp.n_atomic;
+  auto send = [&](auto** dst, size_t* cap, const auto& src, const char* what) -> int {
+    if ((rc = grow(ctx, dst, cap, std::max<size_t>(src.size(), 1), what))) return rc;
+    if (!src.empty())
+      CK(cudaMemcpyAsync(*dst, src.data(), sizeof(src[0]) * src.size(), cudaMemcpyHostToDevice, st), what);
+    return KVPRM_OK;
+  };
+  if ((rc = send(&g.units, &g.units_cap, bp.units, "backward units"))) return rc;
+  if ((rc = send(&g.items, &g.items_cap, bp.items, "backward items"))) return rc;
+  if ((rc = send(&g.item_pages, &g.item_pages_cap, bp.item_pages, "backward item pages"))) return rc;
+  if ((rc = send(&g.item_cands, &g.item_cands_cap, bp.item_cands, "backward item candidates"))) return rc;
+  if ((rc = send(&g.cta_item, &g.cta_item_cap, bp.cta_item, "backward item ranges"))) return rc;
+  if ((rc = send(&g.shared, &g.shared_cap, bp.atomic, "atomic-page flags"))) return rc;
+  if ((rc = send(&g.lists, &g.lists_cap, bp.lists, "page lists"))) return rc;
   g.n_shared = n_shared;
-  g.n_ref = static_cast<int>(lists.size()) - n_shared;
+  g.n_ref = static_cast<int>(bp.lists.size()) - n_shared;
   *n_ref_out = g.n_ref;
   const int64_t page_elems = static_cast<int64_t>(2) * m.n_kv * 16 * m.hd;
   const size_t Bm = static_cast<size_t>(ctx->cfg.max_candidates);
@@ -1253,8 +1255,15 @@ int score_grad_device(kvprm_ctx* ctx, const void* kv_pages, int64_t n_pages, con
       a.dq = g.dq;
       a.dks = g.dks;
       a.dvs = g.dvs;
+      a.items = g.items;
+      a.cta_item = g.cta_item;
+      a.n_ctas = bp.cta_item.empty() ? 0 : static_cast<int>(bp.cta_item.size()) - 1;
+      a.item_pages = g.item_pages;
+      a.item_cands = g.item_cands;
+      a.ops = g.ops;
+      a.meta = g.meta;
       a.units = g.units;
-      a.n_units = static_cast<int>(units.size());
+      a.n_units = static_cast<int>(bp.units.size());
       a.seq_lens = ctx->tables_d;
       a.block_table = ctx->tables_d + ctx->cfg.max_candidates;
       a.max_blocks = mb;
@@ -1262,7 +1271,7 @@ int score_grad_device(kvprm_ctx* ctx, const void* kv_pages, int64_t n_pages, con
       a.shared = g.shared;
       a.grad_layer = grad + l * n_pages * page_elems;
       a.err = ctx->err_d;
-      a.tm_pool = kv_pages && !ctx->grad_cuda_cores ? &ctx->tm_pool : nullptr;   // the forward's map of this pool
+      a.tm_pool_tc = g.ops ? &ctx->tm_pool_tc : nullptr;   // the forward's map of this pool
       a.layer_page0 = static_cast<int64_t>(l) * n_pages;
       CK(kvprm::launch_attn_back(a, s), "attention backward");
       if (l == 0) break;   // below layer 0 lies only the verify token's embedding
@@ -1290,7 +1299,10 @@ int score_grad_device(kvprm_ctx* ctx, const void* kv_pages, int64_t n_pages, con
       ctx->work_host.fuse_cs, ctx->work_host.n_tc > 0 ? 1 : 0, ctx->work_host.n_ctas, ctx->debug_flags,
       ctx->use_pdl ? 1 : 0, ctx->trace ? 1 : 0, ctx->layer_waits ? 1 : 0, ctx->as.layer_pages,
       reinterpret_cast<int64_t>(kv_pages), n_pages, reinterpret_cast<int64_t>(grad),
-      static_cast<int64_t>(units.size()), n_shared, static_cast<int64_t>(lists.size()),
+      static_cast<int64_t>(bp.units.size()), static_cast<int64_t>(bp.cta_item.size()), n_shared,
+      static_cast<int64_t>(bp.lists.size()), reinterpret_cast<int64_t>(g.items),
+      reinterpret_cast<int64_t>(g.item_pages), reinterpret_cast<int64_t>(g.item_cands),
+      reinterpret_cast<int64_t>(g.cta_item),
       reinterpret_cast<int64_t>(g.units), reinterpret_cast<int64_t>(g.lists), reinterpret_cast<int64_t>(g.shared),
       ctx->grad_cuda_cores ? 1 : 0, reinterpret_cast<int64_t>(ctx->pool_ptr)};
   if (!(g.gexec && key == g.gkey)) {

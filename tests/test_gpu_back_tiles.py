@@ -1,0 +1,50 @@
+"""The tensor-core attention backward at the edges of its tiles (8 pages of 16 tokens, 4 candidates a
+step, 8 rows a candidate): shared runs one page short of a tile, one over and several tiles long;
+candidates that fill a step, leave one over or are split over tiles because the pages alone would
+leave the GPU idle; both head widths; the narrowest and widest groups; row counts whose workspace
+arrays do not end on 16 bytes.  Against the fp64 oracle with the gradient's tolerance
+(tests/test_gpu_steering.py), and eagerly against the captured graph."""
+import pytest
+
+import kvsynth as ks
+from tests.gpu_util import require_gpu
+from tests.test_gpu_steering import _compare, _gpu_grad, _oracle
+
+pytestmark = pytest.mark.gpu
+
+
+def arch(hd, group, n_kv=2):
+    return ks.Arch(1, 256, group * n_kv, n_kv, hd, 256)
+
+
+@pytest.mark.parametrize("hd, group, cands, pages, own", [
+    (128, 7, 2, 1, [1, 16]),
+    (128, 7, 3, 7, [0, 5, 33]),
+    (128, 8, 4, 8, [16, 17, 0, 140]),
+    (128, 1, 5, 9, [3] * 5),
+    (128, 6, 9, 17, [0] * 9),
+    (64, 8, 8, 16, [20, 1] * 4),
+    (64, 2, 13, 25, [130] * 13),
+    (64, 7, 5, 8, [15] * 5),
+])
+def test_shared_runs(hd, group, cands, pages, own):
+    require_gpu()
+    t = ks.Tables.make(0.2)
+    segs = [[(1, 16 * pages)] + ([(10 + b, own[b])] if own[b] else []) for b in range(cands)]
+    w = ks.workload_from_segments("back_tiles", arch(hd, group), 700 + pages, segs, gain_std=0.2)
+    p, grad, dev, sc = _gpu_grad(w, t)
+    p_ref, ref, _, _ = _oracle(w, t)
+    _compare(f"hd {hd} G {group}: {cands} candidates, {pages} shared pages", w, p, grad, p_ref, ref)
+    sc.close()
+
+
+@pytest.mark.parametrize("n, group, n_kv", [(65, 7, 1), (27, 7, 2), (3, 5, 1), (66, 3, 1)])
+def test_odd_rows(n, group, n_kv):
+    # n x n_q that is no multiple of four (n >= 64 takes the large-batch projections)
+    require_gpu()
+    t = ks.Tables.make(0.2)
+    w = ks.distinct("back_rows", arch(64, group, n_kv), 720 + n, [(37 * b) % 90 for b in range(n)], gain_std=0.2)
+    p, grad, dev, sc = _gpu_grad(w, t)
+    p_ref, ref, _, _ = _oracle(w, t)
+    _compare(f"{n} candidates of {group * n_kv} heads", w, p, grad, p_ref, ref)
+    sc.close()
