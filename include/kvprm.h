@@ -388,6 +388,14 @@ typedef struct {
  * the candidate's L and partial slot fuse_cs * p + r; rank 0 merges the
  * pair's slots in the same launch, so no combine launch follows. */
 #define KVPRM_PLAN_FUSE 16
+/* share | KVPRM_PLAN_PACK (what scoring contexts do): a partial last page that several candidates
+ * reference with the same number of valid tokens ends the shared run of exactly those candidates
+ * (last_valid of a kind-1 or kind-2 segment may then be below 16), and, when no kind-1 run is
+ * planned and the private runs are short, these are packed: a kind-3 segment holds n_cands <= 8
+ * lanes, one per warp, lane i being six ints from cands[offset + 6 i] on -- candidate, kv head,
+ * offset into pages, pages, valid tokens of the last page, partial slot -- and n_pages is the
+ * longest lane's. */
+#define KVPRM_PLAN_PACK 32
 KVPRM_API int kvprm_plan_attention(const int32_t* block_table, int32_t max_blocks_per_seq, const int32_t* seq_lens,
                                    int32_t n_candidates, int32_t n_kv_heads, int32_t group, int32_t n_ctas,
                                    int32_t share, kvprm_attn_plan* plan);

@@ -41,6 +41,7 @@
 #include <algorithm>
 #include <cstring>
 #include <climits>
+#include <cmath>
 #include <unordered_map>
 #include <vector>
 
@@ -73,6 +74,11 @@ constexpr int64_t kSharedCostPerCand = 2;
 // (8 / n)-th page of a stage and writing its own partial slot: warp w scores candidate w % n,
 // pages p with p % (8 / n) == w / n, into slot w of the segment.  (n <= 4 keeps every warp busy.)
 __host__ __device__ constexpr int shared_reps(int n_cands) { return kConsumerWarps / n_cands; }
+// A packed segment (kind 3): up to eight lanes, one per consumer warp, each a short private run of one
+// (candidate, kv head) that its warp scores alone, a page per stage.  Lane w is kLaneInts ints from
+// cands[seg.cand + w kLaneInts] on: candidate, kv head, page offset, pages, valid tokens of the last
+// page, partial slot.
+constexpr int kLaneInts = 6;
 // The tensor-core launch, in the same units, when it runs beside the private pages' launch: a CTA
 // costs kTcChunkCost per 64-token chunk plus kTcCtaCost once (the first query load and pages'
 // latency, the last output read-out).  Fitted to the SM split that measured fastest on the beam
@@ -116,12 +122,20 @@ struct AttnSmem {
 };
 static_assert(AttnSmem<128>::kDynamic <= 227 * 1024, "attention shared memory exceeds the per-block limit");
 
-template <int HD, bool TWO_ROWS>
+// FORM: what the plan's segments are -- runs (kinds 0 and 1), packs (kind 3) or one private run per CTA
+// of a fused-combine plan.  An image each: a CTA runs its epilogue once and most of its code a few
+// times, so what it does not need only costs instruction fetches (packs inside the runs' image cost the
+// MCTS attention ~2 us per layer).
+constexpr int kFormRuns = 0, kFormPacked = 1, kFormFused = 2;
+
+template <int HD, bool TWO_ROWS, int FORM>
 __global__ void __launch_bounds__(kThreads, 1) attn_kernel(
     const __grid_constant__ CUtensorMap tm_pool, int64_t layer_page0, AttnWork wk,
     const __nv_bfloat16* __restrict__ q_hi, const __nv_bfloat16* __restrict__ q_lo, int n_q, int n_kv, int group,
     float* __restrict__ part_o, float* __restrict__ part_ml, AttnMerge mg, int* err, unsigned long long* ts) {
   using SM = AttnSmem<HD>;
+  constexpr bool packed = FORM == kFormPacked, fused = FORM == kFormFused;
+  static_assert(!TWO_ROWS || FORM == kFormRuns, "packs and the fused combine have groups of at most eight heads");
   trace_begin(ts);
 
   extern __shared__ uint8_t smem_raw[];
@@ -162,16 +176,29 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(
       for (int si = seg0; si < seg1 && ok; ++si) {
         const AttnSeg sg = wk.segs[si];
         const int32_t* pg = wk.pages + sg.page_off;
-        for (int p0 = 0; p0 < sg.n_pages; p0 += kPagesPerStage, ++u) {
+        const int32_t* ln = wk.cands + sg.cand;   // packed: the lanes, longest first
+        int n_lanes = packed ? sg.n_cands : 0;    // those with a page in this stage
+        for (int p0 = 0; p0 < sg.n_pages; p0 += packed ? 1 : kPagesPerStage, ++u) {
           const int slot = static_cast<int>(u % kStages);
           if (u >= static_cast<uint32_t>(kStages) &&
               !mbar_wait(&empty[slot], ((u / kStages) & 1u) ^ 1u, err)) {
             ok = false;
             break;
           }
+          uint8_t* stg = ring + slot * SM::kStageBytes;
+          if (packed) {   // page p0 of every lane that has one
+            while (__ldg(ln + (n_lanes - 1) * kLaneInts + 3) <= p0) --n_lanes;
+            mbar_arrive_expect_tx(&full[slot], static_cast<uint32_t>(n_lanes) * SM::kPageBytes);
+#pragma unroll 1
+            for (int w = 0; w < n_lanes; ++w) {
+              const int32_t page = __ldg(wk.pages + __ldg(ln + w * kLaneInts + 2) + p0);
+              tma_load_5d(stg + w * SM::kPageBytes, &tm_pool, &full[slot], 0, 0, 0, __ldg(ln + w * kLaneInts + 1),
+                          static_cast<int32_t>(2 * (layer_page0 + page)), pol);
+            }
+            continue;
+          }
           const int npg = min(kPagesPerStage, sg.n_pages - p0);
           mbar_arrive_expect_tx(&full[slot], static_cast<uint32_t>(npg) * SM::kPageBytes);
-          uint8_t* stg = ring + slot * SM::kStageBytes;
           for (int pi = 0; pi < npg; ++pi) {
             const int64_t phys = __ldg(pg + p0 + pi);
             tma_load_5d(stg + pi * SM::kPageBytes, &tm_pool, &full[slot], 0, 0, 0, sg.g,
@@ -191,7 +218,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(
     // no warp can arrive for a slot's next use early.
     grid_dep_wait();   // q is written by the preceding kernel
     if (warp == 0 && lane == 0) trace_event(ts, 0);   // the query is ready
-    if (!TWO_ROWS && wk.fuse_cs > 0) {
+    if (fused) {
       // fused combine, before the pages: the verify token's own logit of head `warp`
       // (q . k_self / sqrt(hd), log2 units) and the pair's v_self, into shared memory
       const int pr = blockIdx.x / wk.fuse_cs, b = pr / n_kv, g = pr - b * n_kv;
@@ -213,29 +240,35 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(
     uint32_t u = 0, n_priv = 0;
     for (int si = seg0; si < seg1; ++si) {
       const AttnSeg sg = wk.segs[si];
-      const bool shared = sg.kind == 1;
+      const bool shared = FORM == kFormRuns && sg.kind == 1;
       // the candidate this warp scores in this segment, -1 if none (and, in a shared run, which of the
       // candidate's replica warps it is)
       const int reps = shared ? shared_reps(sg.n_cands) : 1;
-      const int cand = shared ? (warp < reps * sg.n_cands ? wk.cands[sg.cand + warp % sg.n_cands] : -1)
-                              : (warp < sg.n_pages ? sg.cand : -1);
+      const int32_t* ln = wk.cands + sg.cand + warp * kLaneInts;   // packed: warp w scores lane w, a page per stage
+      const bool in_lane = packed && warp < sg.n_cands;
+      const int ln_np = in_lane ? __ldg(ln + 3) : 0, ln_last = in_lane ? __ldg(ln + 4) : 0;
+      const int cand = packed   ? (in_lane ? __ldg(ln) : -1)
+                       : shared ? (warp < reps * sg.n_cands ? wk.cands[sg.cand + warp % sg.n_cands] : -1)
+                                : (warp < sg.n_pages ? sg.cand : -1);
+      const int g = in_lane ? __ldg(ln + 1) : sg.g;
       const int part = shared ? warp / sg.n_cands : 0;
       WarpQ<HD> q;
       if (cand >= 0) {
-        const int64_t q0 = (static_cast<int64_t>(cand) * n_q + static_cast<int64_t>(sg.g) * group) * HD;
+        const int64_t q0 = (static_cast<int64_t>(cand) * n_q + static_cast<int64_t>(g) * group) * HD;
         load_q<HD, TWO_ROWS>(q, q_hi + q0, q_lo + q0, group, lane);
       }
       WarpState<HD> st;
       st.reset();
-      for (int p0 = 0; p0 < sg.n_pages; p0 += kPagesPerStage, ++u) {
+      for (int p0 = 0; p0 < sg.n_pages; p0 += packed ? 1 : kPagesPerStage, ++u) {
         const int slot = static_cast<int>(u % kStages);
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&full[slot], (u / kStages) & 1u, err));
         if (ok && cand >= 0) {
           const uint32_t sbase = smem_u32(ring + slot * SM::kStageBytes);
-          const int npg = min(kPagesPerStage, sg.n_pages - p0);
-          if (!shared) {   // page `warp` of this stage
-            if (warp < npg) {
-              const int valid = p0 + warp == sg.n_pages - 1 ? sg.last_valid : 16;
+          const int npg = packed ? 1 : min(kPagesPerStage, sg.n_pages - p0);
+          if (!shared) {   // page `warp` of this stage (packed: this warp's lane's page p0)
+            if (packed ? p0 < ln_np : warp < npg) {
+              const int valid = packed ? (p0 == ln_np - 1 ? ln_last : 16)
+                                       : (p0 + warp == sg.n_pages - 1 ? sg.last_valid : 16);
               const uint32_t kb = sbase + warp * SM::kPageBytes;
               process_page<HD, TWO_ROWS>(q, kb, kb + SM::kBlockBytes, valid, lane, st);
             }
@@ -259,7 +292,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(
         if (lane == 0) mbar_arrive(&empty[slot]);
       }
       if (cand >= 0 && ok) finish_state<HD, TWO_ROWS>(st);
-      if (!shared && !TWO_ROWS) {
+      if (!shared && !packed && !TWO_ROWS) {
         // hand the warp's state to the merger warp (one slot per private
         // segment); wait only until it has read the previous segment's states
         if (n_priv > 0) ok = __all_sync(0xffffffffu, mbar_wait(seg_free, (n_priv - 1) & 1u, err)) && ok;
@@ -269,12 +302,12 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(
         ++n_priv;
       } else if (cand >= 0 && ok) {
         // this warp's own partial slot
-        const int slot_id = shared ? wk.slots[sg.slot + warp] : sg.slot + warp;
+        const int slot_id = packed ? __ldg(ln + 5) : shared ? wk.slots[sg.slot + warp] : sg.slot + warp;
         store_state_slot<HD, TWO_ROWS>(st, slot_id, group, lane, part_o, part_ml);
       }
     }
     if (lane == 0) trace_event(ts, 1);   // this warp has scored every page of its CTA
-    if (!TWO_ROWS && wk.fuse_cs > 0) {
+    if (fused) {
       // fused combine (one private run per CTA): once every consumer warp has stashed its state and
       // read its last stage, warp r folds query row r of the eight states into the idle ring
       named_bar_sync(3, kConsumerWarps * 32);
@@ -284,14 +317,14 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(
       }
     }
 
-  } else if (warp == kMergerWarp && !TWO_ROWS) {
+  } else if (warp == kMergerWarp && !TWO_ROWS && FORM == kFormRuns) {
     // ------------------------------------------------ merger
     // For every private segment, in order: fold the eight consumer warps'
     // (m, l, O) into the segment's partial slot,
     //   M = max_w m_w, L = sum_w 2^(m_w - M) l_w, O = sum_w 2^(m_w - M) O_w.
     uint32_t k = 0;
     bool ok = true;
-    for (int si = wk.fuse_cs > 0 ? seg1 : seg0; si < seg1; ++si) {   // fused plans: the consumers merge
+    for (int si = seg0; si < seg1; ++si) {   // (fused plans: the consumers merge)
       const AttnSeg sg = wk.segs[si];
       if (sg.kind != 0) continue;
       if (ok) ok = __all_sync(0xffffffffu, mbar_wait(seg_full, k & 1u, err));
@@ -302,7 +335,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(
     }
     if (lane == 0) trace_event(ts, 2);   // every private run of this CTA is merged
   }
-  if (!TWO_ROWS && wk.fuse_cs > 0) {   // fused plans have group <= 8
+  if (fused) {   // fused plans have group <= 8
     // The cluster scored one (candidate, kv head); every rank left its (M, L, O) per query row at
     // the start of its ring and the verify token's own logits in kSelf.  Rank k then produces
     // head-dimension slice k of every row, reading the ranks' states through distributed shared
@@ -324,7 +357,7 @@ __global__ void __launch_bounds__(kThreads, 1) attn_kernel(
       const float* st_o = reinterpret_cast<const float*>(ring);
       const float* st_ml = st_o + 8 * HD;
       const float* s_self = reinterpret_cast<const float*>(base + SM::kSelf);
-#pragma unroll
+#pragma unroll 1
       for (int i = 0; i < kOut; ++i) {
         const int idx = threadIdx.x + i * kMergeThreads;
         if (idx >= group * slice) break;
@@ -757,7 +790,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) attn_tc_kernel(
         long long t0 = tic();
         if (ok) ok = __all_sync(0xffffffffu, mbar_wait(&s_full[b], (u / kTcSBufs) & 1u, err));
         // tokens of my 32 that exist (none after a timeout: x is then never read)
-        const int valid = ok ? min(kTcChunkPages, sg.n_pages - c * kTcChunkPages) * 16 - 32 * hsel : 0;
+        const int valid =
+            ok ? min(16 * kTcChunkPages, 16 * (sg.n_pages - c * kTcChunkPages) - 16 + sg.last_valid) - 32 * hsel : 0;
         tc_fence_after();
         if (lane == 0 && warp == 2) {
           toc(4, t0);
@@ -936,6 +970,92 @@ struct Run {
   int64_t cost;    // per page and kv head
 };
 
+// Short private runs, packed.  A private segment is scored by all eight warps, a page each per stage,
+// and ends with a query load before it and a merge of eight states after it: ~2.5 us that its own
+// pages must hide.  Runs of a dozen pages do not (201 ragged caches of up to 333 tokens, 7B heads: 6.3
+// segments per CTA, 37 us per layer for 79 MB).  Packed, each warp takes a (candidate, kv head) by
+// itself, so eight runs share those costs and nothing is merged: 16.6 us, the combine after it (one or
+// two slots a run) 7.8 -> 6.3 us.  Runs longer than L
+// pages are cut into equal lanes, L the least (but at least kPackMinPages, each lane being a partial
+// slot for the combine) that gives every warp of the launch at most K lanes; lanes of about the same
+// length make a pack.  Chosen when its estimated time is clearly below the other form's: a stage of
+// eight pages streams in ~1.5 us per SM, a warp scores a page in ~1.1 us.  Long runs stream at HBM
+// rate either way and keep the other form.
+constexpr int kPackMinPages = 4;
+
+bool pack_runs(const std::vector<Run>& runs, int n_kv, int n_ctas, int classic_ctas, AttnWorkHost& w,
+               std::vector<int>& seg_cta, int* ctas) {
+  int64_t pages = 0, n_pairs = 0;
+  int most = 0;
+  for (const Run& r : runs) {
+    if (r.kind == 1) return false;
+    if (r.kind != 0) continue;
+    pages += static_cast<int64_t>(r.n_pages) * n_kv;
+    n_pairs += n_kv;
+    most = std::max(most, r.n_pages);
+  }
+  if (n_pairs == 0 || n_ctas < 1 || classic_ctas < 1) return false;
+  const int64_t warps = static_cast<int64_t>(kConsumerWarps) * n_ctas, K = (n_pairs + warps - 1) / warps;
+  auto lanes_of = [&](int L) {
+    int64_t k = 0;
+    for (const Run& r : runs)
+      if (r.kind == 0) k += static_cast<int64_t>((r.n_pages + L - 1) / L) * n_kv;
+    return k;
+  };
+  int lo = std::min(kPackMinPages, most), hi = most;
+  while (lo < hi) {
+    const int mid = (lo + hi) / 2;
+    if (lanes_of(mid) <= warps * K)
+      hi = mid;
+    else
+      lo = mid + 1;
+  }
+  const double segs = static_cast<double>(n_pairs + classic_ctas), per = static_cast<double>(pages) / segs;
+  const double classic = segs / classic_ctas * std::max(0.19 * per, 1.1 * std::ceil(per / kPagesPerStage) + 2.5);
+  if (static_cast<double>(K) * (1.52 * lo + 3.0) >= 0.75 * classic) return false;
+  struct Lane {
+    int32_t cand, g, page_off, n_pages, last_valid;
+  };
+  std::vector<Lane> lanes;
+  lanes.reserve(static_cast<size_t>(lanes_of(lo)));
+  for (const Run& r : runs) {
+    if (r.kind != 0) continue;
+    const int k = (r.n_pages + lo - 1) / lo;
+    for (int g = 0; g < n_kv; ++g)
+      for (int i = 0; i < k; ++i) {
+        const int p0 = static_cast<int>(static_cast<int64_t>(r.n_pages) * i / k);
+        const int p1 = static_cast<int>(static_cast<int64_t>(r.n_pages) * (i + 1) / k);
+        lanes.push_back(Lane{r.cand, g, r.page_off + p0, p1 - p0, i + 1 == k ? r.last_valid : 16});
+      }
+  }
+  std::stable_sort(lanes.begin(), lanes.end(), [](const Lane& a, const Lane& b) { return a.n_pages > b.n_pages; });
+  // packs longest first, to the CTAs in turn and back again
+  const int packs = static_cast<int>((lanes.size() + kConsumerWarps - 1) / kConsumerWarps);
+  const int C = std::min(n_ctas, packs);
+  for (int k = 0; k < C; ++k)
+    for (int round = 0; round * C < packs; ++round) {
+      const int i = round * C + (round % 2 ? C - 1 - k : k);
+      if (i >= packs) continue;
+      const size_t l0 = static_cast<size_t>(i) * kConsumerWarps;
+      const int nl = static_cast<int>(std::min(lanes.size() - l0, static_cast<size_t>(kConsumerWarps)));
+      AttnSeg s{};
+      s.kind = 3;
+      s.cand = static_cast<int32_t>(w.cands.size());
+      s.n_cands = nl;
+      s.n_pages = lanes[l0].n_pages;
+      s.last_valid = 16;
+      for (int x = 0; x < nl; ++x) {
+        const Lane& ln = lanes[l0 + x];
+        w.cands.insert(w.cands.end(), {ln.cand, ln.g, ln.page_off, ln.n_pages, ln.last_valid,
+                                       w.nslots[static_cast<size_t>(ln.cand) * n_kv + ln.g]++});
+      }
+      w.segs.push_back(s);
+      seg_cta.push_back(k);
+    }
+  *ctas = C;
+  return true;
+}
+
 }  // namespace
 
 CUresult encode_pool_map(PFN_cuTensorMapEncodeTiled_v12000 encode, CUtensorMap* map, const void* pool,
@@ -960,6 +1080,11 @@ size_t attn_slot_capacity(int max_candidates, int n_kv, int num_sms) {
   return static_cast<size_t>(kConsumerWarps) * 2 * (static_cast<size_t>(max_candidates) * n_kv + num_sms);
 }
 
+size_t attn_lane_capacity(int max_candidates, int n_kv, int num_sms) {
+  // K lanes per warp, K = ceil(pairs / warps)
+  return static_cast<size_t>(kLaneInts) * (static_cast<size_t>(max_candidates) * n_kv + kConsumerWarps * num_sms);
+}
+
 // Host planner.
 //  1. Shared pages: full pages that >= 2 candidates reference, each exactly
 //     once, grouped by their exact candidate set; each set is cut into chunks
@@ -982,13 +1107,21 @@ size_t attn_slot_capacity(int max_candidates, int n_kv, int num_sms) {
 //     segments, with one slot per candidate.
 //  3. The slots of each (candidate, kv head) are numbered consecutively from
 //     slot_base.
+//  With `pack` set (what scoring contexts use):
+//  - a partial last page that several candidates reference with the same number of valid tokens (the
+//    verify tokens of a depth-k readout always do) ends the shared run of exactly those candidates
+//    instead of being a one-page private run for each (12 ragged caches at depth 4, 1.5B heads: 96 such
+//    runs, each with its query load and merge beside ~13 shared pages per CTA; the attention took 22.5
+//    us per layer with them, 9.9 without);
+//  - when nothing is left to kind-1 runs and the private runs are short, they are packed (pack_runs).
 // Falls back to private runs when sharing would need more than slot_limit
 // slots; returns false if even those do not fit.
 bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks, int n_kv, int group, int n_ctas,
-                     size_t slot_limit, int share, AttnWorkHost& w) {
+                     size_t slot_limit, int share, bool pack, AttnWorkHost& w) {
   w.tc_seg0 = 0;
   w.n_tc = 0;
   w.n_tc_ctas = 0;
+  w.packed = false;
   w.tc_concurrent = false;
   w.tc_cta.clear();
   w.segs.clear();
@@ -1013,6 +1146,7 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
   // ---- 1. runs
   std::vector<uint8_t> in_group_dense;   // by page id (or, sparse, in_group): scored with a group
   std::unordered_map<int32_t, char> in_group;
+  std::vector<uint8_t> tail_shared(pack ? static_cast<size_t>(n) : 0, 0);   // by candidate: its partial last page is
   bool grouped = false;
   std::vector<Run> runs;
   if (share && total_refs > 0) {
@@ -1062,16 +1196,28 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
         }
       }
     }
-    if (any_dup) {
+    // partial last pages by (page, valid tokens): those listed by several candidates
+    struct Tail {
+      int32_t page, valid, cand;
+    };
+    std::vector<Tail> tails;
+    if (pack) {
+      for (int b = 0; b < n; ++b)
+        if (sl[b] % 16) tails.push_back({bt[static_cast<int64_t>(b) * max_blocks + np[b] - 1], sl[b] % 16, b});
+      std::sort(tails.begin(), tails.end(), [](const Tail& x, const Tail& y) {
+        return x.page != y.page ? x.page < y.page : x.valid != y.valid ? x.valid < y.valid : x.cand < y.cand;
+      });
+      auto twins = [](const Tail& x, const Tail& y) { return x.page == y.page && x.valid == y.valid; };
+      if (std::adjacent_find(tails.begin(), tails.end(), twins) == tails.end()) tails.clear();
+    }
+    if (any_dup || !tails.empty()) {
       std::vector<std::vector<int32_t>> group_cands, group_pages;
+      std::vector<std::pair<int32_t, int32_t>> group_tail;   // (page, valid tokens), valid 0: none
       std::unordered_map<uint64_t, int> gidx;
       if (dense) in_group_dense.assign(static_cast<size_t>(max_page) + 1, 0);
       int last = -1;   // the group of the page before: neighbours in a pool often share one
-      // a page referenced (in full) by the candidates c[0 .. len), in increasing order
-      auto consider = [&](int32_t page, const int32_t* c, size_t len) {
-        if (len < 2) return;
-        for (size_t i = 1; i < len; ++i)
-          if (c[i] == c[i - 1]) return;   // a candidate listing the page twice keeps it private
+      // the group of candidates c[0 .. len), in increasing order; -1 after a hash collision
+      auto group_of = [&](const int32_t* c, size_t len) {
         auto same = [&](int gi) {
           const std::vector<int32_t>& g = group_cands[gi];
           return g.size() == len && std::memcmp(g.data(), c, len * sizeof(int32_t)) == 0;
@@ -1081,34 +1227,57 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
           const uint64_t h = hash_list(c, static_cast<int>(len));
           auto itg = gidx.find(h);
           if (itg != gidx.end()) {
-            if (!same(itg->second)) return;   // hash collision: private
+            if (!same(itg->second)) return -1;
             gi = itg->second;
           } else {
             gi = static_cast<int>(group_cands.size());
             gidx.emplace(h, gi);
             group_cands.emplace_back(c, c + len);
             group_pages.emplace_back();
+            group_tail.emplace_back(0, 0);
           }
           last = gi;
         }
+        return gi;
+      };
+      // a page referenced (in full) by the candidates c[0 .. len), in increasing order
+      auto consider = [&](int32_t page, const int32_t* c, size_t len) {
+        if (len < 2) return;
+        for (size_t i = 1; i < len; ++i)
+          if (c[i] == c[i - 1]) return;   // a candidate listing the page twice keeps it private
+        const int gi = group_of(c, len);
+        if (gi < 0) return;
         group_pages[gi].push_back(page);
         if (dense)
           in_group_dense[page] = 1;
         else
           in_group[page] = 1;
       };
-      if (dense) {
+      if (dense && any_dup) {
         for (int32_t pg = 0; pg <= max_page; ++pg)
           consider(pg, ref_list.data() + ref_off[pg], static_cast<size_t>(ref_off[pg + 1] - ref_off[pg]));
       } else {
         for (auto& kv : refs) consider(kv.first, kv.second.data(), kv.second.size());
+      }
+      std::vector<int32_t> tc;   // a tail's candidates (each has one last page, so a group gets at most one tail)
+      for (size_t i = 0, e; i < tails.size(); i = e) {
+        tc.clear();
+        for (e = i; e < tails.size() && tails[e].page == tails[i].page && tails[e].valid == tails[i].valid; ++e)
+          tc.push_back(tails[e].cand);
+        const int gi = tc.size() > 1 ? group_of(tc.data(), tc.size()) : -1;
+        if (gi < 0) continue;
+        group_tail[gi] = {tails[i].page, tails[i].valid};
+        for (int32_t b : tc) tail_shared[b] = 1;
       }
       grouped = !group_cands.empty();
       for (auto& pgs : group_pages) std::sort(pgs.begin(), pgs.end());   // deterministic contents
       std::vector<int> order(group_cands.size());   // deterministic group order
       for (size_t i = 0; i < order.size(); ++i) order[i] = static_cast<int>(i);
       std::sort(order.begin(), order.end(),
-                [&](int a, int b2) { return group_pages[a].front() < group_pages[b2].front(); });
+                [&](int a, int b2) {
+                  auto key = [&](int x) { return group_pages[x].empty() ? group_tail[x].first : group_pages[x].front(); };
+                  return key(a) != key(b2) ? key(a) < key(b2) : group_cands[a].front() < group_cands[b2].front();
+                });
       // Runs: each group's candidates cut into tiles; tiles of the same kind with the same candidate
       // list (an MCTS tile of 16 leaves under a depth-1 edge and the depth-2 edge above those same
       // leaves) become one run over both groups' pages, so that its query rows are loaded and its
@@ -1150,20 +1319,21 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
         r.kind = t.kind;
         r.cand = static_cast<int>(w.cands.size());
         r.n_cands = static_cast<int>(t.cands.size());
-        if (t.groups.size() == 1) {
-          const int gi = t.groups[0];
-          if (group_off[gi] < 0) {
-            group_off[gi] = static_cast<int>(w.pages.size());
-            w.pages.insert(w.pages.end(), group_pages[gi].begin(), group_pages[gi].end());
-          }
-          r.page_off = group_off[gi];
-          r.n_pages = static_cast<int>(group_pages[gi].size());
+        std::pair<int32_t, int32_t> tail{0, 0};   // of the tile's candidates: the run's last page
+        for (int gi : t.groups)
+          if (group_tail[gi].second) tail = group_tail[gi];
+        const int one = t.groups.size() == 1 ? t.groups[0] : -1;
+        if (one >= 0 && group_off[one] >= 0) {
+          r.page_off = group_off[one];
         } else {
           r.page_off = static_cast<int>(w.pages.size());
           for (int gi : t.groups) w.pages.insert(w.pages.end(), group_pages[gi].begin(), group_pages[gi].end());
-          r.n_pages = static_cast<int>(w.pages.size()) - r.page_off;
+          if (tail.second) w.pages.push_back(tail.first);
+          if (one >= 0) group_off[one] = r.page_off;
         }
-        r.last_valid = 16;
+        r.n_pages = tail.second ? 1 : 0;
+        for (int gi : t.groups) r.n_pages += static_cast<int>(group_pages[gi].size());
+        r.last_valid = tail.second ? tail.second : 16;
         r.cost = kSharedCostPerCand * r.n_cands;
         w.cands.insert(w.cands.end(), t.cands.begin(), t.cands.end());
         runs.push_back(r);
@@ -1185,7 +1355,7 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
       const int nfull = sl[b] / 16;   // a last page in part is the candidate's own
       for (int j = 0; j < nfull; ++j)
         if (in_group_dense.empty() ? in_group.count(row[j]) == 0 : in_group_dense[row[j]] == 0) w.pages.push_back(row[j]);
-      if (np[b] > nfull) {
+      if (np[b] > nfull && !(pack && tail_shared[b])) {
         w.pages.push_back(row[nfull]);
         r.last_valid = sl[b] - 16 * nfull;
       }
@@ -1220,7 +1390,7 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
     priv_ctas = n_ctas - tc_ctas;
     w.tc_concurrent = true;
   }
-  const int C = total == 0 ? 0
+  int C = total == 0 ? 0
                            : static_cast<int>(std::max<int64_t>(
                                  1, std::min<int64_t>(priv_ctas, total / (kPagesPerStage * kPrivateCost))));
   // The (run, kv head) pairs in axis order: the pairs of shared runs (bound by their MMAs: a warp
@@ -1255,6 +1425,8 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
     }
   }
   std::vector<int> seg_cta;
+  w.packed = pack && group <= 8 && pack_runs(runs, n_kv, priv_ctas, C, w, seg_cta, &C);
+  if (w.packed) pairs.clear();
   int64_t pos = 0;   // cost position of the current pair's first unit
   for (const auto& pr : pairs) {
     const Run& r = runs[pr.first];
@@ -1320,7 +1492,7 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
           sg.n_cands = r.n_cands;
           sg.page_off = r.page_off + i * kTcChunkPages;
           sg.n_pages = std::min(r.n_pages, e * kTcChunkPages) - i * kTcChunkPages;
-          sg.last_valid = 16;
+          sg.last_valid = e == nch ? r.last_valid : 16;
           sg.slot = static_cast<int>(w.slots.size());
           for (int k2 = 0; k2 < r.n_cands; ++k2)
             w.slots.push_back(w.nslots[static_cast<size_t>(w.cands[r.cand + k2]) * n_kv + g]++);
@@ -1345,13 +1517,18 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
     next += static_cast<size_t>(w.nslots[cg]);
   }
   if (next > slot_limit) {
-    if (share) return build_attn_work(bt, sl, n, max_blocks, n_kv, group, n_ctas, slot_limit, 0, w);
+    if (share) return build_attn_work(bt, sl, n, max_blocks, n_kv, group, n_ctas, slot_limit, 0, pack, w);
     return false;
   }
   w.n_slots = static_cast<int>(next);
   for (AttnSeg& s : w.segs) {
     if (s.kind == 0)
       s.slot += w.slot_base[static_cast<size_t>(s.cand) * n_kv + s.g];
+    else if (s.kind == 3)
+      for (int l = 0; l < s.n_cands; ++l) {
+        int32_t* ln = w.cands.data() + s.cand + l * kLaneInts;
+        ln[5] += w.slot_base[static_cast<size_t>(ln[0]) * n_kv + ln[1]];
+      }
     else   // kind 1: shared_reps(n) * n slots, slot w for candidate w % n; kind 2: one per candidate
       for (int k2 = 0; k2 < (s.kind == 1 ? shared_reps(s.n_cands) : 1) * s.n_cands; ++k2)
         w.slots[s.slot + k2] += w.slot_base[static_cast<size_t>(w.cands[s.cand + k2 % s.n_cands]) * n_kv + s.g];
@@ -1457,11 +1634,15 @@ cudaError_t attention_configure() {
   KVPRM_COMBINE_SMEM(128, 8, 4)
   KVPRM_COMBINE_SMEM(128, 16, 4)
 #undef KVPRM_COMBINE_SMEM
-  if ((e = set_smem(attn_kernel<64, false>, AttnSmem<64>::kDynamic)) != cudaSuccess) return e;
-  if ((e = set_smem(attn_kernel<64, true>, AttnSmem<64>::kDynamic)) != cudaSuccess) return e;
-  if ((e = set_smem(attn_kernel<128, false>, AttnSmem<128>::kDynamic)) != cudaSuccess) return e;
-  if ((e = set_smem(attn_tc_kernel, TcSmem::kDynamic)) != cudaSuccess) return e;
-  return set_smem(attn_kernel<128, true>, AttnSmem<128>::kDynamic);
+  if ((e = set_smem(attn_kernel<64, false, kFormRuns>, AttnSmem<64>::kDynamic)) != cudaSuccess) return e;
+  if ((e = set_smem(attn_kernel<64, false, kFormPacked>, AttnSmem<64>::kDynamic)) != cudaSuccess) return e;
+  if ((e = set_smem(attn_kernel<64, false, kFormFused>, AttnSmem<64>::kDynamic)) != cudaSuccess) return e;
+  if ((e = set_smem(attn_kernel<64, true, kFormRuns>, AttnSmem<64>::kDynamic)) != cudaSuccess) return e;
+  if ((e = set_smem(attn_kernel<128, false, kFormRuns>, AttnSmem<128>::kDynamic)) != cudaSuccess) return e;
+  if ((e = set_smem(attn_kernel<128, false, kFormPacked>, AttnSmem<128>::kDynamic)) != cudaSuccess) return e;
+  if ((e = set_smem(attn_kernel<128, false, kFormFused>, AttnSmem<128>::kDynamic)) != cudaSuccess) return e;
+  if ((e = set_smem(attn_kernel<128, true, kFormRuns>, AttnSmem<128>::kDynamic)) != cudaSuccess) return e;
+  return set_smem(attn_tc_kernel, TcSmem::kDynamic);
 }
 
 cudaError_t launch_attention(const AttnShape& s, const AttnWork& wk, const CUtensorMap* tm_pool, int layer,
@@ -1492,18 +1673,20 @@ cudaError_t launch_attention(const AttnShape& s, const AttnWork& wk, const CUten
   cfg.numAttrs = na;
   const int64_t page0 = static_cast<int64_t>(layer) * s.layer_pages;
   const bool two = s.group > 8;
-  if (s.hd == 128) {
-    if (two)
-      return cudaLaunchKernelEx(&cfg, attn_kernel<128, true>, *tm_pool, page0, wk, q_hi, q_lo, s.n_q, s.n_kv, s.group,
-                                part_o, part_ml, mg, err, ts);
-    return cudaLaunchKernelEx(&cfg, attn_kernel<128, false>, *tm_pool, page0, wk, q_hi, q_lo, s.n_q, s.n_kv, s.group,
-                              part_o, part_ml, mg, err, ts);
-  }
-  if (two)
-    return cudaLaunchKernelEx(&cfg, attn_kernel<64, true>, *tm_pool, page0, wk, q_hi, q_lo, s.n_q, s.n_kv, s.group,
-                              part_o, part_ml, mg, err, ts);
-  return cudaLaunchKernelEx(&cfg, attn_kernel<64, false>, *tm_pool, page0, wk, q_hi, q_lo, s.n_q, s.n_kv, s.group,
-                            part_o, part_ml, mg, err, ts);
+  if (two && (wk.packed || wk.fuse_cs > 0)) return cudaErrorInvalidValue;
+  auto go = [&](auto kern) {
+    return cudaLaunchKernelEx(&cfg, kern, *tm_pool, page0, wk, q_hi, q_lo, s.n_q, s.n_kv, s.group, part_o, part_ml, mg,
+                              err, ts);
+  };
+  if (s.hd == 128)
+    return two              ? go(attn_kernel<128, true, kFormRuns>)
+           : wk.packed      ? go(attn_kernel<128, false, kFormPacked>)
+           : wk.fuse_cs > 0 ? go(attn_kernel<128, false, kFormFused>)
+                            : go(attn_kernel<128, false, kFormRuns>);
+  return two              ? go(attn_kernel<64, true, kFormRuns>)
+         : wk.packed      ? go(attn_kernel<64, false, kFormPacked>)
+         : wk.fuse_cs > 0 ? go(attn_kernel<64, false, kFormFused>)
+                          : go(attn_kernel<64, false, kFormRuns>);
 }
 
 CUresult encode_pool_map_tc(PFN_cuTensorMapEncodeTiled_v12000 encode, CUtensorMap* map, const void* pool,

@@ -134,6 +134,7 @@ struct AttnWork {             // device arrays
   int n_tc_ctas;
   int fuse_cs;                // > 0: CTAs fuse_cs p .. fuse_cs p + fuse_cs - 1 (one cluster) score pair p and
                               // its rank 0 merges the pair's slots (no combine launch)
+  bool packed = false;        // every persistent segment is a pack (kind 3)
 };
 struct AttnWorkHost {
   std::vector<AttnSeg> segs;
@@ -142,6 +143,7 @@ struct AttnWorkHost {
   int tc_seg0 = 0, n_tc = 0;   // tensor-core segments (kind 2): segs[tc_seg0, tc_seg0 + n_tc)
   int n_tc_ctas = 0;
   std::vector<int32_t> tc_cta;   // [n_tc_ctas + 1] first segment (index into segs) of each tensor-core CTA
+  bool packed = false;           // see AttnWork::packed
   bool tc_concurrent = false;    // the two attention launches have disjoint SMs and may run at once
   int fuse_cs = 0;               // see AttnWork::fuse_cs
 };
@@ -151,8 +153,11 @@ struct AttnWorkHost {
 // launch planned over all n_ctas SMs; 3 as 2, with the SMs split between the
 // tensor-core and the private launch so that the later of the two (estimated
 // under a cost model) ends soonest, and the two run concurrently.
+// pack: shared partial pages and packed short runs (kind 3) too (attention.cu).
 bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks, int n_kv, int group, int n_ctas,
-                     size_t slot_limit, int share, AttnWorkHost& w);
+                     size_t slot_limit, int share, bool pack, AttnWorkHost& w);
+// entries of AttnWork::cands that packing may need beyond the candidate lists of shared runs
+size_t attn_lane_capacity(int max_candidates, int n_kv, int num_sms);
 // The plan with the combine fused into the attention launch, for calls where
 // every candidate has about the same number of pages, no page is shared and
 // group <= 8: (candidate, kv head) pair p = b n_kv + g is scored by the fuse_cs

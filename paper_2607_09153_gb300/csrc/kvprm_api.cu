@@ -42,11 +42,13 @@ struct GraphKey {
   int layer_waits = -1;
   int lora_rank = -1;
   int depth = -1;
+  int packed = -1;
   const void* pool = nullptr;
   int64_t n_pages = -1;
   bool operator==(const GraphKey& o) const {
     return n == o.n && n_pad == o.n_pad && attn_ctas == o.attn_ctas && tc_ctas == o.tc_ctas && n_tc == o.n_tc &&
            fuse_cs == o.fuse_cs && layer_waits == o.layer_waits && lora_rank == o.lora_rank && depth == o.depth &&
+           packed == o.packed &&
            debug == o.debug && profile == o.profile && pdl == o.pdl && trace == o.trace && pool == o.pool &&
            n_pages == o.n_pages;
   }
@@ -419,9 +421,10 @@ int plan_work(kvprm_ctx* ctx, const int32_t* bt, const int32_t* sl, int32_t n, b
   if (ctx->fuse_combine && allow_fused &&
       kvprm::build_attn_work_fused(bt, sl, n, mb, nkv, ctx->md.n_q / nkv, ctx->num_sms, ctx->slot_cap, w) && fits())
     return KVPRM_OK;
-  bool ok = kvprm::build_attn_work(bt, sl, n, mb, nkv, ctx->md.n_q / nkv, ctx->num_sms, ctx->slot_cap, ctx->share_mode, w);
-  if (ok && !fits() && ctx->share_mode)
-    ok = kvprm::build_attn_work(bt, sl, n, mb, nkv, ctx->md.n_q / nkv, ctx->num_sms, ctx->slot_cap, 0, w);
+  bool ok = kvprm::build_attn_work(bt, sl, n, mb, nkv, ctx->md.n_q / nkv, ctx->num_sms, ctx->slot_cap, ctx->share_mode,
+                                    true, w);
+  if (ok && !fits())
+    ok = kvprm::build_attn_work(bt, sl, n, mb, nkv, ctx->md.n_q / nkv, ctx->num_sms, ctx->slot_cap, 0, false, w);
   if (!ok || !fits())
     return fail(ctx, KVPRM_ECAPACITY, "attention work list exceeds the context's capacity");
   return KVPRM_OK;
@@ -493,6 +496,7 @@ kvprm::AttnWork device_work(kvprm_ctx* ctx) {
   wk.tc_cta = ctx->tables_d + ctx->off_tc_cta;
   wk.n_tc_ctas = ctx->work_host.n_tc_ctas;
   wk.fuse_cs = ctx->work_host.fuse_cs;
+  wk.packed = ctx->work_host.packed;
   return wk;
 }
 
@@ -1017,6 +1021,7 @@ int score_device(kvprm_ctx* ctx, const void* kv_pages, int64_t n_pages, const in
   key.layer_waits = ctx->layer_waits ? 1 : 0;
   key.lora_rank = ctx->lora_rank;
   key.depth = ctx->depth;
+  key.packed = ctx->work_host.packed ? 1 : 0;
   key.n_tc = ctx->work_host.n_tc > 0 ? 1 : 0;
   key.debug = ctx->debug_flags;
   key.profile = ctx->profile ? 1 : 0;
@@ -1296,7 +1301,8 @@ int score_grad_device(kvprm_ctx* ctx, const void* kv_pages, int64_t n_pages, con
   // the graph of this call: everything its launches take by value or by address
   const std::vector<int64_t> key = {
       n, P.n_pad, P.attn_ctas, ctx->work_host.n_tc_ctas, ctx->work_host.tc_concurrent ? 1 : 0,
-      ctx->work_host.fuse_cs, ctx->work_host.n_tc > 0 ? 1 : 0, ctx->work_host.n_ctas, ctx->debug_flags,
+      ctx->work_host.fuse_cs, ctx->work_host.packed ? 1 : 0, ctx->work_host.n_tc > 0 ? 1 : 0, ctx->work_host.n_ctas,
+      ctx->debug_flags,
       ctx->use_pdl ? 1 : 0, ctx->trace ? 1 : 0, ctx->layer_waits ? 1 : 0, ctx->as.layer_pages,
       reinterpret_cast<int64_t>(kv_pages), n_pages, reinterpret_cast<int64_t>(grad),
       static_cast<int64_t>(bp.units.size()), static_cast<int64_t>(bp.cta_item.size()), n_shared,
@@ -1487,7 +1493,8 @@ int kvprm_create(const kvprm_config* cfg, const kvprm_weights* w, kvprm_ctx** ou
     const size_t bkv = static_cast<size_t>(Bmax) * m.n_kv;
     ctx->cap_segs = 8 * bkv + 4 * static_cast<size_t>(ctx->num_sms);
     ctx->cap_pages = static_cast<size_t>(Bmax) * c.max_blocks_per_seq;
-    ctx->cap_cands = static_cast<size_t>(Bmax) * c.max_blocks_per_seq;
+    ctx->cap_cands = static_cast<size_t>(Bmax) * c.max_blocks_per_seq +
+                     kvprm::attn_lane_capacity(Bmax, m.n_kv, ctx->num_sms);
     ctx->off_segs = al8(tbl);
     ctx->off_cta = al8(ctx->off_segs + ctx->cap_segs * (sizeof(kvprm::AttnSeg) / sizeof(int32_t)));
     ctx->off_pages = al8(ctx->off_cta + ctx->num_sms + 1);
@@ -1906,11 +1913,12 @@ int kvprm_plan_attention(const int32_t* block_table, int32_t max_blocks_per_seq,
       return KVPRM_EINVAL;
   kvprm::AttnWorkHost w;
   const bool fuse = share >= 0 && (share & KVPRM_PLAN_FUSE) != 0;
-  share = share < 0 ? 0 : (share & ~KVPRM_PLAN_FUSE);
+  const bool pack = share >= 0 && (share & KVPRM_PLAN_PACK) != 0;
+  share = share < 0 ? 0 : (share & ~(KVPRM_PLAN_FUSE | KVPRM_PLAN_PACK));
   if (!(fuse && kvprm::build_attn_work_fused(block_table, seq_lens, n_candidates, max_blocks_per_seq, n_kv_heads,
                                              group, n_ctas, SIZE_MAX, w)) &&
       !kvprm::build_attn_work(block_table, seq_lens, n_candidates, max_blocks_per_seq, n_kv_heads, group, n_ctas,
-                              SIZE_MAX, share > 3 ? 3 : share, w))
+                              SIZE_MAX, share > 3 ? 3 : share, pack, w))
     return KVPRM_ECAPACITY;
   plan->fuse_cs = w.fuse_cs;
   plan->n_segs = static_cast<int32_t>(w.segs.size());

@@ -166,8 +166,7 @@ extern "C" int kvprm_attention_noalloc(const void* kv_layer, int64_t n_pages, co
   bool fits = false;
   for (int share = 1; share >= 0 && !fits; --share) {
     if (!kvprm::build_attn_work(block_table, seq_lens, n, max_blocks_per_seq, n_kv_heads, n_q_heads / n_kv_heads, sms,
-                                SIZE_MAX, share != 0,
-                                work))
+                                SIZE_MAX, share != 0, false, work))
       continue;
     cv = carve(n, n_q_heads, n_kv_heads, head_dim, work);
     fits = cv.total <= static_cast<size_t>(KVPRM_NOALLOC_SCRATCH_BYTES);

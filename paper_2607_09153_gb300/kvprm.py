@@ -69,6 +69,7 @@ class KvprmAttnPlan(ctypes.Structure):
                 ("fuse_cs", ctypes.c_int32)]
 
 KVPRM_PLAN_FUSE = 16
+KVPRM_PLAN_PACK = 32
 
 
 _lib = None
