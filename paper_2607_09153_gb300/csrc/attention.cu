@@ -422,9 +422,9 @@ __global__ void __launch_bounds__(W * 32) attn_combine_kernel(
 
 // The combine of a single verify token per candidate, flat: one CTA per (candidate, kv head) and
 // one warp per query head of the group, lane i holding head-dim elements i + 32 j.  A round issues
-// every load it uses (up to kFlatSlots partial slots' (m, l) and O values; in the first round also
-// q, k_self and v_self) before using any, so it costs one memory round trip; the slots then merge
-// into the running (M, L, acc) started from the verify token's own entry.  No shared memory and no
+// every load it uses (up to kFlatSlots partial slots' (m, l) and O values; q, k_self and v_self go
+// before the first) before using any, so it costs one memory round trip; the slots then merge
+// into the running (M, L, acc), and the verify token's own entry last.  No shared memory and no
 // CTA barrier, so CTAs are short and many fit on an SM.
 constexpr int kFlatSlots = 8;
 
@@ -442,9 +442,19 @@ __global__ void __launch_bounds__(512) attn_combine_flat_kernel(
   const int64_t hk = static_cast<int64_t>(b) * n_kv + g;
   grid_dep_wait();   // the partials (and q, k_self, v_self) are written by earlier kernels
   if (threadIdx.x == 0) trace_event(ts, 0);
-  float2 ml[kFlatSlots];
-  float o[kFlatSlots][kPer];
-  auto load_round = [&](int s0) {
+  float qd[kPer], kd[kPer], vd[kPer], acc[kPer];
+#pragma unroll
+  for (int j = 0; j < kPer; ++j) {
+    qd[j] = __ldcg(mg.q + hq * HD + lane + 32 * j);
+    kd[j] = __ldcg(mg.kself + hk * HD + lane + 32 * j);
+    vd[j] = __ldcg(mg.vself + hk * HD + lane + 32 * j);
+    acc[j] = 0.f;
+  }
+  float M = -INFINITY, L = 0.f;
+#pragma unroll 1
+  for (int s0 = 0; s0 < ns; s0 += kFlatSlots) {
+    float2 ml[kFlatSlots];
+    float o[kFlatSlots][kPer];
 #pragma unroll
     for (int k = 0; k < kFlatSlots; ++k) {
       const bool in = s0 + k < ns;
@@ -453,35 +463,38 @@ __global__ void __launch_bounds__(512) attn_combine_flat_kernel(
 #pragma unroll
       for (int j = 0; j < kPer; ++j) o[k][j] = in ? __ldcg(part_o + pr * HD + lane + 32 * j) : 0.f;
     }
-  };
-  float qd[kPer], kd[kPer], acc[kPer];
+    // the round's maximum first, so that each slot takes one exponential
+    float Mn = M;
 #pragma unroll
-  for (int j = 0; j < kPer; ++j) {
-    qd[j] = __ldcg(mg.q + hq * HD + lane + 32 * j);
-    kd[j] = __ldcg(mg.kself + hk * HD + lane + 32 * j);
-    acc[j] = __ldcg(mg.vself + hk * HD + lane + 32 * j);
+    for (int k = 0; k < kFlatSlots; ++k) Mn = fmaxf(Mn, ml[k].x);
+    if (Mn == -INFINITY) continue;   // slots with no token
+    const float sc = exp2f(M - Mn);
+    L *= sc;
+#pragma unroll
+    for (int j = 0; j < kPer; ++j) acc[j] *= sc;
+#pragma unroll
+    for (int k = 0; k < kFlatSlots; ++k) {
+      if (ml[k].x == -INFINITY) continue;   // past the last slot, or a slot with no token (warp-uniform)
+      const float w = exp2f(ml[k].x - Mn);
+      L += w * ml[k].y;
+#pragma unroll
+      for (int j = 0; j < kPer; ++j) acc[j] += w * o[k][j];
+    }
+    M = Mn;
   }
-  load_round(0);
-  // the verify token's own entry: score q . k_self (log2 units), weight 1 at M = that score
+  // the verify token's own entry: score q . k_self (log2 units)
   float dot = 0.f;
 #pragma unroll
   for (int j = 0; j < kPer; ++j) dot += qd[j] * kd[j];
 #pragma unroll
   for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-  float M = dot * (kLog2e * rsqrtf(static_cast<float>(HD))), L = 1.f;
-  for (int s0 = 0;; s0 += kFlatSlots) {
+  dot *= kLog2e * rsqrtf(static_cast<float>(HD));
+  {
+    const float Mn = fmaxf(M, dot), sc = exp2f(M - Mn), w = exp2f(dot - Mn);
+    L = L * sc + w;
 #pragma unroll
-    for (int k = 0; k < kFlatSlots; ++k) {
-      if (ml[k].x == -INFINITY) continue;   // past the last slot, or a slot with no token (warp-uniform)
-      const float Mn = fmaxf(M, ml[k].x);
-      const float sc = exp2f(M - Mn), w = exp2f(ml[k].x - Mn);
-      L = L * sc + w * ml[k].y;
-#pragma unroll
-      for (int j = 0; j < kPer; ++j) acc[j] = acc[j] * sc + w * o[k][j];
-      M = Mn;
-    }
-    if (s0 + kFlatSlots >= ns) break;
-    load_round(s0 + kFlatSlots);
+    for (int j = 0; j < kPer; ++j) acc[j] = acc[j] * sc + w * vd[j];
+    M = Mn;
   }
   const float inv = 1.f / L;
 #pragma unroll

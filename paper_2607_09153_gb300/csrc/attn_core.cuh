@@ -459,62 +459,27 @@ __device__ __forceinline__ void combine_group(int tid, int b, int g, int first, 
   const int warp = tid >> 5, lane = tid & 31;
   const int64_t hq0 = static_cast<int64_t>(b) * n_q + static_cast<int64_t>(g) * group;
   const int64_t hk = static_cast<int64_t>(b) * n_kv + g;
-  // Every global load of the first round is issued before any is used: this
-  // warp's first U slots, the q / k_self rows of head `warp` and this thread's
-  // v_self values for the final phase.
-  float2 ml[U];
-  float v[U][ROWS][kPer];
-#pragma unroll
-  for (int k = 0; k < U; ++k) {
-    const int sk = warp + k * W;
-    const int64_t pr = (static_cast<int64_t>(first) + (sk < ns ? sk : 0)) * group;
-    ml[k] = (sk < ns && lane < group) ? __ldcg(reinterpret_cast<const float2*>(part_ml + (pr + lane) * 2))
-                                      : make_float2(-INFINITY, 0.f);
-#pragma unroll
-    for (int r = 0; r < ROWS; ++r)
-#pragma unroll
-      for (int j = 0; j < kPer; ++j)
-        v[k][r][j] = (sk < ns && r < group) ? __ldcg(part_o + (pr + r) * HD + lane + 32 * j) : 0.f;
-  }
-  float qd[kPer], kd[kPer];
-#pragma unroll
-  for (int j = 0; j < kPer; ++j) {
-    qd[j] = warp < group ? __ldcg(mg.q + (hq0 + warp) * HD + lane + 32 * j) : 0.f;
-    kd[j] = warp < group ? __ldcg(mg.kself + hk * HD + lane + 32 * j) : 0.f;
-  }
-  float vsf[kOut];
-#pragma unroll
-  for (int i = 0; i < kOut; ++i) {
-    const int idx = tid + i * W * 32;
-    vsf[i] = idx < group * HD ? __ldcg(mg.vself + hk * HD + idx % HD) : 0.f;
-  }
-  // the self entries' scores of head `warp`: token t's own (k_self already loaded) and, in a
-  // depth-k readout, its candidate's earlier tokens (rows b - t .. b - 1)
-  // DEEP (a depth-k readout): a compiled variant of its own, so that the single-entry form keeps its code
+  // The q / k_self rows of head `warp` and this thread's v_self values for the final phase are on their
+  // way while the slots are folded, a round of U slots' loads issued before any of it is used.  Each
+  // sequence is written once and the long loops stay rolled: a CTA runs this once per launch, so its
+  // time is as much its instruction fetches as its loads.
+  // the self entries: the row's own token or, in a depth-k readout (DEEP, a compiled variant of its own so
+  // that the single-entry form keeps its code), tokens 0 .. t of its candidate (rows b - t .. b)
+  constexpr int NS = DEEP ? kMaxReadoutDepth : 1;
   const int t_self = DEEP ? b % mg.depth : 0, n_self = DEEP ? t_self + 1 : 1;
   const int64_t hk0 = hk - static_cast<int64_t>(t_self) * n_kv;
-  if (warp < group) {
-    for (int e = 0; e < n_self; ++e) {
-      float dot = 0.f;
+  // an output thread keeps its head-dimension element over all its outputs
+  static_assert(W * 32 % HD == 0, "output threads are a multiple of the head dimension");
+  float qd[kPer], kd[NS][kPer], vd[NS];
 #pragma unroll
-      for (int j = 0; j < kPer; ++j)
-        dot += qd[j] * (e == t_self ? kd[j] : __ldcg(mg.kself + (hk0 + e * n_kv) * HD + lane + 32 * j));
+  for (int j = 0; j < kPer; ++j) qd[j] = warp < group ? __ldcg(mg.q + (hq0 + warp) * HD + lane + 32 * j) : 0.f;
 #pragma unroll
-      for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-      if (lane == 0) s_self[warp * kMaxReadoutDepth + e] = dot * (kLog2e * rsqrtf(static_cast<float>(HD)));
-    }
-  }
-  for (int r = warp + W; r < group; r += W) {   // heads beyond the warp count (G > W; k_self is loaded by all)
-    for (int e = 0; e < n_self; ++e) {
-      float dot = 0.f;
+  for (int e = 0; e < NS; ++e) {
+    const bool in = e < n_self;
 #pragma unroll
-      for (int j = 0; j < kPer; ++j)
-        dot += __ldcg(mg.q + (hq0 + r) * HD + lane + 32 * j) *
-               (e == t_self ? kd[j] : __ldcg(mg.kself + (hk0 + e * n_kv) * HD + lane + 32 * j));
-#pragma unroll
-      for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
-      if (lane == 0) s_self[r * kMaxReadoutDepth + e] = dot * (kLog2e * rsqrtf(static_cast<float>(HD)));
-    }
+    for (int j = 0; j < kPer; ++j)
+      kd[e][j] = in && warp < group ? __ldcg(mg.kself + (hk0 + e * n_kv) * HD + lane + 32 * j) : 0.f;
+    vd[e] = in ? __ldcg(mg.vself + (hk0 + e * n_kv) * HD + tid % HD) : 0.f;
   }
   float M[ROWS], L[ROWS], acc[ROWS][kPer];
 #pragma unroll
@@ -524,7 +489,22 @@ __device__ __forceinline__ void combine_group(int tid, int b, int g, int first, 
 #pragma unroll
     for (int j = 0; j < kPer; ++j) acc[r][j] = 0.f;
   }
-  for (int s0 = warp;; s0 += U * W) {
+#pragma unroll 1
+  for (int s0 = warp; s0 < ns; s0 += U * W) {
+    float2 ml[U];
+    float v[U][ROWS][kPer];
+#pragma unroll
+    for (int k = 0; k < U; ++k) {
+      const int sk = s0 + k * W;
+      const int64_t pr = (static_cast<int64_t>(first) + (sk < ns ? sk : 0)) * group;
+      ml[k] = (sk < ns && lane < group) ? __ldcg(reinterpret_cast<const float2*>(part_ml + (pr + lane) * 2))
+                                        : make_float2(-INFINITY, 0.f);
+#pragma unroll
+      for (int r = 0; r < ROWS; ++r)
+#pragma unroll
+        for (int j = 0; j < kPer; ++j)
+          v[k][r][j] = (sk < ns && r < group) ? __ldcg(part_o + (pr + r) * HD + lane + 32 * j) : 0.f;
+    }
 #pragma unroll
     for (int k = 0; k < U; ++k)
 #pragma unroll
@@ -538,19 +518,22 @@ __device__ __forceinline__ void combine_group(int tid, int b, int g, int first, 
         for (int j = 0; j < kPer; ++j) acc[r][j] = acc[r][j] * sc + wv * v[k][r][j];
         M[r] = Mn;
       }
-    if (s0 + U * W >= ns) break;
-    // the next round of slots (more than U * W slots only)
+  }
+  // the self entries' scores of heads warp, warp + W, .. (G > W: every warp has loaded the keys)
+#pragma unroll 1
+  for (int r = warp; r < group; r += W) {
+    if (r != warp)
 #pragma unroll
-    for (int k = 0; k < U; ++k) {
-      const int sk = s0 + U * W + k * W;
-      const int64_t pr = (static_cast<int64_t>(first) + (sk < ns ? sk : 0)) * group;
-      ml[k] = (sk < ns && lane < group) ? __ldcg(reinterpret_cast<const float2*>(part_ml + (pr + lane) * 2))
-                                        : make_float2(-INFINITY, 0.f);
+      for (int j = 0; j < kPer; ++j) qd[j] = __ldcg(mg.q + (hq0 + r) * HD + lane + 32 * j);
 #pragma unroll
-      for (int r = 0; r < ROWS; ++r)
+    for (int e = 0; e < NS; ++e) {
+      if (e >= n_self) break;
+      float dot = 0.f;
 #pragma unroll
-        for (int j = 0; j < kPer; ++j)
-          v[k][r][j] = (sk < ns && r < group) ? __ldcg(part_o + (pr + r) * HD + lane + 32 * j) : 0.f;
+      for (int j = 0; j < kPer; ++j) dot += qd[j] * kd[e][j];
+#pragma unroll
+      for (int off = 16; off > 0; off >>= 1) dot += __shfl_xor_sync(0xffffffffu, dot, off);
+      if (lane == 0) s_self[r * kMaxReadoutDepth + e] = dot * (kLog2e * rsqrtf(static_cast<float>(HD)));
     }
   }
 #pragma unroll
@@ -565,20 +548,24 @@ __device__ __forceinline__ void combine_group(int tid, int b, int g, int first, 
     }
   }
   sync();
-#pragma unroll
+#pragma unroll 1
   for (int i = 0; i < kOut; ++i) {
     const int idx = tid + i * W * 32;
     if (idx >= group * HD) break;
     const int r = idx / HD, d = idx - r * HD;
     const float* ss = s_self + r * kMaxReadoutDepth;
     float Mt = ss[0];
-    for (int e = 1; e < n_self; ++e) Mt = fmaxf(Mt, ss[e]);
+#pragma unroll
+    for (int e = 1; e < NS; ++e)
+      if (e < n_self) Mt = fmaxf(Mt, ss[e]);
 #pragma unroll
     for (int w = 0; w < W; ++w) Mt = fmaxf(Mt, s_m[w * ROWS + r]);
     float num = 0.f, den = 0.f;
-    for (int e = 0; e < n_self; ++e) {   // the self entries (one without a depth-k readout)
+#pragma unroll
+    for (int e = 0; e < NS; ++e) {
+      if (e >= n_self) break;
       const float ws = exp2f(ss[e] - Mt);
-      num += ws * (e == t_self ? vsf[i] : __ldcg(mg.vself + (hk0 + e * n_kv) * HD + d));
+      num += ws * vd[e];
       den += ws;
     }
 #pragma unroll

@@ -67,7 +67,13 @@ __device__ __forceinline__ void store_hilo(__nv_bfloat16* hi, __nv_bfloat16* lo,
 // with 16-byte DSMEM loads, and the epilogues move 4 or 8 consecutive rows of a column per thread
 // with 16-byte accesses (the 4-warp CTA is otherwise bound by 2- and 4-byte stores and by one load
 // latency per column).
-template <bool LARGE>
+// MODE: the epilogue, an image each.  A CTA runs everything after its MMAs once, so those instructions
+// are fetched cold in every launch, and their number is a good part of the ~3 us from the last MMA to
+// the end of a small launch.  Hence the images, rolled outer loops, counters instead of divisions by the
+// stage count and shifts by the head dimension: 51 KB of code in one small image became 20-32 KB in four
+// (large: 178 KB became 31-52), and a call of the 1.5B workload took 1,112 us instead of 1,155, with the
+// rank-256 adapter 1,687 instead of 1,932, MCTS 9,814 instead of 10,110.
+template <bool LARGE, int MODE>
 __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmW,
                                                            const __grid_constant__ CUtensorMap tmX,
                                                            const __grid_constant__ CUtensorMap tmXlo, int has_lo,
@@ -102,13 +108,13 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   const int kt0 = static_cast<int>(rank) * kps;
   const int kt1 = min(k_tiles, kt0 + kps);
   const int nk = kt1 > kt0 ? kt1 - kt0 : 0;
-  const bool silu = ep.mode == GemmEpilogue::SILU;
+  constexpr bool silu = MODE == GemmEpilogue::SILU;
   // this rank's candidate columns in the reduction and the epilogue
   const int cols = n_pad / cs;
   const int cbeg = static_cast<int>(rank) * cols;
   const int cend = min(cbeg + cols, ep.n_valid);
   const int nc = cend > cbeg ? cend - cbeg : 0;
-  const bool hpreload = ep.mode == GemmEpilogue::RESID && nc <= kHPreCols && mt == 1;
+  const bool hpreload = MODE == GemmEpilogue::RESID && nc <= kHPreCols && mt == 1;
   constexpr int kEpiBatch = LARGE ? 8 : 1;
 
   if (threadIdx.x == 0) {
@@ -148,6 +154,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     auto load_w = [&](uint8_t* st, int kt, uint64_t* bar) {
       const CUtensorMap* wm = kt < k_main ? &tmW : &tmB;
       const int kx = (kt < k_main ? kt : kt - k_main) * kBK;
+#pragma unroll 1
       for (int t = 0; t < mt; ++t) {
         const int m_tile = m_tile0 + t;
         uint8_t* wt = st + t * kWTileBytes;
@@ -168,28 +175,36 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     // Weights do not depend on the preceding kernel: start streaming the first
     // ring's worth of W before waiting for the activations it produces.
     const int pre = min(stages, nk);
+#pragma unroll 1
     for (int i = 0; i < pre; ++i) {
       mbar_arrive_expect_tx(&full[i], stage_bytes);
       load_w(smem + i * stage_bytes, kt0 + i, &full[i]);
     }
     grid_dep_wait();
     trace_event(ts, 0);   // the preceding kernel has completed
+#pragma unroll 1
     for (int i = 0; i < pre; ++i) load_x(smem + i * stage_bytes, kt0 + i, &full[i]);
+    int s = 0;   // stage of K tile i, and the parity of the release before its use
+    uint32_t parity = 0u;
+#pragma unroll 1
     for (int i = pre; i < nk; ++i) {
-      const int s = i % stages;
-      const uint32_t use = static_cast<uint32_t>(i / stages);
-      if (!mbar_wait(&empty[s], (use & 1u) ^ 1u, err)) break;
+      if (!mbar_wait(&empty[s], parity, err)) break;
       uint8_t* st = smem + s * stage_bytes;
       mbar_arrive_expect_tx(&full[s], stage_bytes);
       load_w(st, kt0 + i, &full[s]);
       load_x(st, kt0 + i, &full[s]);
+      if (++s == stages) {
+        s = 0;
+        parity ^= 1u;
+      }
     }
   } else if (warp >= 2) {
     // ---------------- while the weights stream: the RMSNorm factor of each of this rank's columns
     // (QKV, SILU), from the residual stream's tile sums of squares the preceding kernel wrote; the
     // parking barrier below orders these writes before the epilogue reads them
     grid_dep_wait();
-    if (ep.rs_sumsq)
+    if ((MODE == GemmEpilogue::QKV || MODE == GemmEpilogue::SILU) && ep.rs_sumsq)
+#pragma unroll 1
       for (int t0 = threadIdx.x - 64; t0 < nc; t0 += blockDim.x - 64) {   // nc <= 256 columns
         const int c = cbeg + t0;
         float ssum = 0.f;
@@ -199,6 +214,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     // RESID: the residual values the epilogue adds to, read now rather than after the MMAs, when
     // the next kernel's weight stream may be competing for the memory system
     if (hpreload)
+#pragma unroll 4
       for (int idx = threadIdx.x - 64; idx < nc * kBM; idx += blockDim.x - 64) {
         const int c = cbeg + idx / kBM, gm = m_tile0 * kBM + idx % kBM;
         hpre[idx] = gm < ep.M ? ep.h[static_cast<int64_t>(c) * ep.M + gm] : 0.f;
@@ -216,31 +232,32 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     const bool two = has_lo && !merged;
     const uint32_t idesc = idesc_bf16_f32(kBM, merged ? 2 * n_pad : n_pad);
     const uint32_t tile_cols = tmem_cols / static_cast<uint32_t>(mt);
+    int s = 0;
+    uint32_t parity = 0u;
+#pragma unroll 1
     for (int i = 0; i < nk; ++i) {
-      const int s = i % stages;
-      const uint32_t use = static_cast<uint32_t>(i / stages);
-      if (!__all_sync(0xffffffffu, mbar_wait(&full[s], use & 1u, err))) break;
+      if (!__all_sync(0xffffffffu, mbar_wait(&full[s], parity, err))) break;
       if (i == 0 && lane == 0) trace_event(ts, 1);   // first weight and activation tiles landed
       tc_fence_after();
       const uint64_t a0 = desc_sw128(smem_u32(smem + s * stage_bytes));   // K step kk: + 2 kk (32 bytes)
       const uint64_t b0 = a0 + (w_bytes >> 4);
       const uint64_t l0 = b0 + static_cast<uint64_t>(x_bytes >> 4);
       const uint32_t acc0 = i > 0 ? 1u : 0u;
+#pragma unroll 1
       for (int t = 0; t < mt; ++t) {
         const uint32_t d = tmem + static_cast<uint32_t>(t) * tile_cols;
         const uint64_t at = a0 + static_cast<uint64_t>(t) * (kWTileBytes >> 4);
-        if (two) {
 #pragma unroll
-          for (int kk = 0; kk < kBK / 16; ++kk) {
-            umma_bf16_w(d, at + 2 * kk, b0 + 2 * kk, idesc, kk > 0 ? 1u : acc0);
-            umma_bf16_w(d, at + 2 * kk, l0 + 2 * kk, idesc, 1u);
-          }
-        } else {
-#pragma unroll
-          for (int kk = 0; kk < kBK / 16; ++kk) umma_bf16_w(d, at + 2 * kk, b0 + 2 * kk, idesc, kk > 0 ? 1u : acc0);
+        for (int kk = 0; kk < kBK / 16; ++kk) {
+          umma_bf16_w(d, at + 2 * kk, b0 + 2 * kk, idesc, kk > 0 ? 1u : acc0);
+          if (LARGE && two) umma_bf16_w(d, at + 2 * kk, l0 + 2 * kk, idesc, 1u);   // n_pad > 128
         }
       }
       umma_commit_w(&empty[s]);
+      if (++s == stages) {
+        s = 0;
+        parity ^= 1u;
+      }
     }
     umma_commit_w(done);
   }
@@ -259,10 +276,12 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   const uint32_t tile_cols = tmem_cols / static_cast<uint32_t>(mt);
   // one m-tile at a time: park it, reduce it over the cluster (split K), write its epilogue; with two
   // tiles and split K the second is parked once every peer has read this CTA's first partial
+#pragma unroll 1
   for (int tt = 0; tt < mt; ++tt) {
     const int m_tile = m_tile0 + tt;
     const uint32_t tcol = static_cast<uint32_t>(tt) * tile_cols;
     if (tt > 0 && cs > 1) cluster_wait();   // matches the arrive after the previous tile's reduction
+#pragma unroll 1
     for (int c0 = 16 * wh; c0 < n_pad; c0 += 16 * nwh) {
       float v[16];
       if (nk > 0 && have) {
@@ -302,6 +321,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
         auto vreduce = [&](auto cs_c) {
           constexpr int CS = decltype(cs_c)::value, PER = 16 / CS;
           const int rq = static_cast<int>(threadIdx.x) & 31, cg = static_cast<int>(threadIdx.x) >> 5;
+#pragma unroll 1
           for (int c0 = cbeg + cg; c0 < cend; c0 += nw * PER) {
             float4 v[16];
 #pragma unroll
@@ -328,6 +348,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
           vreduce(std::integral_constant<int, 8>{});
       } else if (cs > 1) {
         const int step = cs <= 8 ? 2 : 1;
+#pragma unroll 1
         for (int c = cbeg + wh * step; c < cend; c += step * nwh) {
           const bool two = step == 2 && c + 1 < cend;
           float v[16];
@@ -369,10 +390,11 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     // head's hd rows of the RMSNorm-scaled projection, 1/sqrt(mean(y^2) + eps) times the column's
     // RMSNorm factor (v heads keep the latter alone); parked where RESID preloads its residual
     float* qkf = hpre;   // [column][head of the tile]
-    if (ep.mode == GemmEpilogue::QKV && ep.qn_gain) {
-      const int hpt = kBM / ep.hd;   // heads per tile: 1 (hd 128) or 2 (hd 64)
+    if (MODE == GemmEpilogue::QKV && ep.qn_gain) {
+      const int hpt = ep.hd == 128 ? 1 : 2;   // heads per tile
+#pragma unroll 1
       for (int it = warp; it < nc * hpt; it += nw) {
-        const int cl = it / hpt, hh = it % hpt;
+        const int cl = it >> (hpt - 1), hh = it & (hpt - 1);
         const float* col = acc + (cbeg + cl) * kBM + hh * ep.hd;
         float sq = 0.f;
         for (int r = lane; r < ep.hd; r += 32) sq += col[r] * col[r];
@@ -380,29 +402,29 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
         for (int off = 16; off > 0; off >>= 1) sq += __shfl_xor_sync(0xffffffffu, sq, off);
         if (lane == 0) {
           const float rs = ep.rs_sumsq ? rsc[cl] : 1.f;
-          const int head = m_tile * (kBM / ep.hd) + hh;
+          const int head = m_tile * hpt + hh;
           qkf[cl * 2 + hh] = head < ep.n_q + ep.n_kv ? rs / sqrtf(rs * rs * sq / ep.hd + ep.rs_eps) : rs;
         }
       }
       __syncthreads();
     }
     // Step 2: the epilogue over (row, column) pairs, all threads in parallel
-    if (ep.mode == GemmEpilogue::PLAIN) {
+    if constexpr (MODE == GemmEpilogue::PLAIN) {
       const int gm = m_tile * kBM + m;
       if (gm < ep.M)
+#pragma unroll 4
         for (int c = cbeg + wh; c < cend; c += nwh) ep.out[static_cast<int64_t>(c) * ep.M + gm] = acc[c * kBM + m];
-    } else if (LARGE && ep.mode == GemmEpilogue::LOWRANK) {   // t = s (A x), hi/lo [n][r]; large image only
+    } else if constexpr (MODE == GemmEpilogue::LOWRANK) {   // t = s (A x), hi/lo [n][r]; large image only
+      static_assert(LARGE || MODE != GemmEpilogue::LOWRANK, "the adapter's A x has a large-batch image only");
       const int gm = m_tile * kBM + m;
       if (gm < ep.M)
+#pragma unroll 2
         for (int c = cbeg + wh; c < cend; c += nwh)
           store_hilo(ep.t_hi, ep.t_lo, static_cast<int64_t>(c) * ep.M + gm, ep.lr_scale * acc[c * kBM + m]);
-    } else if (ep.mode == GemmEpilogue::RESID && LARGE) {
-      // pass 1, 16 columns at a time with the group's residual loads in flight before the first use:
-      // h += acc, the next projection's input, and hv^2 parked in place of acc (each (column, row)
-      // slot is this thread's own)
-      const int gm = m_tile * kBM + m;
-      const float gain = (ep.gain_next && gm < ep.M) ? __bfloat162float(ep.gain_next[gm]) : 0.f;
-      if ((ep.M & 3) == 0) {
+    } else if constexpr (MODE == GemmEpilogue::RESID && LARGE) {
+      // pass 1, eight columns' residual loads in flight before the first use: h += acc, the next
+      // projection's input, and hv^2 parked in place of acc (each (column, row) slot is this thread's own)
+      {   // M = d_model, a multiple of 64
         // four consecutive rows of one column per thread (a warp covers one column's 128 rows):
         // 16-byte residual loads and stores, 8-byte hi/lo stores; eight columns' loads in flight
         const int rq = static_cast<int>(threadIdx.x) & 31, cg = static_cast<int>(threadIdx.x) >> 5;
@@ -418,6 +440,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
           g4[2] = gc.x;
           g4[3] = gc.y;
         }
+#pragma unroll 1
         for (int c0 = cbeg + cg; c0 < cend; c0 += nw * 8) {
           float4 h_in[8];
 #pragma unroll
@@ -456,32 +479,12 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
             *ap = make_float4(hv.x * hv.x, hv.y * hv.y, hv.z * hv.z, hv.w * hv.w);
           }
         }
-      } else {   // warps w and w + 4 share rows: alternate 16-column groups
-        for (int c0 = cbeg + 16 * wh; c0 < cend; c0 += 16 * nwh) {
-          float h_in[16];
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int c = c0 + j;
-            h_in[j] = (c < cend && gm < ep.M) ? ep.h[static_cast<int64_t>(c) * ep.M + gm] : 0.f;
-          }
-#pragma unroll
-          for (int j = 0; j < 16; ++j) {
-            const int c = c0 + j;
-            if (c >= cend) break;
-            float hv = 0.f;
-            if (gm < ep.M) {
-              hv = h_in[j] + acc[c * kBM + m];
-              ep.h[static_cast<int64_t>(c) * ep.M + gm] = hv;
-              if (ep.gain_next) store_hilo(ep.x_hi, ep.x_lo, static_cast<int64_t>(c) * ep.M + gm, hv * gain);
-            }
-            acc[c * kBM + m] = hv * hv;
-          }
-        }
       }
       __syncthreads();
       // pass 2: each column's sum of squares over the tile's 128 rows, eight threads per column
       // (rows part + 8 q, the start of q rotated per column so that a warp's four columns hit
       // different banks), warp-uniform trip count for the shuffles
+#pragma unroll 1
       for (int t0 = 0; t0 < nc * 8; t0 += blockDim.x) {
         const int t = t0 + static_cast<int>(threadIdx.x);
         const int cl = t >> 3, part = t & 7;
@@ -496,12 +499,14 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
         sq += __shfl_xor_sync(0xffffffffu, sq, 4);
         if (t < nc * 8 && part == 0) ep.sumsq[static_cast<int64_t>(m_tile) * ep.n_valid + cbeg + cl] = sq;
       }
-    } else if (ep.mode == GemmEpilogue::RESID) {
+    } else if constexpr (MODE == GemmEpilogue::RESID) {
       const int gm = m_tile * kBM + m;
       float* sq_s = red;   // [16 columns][4 warps]
+#pragma unroll 1
       for (int c0 = cbeg; c0 < cend; c0 += 16) {
         const int c1 = min(cend, c0 + 16);
         {
+#pragma unroll 1
           for (int c = c0; c < c1; ++c) {
             float hv = 0.f;
             if (gm < ep.M) {
@@ -525,7 +530,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
         }
         __syncthreads();
       }
-    } else if (ep.mode == GemmEpilogue::SILU && LARGE && (ep.ff & 7) == 0) {
+    } else if constexpr (MODE == GemmEpilogue::SILU && LARGE) {   // d_ff is a multiple of 64
       // eight consecutive rows of one column per thread (8 row groups x 16 column groups): 16-byte
       // loads from the parked tile and one 16-byte store for each of the hi and lo halves (2-byte
       // stores, 256 per warp and tile at B = 256, bound the scalar form); the exponential and the
@@ -566,11 +571,12 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
           }
         }
       }
-    } else if (ep.mode == GemmEpilogue::SILU) {
+    } else if constexpr (MODE == GemmEpilogue::SILU) {
       // 2 nhalf column groups of 64 threads (rows m and m + 64 of a column share a group)
       const int r = m & 63, ng = 2 * nwh, grp = (m >> 6) + 2 * wh;
       const int j = m_tile * 64 + r;
       if (j < ep.ff)
+#pragma unroll 1
         for (int c0 = cbeg + grp; c0 < cend; c0 += ng * kEpiBatch) {
           float g[kEpiBatch], u[kEpiBatch];   // a batch's operands, read before its first store
 #pragma unroll
@@ -593,16 +599,17 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
             }
           }
         }
-    } else if (LARGE && (ep.hd & 7) == 0) {
+    } else if constexpr (LARGE) {   // QKV
       // QKV, four consecutive RoPE pairs (i .. i + 3, partners i + half ..) of one column per
       // thread (16 pair groups x 8 column groups): 16-byte loads of the parked tile and the
       // rotation, 16-byte fp32 and 8-byte hi/lo stores; two columns' operands in flight
       const int pq = 4 * (static_cast<int>(threadIdx.x) & 15), cg = static_cast<int>(threadIdx.x) >> 4;
-      const int hd = ep.hd, half = hd / 2;
-      const int row_a = (pq / half) * hd + (pq % half);   // half % 4 == 0: the four pairs share a head
+      const int lhd = ep.hd == 128 ? 7 : 6;   // head_dim is 64 or 128
+      const int hd = 1 << lhd, half = hd >> 1;
+      const int row_a = ((pq >> (lhd - 1)) << lhd) + (pq & (half - 1));   // half % 4 == 0: the four pairs share a head
       const int row_b = row_a + half;
       const int grow = m_tile * kBM + row_a;
-      const int head = grow / hd, i = grow % hd;
+      const int head = grow >> lhd, i = grow & (hd - 1);
       const bool rot = head < ep.n_q + ep.n_kv;
       // per-head q/k RMSNorm: the gains of these rows (q heads: q_norm, k heads: k_norm)
       const bool qkn = ep.qn_gain != nullptr && rot;
@@ -615,7 +622,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
           gnb[e] = __bfloat162float(gsrc[i + half + e]);
         }
       }
-      const int hh_tile = row_a / hd;   // head of this tile
+      const int hh_tile = row_a >> lhd;   // head of this tile
       auto store4 = [&](float* dst, __nv_bfloat16* dhi, __nv_bfloat16* dlo, int64_t o, const float (&x)[4]) {
         *reinterpret_cast<float4*>(dst + o) = make_float4(x[0], x[1], x[2], x[3]);
         if (dhi) {
@@ -674,11 +681,12 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
       }
     } else {   // QKV: pair p = m & 63 of this tile, 2 nhalf column groups of 64 threads
       const int p = m & 63, ng = 2 * nwh, grp = (m >> 6) + 2 * wh;
-      const int hd = ep.hd, half = hd / 2;
-      const int row_a = (p / half) * hd + (p % half);   // first element of the pair, within the tile
+      const int lhd = ep.hd == 128 ? 7 : 6;               // head_dim is 64 or 128
+      const int hd = 1 << lhd, half = hd >> 1;
+      const int row_a = ((p >> (lhd - 1)) << lhd) + (p & (half - 1));   // first element of the pair, within the tile
       const int row_b = row_a + half;
       const int grow = m_tile * kBM + row_a;              // row of W_qkv
-      const int head = grow / hd, i = grow % hd;          // i < half
+      const int head = grow >> lhd, i = grow & (hd - 1);  // i < half
       const bool rot = head < ep.n_q + ep.n_kv;   // q and k rows take RoPE, v rows do not
       // per-head q/k RMSNorm (q heads: q_norm, k heads: k_norm gains of these two rows)
       float gna = 1.f, gnb = 1.f;
@@ -687,7 +695,8 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
         gna = __bfloat162float(gsrc[i]);
         gnb = __bfloat162float(gsrc[i + half]);
       }
-      const int hh_tile = row_a / hd;
+      const int hh_tile = row_a >> lhd;
+#pragma unroll 1
       for (int c0 = cbeg + grp; c0 < cend; c0 += ng * kEpiBatch) {
         // a batch's operands (accumulator pair and rotation), read before its first store
         float av[kEpiBatch], bv[kEpiBatch];
@@ -832,16 +841,39 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
   return p;
 }
 
+namespace {
+
+typedef decltype(&gemm_cluster_kernel<false, GemmEpilogue::PLAIN>) GemmKernel;
+
+// The kernel image of a batch class and epilogue (null: none).
+GemmKernel gemm_image(bool large, int mode) {
+  switch (mode) {
+    case GemmEpilogue::PLAIN:
+      return large ? gemm_cluster_kernel<true, GemmEpilogue::PLAIN> : gemm_cluster_kernel<false, GemmEpilogue::PLAIN>;
+    case GemmEpilogue::QKV:
+      return large ? gemm_cluster_kernel<true, GemmEpilogue::QKV> : gemm_cluster_kernel<false, GemmEpilogue::QKV>;
+    case GemmEpilogue::RESID:
+      return large ? gemm_cluster_kernel<true, GemmEpilogue::RESID> : gemm_cluster_kernel<false, GemmEpilogue::RESID>;
+    case GemmEpilogue::SILU:
+      return large ? gemm_cluster_kernel<true, GemmEpilogue::SILU> : gemm_cluster_kernel<false, GemmEpilogue::SILU>;
+    case GemmEpilogue::LOWRANK:
+      return large ? gemm_cluster_kernel<true, GemmEpilogue::LOWRANK> : nullptr;
+  }
+  return nullptr;
+}
+
+}  // namespace
+
 cudaError_t gemm_configure() {
-  cudaError_t e = cudaFuncSetAttribute(gemm_cluster_kernel<false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(kGemmMaxSmem));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(gemm_cluster_kernel<true>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(kGemmMaxSmem));
-  if (e != cudaSuccess) return e;
-  e = cudaFuncSetAttribute(gemm_cluster_kernel<false>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
-  if (e != cudaSuccess) return e;
-  return cudaFuncSetAttribute(gemm_cluster_kernel<true>, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  for (int large = 0; large < 2; ++large)
+    for (int mode = GemmEpilogue::PLAIN; mode <= GemmEpilogue::LOWRANK; ++mode) {
+      const GemmKernel k = gemm_image(large != 0, mode);
+      if (!k) continue;
+      cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kGemmMaxSmem));
+      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e != cudaSuccess) return e;
+    }
+  return cudaSuccess;
 }
 
 cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtensorMap* tmX, const CUtensorMap* tmXlo,
@@ -871,14 +903,12 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
   const CUtensorMap& mt = with_lr ? *lr->t_hi : *tmX;
   const CUtensorMap& mtl = with_lr ? (p.has_lo ? *lr->t_lo : *lr->t_hi) : xlo;
   const int k_main = with_lr ? lr->k_main : p.k_tiles;
-  // the adapter's A x (LOWRANK) runs on the large-batch image at every batch size, so that the
-  // small-batch image keeps its register allocation
-  if (large)
-    return cudaLaunchKernelEx(&cfg, gemm_cluster_kernel<true>, *tmW, *tmX, xlo, p.has_lo ? 1 : 0, mb, mt, mtl, k_main,
-                              p.k_tiles, p.cluster, p.stages, p.tmem_cols, n_pad, p.mt, ep, err, ts);
-  if (p.mt != 1) return cudaErrorInvalidValue;   // two m-tiles per CTA exist in the large-batch image only
-  return cudaLaunchKernelEx(&cfg, gemm_cluster_kernel<false>, *tmW, *tmX, xlo, p.has_lo ? 1 : 0, mb, mt, mtl, k_main,
-                            p.k_tiles, p.cluster, p.stages, p.tmem_cols, n_pad, 1, ep, err, ts);
+  // the adapter's A x (LOWRANK) runs on the large-batch image at every batch size; two m-tiles per CTA
+  // exist in the large-batch images only
+  const GemmKernel kern = gemm_image(large, ep.mode);
+  if (!kern || (!large && p.mt != 1)) return cudaErrorInvalidValue;
+  return cudaLaunchKernelEx(&cfg, kern, *tmW, *tmX, xlo, p.has_lo ? 1 : 0, mb, mt, mtl, k_main, p.k_tiles, p.cluster,
+                            p.stages, p.tmem_cols, n_pad, p.mt, ep, err, ts);
 }
 
 }  // namespace kvprm
