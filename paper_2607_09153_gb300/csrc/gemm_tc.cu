@@ -61,7 +61,7 @@ __device__ __forceinline__ void store_hilo(__nv_bfloat16* hi, __nv_bfloat16* lo,
   lo[i] = __float2bfloat16_rn(x - __bfloat162float(h));
 }
 
-// LARGE (n_pad >= 64, one kernel image per batch class so that the small-batch code keeps its own
+// LARGE (n_pad >= 48, one kernel image per batch class so that the small-batch code keeps its own
 // register allocation): the residual epilogue issues a 16-column group's residual loads before
 // using any and sums each column's squares in one pass over the parked tile, clusters of 4 reduce
 // with 16-byte DSMEM loads, and the epilogues move 4 or 8 consecutive rows of a column per thread
@@ -213,12 +213,22 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
       }
     // RESID: the residual values the epilogue adds to, read now rather than after the MMAs, when
     // the next kernel's weight stream may be competing for the memory system
-    if (hpreload)
-#pragma unroll 4
-      for (int idx = threadIdx.x - 64; idx < nc * kBM; idx += blockDim.x - 64) {
-        const int c = cbeg + idx / kBM, gm = m_tile0 * kBM + idx % kBM;
-        hpre[idx] = gm < ep.M ? ep.h[static_cast<int64_t>(c) * ep.M + gm] : 0.f;
+    if (hpreload) {   // warps 2 and 3 take alternate columns, 16 bytes a lane, all in flight at once
+      float4 v[kHPreCols / 2];
+      const int gm = m_tile0 * kBM + 4 * lane;
+#pragma unroll
+      for (int k = 0; k < kHPreCols / 2; ++k) {
+        const int cl = 2 * k + (warp & 1);
+        v[k] = (warp < 4 && cl < nc && gm < ep.M)
+                   ? *reinterpret_cast<const float4*>(ep.h + static_cast<int64_t>(cbeg + cl) * ep.M + gm)
+                   : make_float4(0.f, 0.f, 0.f, 0.f);
       }
+#pragma unroll
+      for (int k = 0; k < kHPreCols / 2; ++k) {
+        const int cl = 2 * k + (warp & 1);
+        if (warp < 4 && cl < nc) *reinterpret_cast<float4*>(hpre + cl * kBM + 4 * lane) = v[k];
+      }
+    }
   } else if (warp == 1 && nk > 0) {
     // ---------------- MMA issuer (the whole warp; one elected lane issues)
     // With the hi and lo activation tiles stored back to back (2 n_pad rows
@@ -414,8 +424,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
       if (gm < ep.M)
 #pragma unroll 4
         for (int c = cbeg + wh; c < cend; c += nwh) ep.out[static_cast<int64_t>(c) * ep.M + gm] = acc[c * kBM + m];
-    } else if constexpr (MODE == GemmEpilogue::LOWRANK) {   // t = s (A x), hi/lo [n][r]; large image only
-      static_assert(LARGE || MODE != GemmEpilogue::LOWRANK, "the adapter's A x has a large-batch image only");
+    } else if constexpr (MODE == GemmEpilogue::LOWRANK) {   // t = s (A x), hi/lo [n][r]
       const int gm = m_tile * kBM + m;
       if (gm < ep.M)
 #pragma unroll 2
@@ -446,8 +455,9 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
             const int c = c0 + nw * k;
-            h_in[k] = (c < cend && rows_ok) ? *reinterpret_cast<const float4*>(ep.h + static_cast<int64_t>(c) * ep.M + gm0)
-                                            : make_float4(0.f, 0.f, 0.f, 0.f);
+            h_in[k] = !(c < cend && rows_ok) ? make_float4(0.f, 0.f, 0.f, 0.f)
+                      : hpreload ? *reinterpret_cast<const float4*>(hpre + (c - cbeg) * kBM + 4 * rq)
+                                 : *reinterpret_cast<const float4*>(ep.h + static_cast<int64_t>(c) * ep.M + gm0);
           }
 #pragma unroll
           for (int k = 0; k < 8; ++k) {
@@ -537,6 +547,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
       // divide take the fast intrinsics
       const int rg = static_cast<int>(threadIdx.x) & 7, cg = static_cast<int>(threadIdx.x) >> 3;
       const int j0 = m_tile * 64 + 8 * rg;   // ff % 8 == 0: a row group is all valid or all past ff
+      const bool few = n_pad < 64;   // the exact functions at batches where their time does not show
       if (j0 < ep.ff) {
 #pragma unroll 2
         for (int c = cbeg + cg; c < cend; c += 4 * nw) {   // 4 nw column groups of 8 threads
@@ -550,8 +561,8 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
 #pragma unroll
           for (int e = 0; e < 4; ++e) {
             const float ga = g[2 * e] * rs, gb = g[2 * e + 1] * rs;
-            const float a = __fdividef(ga, 1.0f + __expf(-ga)) * (u[2 * e] * rs);
-            const float b = __fdividef(gb, 1.0f + __expf(-gb)) * (u[2 * e + 1] * rs);
+            const float a = (few ? ga / (1.0f + expf(-ga)) : __fdividef(ga, 1.0f + __expf(-ga))) * (u[2 * e] * rs);
+            const float b = (few ? gb / (1.0f + expf(-gb)) : __fdividef(gb, 1.0f + __expf(-gb))) * (u[2 * e + 1] * rs);
             const __nv_bfloat162 h2 = __floats2bfloat162_rn(a, b);
             const float2 hf = __bfloat1622float2(h2);
             const __nv_bfloat162 l2 = __floats2bfloat162_rn(a - hf.x, b - hf.y);
@@ -767,16 +778,38 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
   // cluster size: the largest power of two <= 16 that keeps the CTA count within what fits on the
   // SMs at once (two per SM when two CTAs' shared memory fits, else one: at B = 256 a stage holds
   // 64 KB of activations) and gives every rank at least two K tiles
-  const int per_sm = p.smem_bytes + 1024 <= 228u * 1024u / 2 ? 2 : 1;
+  constexpr size_t kHalfSm = 228u * 1024u / 2;
+  int per_sm = p.smem_bytes + 1024 <= kHalfSm ? 2 : 1;
   // A cluster is placed whole on one GPC.  With two CTAs per SM, a grid that needs (nearly) every
   // slot cannot be placed in one wave while the preceding kernel still holds part of the SMs
   // (programmatic dependent launch places this grid's first clusters early, half-filling SMs in a
   // pattern that strands slots): the 7B QKV projection at B = 64, 36 clusters of 8 = 288 of 304
   // slots, had its last clusters start ~10 us after the preceding kernel ended.  Such grids keep
   // within 7/8 of the slots.
-  const int slots = per_sm == 2 ? per_sm * num_sms * 7 / 8 : per_sm * num_sms;
-  int cs = 1;
-  while (cs < 16 && p.m_tiles * cs * 2 <= slots && cs * 4 <= p.k_tiles && cs * 2 <= n_pad) cs *= 2;
+  auto cluster_of = [&](int ctas_per_sm) {
+    const int slots = ctas_per_sm == 2 ? ctas_per_sm * num_sms * 7 / 8 : ctas_per_sm * num_sms;
+    int c = 1;
+    while (c < 16 && p.m_tiles * c * 2 <= slots && c * 4 <= p.k_tiles && c * 2 <= n_pad) c *= 2;
+    return c;
+  };
+  int cs = cluster_of(per_sm);
+  // One stage less can let two CTAs share an SM (48 and 80 padded columns: a few KB too many).  Taken
+  // where it saves a second wave (the 296 CTAs of the 7B gate/up at 48 columns: 52 -> 46 us) or lets a
+  // long K loop run on twice the CTAs (the 7B down projection 31 -> 26 us at 48 columns, 37 -> 35 at 80);
+  // elsewhere the deeper ring of the single CTA is worth more (the 7B QKV at 80 columns: 12.4 us, 17.3
+  // with a stage less).
+  if (per_sm == 1 && p.stages > 2) {
+    size_t less = static_cast<size_t>(p.stages - 1) * stage_bytes;
+    if (less < acc) less = acc;
+    const int cs2 = cluster_of(2);
+    if (less + 1024 + kTailBytes + 1024 <= kHalfSm &&
+        ((n_pad <= 64 && cs == 1 && p.m_tiles > num_sms) || (cs2 > cs && (p.k_tiles + cs - 1) / cs >= 16))) {
+      --p.stages;
+      p.smem_bytes = less + 1024 + kTailBytes;
+      per_sm = 2;
+      cs = cs2;
+    }
+  }
   p.cluster = cs;
   p.splits = cs;
   p.kt_per_split = (p.k_tiles + cs - 1) / cs;
@@ -857,7 +890,7 @@ GemmKernel gemm_image(bool large, int mode) {
     case GemmEpilogue::SILU:
       return large ? gemm_cluster_kernel<true, GemmEpilogue::SILU> : gemm_cluster_kernel<false, GemmEpilogue::SILU>;
     case GemmEpilogue::LOWRANK:
-      return large ? gemm_cluster_kernel<true, GemmEpilogue::LOWRANK> : nullptr;
+      return large ? gemm_cluster_kernel<true, GemmEpilogue::LOWRANK> : gemm_cluster_kernel<false, GemmEpilogue::LOWRANK>;
   }
   return nullptr;
 }
@@ -868,7 +901,6 @@ cudaError_t gemm_configure() {
   for (int large = 0; large < 2; ++large)
     for (int mode = GemmEpilogue::PLAIN; mode <= GemmEpilogue::LOWRANK; ++mode) {
       const GemmKernel k = gemm_image(large != 0, mode);
-      if (!k) continue;
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kGemmMaxSmem));
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
       if (e != cudaSuccess) return e;
@@ -881,7 +913,9 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
                         unsigned long long* ts, const GemmLowRank* lr) {
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3((p.m_tiles + p.mt - 1) / p.mt * p.cluster, 1, 1);
-  const bool large = n_pad >= 64 || ep.mode == GemmEpilogue::LOWRANK;
+  // the vector epilogues win from 48 padded columns on even with four warps (40 candidates of a 7B scorer
+  // 564 -> 532 us for four layers; 24 candidates, 32 columns: 397 us small, 405 large)
+  const bool large = n_pad >= 48;
   if (p.threads != 128 && (p.threads != 256 || !large)) return cudaErrorInvalidValue;
   cfg.blockDim = dim3(static_cast<unsigned>(p.threads), 1, 1);
   cfg.dynamicSmemBytes = p.smem_bytes;
@@ -903,8 +937,7 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
   const CUtensorMap& mt = with_lr ? *lr->t_hi : *tmX;
   const CUtensorMap& mtl = with_lr ? (p.has_lo ? *lr->t_lo : *lr->t_hi) : xlo;
   const int k_main = with_lr ? lr->k_main : p.k_tiles;
-  // the adapter's A x (LOWRANK) runs on the large-batch image at every batch size; two m-tiles per CTA
-  // exist in the large-batch images only
+  // two m-tiles per CTA exist in the large-batch images only
   const GemmKernel kern = gemm_image(large, ep.mode);
   if (!kern || (!large && p.mt != 1)) return cudaErrorInvalidValue;
   return cudaLaunchKernelEx(&cfg, kern, *tmW, *tmX, xlo, p.has_lo ? 1 : 0, mb, mt, mtl, k_main, p.k_tiles, p.cluster,
