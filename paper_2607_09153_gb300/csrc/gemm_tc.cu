@@ -48,6 +48,7 @@ constexpr uint32_t kWTileBytes = kBM * kBK * 2;   // 16 KB
 // after the ring: barriers, TMEM slot and 64 block-sum floats (512 B), then 256
 // per-column RMSNorm factors (1 KB)
 constexpr size_t kTailBytes = 512 + 1024 + 4096;   // barriers, RMSNorm factors, preloaded residual
+constexpr int kHalfBoxCols = 96;                    // padded columns from which activation boxes hold half
 constexpr int kHPreCols = 8;                        // residual columns preloaded per rank (128 rows each)
 constexpr size_t kGemmMaxSmem = 200 * 1024;         // dynamic shared memory the kernel is configured for
 
@@ -73,7 +74,11 @@ __device__ __forceinline__ void store_hilo(__nv_bfloat16* hi, __nv_bfloat16* lo,
 // stage count and shifts by the head dimension: 51 KB of code in one small image became 20-32 KB in four
 // (large: 178 KB became 31-52), and a call of the 1.5B workload took 1,112 us instead of 1,155, with the
 // rank-256 adapter 1,687 instead of 1,932, MCTS 9,814 instead of 10,110.
-template <bool LARGE, int MODE>
+// PAIR (large batches; `plan_gemm` has the rule): a CTA pair's MMA multiplies both CTAs' weight tiles (M = 256)
+// with a B operand that is half in either CTA, so a CTA stages half of the activation rows.  At 256
+// columns a stage is 48 KB instead of 80, four fit instead of two, and a K tile's L2 reads fall from 80 KB
+// to 48: with two stages an m-tile's eight MMAs (0.53 us) waited for loads 0.35 us of every K tile.
+template <bool LARGE, int MODE, bool PAIR>
 __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmW,
                                                            const __grid_constant__ CUtensorMap tmX,
                                                            const __grid_constant__ CUtensorMap tmXlo, int has_lo,
@@ -87,10 +92,11 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
   // m-tiles of this CTA (LARGE only): a stage holds mt weight tiles, then the activation tile(s)
-  const int mt = LARGE ? mt_arg : 1;
+  const int mt = LARGE && !PAIR ? mt_arg : 1;
   const uint32_t x_bytes = static_cast<uint32_t>(n_pad) * kBK * 2;
   const uint32_t w_bytes = kWTileBytes * static_cast<uint32_t>(mt);
-  const uint32_t stage_bytes = w_bytes + x_bytes * (has_lo ? 2u : 1u);
+  // PAIR: half of the pair's activation rows, i.e. one part's n_pad rows or half of each part's
+  const uint32_t stage_bytes = w_bytes + x_bytes * (has_lo && !PAIR ? 2u : 1u);
   const uint32_t acc_bytes = static_cast<uint32_t>(n_pad) * kBM * 4;
   const uint32_t ring_bytes = stages * stage_bytes > acc_bytes ? stages * stage_bytes : acc_bytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + ring_bytes);
@@ -102,8 +108,16 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   float* hpre = rsc + 256;   // RESID: this rank's columns of h for the tile's rows, [c - cbeg][128]
 
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const int m_tile0 = blockIdx.x / cs * mt;   // first m-tile of this CTA
-  const uint32_t rank = cluster_rank();
+  // PAIR: cluster ranks 2 r and 2 r + 1 are split r's CTA pair, with an m-tile each
+  const uint32_t crank = cluster_rank();
+  const uint32_t rank = PAIR ? crank >> 1 : crank, side = PAIR ? crank & 1u : 0u;
+  // of the two m-tiles' n_pad columns, or (n_split 2, n_pad then the half) of one half of the batch's
+  const int n_split = PAIR ? mt_arg : 1, pair_unit = static_cast<int>(blockIdx.x) / (2 * cs);
+  const int m_tile0 = PAIR ? pair_unit / n_split * 2 + static_cast<int>(side)
+                           : static_cast<int>(blockIdx.x) / cs * mt;   // first m-tile of this CTA
+  const int c_off = PAIR ? pair_unit % n_split * n_pad : 0;   // first column
+  // the cluster rank of split r's CTA for this m-tile
+  auto peer = [&](int r) { return PAIR ? 2u * static_cast<uint32_t>(r) + side : static_cast<uint32_t>(r); };
   const int kps = (k_tiles + cs - 1) / cs;
   const int kt0 = static_cast<int>(rank) * kps;
   const int kt1 = min(k_tiles, kt0 + kps);
@@ -111,7 +125,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   constexpr bool silu = MODE == GemmEpilogue::SILU;
   // this rank's candidate columns in the reduction and the epilogue
   const int cols = n_pad / cs;
-  const int cbeg = static_cast<int>(rank) * cols;
+  const int cbeg = c_off + static_cast<int>(rank) * cols;
   const int cend = min(cbeg + cols, ep.n_valid);
   const int nc = cend > cbeg ? cend - cbeg : 0;
   const bool hpreload = MODE == GemmEpilogue::RESID && nc <= kHPreCols && mt == 1;
@@ -134,11 +148,19 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     }
   }
   if (warp == 1) {
-    tmem_alloc(tmem_slot, tmem_cols);
-    tmem_relinquish();
+    if constexpr (PAIR) {
+      tmem_alloc_pair(tmem_slot, tmem_cols);
+      tmem_relinquish_pair();
+    } else {
+      tmem_alloc(tmem_slot, tmem_cols);
+      tmem_relinquish();
+    }
   }
   tc_fence_before();
-  __syncthreads();
+  if constexpr (PAIR)
+    cluster_sync();   // the pair uses each other's barriers and tensor memory
+  else
+    __syncthreads();
   tc_fence_after();
   const uint32_t tmem = *tmem_slot;
   // Let the next kernel in the stream start its own independent prologue and
@@ -151,48 +173,71 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     const uint64_t pol_w = policy_evict_first();
     const uint64_t pol_x = policy_evict_last();
     // K tiles [0, k_main) come from W and x; a scorer adapter's tiles after them from B and t
-    auto load_w = [&](uint8_t* st, int kt, uint64_t* bar) {
+    auto load = [&](uint8_t* dst, const CUtensorMap* map, int stage, int x, int y, uint64_t pol) {
+      if constexpr (PAIR)   // both CTAs' copies complete on the even CTA's barrier, which its MMAs wait for
+        tma_load_2d_pair(dst, map, cluster_addr(&full[stage], crank & ~1u), x, y, pol);
+      else
+        tma_load_2d(dst, map, &full[stage], x, y, pol);
+    };
+    auto load_w = [&](int stage, int kt) {
+      if (!PAIR)
+        mbar_arrive_expect_tx(&full[stage], stage_bytes);
+      else if (side == 0)
+        mbar_arrive_expect_tx(&full[stage], 2 * stage_bytes);
       const CUtensorMap* wm = kt < k_main ? &tmW : &tmB;
       const int kx = (kt < k_main ? kt : kt - k_main) * kBK;
 #pragma unroll 1
       for (int t = 0; t < mt; ++t) {
         const int m_tile = m_tile0 + t;
-        uint8_t* wt = st + t * kWTileBytes;
+        uint8_t* wt = smem + stage * stage_bytes + t * kWTileBytes;
         if (!silu) {
-          tma_load_2d(wt, wm, bar, kx, m_tile * kBM, pol_w);
+          load(wt, wm, stage, kx, m_tile * kBM, pol_w);
         } else {   // 64 gate rows, then the matching 64 up rows
-          tma_load_2d(wt, wm, bar, kx, m_tile * 64, pol_w);
-          tma_load_2d(wt + kWTileBytes / 2, wm, bar, kx, ep.ff + m_tile * 64, pol_w);
+          load(wt, wm, stage, kx, m_tile * 64, pol_w);
+          load(wt + kWTileBytes / 2, wm, stage, kx, ep.ff + m_tile * 64, pol_w);
         }
       }
     };
-    auto load_x = [&](uint8_t* st, int kt, uint64_t* bar) {
+    // the activation maps' boxes hold the batch's columns, from 96 on half of them (gemm_x_box): a stage's
+    // rows are then loaded as halves (hi, hi, lo, lo), of which a pair's CTA takes its own
+    auto load_x = [&](int stage, int kt) {
       const bool main = kt < k_main;
       const int kx = (main ? kt : kt - k_main) * kBK;
-      tma_load_2d(st + w_bytes, main ? &tmX : &tmT, bar, kx, 0, pol_x);
-      if (has_lo) tma_load_2d(st + w_bytes + x_bytes, main ? &tmXlo : &tmTlo, bar, kx, 0, pol_x);
+      const CUtensorMap *xh = main ? &tmX : &tmT, *xl = main ? &tmXlo : &tmTlo;
+      uint8_t* xt = smem + stage * stage_bytes + w_bytes;
+      if (PAIR && n_split == 2) {
+        load(xt, side ? xl : xh, stage, kx, c_off, pol_x);
+      } else if (!LARGE || n_pad < kHalfBoxCols) {
+        if (!PAIR || side == 0) load(xt, xh, stage, kx, 0, pol_x);
+        if (PAIR ? side == 1 : has_lo) load(PAIR ? xt : xt + x_bytes, xl, stage, kx, 0, pol_x);
+      } else {
+        const uint32_t hb = x_bytes / 2;
+        const int hr = n_pad / 2;
+#pragma unroll 1
+        for (int q = 0; q < (PAIR || !has_lo ? 2 : 4); ++q) {
+          // a pair's CTA: both halves of one part where an MMA covers both parts, else its half of each
+          const bool lo_part = PAIR ? (n_pad <= 128 ? side : q) != 0 : q >= 2;
+          const int y = PAIR ? (n_pad <= 128 ? q : static_cast<int>(side)) : (q & 1);
+          load(xt + q * hb, lo_part ? xl : xh, stage, kx, y * hr, pol_x);
+        }
+      }
     };
     // Weights do not depend on the preceding kernel: start streaming the first
     // ring's worth of W before waiting for the activations it produces.
     const int pre = min(stages, nk);
 #pragma unroll 1
-    for (int i = 0; i < pre; ++i) {
-      mbar_arrive_expect_tx(&full[i], stage_bytes);
-      load_w(smem + i * stage_bytes, kt0 + i, &full[i]);
-    }
+    for (int i = 0; i < pre; ++i) load_w(i, kt0 + i);
     grid_dep_wait();
     trace_event(ts, 0);   // the preceding kernel has completed
 #pragma unroll 1
-    for (int i = 0; i < pre; ++i) load_x(smem + i * stage_bytes, kt0 + i, &full[i]);
+    for (int i = 0; i < pre; ++i) load_x(i, kt0 + i);
     int s = 0;   // stage of K tile i, and the parity of the release before its use
     uint32_t parity = 0u;
 #pragma unroll 1
     for (int i = pre; i < nk; ++i) {
       if (!mbar_wait(&empty[s], parity, err)) break;
-      uint8_t* st = smem + s * stage_bytes;
-      mbar_arrive_expect_tx(&full[s], stage_bytes);
-      load_w(st, kt0 + i, &full[s]);
-      load_x(st, kt0 + i, &full[s]);
+      load_w(s, kt0 + i);
+      load_x(s, kt0 + i);
       if (++s == stages) {
         s = 0;
         parity ^= 1u;
@@ -229,7 +274,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
         if (warp < 4 && cl < nc) *reinterpret_cast<float4*>(hpre + cl * kBM + 4 * lane) = v[k];
       }
     }
-  } else if (warp == 1 && nk > 0) {
+  } else if (warp == 1 && nk > 0 && side == 0) {
     // ---------------- MMA issuer (the whole warp; one elected lane issues)
     // With the hi and lo activation tiles stored back to back (2 n_pad rows
     // under the same swizzle), one MMA of N = 2 n_pad reads each weight K
@@ -240,8 +285,15 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     // allocation, a power of two).
     const bool merged = has_lo && 2 * n_pad <= 256;
     const bool two = has_lo && !merged;
-    const uint32_t idesc = idesc_bf16_f32(kBM, merged ? 2 * n_pad : n_pad);
-    const uint32_t tile_cols = tmem_cols / static_cast<uint32_t>(mt);
+    // A pair's MMA (M = 256, both CTAs' weight tiles) takes half of its B rows from either CTA: one part
+    // each when merged, else half of the hi and half of the lo rows.
+    const uint32_t idesc = idesc_bf16_f32(PAIR ? 2 * kBM : kBM, merged ? 2 * n_pad : n_pad);
+    const uint16_t pair_mask = static_cast<uint16_t>(3u << crank);
+    // PAIR: two accumulators, one of the hi and one of the lo part, or when merged one of the first and
+    // one of the second half of the K tiles: half as many fp32 roundings in a row (without them rewards
+    // were 10-20 % further off, a pair's CTA having twice the K tiles of the CTA it replaces).
+    const uint32_t tile_cols = tmem_cols / static_cast<uint32_t>(PAIR ? 2 : mt);
+    const int i_half = PAIR && merged ? (nk + 1) / 2 : nk;   // the second accumulator's first K tile
     int s = 0;
     uint32_t parity = 0u;
 #pragma unroll 1
@@ -251,25 +303,36 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
       tc_fence_after();
       const uint64_t a0 = desc_sw128(smem_u32(smem + s * stage_bytes));   // K step kk: + 2 kk (32 bytes)
       const uint64_t b0 = a0 + (w_bytes >> 4);
-      const uint64_t l0 = b0 + static_cast<uint64_t>(x_bytes >> 4);
-      const uint32_t acc0 = i > 0 ? 1u : 0u;
+      const uint64_t l0 = b0 + static_cast<uint64_t>((PAIR ? x_bytes / 2 : x_bytes) >> 4);
+      const uint32_t acc0 = i > 0 && i != i_half ? 1u : 0u;
 #pragma unroll 1
       for (int t = 0; t < mt; ++t) {
-        const uint32_t d = tmem + static_cast<uint32_t>(t) * tile_cols;
+        const uint32_t d = tmem + (PAIR ? (i >= i_half ? tile_cols : 0u) : static_cast<uint32_t>(t) * tile_cols);
         const uint64_t at = a0 + static_cast<uint64_t>(t) * (kWTileBytes >> 4);
 #pragma unroll
         for (int kk = 0; kk < kBK / 16; ++kk) {
-          umma_bf16_w(d, at + 2 * kk, b0 + 2 * kk, idesc, kk > 0 ? 1u : acc0);
-          if (LARGE && two) umma_bf16_w(d, at + 2 * kk, l0 + 2 * kk, idesc, 1u);   // n_pad > 128
+          if constexpr (PAIR) {
+            umma_bf16_pair_w(d, at + 2 * kk, b0 + 2 * kk, idesc, kk > 0 ? 1u : acc0);
+            if (two) umma_bf16_pair_w(d + tile_cols, at + 2 * kk, l0 + 2 * kk, idesc, kk > 0 ? 1u : acc0);
+          } else {
+            umma_bf16_w(d, at + 2 * kk, b0 + 2 * kk, idesc, kk > 0 ? 1u : acc0);
+            if (LARGE && two) umma_bf16_w(d, at + 2 * kk, l0 + 2 * kk, idesc, 1u);   // n_pad > 128
+          }
         }
       }
-      umma_commit_w(&empty[s]);
+      if constexpr (PAIR)
+        umma_commit_pair_w(&empty[s], pair_mask);
+      else
+        umma_commit_w(&empty[s]);
       if (++s == stages) {
         s = 0;
         parity ^= 1u;
       }
     }
-    umma_commit_w(done);
+    if constexpr (PAIR)
+      umma_commit_pair_w(done, pair_mask);
+    else
+      umma_commit_w(done);
   }
   __syncwarp();
 
@@ -277,48 +340,81 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   const bool have = nk > 0 ? __all_sync(0xffffffffu, mbar_wait(done, 0, err)) : true;
   if (threadIdx.x == 0) trace_event(ts, 2);   // all MMAs of this CTA completed
   tc_fence_after();
-  float* acc = reinterpret_cast<float*>(smem);   // the ring is idle once `done` has fired
+  // the ring is idle once `done` has fired; indexed by the batch's column, this CTA's first at the start
+  float* acc = reinterpret_cast<float*>(smem) - c_off * kBM;
   // 4 warps, or 8 (the large-batch image): warps w and w + 4 share TMEM lane quadrant w,
   // i.e. the tile's rows 32 w .. 32 w + 31, and take alternate 16-column groups (or columns)
   const int nw = static_cast<int>(blockDim.x >> 5), nwh = nw >> 2, wh = warp >> 2;
   const int m = (warp & 3) * 32 + lane;
   const bool merged = has_lo && 2 * n_pad <= 256;
-  const uint32_t tile_cols = tmem_cols / static_cast<uint32_t>(mt);
-  // one m-tile at a time: park it, reduce it over the cluster (split K), write its epilogue; with two
-  // tiles and split K the second is parked once every peer has read this CTA's first partial
+  const uint32_t tile_cols = tmem_cols / static_cast<uint32_t>(PAIR ? 2 : mt);
+  // one m-tile at a time (two without split K only): park it, reduce it over the cluster, write its epilogue
 #pragma unroll 1
   for (int tt = 0; tt < mt; ++tt) {
     const int m_tile = m_tile0 + tt;
     const uint32_t tcol = static_cast<uint32_t>(tt) * tile_cols;
-    if (tt > 0 && cs > 1) cluster_wait();   // matches the arrive after the previous tile's reduction
-#pragma unroll 1
-    for (int c0 = 16 * wh; c0 < n_pad; c0 += 16 * nwh) {
-      float v[16];
-      if (nk > 0 && have) {
-        const uint32_t t = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + tcol + static_cast<uint32_t>(c0);
-        tmem_ld16(t, v);
+    const uint32_t trow = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + tcol;
+    if constexpr (PAIR) {
+      // the two accumulators, a group's loads in flight while the one before it is stored
+      const uint32_t np = static_cast<uint32_t>(n_pad);
+      const bool second = nk > 0 && have && (!merged || nk > 1), any = nk > 0 && have;
+      float v[16], w[16], v2[16], w2[16];
+      auto issue = [&](int c0) {
+        const uint32_t t = trow + static_cast<uint32_t>(c0);
+        tmem_ld16_nowait(t, v);
+        tmem_ld16_nowait(t + tile_cols, v2);
         if (merged) {
-          float w[16];
-          tmem_ld16(t + static_cast<uint32_t>(n_pad), w);
-#pragma unroll
-          for (int j = 0; j < 16; ++j) v[j] += w[j];
+          tmem_ld16_nowait(t + np, w);
+          tmem_ld16_nowait(t + tile_cols + np, w2);
         }
-      } else {
+      };
+      if (16 * wh < n_pad) issue(16 * wh);
+#pragma unroll 1
+      for (int c0 = 16 * wh; c0 < n_pad; c0 += 16 * nwh) {
+        float r[16];
+        tmem_wait_ld();
+        tmem_hold(v);
+        tmem_hold(v2);
 #pragma unroll
-        for (int j = 0; j < 16; ++j) v[j] = 0.f;
+        for (int j = 0; j < 16; ++j) r[j] = (any ? v[j] : 0.f) + (second ? v2[j] : 0.f);
+        if (merged) {
+          tmem_hold(w);
+          tmem_hold(w2);
+#pragma unroll
+          for (int j = 0; j < 16; ++j) r[j] += (any ? w[j] : 0.f) + (second ? w2[j] : 0.f);
+        }
+        if (c0 + 16 * nwh < n_pad) issue(c0 + 16 * nwh);
+#pragma unroll
+        for (int j = 0; j < 16; ++j) acc[(c_off + c0 + j) * kBM + m] = r[j];
       }
+    } else {
+#pragma unroll 1
+      for (int c0 = 16 * wh; c0 < n_pad; c0 += 16 * nwh) {
+        float v[16];
+        if (nk > 0 && have) {
+          const uint32_t t = trow + static_cast<uint32_t>(c0);
+          tmem_ld16(t, v);
+          if (merged) {
+            float w[16];
+            tmem_ld16(t + static_cast<uint32_t>(n_pad), w);
 #pragma unroll
-      for (int j = 0; j < 16; ++j) acc[(c0 + j) * kBM + m] = v[j];
+            for (int j = 0; j < 16; ++j) v[j] += w[j];
+          }
+        } else {
+#pragma unroll
+          for (int j = 0; j < 16; ++j) v[j] = 0.f;
+        }
+#pragma unroll
+        for (int j = 0; j < 16; ++j) acc[(c0 + j) * kBM + m] = v[j];
+      }
     }
     tc_fence_before();
-    if (tt == 0 || cs > 1) {
+    if (tt == 0) {
       cluster_sync();   // every rank's partial is parked
-      if (tt == 0) {
-        if (threadIdx.x == 0) trace_event(ts, 3);
-        if (ep.late_trigger) grid_dep_launch();
-        // ---------------- reduce this rank's candidate columns over the cluster, then the epilogue
-        grid_dep_wait();   // outputs may still be read by kernels that precede this one
-      }
+      if (threadIdx.x == 0) trace_event(ts, 3);
+      if (ep.late_trigger) grid_dep_launch();
+      // ---------------- reduce this rank's candidate columns over the cluster, then the epilogue
+      grid_dep_wait();   // outputs may still be read by kernels that precede this one
       // Step 1: acc[c][m] <- sum over ranks of acc_r[c][m] for this rank's columns
       // (only this rank reads them, so it may overwrite its own copy).  Two columns
       // per round trip when the cluster has <= 8 ranks (four with 16-byte loads in
@@ -337,7 +433,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
 #pragma unroll
             for (int k = 0; k < 16; ++k) {   // rank k % CS of column c0 + nw (k / CS)
               const int cc = c0 + nw * (k / CS);
-              v[k] = cc < cend ? ld_cluster4(acc + cc * kBM + 4 * rq, static_cast<uint32_t>(k % CS))
+              v[k] = cc < cend ? ld_cluster4(acc + cc * kBM + 4 * rq, peer(k % CS))
                                : make_float4(0.f, 0.f, 0.f, 0.f);
             }
 #pragma unroll
@@ -367,7 +463,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
             const int r = step == 2 ? (k & 7) : k;
             const int cc = (step == 2 && k >= 8) ? c + 1 : c;
             const bool use = r < cs && (cc == c || two);
-            v[k] = use ? ld_cluster(acc + cc * kBM + m, static_cast<uint32_t>(r)) : 0.f;
+            v[k] = use ? ld_cluster(acc + cc * kBM + m, peer(r)) : 0.f;
           }
           if (step == 2) {
             float s0 = 0.f, s1 = 0.f;
@@ -389,8 +485,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
       }
       if (threadIdx.x == 0) trace_event(ts, 4);   // this rank's columns are reduced over the cluster
       // no peer reads this tile's partial any more once every rank has arrived here: arrive now and
-      // wait only before this shared memory is reused (the next tile's parking, or the exit), so the
-      // barrier's latency hides behind the epilogue
+      // wait only before the exit, so the barrier's latency hides behind the epilogue
       __syncwarp();
       cluster_arrive();
     }
@@ -755,11 +850,18 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   __syncwarp();
   cluster_wait();   // peers have finished reading this CTA's partial
   if (threadIdx.x == 0) trace_event(ts, 7);
-  if (warp == 1) tmem_dealloc(tmem, tmem_cols);
+  if (warp == 1) {
+    if constexpr (PAIR)
+      tmem_dealloc_pair(tmem, tmem_cols);
+    else
+      tmem_dealloc(tmem, tmem_cols);
+  }
   trace_end(ts);
 }
 
 }  // namespace
+
+uint32_t gemm_x_box(int n_pad) { return static_cast<uint32_t>(n_pad >= kHalfBoxCols ? n_pad / 2 : n_pad); }
 
 GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_up) {
   GemmPlan p;
@@ -785,11 +887,17 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
   // (programmatic dependent launch places this grid's first clusters early, half-filling SMs in a
   // pattern that strands slots): the 7B QKV projection at B = 64, 36 clusters of 8 = 288 of 304
   // slots, had its last clusters start ~10 us after the preceding kernel ended.  Such grids keep
-  // within 7/8 of the slots.
+  // within 7/8 of the slots.  With one CTA per SM, the GPCs (of 18 to 20 SMs, one of fewer) take 36
+  // clusters of 4, 15 of 8 and 7 of 16: what they cannot place starts when the first wave ends (16
+  // clusters of 8 for the 1.5B QKV projection at 256 columns: 12 us later, 22.4 us in all; 12.1 in 4s).
+  auto fit = [&](int c) {
+    return c == 1 ? num_sms : (c == 2 ? num_sms / 2 : num_sms * (c == 4 ? 36 : (c == 8 ? 15 : 7)) / 152);
+  };
   auto cluster_of = [&](int ctas_per_sm) {
-    const int slots = ctas_per_sm == 2 ? ctas_per_sm * num_sms * 7 / 8 : ctas_per_sm * num_sms;
     int c = 1;
-    while (c < 16 && p.m_tiles * c * 2 <= slots && c * 4 <= p.k_tiles && c * 2 <= n_pad) c *= 2;
+    while (c < 16 && c * 4 <= p.k_tiles && c * 2 <= n_pad &&
+           (ctas_per_sm == 2 ? p.m_tiles * c * 2 <= 2 * num_sms * 7 / 8 : p.m_tiles <= fit(2 * c)))
+      c *= 2;
     return c;
   };
   int cs = cluster_of(per_sm);
@@ -841,32 +949,37 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
       p.tmem_cols = 2 * cols;
     }
   }
-  // long split-K loops at large batches (the 7B down projection at B = 256: 74 K tiles per rank): two
-  // m-tiles per CTA over twice the ranks, the same CTA count.  A 96 KB stage then carries 16 MMAs
-  // (~1 us), enough to cover its own loading (~0.8 us), where one tile's 8 MMAs left the tensor pipe
-  // waiting a third of the time; the second tile's parking and cluster reduction cost less than those
-  // stalls once the K loop is long
-  if (!gate_up && n_pad >= 128 && per_sm == 1 && p.mt == 1 && cs >= 2 && cs * 2 <= 8 && p.m_tiles % 2 == 0 &&
-      p.kt_per_split >= 32) {
-    const int cs2 = cs * 2;
-    const uint32_t st2 = 2 * kWTileBytes + static_cast<uint32_t>(n_pad) * kBK * 2 * (has_lo ? 2u : 1u);
-    const int kps2 = (p.k_tiles + cs2 - 1) / cs2;
+  const int pc = cluster_of(1);
+  auto take_pairs = [&](int ranks, int n_split) {
+    const int cols2 = n_pad / n_split;
+    const uint32_t st2 = kWTileBytes + static_cast<uint32_t>(cols2) * kBK * 2;
+    const size_t acc2 = static_cast<size_t>((cols2 + 15) / 16 * 16) * kBM * 4;
+    const int kps = (p.k_tiles + ranks - 1) / ranks;
     int stages2 = static_cast<int>((192u * 1024u) / st2);
     if (stages2 > 8) stages2 = 8;
-    if (stages2 > kps2) stages2 = kps2;
-    size_t ring2 = static_cast<size_t>(stages2) * st2;
-    if (ring2 < acc) ring2 = acc;
-    const size_t smem2 = ring2 + 1024 + kTailBytes;
-    if (stages2 >= 2 && 2 * p.tmem_cols <= 512 && smem2 <= kGemmMaxSmem && (p.m_tiles / 2) * cs2 <= num_sms &&
-        cs2 * 4 <= p.k_tiles && n_pad % cs2 == 0) {
-      p.mt = 2;
-      p.cluster = cs2;
-      p.splits = cs2;
-      p.kt_per_split = kps2;
-      p.stages = stages2;
-      p.smem_bytes = smem2;
-      p.tmem_cols = 2 * p.tmem_cols;
-    }
+    if (stages2 > kps) stages2 = kps < 2 ? 2 : kps;
+    p.pair = true;
+    p.mt = 3 - n_split;
+    p.cluster = p.splits = 2 * ranks;
+    p.kt_per_split = (p.k_tiles + 2 * ranks - 1) / (2 * ranks);
+    p.stages = stages2;
+    ring = static_cast<size_t>(stages2) * st2;
+    p.smem_bytes = (ring < acc2 ? acc2 : ring) + 1024 + kTailBytes;
+    p.tmem_cols = 2 * cols;
+  };
+  // CTA pairs (see the kernel).  The CTAs that one m-tile each over pc ranks would take, as clusters of
+  // 2 pc for two m-tiles; or, where such clusters of 8 do not fit, and without a cluster reduction where pc
+  // is 2, as clusters of pc for two m-tiles and half of the columns.  7B at 256 columns: O 22.7 -> 18.7 us,
+  // down 62.5 -> 51.0 (it was two m-tiles a CTA over 8 ranks), QKV 22.6 -> 19.3 (halves); 8B at 256: QKV
+  // 35.1 -> 26.8 (halves; 35.1 too as whole pairs), O 24.3 -> 20.6 (halves).  Fewer columns, 7B: O 12.2 ->
+  // 10.5 at 80 and 17.2 -> 13.4 at 144, down 35.5 -> 26 and 42.2 -> 32.5, QKV as halves 18.5 -> 13.9 at 96
+  // (but 12.4 -> 13.7 at 80).  8B QKV at 112: whole pairs 19.1, halves 20.7, neither 21.9.  Below 80 only a
+  // K loop over four ranks gains (7B O at 48: 11.4 -> 9.1; 8B QKV over two 14.4 -> 17.2).
+  if (!gate_up && has_lo && n_pad >= 48 && p.m_tiles % 2 == 0 && pc <= 4) {
+    if ((n_pad > 128 && pc == 2) || (n_pad >= kHalfBoxCols && pc == 4 && p.m_tiles / 2 > fit(8)))
+      take_pairs(pc / 2, 2);
+    else if ((n_pad >= 80 || pc == 4) && p.m_tiles / 2 <= fit(2 * pc))
+      take_pairs(pc, 1);
   }
   // the large-batch image runs eight warps instead of four (registers for two such CTAs per SM), so
   // that the parking, the cluster reduction and the epilogue after the MMAs run on twice the warps
@@ -876,21 +989,26 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
 
 namespace {
 
-typedef decltype(&gemm_cluster_kernel<false, GemmEpilogue::PLAIN>) GemmKernel;
+typedef decltype(&gemm_cluster_kernel<false, GemmEpilogue::PLAIN, false>) GemmKernel;
 
+enum GemmImage { kSmall, kLarge, kPair, kGemmImages };
+
+template <int MODE>
+GemmKernel image_of(GemmImage i) {
+  if (i == kPair) {   // gate/up tiles are not paired
+    if constexpr (MODE == GemmEpilogue::SILU) return nullptr;
+    else return gemm_cluster_kernel<true, MODE, true>;
+  }
+  return i == kLarge ? gemm_cluster_kernel<true, MODE, false> : gemm_cluster_kernel<false, MODE, false>;
+}
 // The kernel image of a batch class and epilogue (null: none).
-GemmKernel gemm_image(bool large, int mode) {
+GemmKernel gemm_image(GemmImage i, int mode) {
   switch (mode) {
-    case GemmEpilogue::PLAIN:
-      return large ? gemm_cluster_kernel<true, GemmEpilogue::PLAIN> : gemm_cluster_kernel<false, GemmEpilogue::PLAIN>;
-    case GemmEpilogue::QKV:
-      return large ? gemm_cluster_kernel<true, GemmEpilogue::QKV> : gemm_cluster_kernel<false, GemmEpilogue::QKV>;
-    case GemmEpilogue::RESID:
-      return large ? gemm_cluster_kernel<true, GemmEpilogue::RESID> : gemm_cluster_kernel<false, GemmEpilogue::RESID>;
-    case GemmEpilogue::SILU:
-      return large ? gemm_cluster_kernel<true, GemmEpilogue::SILU> : gemm_cluster_kernel<false, GemmEpilogue::SILU>;
-    case GemmEpilogue::LOWRANK:
-      return large ? gemm_cluster_kernel<true, GemmEpilogue::LOWRANK> : gemm_cluster_kernel<false, GemmEpilogue::LOWRANK>;
+    case GemmEpilogue::PLAIN: return image_of<GemmEpilogue::PLAIN>(i);
+    case GemmEpilogue::QKV: return image_of<GemmEpilogue::QKV>(i);
+    case GemmEpilogue::RESID: return image_of<GemmEpilogue::RESID>(i);
+    case GemmEpilogue::SILU: return image_of<GemmEpilogue::SILU>(i);
+    case GemmEpilogue::LOWRANK: return image_of<GemmEpilogue::LOWRANK>(i);
   }
   return nullptr;
 }
@@ -898,9 +1016,10 @@ GemmKernel gemm_image(bool large, int mode) {
 }  // namespace
 
 cudaError_t gemm_configure() {
-  for (int large = 0; large < 2; ++large)
+  for (int i = 0; i < kGemmImages; ++i)
     for (int mode = GemmEpilogue::PLAIN; mode <= GemmEpilogue::LOWRANK; ++mode) {
-      const GemmKernel k = gemm_image(large != 0, mode);
+      const GemmKernel k = gemm_image(static_cast<GemmImage>(i), mode);
+      if (!k) continue;
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kGemmMaxSmem));
       if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
       if (e != cudaSuccess) return e;
@@ -912,7 +1031,7 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
                         const GemmEpilogue& ep, int n_pad, int* err, cudaStream_t stream, bool pdl,
                         unsigned long long* ts, const GemmLowRank* lr) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((p.m_tiles + p.mt - 1) / p.mt * p.cluster, 1, 1);
+  cfg.gridDim = dim3((p.m_tiles + p.mt - 1) / p.mt * p.cluster, 1, 1);   // a pair's CTAs: m_tiles / 2 clusters too
   // the vector epilogues win from 48 padded columns on even with four warps (40 candidates of a 7B scorer
   // 564 -> 532 us for four layers; 24 candidates, 32 columns: 397 us small, 405 large)
   const bool large = n_pad >= 48;
@@ -937,11 +1056,13 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
   const CUtensorMap& mt = with_lr ? *lr->t_hi : *tmX;
   const CUtensorMap& mtl = with_lr ? (p.has_lo ? *lr->t_lo : *lr->t_hi) : xlo;
   const int k_main = with_lr ? lr->k_main : p.k_tiles;
+  const int n_split = p.pair && p.mt == 1 ? 2 : 1;
   // two m-tiles per CTA exist in the large-batch images only
-  const GemmKernel kern = gemm_image(large, ep.mode);
-  if (!kern || (!large && p.mt != 1)) return cudaErrorInvalidValue;
-  return cudaLaunchKernelEx(&cfg, kern, *tmW, *tmX, xlo, p.has_lo ? 1 : 0, mb, mt, mtl, k_main, p.k_tiles, p.cluster,
-                            p.stages, p.tmem_cols, n_pad, p.mt, ep, err, ts);
+  const GemmKernel kern = gemm_image(p.pair ? kPair : (large ? kLarge : kSmall), ep.mode);
+  if (!kern || (!large && p.mt != 1) || (p.pair && !p.has_lo)) return cudaErrorInvalidValue;
+  return cudaLaunchKernelEx(&cfg, kern, *tmW, *tmX, xlo, p.has_lo ? 1 : 0, mb, mt, mtl, k_main, p.k_tiles,
+                            p.pair ? p.cluster / 2 : p.cluster, p.stages, p.tmem_cols,
+                            n_pad / n_split, p.pair ? n_split : p.mt, ep, err, ts);
 }
 
 }  // namespace kvprm

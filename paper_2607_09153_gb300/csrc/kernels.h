@@ -25,7 +25,10 @@ struct GemmPlan {
   // m-tiles per CTA: 2 for a gate/up projection without split K whose one-tile CTAs would need two
   // waves (large batches); the CTA's stage then holds both weight tiles and one activation tile
   int mt = 1;
-  // threads per CTA: 256 on the large-batch image (n_pad >= 64), else 128
+  // CTA pairs: mt m-tiles over `cluster` CTAs as with mt = 2, a tile per CTA of a pair (cluster / 2 K
+  // splits), the pair's MMAs reading half of the activation tile from either CTA
+  bool pair = false;
+  // threads per CTA: 256 from 64 padded columns, else 128
   int threads = 128;
   uint32_t tmem_cols = 32;
   size_t smem_bytes = 0;
@@ -80,6 +83,8 @@ struct GemmEpilogue {
   bool late_trigger = false;
 };
 GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_up);
+// Rows of an activation operand's tensor-map box: n_pad, or from 96 columns half of them.
+uint32_t gemm_x_box(int n_pad);
 // A scorer adapter's term of a projection, y = W x + B t with t = s A x already computed (LOWRANK):
 // after its k_main K tiles of W and x the projection streams B [out][r] against t [n][r] as further
 // K tiles (the plan counts both: plan_gemm(M, 64 k_main + r, ...)).

@@ -521,12 +521,12 @@ int ensure_x_maps(kvprm_ctx* ctx, int n_pad) {
   if (ctx->tm_x_npad == n_pad) return KVPRM_OK;
   int rc;
   const uint64_t d = ctx->md.d, dq = static_cast<uint64_t>(ctx->md.n_q) * ctx->md.hd, ff = ctx->md.ff;
-  if ((rc = make_map(ctx, &ctx->tm_xhi, ctx->xhi, d, n_pad, 64, n_pad, "x_hi"))) return rc;
-  if ((rc = make_map(ctx, &ctx->tm_xlo, ctx->xlo, d, n_pad, 64, n_pad, "x_lo"))) return rc;
-  if ((rc = make_map(ctx, &ctx->tm_ohi, ctx->ohi, dq, n_pad, 64, n_pad, "o_hi"))) return rc;
-  if ((rc = make_map(ctx, &ctx->tm_olo, ctx->olo, dq, n_pad, 64, n_pad, "o_lo"))) return rc;
-  if ((rc = make_map(ctx, &ctx->tm_ahi, ctx->ahi, ff, n_pad, 64, n_pad, "a_hi"))) return rc;
-  if ((rc = make_map(ctx, &ctx->tm_alo, ctx->alo, ff, n_pad, 64, n_pad, "a_lo"))) return rc;
+  if ((rc = make_map(ctx, &ctx->tm_xhi, ctx->xhi, d, n_pad, 64, kvprm::gemm_x_box(n_pad), "x_hi"))) return rc;
+  if ((rc = make_map(ctx, &ctx->tm_xlo, ctx->xlo, d, n_pad, 64, kvprm::gemm_x_box(n_pad), "x_lo"))) return rc;
+  if ((rc = make_map(ctx, &ctx->tm_ohi, ctx->ohi, dq, n_pad, 64, kvprm::gemm_x_box(n_pad), "o_hi"))) return rc;
+  if ((rc = make_map(ctx, &ctx->tm_olo, ctx->olo, dq, n_pad, 64, kvprm::gemm_x_box(n_pad), "o_lo"))) return rc;
+  if ((rc = make_map(ctx, &ctx->tm_ahi, ctx->ahi, ff, n_pad, 64, kvprm::gemm_x_box(n_pad), "a_hi"))) return rc;
+  if ((rc = make_map(ctx, &ctx->tm_alo, ctx->alo, ff, n_pad, 64, kvprm::gemm_x_box(n_pad), "a_lo"))) return rc;
   ctx->tm_x_npad = n_pad;
   return KVPRM_OK;
 }
@@ -536,8 +536,8 @@ int ensure_t_maps(kvprm_ctx* ctx, int n_pad) {
   if (ctx->lora_rank == 0 || ctx->tm_t_npad == n_pad) return KVPRM_OK;
   int rc;
   const uint64_t r = static_cast<uint64_t>(ctx->lora_rank);
-  if ((rc = make_map(ctx, &ctx->tm_thi, ctx->thi, r, n_pad, 64, n_pad, "t_hi"))) return rc;
-  if ((rc = make_map(ctx, &ctx->tm_tlo, ctx->tlo, r, n_pad, 64, n_pad, "t_lo"))) return rc;
+  if ((rc = make_map(ctx, &ctx->tm_thi, ctx->thi, r, n_pad, 64, kvprm::gemm_x_box(n_pad), "t_hi"))) return rc;
+  if ((rc = make_map(ctx, &ctx->tm_tlo, ctx->tlo, r, n_pad, 64, kvprm::gemm_x_box(n_pad), "t_lo"))) return rc;
   ctx->tm_t_npad = n_pad;
   return KVPRM_OK;
 }
@@ -1146,14 +1146,14 @@ int ensure_grad_maps(kvprm_ctx* ctx, int n_pad) {
   if (g.tm_npad == n_pad) return KVPRM_OK;
   const ModelDims& m = ctx->md;
   int rc;
-  if ((rc = make_map(ctx, &g.tm_d_hi, g.ghi, m.d, n_pad, 64, n_pad, "grad hi (d)"))) return rc;
-  if ((rc = make_map(ctx, &g.tm_d_lo, g.glo, m.d, n_pad, 64, n_pad, "grad lo (d)"))) return rc;
-  if ((rc = make_map(ctx, &g.tm_gu_hi, g.ghi, 2 * static_cast<uint64_t>(m.ff), n_pad, 64, n_pad, "grad hi (gu)")))
+  if ((rc = make_map(ctx, &g.tm_d_hi, g.ghi, m.d, n_pad, 64, kvprm::gemm_x_box(n_pad), "grad hi (d)"))) return rc;
+  if ((rc = make_map(ctx, &g.tm_d_lo, g.glo, m.d, n_pad, 64, kvprm::gemm_x_box(n_pad), "grad lo (d)"))) return rc;
+  if ((rc = make_map(ctx, &g.tm_gu_hi, g.ghi, 2 * static_cast<uint64_t>(m.ff), n_pad, 64, kvprm::gemm_x_box(n_pad), "grad hi (gu)")))
     return rc;
-  if ((rc = make_map(ctx, &g.tm_gu_lo, g.glo, 2 * static_cast<uint64_t>(m.ff), n_pad, 64, n_pad, "grad lo (gu)")))
+  if ((rc = make_map(ctx, &g.tm_gu_lo, g.glo, 2 * static_cast<uint64_t>(m.ff), n_pad, 64, kvprm::gemm_x_box(n_pad), "grad lo (gu)")))
     return rc;
-  if ((rc = make_map(ctx, &g.tm_qkv_hi, g.ghi, m.qkv_rows, n_pad, 64, n_pad, "grad hi (qkv)"))) return rc;
-  if ((rc = make_map(ctx, &g.tm_qkv_lo, g.glo, m.qkv_rows, n_pad, 64, n_pad, "grad lo (qkv)"))) return rc;
+  if ((rc = make_map(ctx, &g.tm_qkv_hi, g.ghi, m.qkv_rows, n_pad, 64, kvprm::gemm_x_box(n_pad), "grad hi (qkv)"))) return rc;
+  if ((rc = make_map(ctx, &g.tm_qkv_lo, g.glo, m.qkv_rows, n_pad, 64, kvprm::gemm_x_box(n_pad), "grad lo (qkv)"))) return rc;
   g.tm_npad = n_pad;
   return KVPRM_OK;
 }
@@ -1779,7 +1779,7 @@ int kvprm_projection(kvprm_ctx* ctx, const void* W, int32_t M, int32_t K, const 
   CUtensorMap tw, tx;
   int rc;
   if ((rc = make_map(ctx, &tw, W, K, M, 64, 128, "W"))) return rc;
-  if ((rc = make_map(ctx, &tx, X, K, n, 64, n_pad, "X"))) return rc;
+  if ((rc = make_map(ctx, &tx, X, K, n, 64, kvprm::gemm_x_box(n_pad), "X"))) return rc;
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   kvprm::GemmEpilogue ep;
   ep.mode = kvprm::GemmEpilogue::PLAIN;

@@ -1,0 +1,44 @@
+"""Projections on CTA pairs (two CTAs, an M = 256 MMA, half of the activation tile read from each): plain pairs
+and pairs that hold half of the columns, with and without a cluster reduction, every epilogue, an adapter's extra
+K tiles and K tiles that do not divide among the ranks, at padded columns around the choice of the form and up to
+the largest.  Against the oracle with the scoring tolerances.  And, on the host, that a plan's clusters are placed
+in one wave."""
+import dataclasses
+
+import pytest
+
+import kvsynth as ks
+import paper_2607_09153_gb300 as kp
+from tests.gpu_util import compare, require_gpu, run_gpu
+
+# QKV and O: pairs at 80 to 128 padded columns, halves beyond; down (11 K tiles over 4 ranks): pairs
+SMALL = ks.Arch(2, 256, 4, 2, 64, 704)
+# QKV (36 m-tiles, 18 clusters of 8 do not fit): halves from 96, two ranks
+WIDE = ks.Arch(1, 512, 28, 4, 128, 1024)
+PLACED = {1: 152, 2: 76, 4: 36, 8: 15, 16: 7}   # clusters of CTAs that fill an SM, on 152 SMs
+
+
+@pytest.mark.parametrize("arch", [ks.ARCH_1P5B, ks.ARCH_7B, ks.ARCH_8B, SMALL, WIDE])
+@pytest.mark.parametrize("rank", [0, 256])
+def test_clusters_are_placed(arch, rank):
+    for n_pad in range(16, 257, 16):
+        for M, K in [(arch.qkv_rows, arch.d_model), (arch.d_model, arch.n_q_heads * arch.head_dim), (arch.d_model, arch.d_ff)]:
+            p = kp.kvprm_plan_projection(M, K + rank, n_pad, 152, True, False)
+            clusters = (p["m_tiles"] + p["tiles_per_cta"] - 1) // p["tiles_per_cta"]
+            if p["smem_bytes"] + 1024 > 228 * 1024 // 2 and p["cluster"] > 1:
+                assert clusters <= PLACED[p["cluster"]], (M, K, n_pad)
+
+
+@pytest.mark.gpu
+@pytest.mark.parametrize("arch, n, rank", [(SMALL, 48, 0), (SMALL, 64, 64), (SMALL, 65, 0), (SMALL, 128, 64),
+                                           (SMALL, 129, 0), (SMALL, 145, 256),
+                                           (SMALL, 208, 64), (SMALL, 256, 0), (WIDE, 88, 0), (WIDE, 129, 64), (WIDE, 176, 0),
+                                           (WIDE, 250, 0)])
+def test_layers(arch, n, rank):
+    require_gpu()
+    w = ks.distinct("pairs", dataclasses.replace(arch, lora_rank=rank), 700 + n, [(5 * b) % 40 for b in range(n)],
+                    gain_std=0.2)
+    t = ks.Tables.make(0.2)
+    r, attn, _, sc = run_gpu(w, t)
+    compare(w, t, gpu_rewards=r, gpu_attn=attn, label=f"d {arch.d_model} n {n} rank {rank}")
+    sc.close()
