@@ -86,13 +86,15 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
                                                            const __grid_constant__ CUtensorMap tmT,
                                                            const __grid_constant__ CUtensorMap tmTlo, int k_main,
                                                            int k_tiles, int cs, int stages, uint32_t tmem_cols,
-                                                           int n_pad, int mt_arg, GemmEpilogue ep, int* err,
+                                                           int n_pad, int n_split, GemmEpilogue ep, int* err,
                                                            unsigned long long* ts) {
   trace_begin(ts);
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = align1024(smem_raw);
-  // m-tiles of this CTA (LARGE only): a stage holds mt weight tiles, then the activation tile(s)
-  const int mt = LARGE && !PAIR ? mt_arg : 1;
+  constexpr bool silu = MODE == GemmEpilogue::SILU;
+  // weight tiles of this CTA, which a stage holds ahead of the activation tile(s): a gate/up pair's CTA
+  // has 128 gate rows and the matching 128 up rows, so that either is the other's TMEM lane for lane
+  constexpr int mt = PAIR && silu ? 2 : 1;
   const uint32_t x_bytes = static_cast<uint32_t>(n_pad) * kBK * 2;
   const uint32_t w_bytes = kWTileBytes * static_cast<uint32_t>(mt);
   // PAIR: half of the pair's activation rows, i.e. one part's n_pad rows or half of each part's
@@ -112,9 +114,9 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   const uint32_t crank = cluster_rank();
   const uint32_t rank = PAIR ? crank >> 1 : crank, side = PAIR ? crank & 1u : 0u;
   // of the two m-tiles' n_pad columns, or (n_split 2, n_pad then the half) of one half of the batch's
-  const int n_split = PAIR ? mt_arg : 1, pair_unit = static_cast<int>(blockIdx.x) / (2 * cs);
-  const int m_tile0 = PAIR ? pair_unit / n_split * 2 + static_cast<int>(side)
-                           : static_cast<int>(blockIdx.x) / cs * mt;   // first m-tile of this CTA
+  const int pair_unit = static_cast<int>(blockIdx.x) / (2 * cs);
+  const int m_tile = PAIR ? pair_unit / n_split * 2 + static_cast<int>(side)
+                           : static_cast<int>(blockIdx.x) / cs;   // (gate/up pairs: of 128 gate rows)
   const int c_off = PAIR ? pair_unit % n_split * n_pad : 0;   // first column
   // the cluster rank of split r's CTA for this m-tile
   auto peer = [&](int r) { return PAIR ? 2u * static_cast<uint32_t>(r) + side : static_cast<uint32_t>(r); };
@@ -122,13 +124,12 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   const int kt0 = static_cast<int>(rank) * kps;
   const int kt1 = min(k_tiles, kt0 + kps);
   const int nk = kt1 > kt0 ? kt1 - kt0 : 0;
-  constexpr bool silu = MODE == GemmEpilogue::SILU;
   // this rank's candidate columns in the reduction and the epilogue
   const int cols = n_pad / cs;
   const int cbeg = c_off + static_cast<int>(rank) * cols;
   const int cend = min(cbeg + cols, ep.n_valid);
   const int nc = cend > cbeg ? cend - cbeg : 0;
-  const bool hpreload = MODE == GemmEpilogue::RESID && nc <= kHPreCols && mt == 1;
+  const bool hpreload = MODE == GemmEpilogue::RESID && nc <= kHPreCols;
   constexpr int kEpiBatch = LARGE ? 8 : 1;
 
   if (threadIdx.x == 0) {
@@ -186,16 +187,14 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
         mbar_arrive_expect_tx(&full[stage], 2 * stage_bytes);
       const CUtensorMap* wm = kt < k_main ? &tmW : &tmB;
       const int kx = (kt < k_main ? kt : kt - k_main) * kBK;
+      uint8_t* wt = smem + stage * stage_bytes;
+      if constexpr (!silu) {
+        load(wt, wm, stage, kx, m_tile * kBM, pol_w);
+      } else {   // mt x 64 gate rows, then the matching up rows, in boxes of 64
 #pragma unroll 1
-      for (int t = 0; t < mt; ++t) {
-        const int m_tile = m_tile0 + t;
-        uint8_t* wt = smem + stage * stage_bytes + t * kWTileBytes;
-        if (!silu) {
-          load(wt, wm, stage, kx, m_tile * kBM, pol_w);
-        } else {   // 64 gate rows, then the matching 64 up rows
-          load(wt, wm, stage, kx, m_tile * 64, pol_w);
-          load(wt + kWTileBytes / 2, wm, stage, kx, ep.ff + m_tile * 64, pol_w);
-        }
+        for (int t = 0; t < 2 * mt; ++t)
+          load(wt + t * (kWTileBytes / 2), wm, stage, kx,
+               (t < mt ? 0 : ep.ff) + (m_tile * mt + (t < mt ? t : t - mt)) * 64, pol_w);
       }
     };
     // the activation maps' boxes hold the batch's columns, from 96 on half of them (gemm_x_box): a stage's
@@ -260,7 +259,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     // the next kernel's weight stream may be competing for the memory system
     if (hpreload) {   // warps 2 and 3 take alternate columns, 16 bytes a lane, all in flight at once
       float4 v[kHPreCols / 2];
-      const int gm = m_tile0 * kBM + 4 * lane;
+      const int gm = m_tile * kBM + 4 * lane;
 #pragma unroll
       for (int k = 0; k < kHPreCols / 2; ++k) {
         const int cl = 2 * k + (warp & 1);
@@ -281,19 +280,18 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     // slice from shared memory once: columns [0, n_pad) accumulate W hi,
     // [n_pad, 2 n_pad) accumulate W lo, summed when the accumulator is read.
     // Beyond N = 256 the two halves take one MMA each into the same columns.
-    // With two m-tiles per CTA, tile t accumulates from TMEM column t tile_cols (half the
-    // allocation, a power of two).
+    // A gate/up pair's up tile accumulates in the second half of the allocation.
     const bool merged = has_lo && 2 * n_pad <= 256;
     const bool two = has_lo && !merged;
     // A pair's MMA (M = 256, both CTAs' weight tiles) takes half of its B rows from either CTA: one part
     // each when merged, else half of the hi and half of the lo rows.
     const uint32_t idesc = idesc_bf16_f32(PAIR ? 2 * kBM : kBM, merged ? 2 * n_pad : n_pad);
     const uint16_t pair_mask = static_cast<uint16_t>(3u << crank);
-    // PAIR: two accumulators, one of the hi and one of the lo part, or when merged one of the first and
+    // PAIR without gate/up: two accumulators, one of the hi and one of the lo part, or when merged one of the first and
     // one of the second half of the K tiles: half as many fp32 roundings in a row (without them rewards
     // were 10-20 % further off, a pair's CTA having twice the K tiles of the CTA it replaces).
-    const uint32_t tile_cols = tmem_cols / static_cast<uint32_t>(PAIR ? 2 : mt);
-    const int i_half = PAIR && merged ? (nk + 1) / 2 : nk;   // the second accumulator's first K tile
+    const uint32_t tile_cols = tmem_cols / (PAIR ? 2u : 1u);
+    const int i_half = PAIR && !silu && merged ? (nk + 1) / 2 : nk;   // the second accumulator's first K tile
     int s = 0;
     uint32_t parity = 0u;
 #pragma unroll 1
@@ -307,13 +305,18 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
       const uint32_t acc0 = i > 0 && i != i_half ? 1u : 0u;
 #pragma unroll 1
       for (int t = 0; t < mt; ++t) {
-        const uint32_t d = tmem + (PAIR ? (i >= i_half ? tile_cols : 0u) : static_cast<uint32_t>(t) * tile_cols);
+        const uint32_t d = tmem + (t > 0 || i >= i_half ? tile_cols : 0u);
         const uint64_t at = a0 + static_cast<uint64_t>(t) * (kWTileBytes >> 4);
 #pragma unroll
         for (int kk = 0; kk < kBK / 16; ++kk) {
           if constexpr (PAIR) {
             umma_bf16_pair_w(d, at + 2 * kk, b0 + 2 * kk, idesc, kk > 0 ? 1u : acc0);
-            if (two) umma_bf16_pair_w(d + tile_cols, at + 2 * kk, l0 + 2 * kk, idesc, kk > 0 ? 1u : acc0);
+            if (two) {
+              if constexpr (silu)
+                umma_bf16_pair_w(d, at + 2 * kk, l0 + 2 * kk, idesc, 1u);
+              else
+                umma_bf16_pair_w(d + tile_cols, at + 2 * kk, l0 + 2 * kk, idesc, kk > 0 ? 1u : acc0);
+            }
           } else {
             umma_bf16_w(d, at + 2 * kk, b0 + 2 * kk, idesc, kk > 0 ? 1u : acc0);
             if (LARGE && two) umma_bf16_w(d, at + 2 * kk, l0 + 2 * kk, idesc, 1u);   // n_pad > 128
@@ -347,13 +350,99 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   const int nw = static_cast<int>(blockDim.x >> 5), nwh = nw >> 2, wh = warp >> 2;
   const int m = (warp & 3) * 32 + lane;
   const bool merged = has_lo && 2 * n_pad <= 256;
-  const uint32_t tile_cols = tmem_cols / static_cast<uint32_t>(PAIR ? 2 : mt);
-  // one m-tile at a time (two without split K only): park it, reduce it over the cluster, write its epilogue
+  const uint32_t tile_cols = tmem_cols / (PAIR ? 2u : 1u);
+  const uint32_t trow = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16);
+  if constexpr (PAIR && silu) {
+    // Gate and up of a row sit in the same TMEM lane, so their product needs no parked accumulator: 16
+    // columns at a time to shared memory as (hi, lo) words, and from there 16 bytes of rows a thread to
+    // global memory.  Bound by those stores: 8 us after the last MMA at 256 columns, 7 without any of the
+    // arithmetic; storing from the lanes (4 bytes of two rows) took 9.3.
+    const bool few = n_pad < 64;   // the exact functions at batches where their time does not show
+    grid_dep_wait();    // outputs may still be read by kernels that precede this one
+    __syncthreads();    // the columns' RMSNorm factors
+    if (threadIdx.x == 0) trace_event(ts, 5);
+    const int j = m_tile * kBM + m;
+    // stores: 16 row groups of 8 x 8 columns a step; the halves are read in the order free of bank conflicts
+    const int rg = static_cast<int>(threadIdx.x) & 15, tq = (static_cast<int>(threadIdx.x) & 127) >> 4;
+    const int row = m_tile * kBM + 8 * rg, flip = (rg >> 2) & 1;   // ff % 8 == 0
+    const uint32_t np = static_cast<uint32_t>(n_pad);
 #pragma unroll 1
-  for (int tt = 0; tt < mt; ++tt) {
-    const int m_tile = m_tile0 + tt;
-    const uint32_t tcol = static_cast<uint32_t>(tt) * tile_cols;
-    const uint32_t trow = tmem + (static_cast<uint32_t>((warp & 3) * 32) << 16) + tcol;
+    for (int c0 = 16 * wh; c0 < cend; c0 += 16 * nwh) {
+      float g[16], u[16];
+      const uint32_t t = trow + static_cast<uint32_t>(c0);
+      tmem_ld16_nowait(t, g);
+      tmem_ld16_nowait(t + tile_cols, u);
+      if (merged) {
+        float gl[16], ul[16];
+        tmem_ld16_nowait(t + np, gl);
+        tmem_ld16_nowait(t + tile_cols + np, ul);
+        tmem_wait_ld();
+        tmem_hold(g);
+        tmem_hold(u);
+        tmem_hold(gl);
+        tmem_hold(ul);
+#pragma unroll
+        for (int k = 0; k < 16; ++k) {
+          g[k] += gl[k];
+          u[k] += ul[k];
+        }
+      } else {
+        tmem_wait_ld();
+        tmem_hold(g);
+        tmem_hold(u);
+      }
+      if (ep.rs_sumsq) {
+#pragma unroll
+        for (int k = 0; k < 16; k += 4) {   // columns past the batch: whatever the slot holds, and not stored
+          const float4 rs = *reinterpret_cast<const float4*>(rsc + c0 + k);
+          g[k] *= rs.x, g[k + 1] *= rs.y, g[k + 2] *= rs.z, g[k + 3] *= rs.w;
+          u[k] *= rs.x, u[k + 1] *= rs.y, u[k + 2] *= rs.z, u[k + 3] *= rs.w;
+        }
+      }
+      if (ep.gu_save && j < ep.ff) {   // pre-activations for a backward pass
+        float* gs = ep.gu_save + static_cast<int64_t>(c0) * 2 * ep.ff + j;
+#pragma unroll
+        for (int k = 0; k < 16; ++k)
+          if (c0 + k < cend) {
+            gs[static_cast<int64_t>(2 * k) * ep.ff] = g[k];
+            gs[static_cast<int64_t>(2 * k + 1) * ep.ff] = u[k];
+          }
+      }
+      uint32_t* xc = reinterpret_cast<uint32_t*>(smem) + c0 * kBM;   // (hi, lo) of 16 columns, in the idle ring
+#pragma unroll
+      for (int k = 0; k < 16; k += 2) {
+        float a[2];
+#pragma unroll
+        for (int e = 0; e < 2; ++e)
+          a[e] = (few ? g[k + e] / (1.0f + expf(-g[k + e]))
+                      : g[k + e] * rcp_ftz(1.0f + ex2_ftz(-1.4426950408889634f * g[k + e]))) * u[k + e];
+        const __nv_bfloat162 h2 = __floats2bfloat162_rn(a[0], a[1]);
+        const float2 hf = __bfloat1622float2(h2);
+        const __nv_bfloat162 l2 = __floats2bfloat162_rn(a[0] - hf.x, a[1] - hf.y);
+        const uint32_t h = *reinterpret_cast<const uint32_t*>(&h2), l = *reinterpret_cast<const uint32_t*>(&l2);
+        xc[k * kBM + m] = __byte_perm(h, l, 0x5410);
+        xc[(k + 1) * kBM + m] = __byte_perm(h, l, 0x7632);
+      }
+      named_bar_sync(1 + wh, 128);   // the four warps of these columns
+#pragma unroll
+      for (int k = 0; k < 2; ++k) {
+        const int cl = tq + 8 * k;
+        const uint4* xp = reinterpret_cast<const uint4*>(xc + cl * kBM + 8 * rg);
+        const uint4 w0 = xp[flip], w1 = xp[1 - flip], v0 = flip ? w1 : w0, v1 = flip ? w0 : w1;
+        if (c0 + cl < cend && row < ep.ff) {
+          const int64_t o = static_cast<int64_t>(c0 + cl) * ep.ff + row;
+          *reinterpret_cast<uint4*>(ep.a_hi + o) = make_uint4(__byte_perm(v0.x, v0.y, 0x5410), __byte_perm(v0.z, v0.w, 0x5410),
+                                                              __byte_perm(v1.x, v1.y, 0x5410), __byte_perm(v1.z, v1.w, 0x5410));
+          *reinterpret_cast<uint4*>(ep.a_lo + o) = make_uint4(__byte_perm(v0.x, v0.y, 0x7632), __byte_perm(v0.z, v0.w, 0x7632),
+                                                              __byte_perm(v1.x, v1.y, 0x7632), __byte_perm(v1.z, v1.w, 0x7632));
+        }
+      }
+    }
+    tc_fence_before();
+    __syncwarp();
+    cluster_arrive();
+  } else {
+    // park the tile, reduce it over the cluster, write its epilogue
     if constexpr (PAIR) {
       // the two accumulators, a group's loads in flight while the one before it is stored
       const uint32_t np = static_cast<uint32_t>(n_pad);
@@ -409,7 +498,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
       }
     }
     tc_fence_before();
-    if (tt == 0) {
+    {
       cluster_sync();   // every rank's partial is parked
       if (threadIdx.x == 0) trace_event(ts, 3);
       if (ep.late_trigger) grid_dep_launch();
@@ -843,7 +932,6 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
         }
       }
     }
-    if (tt + 1 < mt) __syncthreads();   // every thread is done with acc before the next tile is parked
   }
   (void)nc;
   if (threadIdx.x == 0) trace_event(ts, 6);   // this thread's epilogue written
@@ -931,23 +1019,21 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
   const int need = (has_lo && 2 * n_pad <= 256) ? 2 * n_pad : n_pad;   // merged hi/lo accumulator halves
   while (cols < static_cast<uint32_t>(need)) cols <<= 1;
   p.tmem_cols = cols;
-  // gate/up at large batches without split K: when one-tile CTAs would need two waves, a CTA takes
-  // two m-tiles, so that every stage's activation tile (four times the weight tile at B = 256 with
-  // the lo half) serves both, and the grid fits on the SMs at once
-  if (gate_up && n_pad > 64 && cs == 1 && p.m_tiles % 2 == 0 && p.m_tiles > per_sm * num_sms) {
-    const uint32_t st2 = 2 * kWTileBytes + static_cast<uint32_t>(n_pad) * kBK * 2 * (has_lo ? 2u : 1u);
+  // gate/up without split K, more tiles than SMs: pairs of CTAs with two tiles each.  The 7B gate/up, 296
+  // tiles: one-tile CTAs two to an SM took 51.6 us at 96 columns and 56.5 at 144, two tiles a CTA without
+  // pairs 47.5 at 80, 66.5 at 160 and 80.0 at 256; pairs take 44.1, 50.1, 44.7, 52.9 and 75.4 (the weights'
+  // bytes alone 40.7, the MMAs 71 at 256).  At 64 columns 45.0 -> 43.7, at 48 45.6 -> 43.1.
+  if (gate_up && has_lo && n_pad >= 48 && cs == 1 && p.m_tiles % 2 == 0 && p.m_tiles > num_sms &&
+      (p.m_tiles / 2 + 1) / 2 <= fit(2)) {
+    const uint32_t st2 = 2 * kWTileBytes + static_cast<uint32_t>(n_pad) * kBK * 2;
     int stages2 = static_cast<int>((192u * 1024u) / st2);
     if (stages2 > 8) stages2 = 8;
-    if (stages2 > p.kt_per_split) stages2 = p.kt_per_split;
-    size_t ring2 = static_cast<size_t>(stages2) * st2;
-    if (ring2 < acc) ring2 = acc;
-    const size_t smem2 = ring2 + 1024 + kTailBytes;
-    if (stages2 >= 2 && 2 * cols <= 512 && smem2 <= kGemmMaxSmem && (p.m_tiles / 2) <= num_sms) {
-      p.mt = 2;
-      p.stages = stages2;
-      p.smem_bytes = smem2;
-      p.tmem_cols = 2 * cols;
-    }
+    if (stages2 > p.k_tiles) stages2 = p.k_tiles < 2 ? 2 : p.k_tiles;
+    p.pair = true;
+    p.mt = 2;
+    p.stages = stages2;
+    p.smem_bytes = static_cast<size_t>(stages2) * st2 + 1024 + kTailBytes;
+    p.tmem_cols = 2 * cols;
   }
   const int pc = cluster_of(1);
   auto take_pairs = [&](int ranks, int n_split) {
@@ -995,10 +1081,7 @@ enum GemmImage { kSmall, kLarge, kPair, kGemmImages };
 
 template <int MODE>
 GemmKernel image_of(GemmImage i) {
-  if (i == kPair) {   // gate/up tiles are not paired
-    if constexpr (MODE == GemmEpilogue::SILU) return nullptr;
-    else return gemm_cluster_kernel<true, MODE, true>;
-  }
+  if (i == kPair) return gemm_cluster_kernel<true, MODE, true>;
   return i == kLarge ? gemm_cluster_kernel<true, MODE, false> : gemm_cluster_kernel<false, MODE, false>;
 }
 // The kernel image of a batch class and epilogue (null: none).
@@ -1031,7 +1114,9 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
                         const GemmEpilogue& ep, int n_pad, int* err, cudaStream_t stream, bool pdl,
                         unsigned long long* ts, const GemmLowRank* lr) {
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3((p.m_tiles + p.mt - 1) / p.mt * p.cluster, 1, 1);   // a pair's CTAs: m_tiles / 2 clusters too
+  const int units = (p.m_tiles + p.mt - 1) / p.mt;   // launched by the cluster, gate/up pairs' by two
+  const int cluster = p.pair && p.gate_up ? 2 : p.cluster;
+  cfg.gridDim = dim3(p.pair && p.gate_up ? (units + 1) / 2 * 2 : units * p.cluster, 1, 1);
   // the vector epilogues win from 48 padded columns on even with four warps (40 candidates of a 7B scorer
   // 564 -> 532 us for four layers; 24 candidates, 32 columns: 397 us small, 405 large)
   const bool large = n_pad >= 48;
@@ -1041,7 +1126,7 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = p.cluster;
+  attr[0].val.clusterDim.x = cluster;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
   attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -1057,12 +1142,11 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
   const CUtensorMap& mtl = with_lr ? (p.has_lo ? *lr->t_lo : *lr->t_hi) : xlo;
   const int k_main = with_lr ? lr->k_main : p.k_tiles;
   const int n_split = p.pair && p.mt == 1 ? 2 : 1;
-  // two m-tiles per CTA exist in the large-batch images only
   const GemmKernel kern = gemm_image(p.pair ? kPair : (large ? kLarge : kSmall), ep.mode);
-  if (!kern || (!large && p.mt != 1) || (p.pair && !p.has_lo)) return cudaErrorInvalidValue;
+  if (!kern || (p.pair && (!large || !p.has_lo || p.gate_up != (ep.mode == GemmEpilogue::SILU))))
+    return cudaErrorInvalidValue;
   return cudaLaunchKernelEx(&cfg, kern, *tmW, *tmX, xlo, p.has_lo ? 1 : 0, mb, mt, mtl, k_main, p.k_tiles,
-                            p.pair ? p.cluster / 2 : p.cluster, p.stages, p.tmem_cols,
-                            n_pad / n_split, p.pair ? n_split : p.mt, ep, err, ts);
+                            p.pair ? cluster / 2 : cluster, p.stages, p.tmem_cols, n_pad / n_split, n_split, ep, err, ts);
 }
 
 }  // namespace kvprm

@@ -22,11 +22,11 @@ struct GemmPlan {
   bool has_lo = true;    // activation given as a bf16 (hi, lo) pair
   bool gate_up = false;  // tiles of 64 gate rows + the matching 64 up rows
   int m_tiles = 0, k_tiles = 0, kt_per_split = 0, splits = 0, stages = 0, cluster = 1;
-  // m-tiles per CTA: 2 for a gate/up projection without split K whose one-tile CTAs would need two
-  // waves (large batches); the CTA's stage then holds both weight tiles and one activation tile
+  // m-tiles that one activation tile serves, over `cluster` CTAs: 2 with `pair`, else 1
   int mt = 1;
-  // CTA pairs: mt m-tiles over `cluster` CTAs as with mt = 2, a tile per CTA of a pair (cluster / 2 K
-  // splits), the pair's MMAs reading half of the activation tile from either CTA
+  // CTA pairs.  gate/up: two neighbouring CTAs with 128 gate and the matching 128 up rows each (a launch
+  // cluster of two, cluster = 1 K split).  Otherwise a tile each over cluster / 2 K splits; or, with
+  // mt = 1, of half of the columns.
   bool pair = false;
   // threads per CTA: 256 from 64 padded columns, else 128
   int threads = 128;

@@ -328,6 +328,12 @@ __device__ __forceinline__ float ex2_ftz(float x) {
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
 }
+// 1 / x by the hardware approximation (rcp.approx, relative error 2^-23), subnormals flushed to zero.
+__device__ __forceinline__ float rcp_ftz(float x) {
+  float y;
+  asm("rcp.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
 // tmem_ld16 without the wait: several loads in flight, then one tmem_wait_ld
 // before any of the values is used.
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, float (&v)[16]) {

@@ -10,11 +10,15 @@ import pytest
 import kvsynth as ks
 import paper_2607_09153_gb300 as kp
 from tests.gpu_util import compare, require_gpu, run_gpu
+from tests.test_gpu_steering import _compare, _gpu_grad, _oracle
 
 # QKV and O: pairs at 80 to 128 padded columns, halves beyond; down (11 K tiles over 4 ranks): pairs
 SMALL = ks.Arch(2, 256, 4, 2, 64, 704)
 # QKV (36 m-tiles, 18 clusters of 8 do not fit): halves from 96, two ranks
 WIDE = ks.Arch(1, 512, 28, 4, 128, 1024)
+# gate/up has more tiles than the chip has SMs: pairs, of an even and of an odd number of 128-row units
+GATE_UP = ks.Arch(1, 128, 2, 2, 64, 9984)
+GATE_UP_ODD = ks.Arch(1, 128, 2, 2, 64, 9856)
 PLACED = {1: 152, 2: 76, 4: 36, 8: 15, 16: 7}   # clusters of CTAs that fill an SM, on 152 SMs
 
 
@@ -33,7 +37,9 @@ def test_clusters_are_placed(arch, rank):
 @pytest.mark.parametrize("arch, n, rank", [(SMALL, 48, 0), (SMALL, 64, 64), (SMALL, 65, 0), (SMALL, 128, 64),
                                            (SMALL, 129, 0), (SMALL, 145, 256),
                                            (SMALL, 208, 64), (SMALL, 256, 0), (WIDE, 88, 0), (WIDE, 129, 64), (WIDE, 176, 0),
-                                           (WIDE, 250, 0)])
+                                           (WIDE, 250, 0), (GATE_UP, 48, 0), (GATE_UP, 128, 64), (GATE_UP, 161, 0),
+                                           (GATE_UP_ODD, 49, 0), (GATE_UP_ODD, 80, 64),
+                                           (GATE_UP_ODD, 256, 0)])
 def test_layers(arch, n, rank):
     require_gpu()
     w = ks.distinct("pairs", dataclasses.replace(arch, lora_rank=rank), 700 + n, [(5 * b) % 40 for b in range(n)],
@@ -41,4 +47,16 @@ def test_layers(arch, n, rank):
     t = ks.Tables.make(0.2)
     r, attn, _, sc = run_gpu(w, t)
     compare(w, t, gpu_rewards=r, gpu_attn=attn, label=f"d {arch.d_model} n {n} rank {rank}")
+    sc.close()
+
+
+@pytest.mark.gpu
+def test_gradient():
+    """The backward's products and the gate and up values that the forward keeps for it."""
+    require_gpu()
+    w = ks.distinct("pairs_grad", GATE_UP, 790, [(7 * b) % 20 for b in range(166)], gain_std=0.2)
+    t = ks.Tables.make(0.2)
+    p, grad, dev, sc = _gpu_grad(w, t)
+    p_ref, ref, _, _ = _oracle(w, t)
+    _compare("166 candidates", w, p, grad, p_ref, ref)
     sc.close()
