@@ -167,7 +167,8 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   // Let the next kernel in the stream start its own independent prologue and
   // streaming now (or, with late_trigger, once the partials are parked); it
   // waits for this grid's completion before touching what this grid writes.
-  if (!ep.late_trigger) grid_dep_launch();
+  // LOWRANK lets it start once the activations it reads are there (below).
+  if (MODE != GemmEpilogue::LOWRANK && !ep.late_trigger) grid_dep_launch();
 
   if (warp == 0 && lane == 0 && nk > 0) {
     // ---------------- TMA producer
@@ -226,17 +227,30 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     const int pre = min(stages, nk);
 #pragma unroll 1
     for (int i = 0; i < pre; ++i) load_w(i, kt0 + i);
-    grid_dep_wait();
+    // With an adapter the preceding kernel is its A x, which starts this one after its own wait for the
+    // kernel that wrote x: only the last K tiles, t's, wait for it.  The weights' products then run beside
+    // A x (1.5B, 16 candidates: rank 256 1,582 -> 1,550 us a call, rank 64 414 -> 391 for eight layers; 48
+    // candidates at rank 256 577 -> 542; ranks 512 and 1,024 -3 to +1 %).  Starting it from A x's last
+    // landed tile instead: 1,607.
+    bool waited = k_main == k_tiles;
+    if (waited) grid_dep_wait();
     trace_event(ts, 0);   // the preceding kernel has completed
+    auto load_act = [&](int stage, int kt) {
+      if (!waited && kt >= k_main) {
+        grid_dep_wait();
+        waited = true;
+      }
+      load_x(stage, kt);
+    };
 #pragma unroll 1
-    for (int i = 0; i < pre; ++i) load_x(i, kt0 + i);
+    for (int i = 0; i < pre; ++i) load_act(i, kt0 + i);
     int s = 0;   // stage of K tile i, and the parity of the release before its use
     uint32_t parity = 0u;
 #pragma unroll 1
     for (int i = pre; i < nk; ++i) {
       if (!mbar_wait(&empty[s], parity, err)) break;
       load_w(s, kt0 + i);
-      load_x(s, kt0 + i);
+      load_act(s, kt0 + i);
       if (++s == stages) {
         s = 0;
         parity ^= 1u;
@@ -247,6 +261,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     // (QKV, SILU), from the residual stream's tile sums of squares the preceding kernel wrote; the
     // parking barrier below orders these writes before the epilogue reads them
     grid_dep_wait();
+    if (MODE == GemmEpilogue::LOWRANK) grid_dep_launch();
     if ((MODE == GemmEpilogue::QKV || MODE == GemmEpilogue::SILU) && ep.rs_sumsq)
 #pragma unroll 1
       for (int t0 = threadIdx.x - 64; t0 < nc; t0 += blockDim.x - 64) {   // nc <= 256 columns

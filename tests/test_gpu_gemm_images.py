@@ -1,6 +1,7 @@
 """The projections where the choice of kernel image and ring depth changes: 32, 33, 48, 49 and 64, 65, 80, 81
 candidates (the padded columns step by 16), a gate/up that only fits one wave with a stage less, a down
-projection whose K loop gets twice the CTAs, and the adapter's A x on either image.  One kernel alone
+projection whose K loop gets twice the CTAs, the adapter's A x on either image, and an adapter with more K
+tiles than the weights.  One kernel alone
 against an fp64 product (fp32 accumulation over K = 18,944: below 1e-5 of the largest output), and whole
 layers against the oracle with the scoring tolerances."""
 import dataclasses
@@ -38,7 +39,7 @@ def test_projection(ctx, M, K, n):
     assert np.abs(Y.cpu().numpy().astype(np.float64) - ref).max() / np.abs(ref).max() < 1e-5
 
 
-@pytest.mark.parametrize("n, rank", [(32, 64), (33, 0), (48, 128), (49, 0), (65, 64), (80, 0), (81, 64)])
+@pytest.mark.parametrize("n, rank", [(5, 512), (32, 64), (33, 0), (48, 128), (49, 0), (65, 64), (80, 0), (81, 64)])
 def test_layers(n, rank):
     require_gpu()
     arch = dataclasses.replace(ks.Arch(2, 320, 5, 5, 64, 9792), lora_rank=rank)
