@@ -12,7 +12,9 @@
 // sit back to back in shared memory and one MMA of N = 2 n_pad covers both
 // (each weight K slice is read from shared memory once -- the MMA issue rate
 // is bounded by those reads at this small N); the two accumulator halves are
-// added when TMEM is read.  Beyond N = 256 each half takes its own MMA.
+// added when TMEM is read.  Beyond N = 256 each half takes its own MMA.  From
+// 48 columns on two CTAs may share an M = 256 MMA (cta_group::2), each staging
+// half of its activation rows.
 //
 // K is split across the CTAs of a thread-block cluster (one cluster per
 // 128-row tile) so that every SM streams weights.  The splits are reduced
@@ -27,7 +29,10 @@
 //          candidate, and h ⊙ g (g = the next RMSNorm's gain) as the next
 //          projection's bf16 hi/lo input
 //   SILU   rows are 64 gate rows and the matching 64 up rows (two TMA boxes
-//          per stage); a = SiLU(gate) * up as a bf16 hi/lo pair
+//          per stage; CTA pairs: 128 and 128 as two tiles); a = SiLU(gate) * up
+//          as a bf16 hi/lo pair
+//   LOWRANK  t = s (A x) of a scorer adapter as a bf16 hi/lo pair, the next
+//          projection's last K tiles
 // An RMSNorm x = g ⊙ h / sqrt(mean(h^2) + eps) between two projections is
 // thereby split: the per-candidate factor r = 1/sqrt(mean(h^2) + eps) is a
 // scalar of the column, so W x = r (W (h ⊙ g)); the residual epilogue writes
@@ -48,6 +53,7 @@ constexpr uint32_t kWTileBytes = kBM * kBK * 2;   // 16 KB
 // after the ring: barriers, TMEM slot and 64 block-sum floats (512 B), then 256
 // per-column RMSNorm factors (1 KB)
 constexpr size_t kTailBytes = 512 + 1024 + 4096;   // barriers, RMSNorm factors, preloaded residual
+constexpr int kLargeCols = 48;                      // padded columns from which the large-batch images run
 constexpr int kHalfBoxCols = 96;                    // padded columns from which activation boxes hold half
 constexpr int kHPreCols = 8;                        // residual columns preloaded per rank (128 rows each)
 constexpr size_t kGemmMaxSmem = 200 * 1024;         // dynamic shared memory the kernel is configured for
@@ -64,15 +70,15 @@ __device__ __forceinline__ void store_hilo(__nv_bfloat16* hi, __nv_bfloat16* lo,
 
 // LARGE (n_pad >= 48, one kernel image per batch class so that the small-batch code keeps its own
 // register allocation): the residual epilogue issues a 16-column group's residual loads before
-// using any and sums each column's squares in one pass over the parked tile, clusters of 4 reduce
-// with 16-byte DSMEM loads, and the epilogues move 4 or 8 consecutive rows of a column per thread
+// using any and sums each column's squares in one pass over the parked tile, clusters reduce with
+// 16-byte DSMEM loads, and the epilogues move 4 or 8 consecutive rows of a column per thread
 // with 16-byte accesses (the 4-warp CTA is otherwise bound by 2- and 4-byte stores and by one load
 // latency per column).
 // MODE: the epilogue, an image each.  A CTA runs everything after its MMAs once, so those instructions
 // are fetched cold in every launch, and their number is a good part of the ~3 us from the last MMA to
 // the end of a small launch.  Hence the images, rolled outer loops, counters instead of divisions by the
-// stage count and shifts by the head dimension: 51 KB of code in one small image became 20-32 KB in four
-// (large: 178 KB became 31-52), and a call of the 1.5B workload took 1,112 us instead of 1,155, with the
+// stage count and shifts by the head dimension: 51 KB of code in one small image became 20-33 KB each
+// (large: 178 KB became 25-53), and a call of the 1.5B workload took 1,112 us instead of 1,155, with the
 // rank-256 adapter 1,687 instead of 1,932, MCTS 9,814 instead of 10,110.
 // PAIR (large batches; `plan_gemm` has the rule): a CTA pair's MMA multiplies both CTAs' weight tiles (M = 256)
 // with a B operand that is half in either CTA, so a CTA stages half of the activation rows.  At 256
@@ -1032,7 +1038,7 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
   // tiles: one-tile CTAs two to an SM took 51.6 us at 96 columns and 56.5 at 144, two tiles a CTA without
   // pairs 47.5 at 80, 66.5 at 160 and 80.0 at 256; pairs take 44.1, 50.1, 44.7, 52.9 and 75.4 (the weights'
   // bytes alone 40.7, the MMAs 71 at 256).  At 64 columns 45.0 -> 43.7, at 48 45.6 -> 43.1.
-  if (gate_up && has_lo && n_pad >= 48 && cs == 1 && p.m_tiles % 2 == 0 && p.m_tiles > num_sms &&
+  if (gate_up && has_lo && n_pad >= kLargeCols && cs == 1 && p.m_tiles % 2 == 0 && p.m_tiles > num_sms &&
       (p.m_tiles / 2 + 1) / 2 <= fit(2)) {
     const uint32_t st2 = 2 * kWTileBytes + static_cast<uint32_t>(n_pad) * kBK * 2;
     int stages2 = static_cast<int>((192u * 1024u) / st2);
@@ -1070,7 +1076,7 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
   // 10.5 at 80 and 17.2 -> 13.4 at 144, down 35.5 -> 26 and 42.2 -> 32.5, QKV as halves 18.5 -> 13.9 at 96
   // (but 12.4 -> 13.7 at 80).  8B QKV at 112: whole pairs 19.1, halves 20.7, neither 21.9.  Below 80 only a
   // K loop over four ranks gains (7B O at 48: 11.4 -> 9.1; 8B QKV over two 14.4 -> 17.2).
-  if (!gate_up && has_lo && n_pad >= 48 && p.m_tiles % 2 == 0 && pc <= 4) {
+  if (!gate_up && has_lo && n_pad >= kLargeCols && p.m_tiles % 2 == 0 && pc <= 4) {
     if ((n_pad > 128 && pc == 2) || (n_pad >= kHalfBoxCols && pc == 4 && p.m_tiles / 2 > fit(8)))
       take_pairs(pc / 2, 2);
     else if ((n_pad >= 80 || pc == 4) && p.m_tiles / 2 <= fit(2 * pc))
@@ -1107,13 +1113,13 @@ GemmKernel gemm_image(GemmImage i, int mode) {
 
 }  // namespace
 
-cudaError_t gemm_configure() {
-  for (int i = 0; i < kGemmImages; ++i)
+cudaError_t gemm_configure(int n_pad_max) {
+  for (int i = 0; i < (n_pad_max >= kLargeCols ? kGemmImages : kLarge); ++i)
     for (int mode = GemmEpilogue::PLAIN; mode <= GemmEpilogue::LOWRANK; ++mode) {
       const GemmKernel k = gemm_image(static_cast<GemmImage>(i), mode);
       if (!k) continue;
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kGemmMaxSmem));
-      if (e == cudaSuccess) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+      if (e == cudaSuccess && i != kPair) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
       if (e != cudaSuccess) return e;
     }
   return cudaSuccess;
@@ -1128,7 +1134,7 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
   cfg.gridDim = dim3(p.pair && p.gate_up ? (units + 1) / 2 * 2 : units * p.cluster, 1, 1);
   // the vector epilogues win from 48 padded columns on even with four warps (40 candidates of a 7B scorer
   // 564 -> 532 us for four layers; 24 candidates, 32 columns: 397 us small, 405 large)
-  const bool large = n_pad >= 48;
+  const bool large = n_pad >= kLargeCols;
   if (p.threads != 128 && (p.threads != 256 || !large)) return cudaErrorInvalidValue;
   cfg.blockDim = dim3(static_cast<unsigned>(p.threads), 1, 1);
   cfg.dynamicSmemBytes = p.smem_bytes;

@@ -94,7 +94,8 @@ struct GemmLowRank {
   const CUtensorMap* t_lo = nullptr;
   int k_main = 0;
 };
-cudaError_t gemm_configure();
+// Attributes of the kernel images that batches of up to n_pad_max padded columns take.
+cudaError_t gemm_configure(int n_pad_max);
 cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtensorMap* tmX, const CUtensorMap* tmXlo,
                         const GemmEpilogue& ep, int n_pad, int* err, cudaStream_t stream, bool pdl,
                         unsigned long long* ts = nullptr, const GemmLowRank* lr = nullptr);

@@ -1403,7 +1403,7 @@ int kvprm_create(const kvprm_config* cfg, const kvprm_weights* w, kvprm_ctx** ou
     }
     ctx->encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
-  CREATE_CK(cu(kvprm::gemm_configure(), "gemm_configure"));
+  CREATE_CK(cu(kvprm::gemm_configure((ctx->cfg.max_candidates + 15) / 16 * 16), "gemm_configure"));
   CREATE_CK(cu(kvprm::attention_configure(), "attention_configure"));
   CREATE_CK(cu(kvprm::grad_configure(), "grad_configure"));
 
