@@ -336,7 +336,7 @@ KVPRM_API int kvprm_resolve(kvprm_ctx* ctx, int32_t b, int64_t* phys_row);
  * per CTA of a separate launch (at most n_ctas of them); 3 (what scoring
  * contexts with head_dim 128 use) as 2, with the n_ctas SMs split between the
  * two launches so that the later one, estimated under a cost model (a
- * tensor-core CTA: 29 units per chunk plus 180; a private page 4, a shared
+ * tensor-core CTA: 26 units per chunk plus 180; a private page 4, a shared
  * page 2 per candidate), ends soonest (n_ctas + n_tc_ctas <= the given
  * n_ctas), so that they run side by side.  Shared tiles of different groups
  * with the same candidates form one run over all their pages.  Kind-2 segments follow
@@ -405,11 +405,15 @@ KVPRM_API int kvprm_plan_attention(const int32_t* block_table, int32_t max_block
  * device call), so that its invariants can be checked without a GPU.  gate_up: W holds the gate rows
  * then the up rows (M = d_ff pairs, 64 of each per tile).
  *  m_tiles       128-row tiles (gate/up: 64-pair tiles)
- *  k_tiles       64-wide K tiles; kt_per_split per rank of a split-K cluster
- *  cluster       CTAs per thread-block cluster (split-K ranks)
- *  tiles_per_cta m-tiles each CTA takes (1, or 2 for large batches)
+ *  k_tiles       64-wide K tiles; kt_per_split = ceil(k_tiles / cluster)
+ *  cluster       CTAs that share tiles_per_cta m-tiles: split-K ranks of one cluster; at larger
+ *                batches CTA pairs, which divide two m-tiles (tiles_per_cta 2) or the columns (1)
+ *                between them and K over cluster / 2 ranks.  gate/up with tiles_per_cta 2: no split
+ *                K, two such CTAs a pair
+ *  tiles_per_cta m-tiles that one activation tile serves (1 or 2)
  *  stages        shared-memory ring stages; tmem_cols tensor-memory columns; smem_bytes per CTA
- *  threads       threads per CTA: 256 for n_pad >= 64 (the large-batch kernel image), else 128
+ *  threads       threads per CTA: 256 for n_pad >= 64, else 128 (the large-batch kernel image starts
+ *                at 48 columns)
  * Errors: KVPRM_EINVAL (M, K or num_sms < 1, n_pad not a positive multiple of 16, out NULL). */
 typedef struct {
   int32_t m_tiles, k_tiles, kt_per_split, cluster, tiles_per_cta, stages, tmem_cols;
