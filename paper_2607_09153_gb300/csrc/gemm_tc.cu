@@ -57,6 +57,7 @@ constexpr int kLargeCols = 48;                      // padded columns from which
 constexpr int kHalfBoxCols = 96;                    // padded columns from which activation boxes hold half
 constexpr int kHPreCols = 8;                        // residual columns preloaded per rank (128 rows each)
 constexpr size_t kGemmMaxSmem = 200 * 1024;         // dynamic shared memory the kernel is configured for
+constexpr size_t kAloneSmem = 120 * 1024;           // with which no second CTA fits on an SM
 
 __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
   return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~static_cast<uintptr_t>(1023));
@@ -1138,6 +1139,11 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
   if (p.threads != 128 && (p.threads != 256 || !large)) return cudaErrorInvalidValue;
   cfg.blockDim = dim3(static_cast<unsigned>(p.threads), 1, 1);
   cfg.dynamicSmemBytes = p.smem_bytes;
+  // An adapter's A x keeps its few SMs (16 to 64 CTAs) to itself, over half of an SM's shared memory a
+  // CTA: beside CTAs of the projection that it lets start, its K loop and its parking took twice as long
+  // (gate/up's A x 8.8 us, 3.9 alone).  Eight 1.5B layers at rank 64 392 -> 370 us, rank 512 433 -> 411;
+  // four 7B layers, 16 candidates, rank 256 452 -> 431; rank 256 over 28 1.5B layers the same (1,550).
+  if (ep.mode == GemmEpilogue::LOWRANK && cfg.dynamicSmemBytes < kAloneSmem) cfg.dynamicSmemBytes = kAloneSmem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
