@@ -1478,13 +1478,11 @@ int kvprm_create(const kvprm_config* cfg, const kvprm_weights* w, kvprm_ctx** ou
   CREATE_CK(dalloc(ctx, &ctx->apart_o, ctx->slot_cap * group * m.hd, "attn partials"));
   CREATE_CK(dalloc(ctx, &ctx->apart_ml, ctx->slot_cap * group * 2, "attn stats"));
   CREATE_CK(dalloc(ctx, &ctx->rope, static_cast<size_t>(Bmax) * (m.hd / 2), "rope table"));
-  {
-    double f[64];
-    for (int i = 0; i < m.hd / 2; ++i) f[i] = std::pow(static_cast<double>(c.rope_base), -2.0 * i / m.hd);
-    CREATE_CK(dalloc(ctx, &ctx->inv_freq, static_cast<size_t>(m.hd / 2), "rotary frequencies"));
-    CREATE_CK(cu(cudaMemcpy(ctx->inv_freq, f, sizeof(double) * (m.hd / 2), cudaMemcpyHostToDevice),
-                 "cudaMemcpy(rotary frequencies)"));
-  }
+  double freq[64];   // read by its copy until the synchronisation below at the latest
+  for (int i = 0; i < m.hd / 2; ++i) freq[i] = std::pow(static_cast<double>(c.rope_base), -2.0 * i / m.hd);
+  CREATE_CK(dalloc(ctx, &ctx->inv_freq, static_cast<size_t>(m.hd / 2), "rotary frequencies"));
+  CREATE_CK(cu(cudaMemcpyAsync(ctx->inv_freq, freq, sizeof(double) * (m.hd / 2), cudaMemcpyHostToDevice, nullptr),
+               "cudaMemcpyAsync(rotary frequencies)"));   // behind dalloc's memset, and no wait for the device here
   {
     const size_t tbl = static_cast<size_t>(Bmax) * (1 + c.max_blocks_per_seq);
     auto al8 = [](size_t x) { return (x + 7) & ~static_cast<size_t>(7); };
