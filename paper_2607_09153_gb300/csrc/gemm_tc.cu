@@ -1144,6 +1144,10 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
   // (gate/up's A x 8.8 us, 3.9 alone).  Eight 1.5B layers at rank 64 392 -> 370 us, rank 512 433 -> 411;
   // four 7B layers, 16 candidates, rank 256 452 -> 431; rank 256 over 28 1.5B layers the same (1,550).
   if (ep.mode == GemmEpilogue::LOWRANK && cfg.dynamicSmemBytes < kAloneSmem) cfg.dynamicSmemBytes = kAloneSmem;
+  // A pair's CTA takes all it may: its tensor memory (up to 512 columns) is allocated in two SMs at once, and
+  // beside a cluster of another stream's launch either could hold the columns the other's second CTA waits
+  // for.  What is left (27 KB) is too little for any other launch that allocates tensor memory.
+  if (p.pair) cfg.dynamicSmemBytes = kGemmMaxSmem;
   cfg.stream = stream;
   cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;

@@ -9,7 +9,7 @@ import pytest
 
 import kvsynth as ks
 import paper_2607_09153_gb300 as kp
-from tests.gpu_util import compare, require_gpu, run_gpu
+from tests.gpu_util import compare, make_scorer, require_gpu, run_gpu
 from tests.test_gpu_steering import _compare, _gpu_grad, _oracle
 
 # QKV and O: pairs at 80 to 128 padded columns, halves beyond; down (11 K tiles over 4 ranks): pairs
@@ -60,3 +60,25 @@ def test_gradient():
     p_ref, ref, _, _ = _oracle(w, t)
     _compare("166 candidates", w, p, grad, p_ref, ref)
     sc.close()
+
+
+@pytest.mark.gpu
+def test_two_streams():
+    """Two contexts' pairs on two streams at once: the rewards of either alone, bit for bit."""
+    torch = require_gpu()
+    t = ks.Tables.make(0.2)
+    runs = []
+    for arch, n in [(GATE_UP, 96), (WIDE, 130)]:
+        w = ks.distinct("pairs_streams", arch, 800 + n, [(5 * b) % 40 for b in range(n)], gain_std=0.2)
+        dev = ks.DeviceInputs(w, t)
+        sc = make_scorer(dev, n, w.max_blocks)
+        alone = torch.tensor(sc.score(dev.pool, w.block_table, w.seq_lens))
+        runs.append((w, dev, sc, alone, torch.zeros(n, device="cuda"), torch.cuda.Stream()))
+    torch.cuda.synchronize()
+    for _ in range(8):
+        for w, dev, sc, _, out, st in runs:
+            sc.score_async(dev.pool, w.block_table, w.seq_lens, out, stream=st)
+    torch.cuda.synchronize()
+    for _, _, sc, alone, out, _ in runs:
+        assert torch.equal(out.cpu(), alone)
+        sc.close()
