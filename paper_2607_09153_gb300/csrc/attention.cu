@@ -425,8 +425,11 @@ __global__ void __launch_bounds__(W * 32) attn_combine_kernel(
 // every load it uses (up to kFlatSlots partial slots' (m, l) and O values; q, k_self and v_self go
 // before the first) before using any, so it costs one memory round trip; the slots then merge
 // into the running (M, L, acc), and the verify token's own entry last.  No shared memory and no
-// CTA barrier, so CTAs are short and many fit on an SM.
-constexpr int kFlatSlots = 8;
+// CTA barrier, so CTAs are short and many fit on an SM.  Five slots a round: 64 registers, so four CTAs of
+// 7 warps on an SM where eight slots (91 registers) let three, and MCTS's 1,024 CTAs start in fewer waves
+// (12.6 -> 9.8 us a layer; its pairs average 4.7 slots).  Six slots 11.4; four in 54 registers 9.5, but beam's
+// 256 CTAs, one wave either way, then 7.1 instead of 6.1.
+constexpr int kFlatSlots = 5;
 
 template <int HD>
 __global__ void __launch_bounds__(512) attn_combine_flat_kernel(
