@@ -79,7 +79,8 @@ struct GemmEpilogue {
   __nv_bfloat16* t_lo = nullptr;
   // let the next kernel in the stream launch only once this one's partials are parked (after its
   // first cluster barrier) instead of at entry: a next kernel whose CTAs fit beside this one's on
-  // an SM otherwise slows that barrier by ~2.5 us (measured for the O projection before gate/up)
+  // an SM otherwise slows that barrier by ~2.5 us (measured for the O projection before gate/up; the
+  // down projection and, from 64 columns, QKV do the same)
   bool late_trigger = false;
 };
 GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_up);
