@@ -46,16 +46,6 @@ __device__ __forceinline__ void store_hilo4(HiLo o, int64_t i, float4 x) {
   *reinterpret_cast<uint2*>(o.lo + i) = lo;
 }
 
-// Four consecutive bf16 of a caller's vector as fp32 (8 bytes at a time when it is aligned).
-__device__ __forceinline__ float4 load_bf16x4(const __nv_bfloat16* p) {
-  if (reinterpret_cast<uintptr_t>(p) & 7u)
-    return make_float4(__bfloat162float(p[0]), __bfloat162float(p[1]), __bfloat162float(p[2]), __bfloat162float(p[3]));
-  const uint2 r = *reinterpret_cast<const uint2*>(p);
-  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r.x));
-  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r.y));
-  return make_float4(a.x, a.y, b.x, b.y);
-}
-
 // The call's tables, read by the GPU from the pinned staging buffer (one launch instead of a copy per
 // table: seven to nine small copies took ~2 us each on the stream, ahead of every call), and for the
 // attention entry point the query as a bf16 pair.  Measured per call with calls queued back to back:

@@ -641,13 +641,11 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
         const bool rows_ok = gm0 < ep.M;   // M % 4 == 0: the four rows are all valid or all past M
         float g4[4] = {0.f, 0.f, 0.f, 0.f};
         if (ep.gain_next && rows_ok) {
-          const uint2 gb = *reinterpret_cast<const uint2*>(ep.gain_next + gm0);
-          const float2 ga = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gb.x));
-          const float2 gc = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&gb.y));
-          g4[0] = ga.x;
-          g4[1] = ga.y;
-          g4[2] = gc.x;
-          g4[3] = gc.y;
+          const float4 g = load_bf16x4(ep.gain_next + gm0);
+          g4[0] = g.x;
+          g4[1] = g.y;
+          g4[2] = g.z;
+          g4[3] = g.w;
         }
 #pragma unroll 1
         for (int c0 = cbeg + cg; c0 < cend; c0 += nw * 8) {

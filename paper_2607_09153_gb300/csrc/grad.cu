@@ -48,16 +48,6 @@ __device__ __forceinline__ void put_hilo4(bf16* hi, bf16* lo, int64_t i, float4 
   *reinterpret_cast<uint2*>(lo + i) = b;
 }
 
-// Four consecutive bf16 of a caller's vector as fp32 (8 bytes at a time when it is aligned).
-__device__ __forceinline__ float4 bf16x4(const bf16* p) {
-  if (reinterpret_cast<uintptr_t>(p) & 7u)
-    return make_float4(__bfloat162float(p[0]), __bfloat162float(p[1]), __bfloat162float(p[2]), __bfloat162float(p[3]));
-  const uint2 r = *reinterpret_cast<const uint2*>(p);
-  const float2 a = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r.x));
-  const float2 b = __bfloat1622float2(*reinterpret_cast<const __nv_bfloat162*>(&r.y));
-  return make_float4(a.x, a.y, b.x, b.y);
-}
-
 // two block-wide sums at once (blockDim.x a multiple of 32, <= 1024); every thread gets both
 __device__ __forceinline__ float2 block_sum2(float a, float b, float2* red) {
 #pragma unroll
@@ -140,7 +130,7 @@ __global__ void __launch_bounds__(1024) head_back_kernel(
   const int64_t row = static_cast<int64_t>(blockIdx.x) * d;
   const float q = 1.f - p_plus[blockIdx.x];   // d(-log P)/dz_- = 1 - P = -d(-log P)/dz_+
   auto load = [&](int c) {
-    const float4 g = bf16x4(gain + c), p = bf16x4(w_plus + c), m = bf16x4(w_minus + c);
+    const float4 g = load_bf16x4(gain + c), p = load_bf16x4(w_plus + c), m = load_bf16x4(w_minus + c);
     NormBack v;
     v.h = *reinterpret_cast<const float4*>(h + row + c);
     v.gdy = make_float4(g.x * q * (m.x - p.x), g.y * q * (m.y - p.y), g.z * q * (m.z - p.z), g.w * q * (m.w - p.w));
@@ -161,9 +151,9 @@ __global__ void __launch_bounds__(1024) rms_back_kernel(const float* __restrict_
   grid_dep_wait();
   const int64_t row = static_cast<int64_t>(blockIdx.x) * d;
   auto load = [&](int c) {
-    const float4 g = bf16x4(gain + c), y = *reinterpret_cast<const float4*>(dy + row + c);
+    const float4 g = load_bf16x4(gain + c), y = *reinterpret_cast<const float4*>(dy + row + c);
     NormBack v;
-    v.h = h_bf16 ? bf16x4(h_bf16 + c) : *reinterpret_cast<const float4*>(h + row + c);
+    v.h = h_bf16 ? load_bf16x4(h_bf16 + c) : *reinterpret_cast<const float4*>(h + row + c);
     v.gdy = make_float4(g.x * y.x, g.y * y.y, g.z * y.z, g.w * y.w);
     v.dres = *reinterpret_cast<const float4*>(dres + row + c);
     return v;

@@ -1,7 +1,8 @@
 """The call's tables on their way to the device (one kernel reading pinned host memory) and the
 rewards on their way out: odd table sizes (parts that end inside a 16-byte quad, empty parts, more
 than one launch round of quads), two calls in flight that share the staging buffer, and the
-caller's device buffer written by the head kernel instead of a copy."""
+caller's device buffer written by the head kernel instead of a copy; and the caller's vectors (embedding,
+gains, head rows), which may start at any element, on every image that reads them."""
 import numpy as np
 import pytest
 
@@ -63,3 +64,28 @@ def test_vectors_at_any_address(shift):
     sc = make_scorer(dev, 3, w.max_blocks)
     assert np.array_equal(sc.score(dev.pool, w.block_table, w.seq_lens), want)
     sc.close()
+
+
+# a residual epilogue of each image: 32 padded columns (small), 48 (the fewest of the large one, also as 12
+# candidates of four verify tokens), 64, 80 (CTA pairs), 144 (pairs of half of the columns)
+@pytest.mark.parametrize("n, depth", [(32, 1), (33, 1), (12, 4), (49, 1), (80, 1), (129, 1)])
+@pytest.mark.parametrize("shift", [1, 2])
+def test_gains_at_any_address(n, depth, shift):
+    require_gpu()
+    w = ks.distinct("gains", ks.Arch(2, 256, 4, 2, 64, 704), 95 + n, [(11 * b) % 50 for b in range(n)], gain_std=0.2)
+    dev = ks.DeviceInputs(w, ks.Tables.make(0.2))
+
+    def rewards():
+        sc = make_scorer(dev, n * depth, w.max_blocks)
+        sc.set_depth(depth)
+        r = sc.score(dev.pool, w.block_table, w.seq_lens)
+        sc.close()
+        return r
+
+    want = rewards()
+    for layer in dev.layers:
+        for k in (ks.ATTN_NORM, ks.MLP_NORM):
+            buf = layer[k].new_zeros(layer[k].numel() + 8)
+            buf[shift:shift + layer[k].numel()] = layer[k].reshape(-1)
+            layer[k] = buf[shift:shift + layer[k].numel()]
+    assert np.array_equal(rewards(), want)
