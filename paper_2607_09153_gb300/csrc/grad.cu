@@ -532,9 +532,9 @@ __device__ __forceinline__ void split8(const float (&x)[8], uint4* hi, uint4* lo
 template <int HD>
 __global__ void __launch_bounds__(kBackThreads, 1) attn_back_tc_kernel(
     const __grid_constant__ CUtensorMap tm_pool_tc, int64_t layer_page0, const BackItem* __restrict__ items,
-    const int32_t* __restrict__ cta_item, const uint32_t* __restrict__ pages, const int32_t* __restrict__ cands, const uint8_t* __restrict__ ops,
-    const float2* __restrict__ meta, int n_q, int n_kv, float* __restrict__ grad_layer,
-    float* __restrict__ dq, int* err) {
+    const int32_t* __restrict__ cta_item, const uint32_t* __restrict__ pages, const int32_t* __restrict__ cands,
+    const uint8_t* __restrict__ ops, const uint8_t* __restrict__ zero_rows, const float2* __restrict__ meta, int n_q,
+    int n_kv, float* __restrict__ grad_layer, float* __restrict__ dq, int* err) {
   using SM = BackSmem<HD>;
   extern __shared__ uint8_t smem_raw[];
   uint8_t* base = align1024(smem_raw);
@@ -574,7 +574,8 @@ __global__ void __launch_bounds__(kBackThreads, 1) attn_back_tc_kernel(
     fence_mbar_init();
     tma_prefetch_desc(&tm_pool_tc);
   }
-  // rows that no candidate of a step fills meet zero weights: they only have to be finite
+  // The partner rows of an odd candidate meet zero weights, but 0 x Inf is NaN: they are zero, here and
+  // (load_rows) whenever an earlier step left a candidate's rows there.
   for (uint32_t i = threadIdx.x; i < kBackRowStages * 2 * SM::kRows / 16; i += blockDim.x)
     reinterpret_cast<uint4*>(base + SM::kRowBuf)[i] = make_uint4(0u, 0u, 0u, 0u);
   fence_proxy_async_smem();
@@ -595,6 +596,7 @@ __global__ void __launch_bounds__(kBackThreads, 1) attn_back_tc_kernel(
       const bool keys = warp == 0;
       const uint64_t pol = policy_evict_first();
       uint32_t it = 0, ki = 0;
+      uint32_t filled = 0;   // bit 4 rb + i: candidate slot i of row stage rb holds some candidate's rows
       bool ok = true;
       auto load_pages = [&](const BackItem& w) -> bool {
         uint64_t* full = keys ? &k_full[ki & 1u] : v_full;
@@ -618,8 +620,16 @@ __global__ void __launch_bounds__(kBackThreads, 1) attn_back_tc_kernel(
         const uint32_t rb = it % kBackRowStages, use = it / kBackRowStages;
         if (use > 0 && !mbar_wait(&r_empty[rb], (use - 1) & 1u, err)) return false;
         const int nc = min(kBackRowsCands, w.n_cands - c0);
-        mbar_arrive_expect_tx(&r_full[rb], static_cast<uint32_t>(nc) * (2 * SM::kCand + 64));
+        // an odd candidate's partner in its 16-row MMA
+        const uint32_t partner = (nc & 1) ? 1u << (kBackRowsCands * rb + nc) : 0u;
+        const bool clear = (filled & partner) != 0u;
+        mbar_arrive_expect_tx(&r_full[rb], static_cast<uint32_t>(nc) * (2 * SM::kCand + 64) + (clear ? 2 * SM::kCand : 0u));
         uint8_t* rows = base + SM::kRowBuf + rb * 2 * SM::kRows;
+        if (clear) {
+          bulk_load(rows + nc * SM::kCand, zero_rows, SM::kCand, &r_full[rb]);
+          bulk_load(rows + SM::kRows + nc * SM::kCand, zero_rows, SM::kCand, &r_full[rb]);
+        }
+        filled = (filled & ~partner) | ((1u << nc) - 1u) << (kBackRowsCands * rb);
 #pragma unroll 1
         for (int i = 0; i < nc; ++i) {
           const int64_t bg = static_cast<int64_t>(__ldg(cands + w.cand_off + c0 + i)) * n_kv + w.g;
@@ -1047,11 +1057,11 @@ cudaError_t launch_attn_back(const AttnBackArgs& a, cudaStream_t st) {
     const dim3 grid(a.n_ctas);
     if (a.hd == 128)
       return launch_pdl(attn_back_tc_kernel<128>, grid, dim3(kBackThreads), BackSmem<128>::kBytes, st, *a.tm_pool_tc,
-                        a.layer_page0, a.items, a.cta_item, a.item_pages, a.item_cands, a.ops, a.meta, a.n_q, a.n_kv,
-                        a.grad_layer, a.dq, a.err);
+                        a.layer_page0, a.items, a.cta_item, a.item_pages, a.item_cands, a.ops, a.zero_rows, a.meta, a.n_q,
+                        a.n_kv, a.grad_layer, a.dq, a.err);
     return launch_pdl(attn_back_tc_kernel<64>, grid, dim3(kBackThreads), BackSmem<64>::kBytes, st, *a.tm_pool_tc,
-                      a.layer_page0, a.items, a.cta_item, a.item_pages, a.item_cands, a.ops, a.meta, a.n_q, a.n_kv,
-                      a.grad_layer, a.dq, a.err);
+                      a.layer_page0, a.items, a.cta_item, a.item_pages, a.item_cands, a.ops, a.zero_rows, a.meta, a.n_q,
+                      a.n_kv, a.grad_layer, a.dq, a.err);
   }
   if (a.n_units == 0) return e;
   const size_t smem = a.hd == 128 ? back_pages_smem<128>() : back_pages_smem<64>();

@@ -320,6 +320,7 @@ struct AttnBackArgs {
   const uint32_t* item_pages;
   const int32_t* item_cands;
   uint8_t* ops;
+  const uint8_t* zero_rows;   // attn_back_zero_bytes(hd) of zeros
   float2* meta;
   const CUtensorMap* tm_pool_tc = nullptr;
   int64_t layer_page0 = 0;
@@ -336,6 +337,8 @@ struct AttnBackArgs {
 };
 // bytes of AttnBackArgs::ops for n rows
 inline size_t attn_back_ops_bytes(size_t n, int n_kv, int hd) { return n * n_kv * 4 * (hd / 64) * 1024; }
+// the hi and lo rows of one candidate
+inline size_t attn_back_zero_bytes(int hd) { return static_cast<size_t>(2) * (hd / 64) * 1024; }
 // units hold at most this many pages (the pages kernel stages them all in shared memory)
 constexpr int kBackUnitPagesMax = 8;
 cudaError_t grad_configure();

@@ -81,6 +81,7 @@ struct GradState {
   int tm_npad = -1;
   CUtensorMap tm_d_hi{}, tm_d_lo{}, tm_gu_hi{}, tm_gu_lo{}, tm_qkv_hi{}, tm_qkv_lo{};
   uint8_t* ops = nullptr;    // tensor-core attention backward: the rows' operand blocks, their (lse, D)
+  const uint8_t* zero_rows = nullptr;   // in ops
   float2* meta = nullptr;
   // per call: the attention backward's schedule, atomic-page flags and page lists (BackPlan)
   kvprm::BackPlan plan;
@@ -1119,7 +1120,10 @@ int ensure_grad(kvprm_ctx* ctx, cudaStream_t st) {
   if ((rc = dalloc(ctx, &g.ghi, static_cast<size_t>(ctx->npad_max) * gmax, "backward hi"))) return rc;
   if ((rc = dalloc(ctx, &g.glo, static_cast<size_t>(ctx->npad_max) * gmax, "backward lo"))) return rc;
   if (m.n_q / m.n_kv <= 8 && !ctx->grad_cuda_cores) {
-    if ((rc = dalloc(ctx, &g.ops, kvprm::attn_back_ops_bytes(Bm, m.n_kv, m.hd), "backward operands"))) return rc;
+    // and after them the zero rows
+    const size_t ops = kvprm::attn_back_ops_bytes(Bm, m.n_kv, m.hd);
+    if ((rc = dalloc(ctx, &g.ops, ops + kvprm::attn_back_zero_bytes(m.hd), "backward operands"))) return rc;
+    g.zero_rows = g.ops + ops;
     if ((rc = dalloc(ctx, &g.meta, Bm * m.n_kv * 8, "backward row statistics"))) return rc;
   }
   // transposed weights: W [out][in] -> W^T [in][out], from the borrowed weights' tensor-map bases
@@ -1271,6 +1275,7 @@ int score_grad_device(kvprm_ctx* ctx, const void* kv_pages, int64_t n_pages, con
       a.item_pages = g.item_pages;
       a.item_cands = g.item_cands;
       a.ops = g.ops;
+      a.zero_rows = g.zero_rows;
       a.meta = g.meta;
       a.units = g.units;
       a.n_units = static_cast<int>(bp.units.size());

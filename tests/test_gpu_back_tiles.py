@@ -3,7 +3,9 @@ step, 8 rows a candidate): shared runs one page short of a tile, one over and se
 candidates that fill a step, leave one over or are split over tiles because the pages alone would
 leave the GPU idle; both head widths; the narrowest and widest groups; row counts whose workspace
 arrays do not end on 16 bytes.  Against the fp64 oracle with the gradient's tolerance
-(tests/test_gpu_steering.py), and eagerly against the captured graph."""
+(tests/test_gpu_steering.py), and eagerly against the captured graph.  And a candidate that is not finite, whose
+rows must not reach the gradient of pages that it does not read."""
+import numpy as np
 import pytest
 
 import kvsynth as ks
@@ -48,3 +50,24 @@ def test_odd_rows(n, group, n_kv):
     p_ref, ref, _, _ = _oracle(w, t)
     _compare(f"{n} candidates of {group * n_kv} heads", w, p, grad, p_ref, ref)
     sc.close()
+
+
+# The bad candidate's rows stay in shared memory, in its place of a step of four; three row stages on, the same CTA
+# takes a step that leaves this place empty beside a candidate: a private page's (places 0, 1), or a step of three.
+@pytest.mark.parametrize("groups, bad, own", [([(4, 128)], 1, 9728), ([(8, 608 * 16), (3, 1216 * 16)], 3, 16)])
+@pytest.mark.parametrize("which, value", [(0, "inf"), (1, "nan")])
+def test_a_candidate_that_is_not_finite(groups, bad, own, which, value):
+    torch = require_gpu()
+    t = ks.Tables.make(0.2)
+    segs = [[(1 + i, shared), (10 + 10 * i + b, own)] for i, (cands, shared) in enumerate(groups) for b in range(cands)]
+    w = ks.workload_from_segments("back_nan", arch(64, 2), 750, segs, gain_std=0.2)
+    p, grad, dev, sc = _gpu_grad(w, t)
+    sc.close()
+    pages = [set(w.block_table[b, :int(w.seq_lens[b]) // 16].tolist()) for b in range(len(segs))]
+    dev.pool[0, int(w.block_table[bad, int(w.seq_lens[bad]) // 16 - 1]), which, :, 3, :] = float(value)
+    p2, grad2, _, sc = _gpu_grad(w, t, dev)
+    sc.close()
+    others = [b for b in range(len(segs)) if b != bad]
+    assert not np.isfinite(p2[bad]) and np.array_equal(p2[others], p[others])
+    clean = sorted(set().union(*pages) - pages[bad])
+    assert torch.equal(grad2[0][clean], grad[0][clean])
