@@ -238,10 +238,15 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     // kernel that wrote x: only the last K tiles, t's, wait for it.  The weights' products then run beside
     // A x (1.5B, 16 candidates: rank 256 1,582 -> 1,550 us a call, rank 64 414 -> 391 for eight layers; 48
     // candidates at rank 256 577 -> 542; ranks 512 and 1,024 -3 to +1 %).  Starting it from A x's last
-    // landed tile instead: 1,607.
+    // landed tile instead: 1,607.  That A x has waited does not by itself order x before the reads here, so
+    // one of its threads leaves a mark after its wait (0.1 us a launch: 1,509 -> 1,521; 8B, 4 candidates,
+    // rank 64, four layers 375 -> 379; 1,563 and 395 with x behind A x's end).
     bool waited = k_main == k_tiles;
-    if (waited) grid_dep_wait();
-    trace_event(ts, 0);   // the preceding kernel has completed
+    if (waited)
+      grid_dep_wait();
+    else
+      mark_acquire(ep.x_ready, *ep.call, err);
+    trace_event(ts, 0);   // the preceding kernel has completed (with an adapter: the one before A x)
     auto load_act = [&](int stage, int kt) {
       if (!waited && kt >= k_main) {
         grid_dep_wait();
@@ -267,8 +272,13 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     // ---------------- while the weights stream: the RMSNorm factor of each of this rank's columns
     // (QKV, SILU), from the residual stream's tile sums of squares the preceding kernel wrote; the
     // parking barrier below orders these writes before the epilogue reads them
+    const bool marks = MODE == GemmEpilogue::LOWRANK && blockIdx.x == 0 && threadIdx.x == 64;
+    const int call = marks ? *ep.call : 0;
     grid_dep_wait();
-    if (MODE == GemmEpilogue::LOWRANK) grid_dep_launch();
+    if (MODE == GemmEpilogue::LOWRANK) {
+      if (marks) mark_release(ep.x_ready, call);
+      grid_dep_launch();
+    }
     if ((MODE == GemmEpilogue::QKV || MODE == GemmEpilogue::SILU) && ep.rs_sumsq)
 #pragma unroll 1
       for (int t0 = threadIdx.x - 64; t0 < nc; t0 += blockDim.x - 64) {   // nc <= 256 columns
@@ -1164,12 +1174,17 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
   const CUtensorMap& mt = with_lr ? *lr->t_hi : *tmX;
   const CUtensorMap& mtl = with_lr ? (p.has_lo ? *lr->t_lo : *lr->t_hi) : xlo;
   const int k_main = with_lr ? lr->k_main : p.k_tiles;
+  GemmEpilogue e = ep;
+  if (with_lr) {
+    e.x_ready = lr->x_ready;
+    e.call = lr->call;
+  }
   const int n_split = p.pair && p.mt == 1 ? 2 : 1;
   const GemmKernel kern = gemm_image(p.pair ? kPair : (large ? kLarge : kSmall), ep.mode);
   if (!kern || (p.pair && (!large || !p.has_lo || p.gate_up != (ep.mode == GemmEpilogue::SILU))))
     return cudaErrorInvalidValue;
   return cudaLaunchKernelEx(&cfg, kern, *tmW, *tmX, xlo, p.has_lo ? 1 : 0, mb, mt, mtl, k_main, p.k_tiles,
-                            p.pair ? cluster / 2 : cluster, p.stages, p.tmem_cols, n_pad / n_split, n_split, ep, err, ts);
+                            p.pair ? cluster / 2 : cluster, p.stages, p.tmem_cols, n_pad / n_split, n_split, e, err, ts);
 }
 
 }  // namespace kvprm

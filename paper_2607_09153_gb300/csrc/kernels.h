@@ -77,6 +77,10 @@ struct GemmEpilogue {
   float lr_scale = 0.f;
   __nv_bfloat16* t_hi = nullptr;
   __nv_bfloat16* t_lo = nullptr;
+  // LOWRANK: *x_ready becomes the call's number *call once x may be read; the projection that takes t waits for
+  // that, instead of for its predecessor's end, before it reads x
+  int* x_ready = nullptr;
+  const int* call = nullptr;
   // let the next kernel in the stream launch only once this one's partials are parked (after its
   // first cluster barrier) instead of at entry: a next kernel whose CTAs fit beside this one's on
   // an SM otherwise slows that barrier by ~2.5 us (measured for the O projection before gate/up; the
@@ -94,6 +98,8 @@ struct GemmLowRank {
   const CUtensorMap* t_hi = nullptr;   // t hi / lo, box of its activation tile
   const CUtensorMap* t_lo = nullptr;
   int k_main = 0;
+  int* x_ready = nullptr;              // of the A x launch, and the call's number (GemmEpilogue)
+  const int* call = nullptr;
 };
 // Attributes of the kernel images that batches of up to n_pad_max padded columns take.
 cudaError_t gemm_configure(int n_pad_max);

@@ -130,6 +130,8 @@ struct kvprm_ctx {
   std::vector<CUtensorMap> tm_la[4], tm_lb[4];
   bf16 *thi = nullptr, *tlo = nullptr;
   size_t t_cap = 0;
+  int* x_ready = nullptr;   // [n_layers][4] the last call whose A x of that projection had its x
+  int32_t call = 0;         // number of the current call (in its tables)
   int tm_t_npad = -1;
   CUtensorMap tm_thi{}, tm_tlo{};
   // workspace
@@ -311,6 +313,7 @@ void free_ctx(kvprm_ctx* c) {
   cudaFree(c->apart_ml);
   cudaFree(c->rope);
   cudaFree(c->inv_freq);
+  cudaFree(c->x_ready);
   cudaFree(c->tables_d);
   cudaFree(c->rewards_d);
   cudaFree(c->err_d);
@@ -431,8 +434,8 @@ int plan_work(kvprm_ctx* ctx, const int32_t* bt, const int32_t* sl, int32_t n, b
   return KVPRM_OK;
 }
 
-// Put the tables, the planned work and the address of the caller's reward buffer (or null) into the
-// pinned staging buffer and enqueue the kernel that pulls them to the device; q_count > 0: that launch
+// Put the tables, the planned work, the address of the caller's reward buffer (or null) and the call's
+// number into the pinned staging buffer and enqueue the kernel that pulls them to the device; q_count > 0: that launch
 // also splits the caller's query into ctx->qhi / qlo.
 int upload_tables(kvprm_ctx* ctx, const int32_t* bt, const int32_t* sl, int32_t n, cudaStream_t st,
                   float* rewards_out = nullptr, const float* q = nullptr, int64_t q_count = 0) {
@@ -444,6 +447,11 @@ int upload_tables(kvprm_ctx* ctx, const int32_t* bt, const int32_t* sl, int32_t 
   const kvprm::AttnWorkHost& w = ctx->work_host;
   int32_t* S = ctx->staging;
   constexpr size_t kSegInts = sizeof(kvprm::AttnSeg) / sizeof(int32_t);
+  if (++ctx->call == 0) ++ctx->call;   // x_ready's marks start at 0
+  const struct {
+    float* rewards;
+    int32_t call, pad;
+  } out{rewards_out, ctx->call, 0};
   std::memcpy(S, sl, sizeof(int32_t) * n);
   std::memcpy(S + Bmax, bt, sizeof(int32_t) * static_cast<size_t>(n) * mb);
   struct Part {
@@ -460,7 +468,7 @@ int upload_tables(kvprm_ctx* ctx, const int32_t* bt, const int32_t* sl, int32_t 
       {ctx->off_base, w.slot_base.data(), w.slot_base.size()},
       {ctx->off_nslots, w.nslots.data(), w.nslots.size()},
       {ctx->off_tc_cta, w.tc_cta.data(), w.tc_cta.size()},
-      {ctx->off_out, &rewards_out, sizeof(rewards_out) / sizeof(int32_t)},
+      {ctx->off_out, &out, sizeof(out) / sizeof(int32_t)},
   };
   // every part starts at a multiple of eight ints, so a part rounded up to whole quads ends before the next
   kvprm::TableParts tp;
@@ -724,6 +732,8 @@ int enqueue_forward(kvprm_ctx* ctx, const CallPlan& P, Enq& E, const FwdSaves* s
   auto adapter = [&](int j, int l, const GemmPlan& g, const CUtensorMap* xh, const CUtensorMap* xl, int k_main,
                      kvprm::GemmLowRank* lr) -> int {
     static const char* what[4] = {"adapter_qkv", "adapter_o", "adapter_gate_up", "adapter_down"};
+    et.x_ready = lr->x_ready = ctx->x_ready + 4 * l + j;
+    et.call = lr->call = ctx->tables_d + ctx->off_out + 2;
     LAUNCH(KVPRM_PROF_LORA, kvprm::launch_gemm(g, &ctx->tm_la[j][l], xh, xl, et, np, ctx->err_d, st, pdl, TS), what[j]);
     lr->b = &ctx->tm_lb[j][l];
     lr->t_hi = &ctx->tm_thi;
@@ -1512,7 +1522,7 @@ int kvprm_create(const kvprm_config* cfg, const kvprm_weights* w, kvprm_ctx** ou
     ctx->off_nslots = al8(ctx->off_base + bkv);
     ctx->off_tc_cta = al8(ctx->off_nslots + bkv);
     ctx->off_out = al8(ctx->off_tc_cta + ctx->num_sms + 1);
-    ctx->tables_ints = al8(ctx->off_out + 2);
+    ctx->tables_ints = al8(ctx->off_out + 4);
   }
   CREATE_CK(dalloc(ctx, &ctx->tables_d, ctx->tables_ints, "tables and attention work"));
   CREATE_CK(dalloc(ctx, &ctx->rewards_d, static_cast<size_t>(Bmax), "rewards"));
@@ -1610,6 +1620,7 @@ int kvprm_set_lora(kvprm_ctx* ctx, int32_t rank, float scale, const kvprm_lora* 
         return rc;
     }
   }
+  if (!ctx->x_ready && (rc = dalloc(ctx, &ctx->x_ready, 4 * static_cast<size_t>(NL), "adapter marks"))) return rc;
   const size_t need = static_cast<size_t>(ctx->npad_max) * rank;
   if (need > ctx->t_cap) {
     bf16 *th = nullptr, *tl = nullptr;

@@ -126,6 +126,28 @@ __device__ __forceinline__ bool flag_wait(const int* flag, int* err, unsigned lo
   }
 }
 
+// A mark that one grid leaves for a later one of the same stream, which may start while the first still runs: the
+// release orders everything the marking thread may rely on (the writes of grids it has waited for among them)
+// before the mark.
+__device__ __forceinline__ void mark_release(int* mark, int value) {
+  asm volatile("st.release.gpu.global.b32 [%0], %1;" ::"l"(mark), "r"(value) : "memory");
+}
+// Until *mark is `value`; then what was written before the mark may be read, by plain accesses and by bulk copies.
+// Bounded like every wait: after the limit the error word is set and the caller goes on, with whatever it reads.
+__device__ __forceinline__ int mark_read(const int* mark) {
+  int v;
+  asm volatile("ld.acquire.gpu.global.b32 %0, [%1];" : "=r"(v) : "l"(mark) : "memory");
+  return v;
+}
+__device__ __forceinline__ void mark_acquire(const int* mark, int value, int* err) {
+  if (mark_read(mark) != value) {
+    const uint64_t t0 = global_timer_ns();
+    while (mark_read(mark) != value && *(volatile int*)err == 0)
+      if (global_timer_ns() - t0 > kWaitTimeoutNs) atomicCAS(err, 0, kDevTimeout);
+  }
+  asm volatile("fence.proxy.async.global;" ::: "memory");
+}
+
 // ---------------------------------------------------------------- TMA
 // One-dimensional bulk copy global -> this CTA's shared memory, completing `bytes` on `bar`
 // (src and dst 16-byte aligned, bytes a multiple of 16).

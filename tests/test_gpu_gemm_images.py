@@ -3,7 +3,8 @@ candidates (the padded columns step by 16), a gate/up that only fits one wave wi
 projection whose K loop gets twice the CTAs, the adapter's A x on either image, and an adapter with more K
 tiles than the weights.  One kernel alone
 against an fp64 product (fp32 accumulation over K = 18,944: below 1e-5 of the largest output), and whole
-layers against the oracle with the scoring tolerances."""
+layers against the oracle with the scoring tolerances.  And an adapter's launches beside one another against the
+same launches one after the other."""
 import dataclasses
 
 import numpy as np
@@ -47,4 +48,31 @@ def test_layers(n, rank):
     t = ks.Tables.make(0.2)
     r, attn, _, sc = run_gpu(w, t)
     compare(w, t, gpu_rewards=r, gpu_attn=attn, label=f"n {n} rank {rank}")
+    sc.close()
+
+
+@pytest.mark.parametrize("arch, n", [(ks.Arch(3, 1536, 12, 2, 128, 8960), 16), (ks.Arch(3, 1536, 12, 2, 128, 8960), 48),
+                                     (ks.Arch(2, 256, 4, 2, 64, 704), 201)])
+@pytest.mark.parametrize("rank", [64, 256])
+def test_adapter_beside_the_weights(monkeypatch, arch, n, rank):
+    """A projection with an adapter starts while its A x still runs and reads x after the mark that A x leaves: calls
+    of two different batches in turn, queued behind one another, against launches that wait for their predecessor's
+    end.  The same kernels in the same order of sums, so bit for bit."""
+    torch = require_gpu()
+    w = ks.distinct("beside", dataclasses.replace(arch, lora_rank=rank), 950 + n, [(7 * b) % 90 for b in range(n)],
+                    gain_std=0.2)
+    dev = ks.DeviceInputs(w, ks.Tables.make(0.2))
+    bt, sl = np.asarray(w.block_table), np.asarray(w.seq_lens)
+    batches = [(bt, sl), (np.ascontiguousarray(np.roll(bt, 1, 0)), np.ascontiguousarray(np.roll(sl, 1)))]
+    sc = make_scorer(dev, n, w.max_blocks)
+    out = torch.zeros((40, n), dtype=torch.float32, device="cuda")
+    for i in range(40):
+        sc.score_async(dev.pool, *batches[i % 2], out[i])
+    torch.cuda.synchronize()
+    sc.close()
+    monkeypatch.setenv("KVPRM_NO_PDL", "1")
+    sc = make_scorer(dev, n, w.max_blocks)
+    for k, b in enumerate(batches):
+        want = torch.from_numpy(sc.score(dev.pool, *b))
+        assert all(torch.equal(o, want) for o in out[k::2].cpu())
     sc.close()
