@@ -405,7 +405,8 @@ KVPRM_API int kvprm_plan_attention(const int32_t* block_table, int32_t max_block
  * device call), so that its invariants can be checked without a GPU.  gate_up: W holds the gate rows
  * then the up rows (M = d_ff pairs, 64 of each per tile).
  *  m_tiles       128-row tiles (gate/up: 64-pair tiles)
- *  k_tiles       64-wide K tiles; kt_per_split = ceil(k_tiles / cluster)
+ *  k_tiles       64-wide K tiles; kt_per_split = ceil(k_tiles / cluster): a CTA's K tiles where CTAs
+ *                are not paired (see kt_per_rank)
  *  cluster       CTAs that share tiles_per_cta m-tiles: split-K ranks of one cluster; at larger
  *                batches CTA pairs, which divide two m-tiles (tiles_per_cta 2) or the columns (1)
  *                between them and K over cluster / 2 ranks.  gate/up with tiles_per_cta 2: no split
@@ -414,11 +415,17 @@ KVPRM_API int kvprm_plan_attention(const int32_t* block_table, int32_t max_block
  *  stages        shared-memory ring stages; tmem_cols tensor-memory columns; smem_bytes per CTA
  *  threads       threads per CTA: 256 for n_pad >= 64, else 128 (the large-batch kernel image starts
  *                at 48 columns)
+ *  pair          1: CTAs are paired, two of neighbouring cluster ranks to an MMA
+ *  k_ranks       K splits that are reduced over the cluster; each streams kt_per_rank K tiles (the last
+ *                ones fewer, or none)
+ *  col_parts     2: the columns go in halves to clusters of their own, else 1; each rank writes
+ *                n_pad / col_parts / k_ranks columns
  * Errors: KVPRM_EINVAL (M, K or num_sms < 1, n_pad not a positive multiple of 16, out NULL). */
 typedef struct {
   int32_t m_tiles, k_tiles, kt_per_split, cluster, tiles_per_cta, stages, tmem_cols;
   int64_t smem_bytes;
   int32_t threads;
+  int32_t pair, k_ranks, kt_per_rank, col_parts;
 } kvprm_projection_plan;
 KVPRM_API int kvprm_plan_projection(int32_t M, int32_t K, int32_t n_pad, int32_t num_sms, int32_t has_lo,
                                     int32_t gate_up, kvprm_projection_plan* out);

@@ -59,6 +59,9 @@ constexpr int kHPreCols = 8;                        // residual columns preloade
 constexpr size_t kGemmMaxSmem = 200 * 1024;         // dynamic shared memory the kernel is configured for
 constexpr size_t kAloneSmem = 120 * 1024;           // with which no second CTA fits on an SM
 
+// The parked accumulator of a CTA with `cols` columns: 16 of them at a time, 128 fp32 rows each.
+__host__ __device__ constexpr uint32_t park_bytes(int cols) { return static_cast<uint32_t>((cols + 15) / 16 * 16) * kBM * 4; }
+
 __device__ __forceinline__ uint8_t* align1024(uint8_t* p) {
   return reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(p) + 1023) & ~static_cast<uintptr_t>(1023));
 }
@@ -106,7 +109,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   const uint32_t w_bytes = kWTileBytes * static_cast<uint32_t>(mt);
   // PAIR: half of the pair's activation rows, i.e. one part's n_pad rows or half of each part's
   const uint32_t stage_bytes = w_bytes + x_bytes * (has_lo && !PAIR ? 2u : 1u);
-  const uint32_t acc_bytes = static_cast<uint32_t>(n_pad) * kBM * 4;
+  const uint32_t acc_bytes = park_bytes(n_pad);
   const uint32_t ring_bytes = stages * stage_bytes > acc_bytes ? stages * stage_bytes : acc_bytes;
   uint64_t* full = reinterpret_cast<uint64_t*>(smem + ring_bytes);
   uint64_t* empty = full + stages;
@@ -986,7 +989,7 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
   p.stages = stages < 2 ? 2 : (stages > 8 ? 8 : stages);
   // the parked accumulator (n_pad x 128 fp32) reuses the ring
   size_t ring = static_cast<size_t>(p.stages) * stage_bytes;
-  const size_t acc = static_cast<size_t>(n_pad) * kBM * 4;
+  const size_t acc = park_bytes(n_pad);
   if (ring < acc) ring = acc;
   p.smem_bytes = ring + 1024 /*align*/ + kTailBytes;
   // cluster size: the largest power of two <= 16 that keeps the CTA count within what fits on the
@@ -1030,12 +1033,11 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
       cs = cs2;
     }
   }
-  p.cluster = cs;
-  p.splits = cs;
-  p.kt_per_split = (p.k_tiles + cs - 1) / cs;
+  p.cluster = p.ranks = cs;
+  p.kt_per_rank = (p.k_tiles + cs - 1) / cs;
   // a ring deeper than the K tiles one CTA streams only holds shared memory
   // that overlapping kernels could use
-  if (p.stages > p.kt_per_split) p.stages = p.kt_per_split < 2 ? 2 : p.kt_per_split;
+  if (p.stages > p.kt_per_rank) p.stages = p.kt_per_rank < 2 ? 2 : p.kt_per_rank;
   ring = static_cast<size_t>(p.stages) * stage_bytes;
   if (ring < acc) ring = acc;
   p.smem_bytes = ring + 1024 /*align*/ + kTailBytes;
@@ -1056,22 +1058,25 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
     p.pair = true;
     p.mt = 2;
     p.stages = stages2;
-    p.smem_bytes = static_cast<size_t>(stages2) * st2 + 1024 + kTailBytes;
+    ring = static_cast<size_t>(stages2) * st2;
+    p.smem_bytes = (ring < acc ? acc : ring) + 1024 + kTailBytes;
     p.tmem_cols = 2 * cols;
   }
   const int pc = cluster_of(1);
   auto take_pairs = [&](int ranks, int n_split) {
     const int cols2 = n_pad / n_split;
     const uint32_t st2 = kWTileBytes + static_cast<uint32_t>(cols2) * kBK * 2;
-    const size_t acc2 = static_cast<size_t>((cols2 + 15) / 16 * 16) * kBM * 4;
+    const size_t acc2 = park_bytes(cols2);
     const int kps = (p.k_tiles + ranks - 1) / ranks;
     int stages2 = static_cast<int>((192u * 1024u) / st2);
     if (stages2 > 8) stages2 = 8;
     if (stages2 > kps) stages2 = kps < 2 ? 2 : kps;
     p.pair = true;
     p.mt = 3 - n_split;
-    p.cluster = p.splits = 2 * ranks;
-    p.kt_per_split = (p.k_tiles + 2 * ranks - 1) / (2 * ranks);
+    p.cluster = 2 * ranks;
+    p.ranks = ranks;
+    p.kt_per_rank = kps;
+    p.col_parts = n_split;
     p.stages = stages2;
     ring = static_cast<size_t>(stages2) * st2;
     p.smem_bytes = (ring < acc2 ? acc2 : ring) + 1024 + kTailBytes;
@@ -1179,12 +1184,11 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
     e.x_ready = lr->x_ready;
     e.call = lr->call;
   }
-  const int n_split = p.pair && p.mt == 1 ? 2 : 1;
   const GemmKernel kern = gemm_image(p.pair ? kPair : (large ? kLarge : kSmall), ep.mode);
   if (!kern || (p.pair && (!large || !p.has_lo || p.gate_up != (ep.mode == GemmEpilogue::SILU))))
     return cudaErrorInvalidValue;
   return cudaLaunchKernelEx(&cfg, kern, *tmW, *tmX, xlo, p.has_lo ? 1 : 0, mb, mt, mtl, k_main, p.k_tiles,
-                            p.pair ? cluster / 2 : cluster, p.stages, p.tmem_cols, n_pad / n_split, n_split, e, err, ts);
+                            p.ranks, p.stages, p.tmem_cols, n_pad / p.col_parts, p.col_parts, e, err, ts);
 }
 
 }  // namespace kvprm

@@ -21,12 +21,14 @@ constexpr int kTraceStride = 2 + kTraceEvents;
 struct GemmPlan {
   bool has_lo = true;    // activation given as a bf16 (hi, lo) pair
   bool gate_up = false;  // tiles of 64 gate rows + the matching 64 up rows
-  int m_tiles = 0, k_tiles = 0, kt_per_split = 0, splits = 0, stages = 0, cluster = 1;
-  // m-tiles that one activation tile serves, over `cluster` CTAs: 2 with `pair`, else 1
+  int m_tiles = 0, k_tiles = 0, stages = 0, cluster = 1;
+  int ranks = 1, kt_per_rank = 0;   // K splits: rank r streams K tiles [r kt_per_rank, (r + 1) kt_per_rank)
+  int col_parts = 1;                // parts of the batch's columns, a cluster each
+  // m-tiles that one activation tile serves, over `cluster` CTAs: 2 with `pair` and all columns, else 1
   int mt = 1;
   // CTA pairs.  gate/up: two neighbouring CTAs with 128 gate and the matching 128 up rows each (a launch
-  // cluster of two, cluster = 1 K split).  Otherwise a tile each over cluster / 2 K splits; or, with
-  // mt = 1, of half of the columns.
+  // cluster of two, cluster = 1 K split).  Otherwise a tile each over cluster / 2 K splits, of all columns
+  // or (col_parts 2) of half of them.
   bool pair = false;
   // threads per CTA: 256 from 64 padded columns, else 128
   int threads = 128;

@@ -1910,13 +1910,17 @@ int kvprm_plan_projection(int32_t M, int32_t K, int32_t n_pad, int32_t num_sms, 
   const GemmPlan g = kvprm::plan_gemm(M, K, n_pad, num_sms, has_lo != 0, gate_up != 0);
   out->m_tiles = g.m_tiles;
   out->k_tiles = g.k_tiles;
-  out->kt_per_split = g.kt_per_split;
+  out->kt_per_split = (g.k_tiles + g.cluster - 1) / g.cluster;
   out->cluster = g.cluster;
   out->tiles_per_cta = g.mt;
   out->stages = g.stages;
   out->tmem_cols = static_cast<int32_t>(g.tmem_cols);
   out->smem_bytes = static_cast<int64_t>(g.smem_bytes);
   out->threads = g.threads;
+  out->pair = g.pair ? 1 : 0;
+  out->k_ranks = g.ranks;
+  out->kt_per_rank = g.kt_per_rank;
+  out->col_parts = g.col_parts;
   return KVPRM_OK;
 }
 

@@ -42,7 +42,8 @@ def test_projection_plan_invariants(arch, n_pad, rank):
 
 
 def test_projection_plan_large_batch_choices():
-    """The plans the 7B scorer at 256 candidates runs: gate/up and down take two m-tiles per CTA."""
+    """The plans the 7B scorer at 256 candidates runs, all on CTA pairs: gate/up with two tiles a CTA, down with
+    one over four K ranks, QKV with half of the columns over two."""
     a = ks.ARCH_7B
     gu = kp.kvprm_plan_projection(a.d_ff, a.d_model, 256, SMS, True, True)
     down = kp.kvprm_plan_projection(a.d_model, a.d_ff, 256, SMS, True, False)
@@ -51,6 +52,40 @@ def test_projection_plan_large_batch_choices():
     assert (down["tiles_per_cta"], down["cluster"]) == (2, 8)
     assert (qkv["tiles_per_cta"], qkv["cluster"]) == (1, 4)
     assert gu["threads"] == down["threads"] == qkv["threads"] == 256
+
+
+@pytest.mark.parametrize("has_lo", [True, False])
+def test_what_the_kernel_relies_on(has_lo):
+    """For every padded batch and K from one tile to the longest (and tile counts that leave ranks short of K
+    tiles): the K ranks cover K, their columns divide among them, a stage's tiles and the parked accumulator (16
+    columns at a time) fit ahead of the barriers, and the accumulators fit the tensor memory.  A CTA streams what
+    the plan says: 74 K tiles each for the 7B down projection at 256 columns."""
+    shapes = [(M, K, gu) for a in (ks.ARCH_1P5B, ks.ARCH_7B, ks.ARCH_8B) for _, M, K, gu in _shapes(a)]
+    shapes += [(M, 64 * k, gu) for M in (128, 256, 512, 2048, 3584, 4608, 6144) for k in (1, 2, 3, 4, 5, 8, 9, 11, 16, 33, 50)
+               for gu in (False, True)]
+    shapes += [(9984, 64 * k, True) for k in (1, 2, 3, 7)]
+    for M, K, gu in shapes:
+        for n_pad in range(16, 257, 16):
+            p = kp.kvprm_plan_projection(M, K, n_pad, SMS, has_lo, gu)
+            tag = f"M={M} K={K} n_pad={n_pad} gate_up={gu}: {p}"
+            cols, ranks = n_pad // p["col_parts"], p["k_ranks"]
+            assert n_pad % p["col_parts"] == 0 and cols % ranks == 0 and cols % 8 == 0, tag
+            assert p["kt_per_rank"] == -(-p["k_tiles"] // ranks), tag
+            split_ctas = 2 if p["pair"] and not gu else 1   # of one rank
+            assert p["cluster"] == split_ctas * ranks, tag
+            assert p["tiles_per_cta"] == (2 if p["pair"] and p["col_parts"] == 1 else 1), tag
+            assert not p["pair"] or (has_lo and n_pad >= 48 and p["m_tiles"] % 2 == 0), tag
+            stage = 16384 * (2 if p["pair"] and gu else 1) + cols * 128 * (2 if has_lo and not p["pair"] else 1)
+            ring = max(p["stages"] * stage, -(-cols // 16) * 16 * 512)
+            assert p["smem_bytes"] >= ring + 1024 + 512 + 1024 + 4096 and p["smem_bytes"] <= MAX_SMEM, tag
+            assert 2 <= p["stages"] <= max(2, p["kt_per_rank"]), tag
+            parts = 2 if has_lo and 2 * cols <= 256 else 1   # hi and lo beside each other, else one after the other
+            assert p["tmem_cols"] // (2 if p["pair"] else 1) >= parts * cols, tag
+    a = ks.ARCH_7B
+    down = kp.kvprm_plan_projection(a.d_model, a.d_ff, 256, SMS, True, False)
+    assert (down["pair"], down["k_ranks"], down["kt_per_rank"], down["col_parts"]) == (1, 4, 74, 1)
+    qkv = kp.kvprm_plan_projection(a.qkv_rows, a.d_model, 256, SMS, True, False)
+    assert (qkv["pair"], qkv["k_ranks"], qkv["kt_per_rank"], qkv["col_parts"]) == (1, 2, 28, 2)
 
 
 def test_projection_plan_errors():
