@@ -88,7 +88,10 @@ __device__ __forceinline__ void store_hilo(__nv_bfloat16* hi, __nv_bfloat16* lo,
 // with a B operand that is half in either CTA, so a CTA stages half of the activation rows.  At 256
 // columns a stage is 48 KB instead of 80, four fit instead of two, and a K tile's L2 reads fall from 80 KB
 // to 48: with two stages an m-tile's eight MMAs (0.53 us) waited for loads 0.35 us of every K tile.
-template <bool LARGE, int MODE, bool PAIR>
+// LORA: the projection takes a scorer adapter's K tiles after its own (QKV, RESID, SILU).  Images of their own: in
+// shared ones the loader's choices and the mark's acquire cost both kinds of call (1.5B, 16 candidates, rank 256:
+// 1,518 us a call, apart 1,511; beam without an adapter 3,428, apart 3,418).
+template <bool LARGE, int MODE, bool PAIR, bool LORA>
 __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_constant__ CUtensorMap tmW,
                                                            const __grid_constant__ CUtensorMap tmX,
                                                            const __grid_constant__ CUtensorMap tmXlo, int has_lo,
@@ -152,7 +155,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     tma_prefetch_desc(&tmW);
     tma_prefetch_desc(&tmX);
     if (has_lo) tma_prefetch_desc(&tmXlo);
-    if (k_main < k_tiles) {
+    if constexpr (LORA) {
       tma_prefetch_desc(&tmB);
       tma_prefetch_desc(&tmT);
       if (has_lo) tma_prefetch_desc(&tmTlo);
@@ -196,8 +199,9 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
         mbar_arrive_expect_tx(&full[stage], stage_bytes);
       else if (side == 0)
         mbar_arrive_expect_tx(&full[stage], 2 * stage_bytes);
-      const CUtensorMap* wm = kt < k_main ? &tmW : &tmB;
-      const int kx = (kt < k_main ? kt : kt - k_main) * kBK;
+      const bool main = !LORA || kt < k_main;
+      const CUtensorMap* wm = main ? &tmW : &tmB;
+      const int kx = (main ? kt : kt - k_main) * kBK;
       uint8_t* wt = smem + stage * stage_bytes;
       if constexpr (!silu) {
         load(wt, wm, stage, kx, m_tile * kBM, pol_w);
@@ -211,7 +215,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     // the activation maps' boxes hold the batch's columns, from 96 on half of them (gemm_x_box): a stage's
     // rows are then loaded as halves (hi, hi, lo, lo), of which a pair's CTA takes its own
     auto load_x = [&](int stage, int kt) {
-      const bool main = kt < k_main;
+      const bool main = !LORA || kt < k_main;
       const int kx = (main ? kt : kt - k_main) * kBK;
       const CUtensorMap *xh = main ? &tmX : &tmT, *xl = main ? &tmXlo : &tmTlo;
       uint8_t* xt = smem + stage * stage_bytes + w_bytes;
@@ -242,16 +246,16 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
     // A x (1.5B, 16 candidates: rank 256 1,582 -> 1,550 us a call, rank 64 414 -> 391 for eight layers; 48
     // candidates at rank 256 577 -> 542; ranks 512 and 1,024 -3 to +1 %).  Starting it from A x's last
     // landed tile instead: 1,607.  That A x has waited does not by itself order x before the reads here, so
-    // one of its threads leaves a mark after its wait (0.1 us a launch: 1,509 -> 1,521; 8B, 4 candidates,
-    // rank 64, four layers 375 -> 379; 1,563 and 395 with x behind A x's end).
-    bool waited = k_main == k_tiles;
-    if (waited)
-      grid_dep_wait();
-    else
+    // one of its threads leaves a mark after its wait (1,506 -> 1,511; 8B, 4 candidates, rank 64,
+    // four layers 375 -> 378; with x behind A x's end 1,563 and 395).
+    bool waited = !LORA;
+    if constexpr (LORA)
       mark_acquire(ep.x_ready, *ep.call, err);
+    else
+      grid_dep_wait();
     trace_event(ts, 0);   // the preceding kernel has completed (with an adapter: the one before A x)
     auto load_act = [&](int stage, int kt) {
-      if (!waited && kt >= k_main) {
+      if (LORA && !waited && kt >= k_main) {
         grid_dep_wait();
         waited = true;
       }
@@ -1104,33 +1108,34 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
 
 namespace {
 
-typedef decltype(&gemm_cluster_kernel<false, GemmEpilogue::PLAIN, false>) GemmKernel;
+typedef decltype(&gemm_cluster_kernel<false, GemmEpilogue::PLAIN, false, false>) GemmKernel;
 
 enum GemmImage { kSmall, kLarge, kPair, kGemmImages };
 
-template <int MODE>
+template <int MODE, bool LORA = false>
 GemmKernel image_of(GemmImage i) {
-  if (i == kPair) return gemm_cluster_kernel<true, MODE, true>;
-  return i == kLarge ? gemm_cluster_kernel<true, MODE, false> : gemm_cluster_kernel<false, MODE, false>;
+  if (i == kPair) return gemm_cluster_kernel<true, MODE, true, LORA>;
+  return i == kLarge ? gemm_cluster_kernel<true, MODE, false, LORA> : gemm_cluster_kernel<false, MODE, false, LORA>;
 }
-// The kernel image of a batch class and epilogue (null: none).
-GemmKernel gemm_image(GemmImage i, int mode) {
+// The kernel image of a batch class and epilogue, with an adapter's K tiles or without (null: none).
+GemmKernel gemm_image(GemmImage i, int mode, bool lora) {
   switch (mode) {
-    case GemmEpilogue::PLAIN: return image_of<GemmEpilogue::PLAIN>(i);
-    case GemmEpilogue::QKV: return image_of<GemmEpilogue::QKV>(i);
-    case GemmEpilogue::RESID: return image_of<GemmEpilogue::RESID>(i);
-    case GemmEpilogue::SILU: return image_of<GemmEpilogue::SILU>(i);
-    case GemmEpilogue::LOWRANK: return image_of<GemmEpilogue::LOWRANK>(i);
+    case GemmEpilogue::PLAIN: return lora ? nullptr : image_of<GemmEpilogue::PLAIN>(i);
+    case GemmEpilogue::QKV: return lora ? image_of<GemmEpilogue::QKV, true>(i) : image_of<GemmEpilogue::QKV>(i);
+    case GemmEpilogue::RESID: return lora ? image_of<GemmEpilogue::RESID, true>(i) : image_of<GemmEpilogue::RESID>(i);
+    case GemmEpilogue::SILU: return lora ? image_of<GemmEpilogue::SILU, true>(i) : image_of<GemmEpilogue::SILU>(i);
+    case GemmEpilogue::LOWRANK: return lora ? nullptr : image_of<GemmEpilogue::LOWRANK>(i);
   }
   return nullptr;
 }
 
 }  // namespace
 
-cudaError_t gemm_configure(int n_pad_max) {
+cudaError_t gemm_configure(int n_pad_max, bool lora) {
   for (int i = 0; i < (n_pad_max >= kLargeCols ? kGemmImages : kLarge); ++i)
     for (int mode = GemmEpilogue::PLAIN; mode <= GemmEpilogue::LOWRANK; ++mode) {
-      const GemmKernel k = gemm_image(static_cast<GemmImage>(i), mode);
+      const bool ax = mode == GemmEpilogue::LOWRANK;   // an adapter's other launch
+      const GemmKernel k = ax && !lora ? nullptr : gemm_image(static_cast<GemmImage>(i), mode, lora && !ax);
       if (!k) continue;
       cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, static_cast<int>(kGemmMaxSmem));
       if (e == cudaSuccess && i != kPair) e = cudaFuncSetAttribute(k, cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
@@ -1184,7 +1189,7 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
     e.x_ready = lr->x_ready;
     e.call = lr->call;
   }
-  const GemmKernel kern = gemm_image(p.pair ? kPair : (large ? kLarge : kSmall), ep.mode);
+  const GemmKernel kern = gemm_image(p.pair ? kPair : (large ? kLarge : kSmall), ep.mode, with_lr);
   if (!kern || (p.pair && (!large || !p.has_lo || p.gate_up != (ep.mode == GemmEpilogue::SILU))))
     return cudaErrorInvalidValue;
   return cudaLaunchKernelEx(&cfg, kern, *tmW, *tmX, xlo, p.has_lo ? 1 : 0, mb, mt, mtl, k_main, p.k_tiles,

@@ -103,8 +103,9 @@ struct GemmLowRank {
   int* x_ready = nullptr;              // of the A x launch, and the call's number (GemmEpilogue)
   const int* call = nullptr;
 };
-// Attributes of the kernel images that batches of up to n_pad_max padded columns take.
-cudaError_t gemm_configure(int n_pad_max);
+// Attributes of the kernel images that batches of up to n_pad_max padded columns take: those of calls without an
+// adapter, or with lora set an adapter's.
+cudaError_t gemm_configure(int n_pad_max, bool lora);
 cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtensorMap* tmX, const CUtensorMap* tmXlo,
                         const GemmEpilogue& ep, int n_pad, int* err, cudaStream_t stream, bool pdl,
                         unsigned long long* ts = nullptr, const GemmLowRank* lr = nullptr);

@@ -1423,7 +1423,7 @@ int kvprm_create(const kvprm_config* cfg, const kvprm_weights* w, kvprm_ctx** ou
     }
     ctx->encode = reinterpret_cast<PFN_cuTensorMapEncodeTiled_v12000>(fn);
   }
-  CREATE_CK(cu(kvprm::gemm_configure((ctx->cfg.max_candidates + 15) / 16 * 16), "gemm_configure"));
+  CREATE_CK(cu(kvprm::gemm_configure((ctx->cfg.max_candidates + 15) / 16 * 16, false), "gemm_configure"));
   CREATE_CK(cu(kvprm::attention_configure(), "attention_configure"));
   CREATE_CK(cu(kvprm::grad_configure(), "grad_configure"));
 
@@ -1620,6 +1620,7 @@ int kvprm_set_lora(kvprm_ctx* ctx, int32_t rank, float scale, const kvprm_lora* 
         return rc;
     }
   }
+  CK(kvprm::gemm_configure((ctx->cfg.max_candidates + 15) / 16 * 16, true), "gemm_configure(adapter)");
   if (!ctx->x_ready && (rc = dalloc(ctx, &ctx->x_ready, 4 * static_cast<size_t>(NL), "adapter marks"))) return rc;
   const size_t need = static_cast<size_t>(ctx->npad_max) * rank;
   if (need > ctx->t_cap) {
