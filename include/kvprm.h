@@ -412,7 +412,8 @@ KVPRM_API int kvprm_plan_attention(const int32_t* block_table, int32_t max_block
  *                between them and K over cluster / 2 ranks.  gate/up with tiles_per_cta 2: no split
  *                K, two such CTAs a pair
  *  tiles_per_cta m-tiles that one activation tile serves (1 or 2)
- *  stages        shared-memory ring stages; tmem_cols tensor-memory columns; smem_bytes per CTA
+ *  stages        shared-memory ring stages; tmem_cols tensor-memory columns; smem_bytes per CTA, as
+ *                launched (a pair's CTAs take all that a CTA may, 200 KB)
  *  threads       threads per CTA: 256 for n_pad >= 64, else 128 (the large-batch kernel image starts
  *                at 48 columns)
  *  pair          1: CTAs are paired, two of neighbouring cluster ranks to an MMA
@@ -429,6 +430,13 @@ typedef struct {
 } kvprm_projection_plan;
 KVPRM_API int kvprm_plan_projection(int32_t M, int32_t K, int32_t n_pad, int32_t num_sms, int32_t has_lo,
                                     int32_t gate_up, kvprm_projection_plan* out);
+/* The clusters of that launch for n candidates on ctx's device (hi/lo input), and how many of them the device
+ * holds at once at one CTA per SM (cudaOccupancyMaxActiveClusters for the kernel with the launch's shared memory
+ * and cluster size, which counts one CTA per SM for any kernel that allocates tensor memory; two that fit do run
+ * beside each other).  Nothing runs.
+ * Errors: KVPRM_EINVAL, KVPRM_ECAPACITY (n outside [1, max_candidates]), KVPRM_ECUDA. */
+KVPRM_API int kvprm_debug_projection_placement(kvprm_ctx* ctx, int32_t M, int32_t K, int32_t n, int32_t gate_up,
+                                               int32_t* clusters, int32_t* placed);
 
 /* Device-side status: returns KVPRM_OK, or KVPRM_ETIMEOUT if an in-kernel
  * bounded wait gave up since the last check (the flag is then cleared).

@@ -1049,6 +1049,10 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
   const int need = (has_lo && 2 * n_pad <= 256) ? 2 * n_pad : n_pad;   // merged hi/lo accumulator halves
   while (cols < static_cast<uint32_t>(need)) cols <<= 1;
   p.tmem_cols = cols;
+  // A pair's CTA takes all shared memory it may (its ring and the parked accumulator are well below): its tensor
+  // memory (up to 512 columns) is allocated in two SMs at once, and beside a cluster of another stream's launch
+  // either could hold the columns the other's second CTA waits for.  What is left (26 KB) is too little for any
+  // other launch that allocates tensor memory.
   // gate/up without split K, more tiles than SMs: pairs of CTAs with two tiles each.  The 7B gate/up, 296
   // tiles: one-tile CTAs two to an SM took 51.6 us at 96 columns and 56.5 at 144, two tiles a CTA without
   // pairs 47.5 at 80, 66.5 at 160 and 80.0 at 256; pairs take 44.1, 50.1, 44.7, 52.9 and 75.4 (the weights'
@@ -1062,15 +1066,13 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
     p.pair = true;
     p.mt = 2;
     p.stages = stages2;
-    ring = static_cast<size_t>(stages2) * st2;
-    p.smem_bytes = (ring < acc ? acc : ring) + 1024 + kTailBytes;
+    p.smem_bytes = kGemmMaxSmem;
     p.tmem_cols = 2 * cols;
   }
   const int pc = cluster_of(1);
   auto take_pairs = [&](int ranks, int n_split) {
     const int cols2 = n_pad / n_split;
     const uint32_t st2 = kWTileBytes + static_cast<uint32_t>(cols2) * kBK * 2;
-    const size_t acc2 = park_bytes(cols2);
     const int kps = (p.k_tiles + ranks - 1) / ranks;
     int stages2 = static_cast<int>((192u * 1024u) / st2);
     if (stages2 > 8) stages2 = 8;
@@ -1082,8 +1084,7 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
     p.kt_per_rank = kps;
     p.col_parts = n_split;
     p.stages = stages2;
-    ring = static_cast<size_t>(stages2) * st2;
-    p.smem_bytes = (ring < acc2 ? acc2 : ring) + 1024 + kTailBytes;
+    p.smem_bytes = kGemmMaxSmem;
     p.tmem_cols = 2 * cols;
   };
   // CTA pairs (see the kernel).  The CTAs that one m-tile each over pc ranks would take, as clusters of
@@ -1103,6 +1104,16 @@ GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_
   // the large-batch image runs eight warps instead of four (registers for two such CTAs per SM), so
   // that the parking, the cluster reduction and the epilogue after the MMAs run on twice the warps
   p.threads = n_pad >= 64 ? 256 : 128;
+  return p;
+}
+
+// An adapter's A x keeps its few SMs (16 to 64 CTAs) to itself, over half of an SM's shared memory a CTA:
+// beside CTAs of the projection that it lets start, its K loop and its parking took twice as long (gate/up's
+// A x 8.8 us, 3.9 alone).  Eight 1.5B layers at rank 64 392 -> 370 us, rank 512 433 -> 411; four 7B layers,
+// 16 candidates, rank 256 452 -> 431; rank 256 over 28 1.5B layers the same (1,550).
+GemmPlan plan_lowrank(int rank, int K, int n_pad, int num_sms) {
+  GemmPlan p = plan_gemm(rank, K, n_pad, num_sms, true, false);
+  if (p.smem_bytes < kAloneSmem) p.smem_bytes = kAloneSmem;
   return p;
 }
 
@@ -1144,42 +1155,58 @@ cudaError_t gemm_configure(int n_pad_max, bool lora) {
   return cudaSuccess;
 }
 
-cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtensorMap* tmX, const CUtensorMap* tmXlo,
-                        const GemmEpilogue& ep, int n_pad, int* err, cudaStream_t stream, bool pdl,
-                        unsigned long long* ts, const GemmLowRank* lr) {
-  cudaLaunchConfig_t cfg = {};
-  const int units = (p.m_tiles + p.mt - 1) / p.mt;   // launched by the cluster, gate/up pairs' by two
-  const int cluster = p.pair && p.gate_up ? 2 : p.cluster;
-  cfg.gridDim = dim3(p.pair && p.gate_up ? (units + 1) / 2 * 2 : units * p.cluster, 1, 1);
+namespace {
+
+// The image and launch configuration of a plan (null: none), but for the stream and its order; attr: two, the first
+// of them set here.
+GemmKernel gemm_config(const GemmPlan& p, int mode, int n_pad, bool lora, cudaLaunchConfig_t& cfg,
+                       cudaLaunchAttribute* attr) {
   // the vector epilogues win from 48 padded columns on even with four warps (40 candidates of a 7B scorer
   // 564 -> 532 us for four layers; 24 candidates, 32 columns: 397 us small, 405 large)
   const bool large = n_pad >= kLargeCols;
-  if (p.threads != 128 && (p.threads != 256 || !large)) return cudaErrorInvalidValue;
+  if (p.threads != 128 && (p.threads != 256 || !large)) return nullptr;
+  if (p.pair && (!large || !p.has_lo || p.gate_up != (mode == GemmEpilogue::SILU))) return nullptr;
+  const int units = (p.m_tiles + p.mt - 1) / p.mt;   // launched by the cluster, gate/up pairs' by two
+  const bool gu_pair = p.pair && p.gate_up;
+  cfg = cudaLaunchConfig_t{};
+  cfg.gridDim = dim3(gu_pair ? (units + 1) / 2 * 2 : units * p.cluster, 1, 1);
   cfg.blockDim = dim3(static_cast<unsigned>(p.threads), 1, 1);
   cfg.dynamicSmemBytes = p.smem_bytes;
-  // An adapter's A x keeps its few SMs (16 to 64 CTAs) to itself, over half of an SM's shared memory a
-  // CTA: beside CTAs of the projection that it lets start, its K loop and its parking took twice as long
-  // (gate/up's A x 8.8 us, 3.9 alone).  Eight 1.5B layers at rank 64 392 -> 370 us, rank 512 433 -> 411;
-  // four 7B layers, 16 candidates, rank 256 452 -> 431; rank 256 over 28 1.5B layers the same (1,550).
-  if (ep.mode == GemmEpilogue::LOWRANK && cfg.dynamicSmemBytes < kAloneSmem) cfg.dynamicSmemBytes = kAloneSmem;
-  // A pair's CTA takes all it may: its tensor memory (up to 512 columns) is allocated in two SMs at once, and
-  // beside a cluster of another stream's launch either could hold the columns the other's second CTA waits
-  // for.  What is left (27 KB) is too little for any other launch that allocates tensor memory.
-  if (p.pair) cfg.dynamicSmemBytes = kGemmMaxSmem;
-  cfg.stream = stream;
-  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
-  attr[0].val.clusterDim.x = cluster;
+  attr[0].val.clusterDim.x = gu_pair ? 2 : p.cluster;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
-  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
-  cfg.numAttrs = pdl ? 2 : 1;
-  const CUtensorMap& xlo = p.has_lo ? *tmXlo : *tmX;
+  cfg.numAttrs = 1;
+  return gemm_image(p.pair ? kPair : (large ? kLarge : kSmall), mode, lora);
+}
+
+}  // namespace
+
+cudaError_t gemm_placement(const GemmPlan& p, int n_pad, int* clusters, int* placed) {
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  const GemmKernel kern = gemm_config(p, p.gate_up ? GemmEpilogue::SILU : GemmEpilogue::RESID, n_pad, false, cfg, attr);
+  if (!kern) return cudaErrorInvalidValue;
+  *clusters = static_cast<int>(cfg.gridDim.x / attr[0].val.clusterDim.x);
+  return cudaOccupancyMaxActiveClusters(placed, kern, &cfg);
+}
+
+cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtensorMap* tmX, const CUtensorMap* tmXlo,
+                        const GemmEpilogue& ep, int n_pad, int* err, cudaStream_t stream, bool pdl,
+                        unsigned long long* ts, const GemmLowRank* lr) {
   // without an adapter every K tile is W's and x's (the extra maps are never read)
   const bool with_lr = lr && lr->b && lr->t_hi && (!p.has_lo || lr->t_lo);
   if (with_lr && (lr->k_main < 1 || lr->k_main >= p.k_tiles)) return cudaErrorInvalidValue;
+  cudaLaunchConfig_t cfg;
+  cudaLaunchAttribute attr[2];
+  const GemmKernel kern = gemm_config(p, ep.mode, n_pad, with_lr, cfg, attr);
+  if (!kern) return cudaErrorInvalidValue;
+  cfg.stream = stream;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
+  cfg.numAttrs = pdl ? 2 : 1;
+  const CUtensorMap& xlo = p.has_lo ? *tmXlo : *tmX;
   const CUtensorMap& mb = with_lr ? *lr->b : *tmW;
   const CUtensorMap& mt = with_lr ? *lr->t_hi : *tmX;
   const CUtensorMap& mtl = with_lr ? (p.has_lo ? *lr->t_lo : *lr->t_hi) : xlo;
@@ -1189,9 +1216,6 @@ cudaError_t launch_gemm(const GemmPlan& p, const CUtensorMap* tmW, const CUtenso
     e.x_ready = lr->x_ready;
     e.call = lr->call;
   }
-  const GemmKernel kern = gemm_image(p.pair ? kPair : (large ? kLarge : kSmall), ep.mode, with_lr);
-  if (!kern || (p.pair && (!large || !p.has_lo || p.gate_up != (ep.mode == GemmEpilogue::SILU))))
-    return cudaErrorInvalidValue;
   return cudaLaunchKernelEx(&cfg, kern, *tmW, *tmX, xlo, p.has_lo ? 1 : 0, mb, mt, mtl, k_main, p.k_tiles,
                             p.ranks, p.stages, p.tmem_cols, n_pad / p.col_parts, p.col_parts, e, err, ts);
 }

@@ -90,6 +90,10 @@ struct GemmEpilogue {
   bool late_trigger = false;
 };
 GemmPlan plan_gemm(int M, int K, int n_pad, int num_sms, bool has_lo, bool gate_up);
+// An adapter's A x (LOWRANK), A [rank][K].
+GemmPlan plan_lowrank(int rank, int K, int n_pad, int num_sms);
+// Clusters of the plan's launch (QKV, RESID or SILU), and how many the current device takes at once.
+cudaError_t gemm_placement(const GemmPlan& p, int n_pad, int* clusters, int* placed);
 // Rows of an activation operand's tensor-map box: n_pad, or from 96 columns half of them.
 uint32_t gemm_x_box(int n_pad);
 // A scorer adapter's term of a projection, y = W x + B t with t = s A x already computed (LOWRANK):

@@ -566,10 +566,10 @@ CallPlan make_plan(kvprm_ctx* ctx, int n, int max_pages) {
   p.g_gu = kvprm::plan_gemm(m.ff, keff(m.d), p.n_pad, ctx->num_sms, true, true);
   p.g_down = kvprm::plan_gemm(m.d, keff(m.ff), p.n_pad, ctx->num_sms, true, false);
   if (r) {
-    p.l_qkv = kvprm::plan_gemm(r, m.d, p.n_pad, ctx->num_sms, true, false);
-    p.l_o = kvprm::plan_gemm(r, m.n_q * m.hd, p.n_pad, ctx->num_sms, true, false);
-    p.l_gu = kvprm::plan_gemm(r, m.d, p.n_pad, ctx->num_sms, true, false);
-    p.l_down = kvprm::plan_gemm(r, m.ff, p.n_pad, ctx->num_sms, true, false);
+    p.l_qkv = kvprm::plan_lowrank(r, m.d, p.n_pad, ctx->num_sms);
+    p.l_o = kvprm::plan_lowrank(r, m.n_q * m.hd, p.n_pad, ctx->num_sms);
+    p.l_gu = kvprm::plan_lowrank(r, m.d, p.n_pad, ctx->num_sms);
+    p.l_down = kvprm::plan_lowrank(r, m.ff, p.n_pad, ctx->num_sms);
     p.k_qkv = kt(m.d);
     p.k_o = kt(m.n_q * m.hd);
     p.k_gu = kt(m.d);
@@ -1922,6 +1922,21 @@ int kvprm_plan_projection(int32_t M, int32_t K, int32_t n_pad, int32_t num_sms, 
   out->k_ranks = g.ranks;
   out->kt_per_rank = g.kt_per_rank;
   out->col_parts = g.col_parts;
+  return KVPRM_OK;
+}
+
+int kvprm_debug_projection_placement(kvprm_ctx* ctx, int32_t M, int32_t K, int32_t n, int32_t gate_up, int32_t* clusters,
+                                     int32_t* placed) {
+  if (!ctx) return KVPRM_EINVAL;
+  if (!clusters || !placed || M < 1 || K < 1) return fail(ctx, KVPRM_EINVAL, "bad projection placement arguments");
+  if (n < 1 || n > ctx->cfg.max_candidates)
+    return fail(ctx, KVPRM_ECAPACITY, "n = %d outside [1, max_candidates = %d]", n, ctx->cfg.max_candidates);
+  const int n_pad = (n + 15) / 16 * 16;
+  const GemmPlan g = kvprm::plan_gemm(M, K, n_pad, ctx->num_sms, true, gate_up != 0);
+  int c = 0, p = 0;
+  CK(kvprm::gemm_placement(g, n_pad, &c, &p), "cudaOccupancyMaxActiveClusters");
+  *clusters = c;
+  *placed = p;
   return KVPRM_OK;
 }
 

@@ -96,6 +96,8 @@ def lib() -> ctypes.CDLL:
         L.kvprm_set_lora.argtypes = [vp, i32, ctypes.c_float, ctypes.POINTER(KvprmLora)]
         L.kvprm_set_readout_depth.argtypes = [vp, i32]
         L.kvprm_plan_projection.argtypes = [i32, i32, i32, i32, i32, i32, ctypes.POINTER(KvprmProjectionPlan)]
+        L.kvprm_debug_projection_placement.argtypes = [vp, i32, i32, i32, i32, ctypes.POINTER(i32),
+                                                       ctypes.POINTER(i32)]
         L.kvprm_debug_hidden.argtypes = [vp, vp]
         L.kvprm_attention_noalloc.argtypes = [vp, i64, i32p, i32, i32p, i32, i32, i32, i32, vp, vp, vp, vp, vp]
         L.kvprm_set_debug.argtypes = [vp, ctypes.c_int]
@@ -222,6 +224,14 @@ def kvprm_plan_projection(M: int, K: int, n_pad: int, num_sms: int, has_lo: bool
     if rc != 0:
         raise KvprmError(rc, "kvprm_plan_projection: bad arguments")
     return {k: getattr(out, k) for k, _ in KvprmProjectionPlan._fields_}
+
+
+def kvprm_debug_projection_placement(ctx, M: int, K: int, n: int, gate_up: bool = False) -> tuple[int, int]:
+    """(clusters of the launch, clusters the device holds at once) of a projection for n candidates."""
+    c, p = ctypes.c_int32(), ctypes.c_int32()
+    _check(ctx, lib().kvprm_debug_projection_placement(ctx, int(M), int(K), int(n), int(gate_up), ctypes.byref(c),
+                                                       ctypes.byref(p)))
+    return c.value, p.value
 
 
 def kvprm_set_readout_depth(ctx, depth: int) -> None:

@@ -34,6 +34,28 @@ def test_clusters_are_placed(arch, rank):
 
 
 @pytest.mark.gpu
+@pytest.mark.parametrize("arch", [ks.ARCH_1P5B, ks.ARCH_7B, ks.ARCH_8B, SMALL, WIDE, GATE_UP])
+def test_clusters_are_placed_by_the_device(arch):
+    """The same of the launches themselves: where a CTA fills an SM, no more clusters than the device holds at once
+    with the shared memory and cluster size that the launch has (not the plan's table of what GPCs place)."""
+    require_gpu()
+    w = ks.distinct("placed", ks.Arch(1, 128, 2, 2, 64, 128), 810, [16])
+    sc = make_scorer(ks.DeviceInputs(w, ks.Tables.make(0.2)), 256, w.max_blocks)
+    checked = 0
+    for n_pad in range(16, 257, 16):
+        for M, K, gu in [(arch.qkv_rows, arch.d_model, False), (arch.d_model, arch.n_q_heads * arch.head_dim, False),
+                         (arch.d_model, arch.d_ff, False), (arch.d_ff, arch.d_model, True)]:
+            for rank in (0, 64, 256):
+                p = kp.kvprm_plan_projection(M, K + rank, n_pad, 152, True, gu)
+                if p["smem_bytes"] + 1024 > 228 * 1024 // 2 and p["cluster"] * (1 + p["pair"]) > 1:
+                    clusters, placed = kp.kvprm_debug_projection_placement(sc.ctx, M, K + rank, n_pad, gu)
+                    assert 0 < clusters <= placed, (M, K, n_pad, gu, rank, p)
+                    checked += 1
+    assert checked
+    sc.close()
+
+
+@pytest.mark.gpu
 @pytest.mark.parametrize("arch, n, rank", [(SMALL, 48, 0), (SMALL, 64, 64), (SMALL, 65, 0), (SMALL, 128, 64),
                                            (SMALL, 129, 0), (SMALL, 145, 256),
                                            (SMALL, 208, 64), (SMALL, 256, 0), (WIDE, 88, 0), (WIDE, 129, 64), (WIDE, 176, 0),
