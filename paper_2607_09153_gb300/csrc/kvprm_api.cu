@@ -273,8 +273,10 @@ bool take_budget(size_t bytes) {
   return true;
 }
 
+// The buffer is zeroed in the order of `st`, the stream whose work uses it next (kvprm_create's, on the legacy
+// stream, are waited for before it returns).
 template <typename T>
-int dalloc(kvprm_ctx* ctx, T** p, size_t count, const char* what) {
+int dalloc(kvprm_ctx* ctx, T** p, size_t count, const char* what, cudaStream_t st = nullptr) {
   if (!take_budget(count * sizeof(T))) {
     *p = nullptr;
     return fail(ctx, KVPRM_ENOMEM, "allocation of %s (%zu bytes) exceeds the allocation budget", what,
@@ -286,9 +288,17 @@ int dalloc(kvprm_ctx* ctx, T** p, size_t count, const char* what) {
     cudaGetLastError();
     return fail(ctx, KVPRM_ENOMEM, "cudaMalloc(%s, %zu bytes): %s", what, count * sizeof(T), cudaGetErrorString(e));
   }
-  e = cudaMemset(*p, 0, count * sizeof(T) > 0 ? count * sizeof(T) : 16);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemset");
+  e = cudaMemsetAsync(*p, 0, count * sizeof(T) > 0 ? count * sizeof(T) : 16, st);
+  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemsetAsync");
   return KVPRM_OK;
+}
+
+// For a buffer made between calls, whatever stream the next one uses: zeroed on return.
+template <typename T>
+int dalloc_wait(kvprm_ctx* ctx, T** p, size_t count, const char* what) {
+  int rc = dalloc(ctx, p, count, what);
+  if (rc == KVPRM_OK) CK(cudaStreamSynchronize(nullptr), what);
+  return rc;
 }
 
 void free_ctx(kvprm_ctx* c) {
@@ -1108,7 +1118,7 @@ int ensure_grad(kvprm_ctx* ctx, cudaStream_t st) {
   size_t save_total = 0;
   for (size_t e : save_elems) save_total += al64(e * NL);
   float* base = nullptr;
-  if ((rc = dalloc(ctx, &base, save_total, "backward saves"))) return rc;
+  if ((rc = dalloc(ctx, &base, save_total, "backward saves", st))) return rc;
   FwdSaves& sv = g.sv;
   float* p = base;
   float** const save_ptr[8] = {&sv.q, &sv.k, &sv.v, &sv.o, &sv.lse, &sv.hmid, &sv.hout, &sv.gu};
@@ -1120,21 +1130,21 @@ int ensure_grad(kvprm_ctx* ctx, cudaStream_t st) {
   const size_t wmax = std::max<size_t>(std::max<size_t>(m.ff, m.d), nqh);
   const size_t gmax = std::max<size_t>(std::max<size_t>(2 * static_cast<size_t>(m.ff), m.qkv_rows), m.d);
   float* bb = nullptr;
-  if ((rc = dalloc(ctx, &bb, Bm * (m.d + wmax + nqh + 2 * nkh) + al64(Bm * m.n_q), "backward buffers"))) return rc;
+  if ((rc = dalloc(ctx, &bb, Bm * (m.d + wmax + nqh + 2 * nkh) + al64(Bm * m.n_q), "backward buffers", st))) return rc;
   g.dh = bb;
   g.tmp = g.dh + Bm * m.d;
   g.D = g.tmp + Bm * wmax;
   g.dq = g.D + al64(Bm * m.n_q);
   g.dks = g.dq + Bm * nqh;
   g.dvs = g.dks + Bm * nkh;
-  if ((rc = dalloc(ctx, &g.ghi, static_cast<size_t>(ctx->npad_max) * gmax, "backward hi"))) return rc;
-  if ((rc = dalloc(ctx, &g.glo, static_cast<size_t>(ctx->npad_max) * gmax, "backward lo"))) return rc;
+  if ((rc = dalloc(ctx, &g.ghi, static_cast<size_t>(ctx->npad_max) * gmax, "backward hi", st))) return rc;
+  if ((rc = dalloc(ctx, &g.glo, static_cast<size_t>(ctx->npad_max) * gmax, "backward lo", st))) return rc;
   if (m.n_q / m.n_kv <= 8 && !ctx->grad_cuda_cores) {
     // and after them the zero rows
     const size_t ops = kvprm::attn_back_ops_bytes(Bm, m.n_kv, m.hd);
-    if ((rc = dalloc(ctx, &g.ops, ops + kvprm::attn_back_zero_bytes(m.hd), "backward operands"))) return rc;
+    if ((rc = dalloc(ctx, &g.ops, ops + kvprm::attn_back_zero_bytes(m.hd), "backward operands", st))) return rc;
     g.zero_rows = g.ops + ops;
-    if ((rc = dalloc(ctx, &g.meta, Bm * m.n_kv * 8, "backward row statistics"))) return rc;
+    if ((rc = dalloc(ctx, &g.meta, Bm * m.n_kv * 8, "backward row statistics", st))) return rc;
   }
   // transposed weights: W [out][in] -> W^T [in][out], from the borrowed weights' tensor-map bases
   g.tm_qkv.resize(NL);
@@ -1149,7 +1159,7 @@ int ensure_grad(kvprm_ctx* ctx, cudaStream_t st) {
     CUtensorMap* maps[4] = {&g.tm_qkv[l], &g.tm_o[l], &g.tm_gu[l], &g.tm_down[l]};
     for (int j = 0; j < 4; ++j) {
       bf16* wt = nullptr;
-      if ((rc = dalloc(ctx, &wt, static_cast<size_t>(mats[j].out) * mats[j].in, "transposed weights"))) return rc;
+      if ((rc = dalloc(ctx, &wt, static_cast<size_t>(mats[j].out) * mats[j].in, "transposed weights", st))) return rc;
       g.wt.push_back(wt);
       CK(kvprm::launch_transpose(static_cast<const bf16*>(src[j]), wt, mats[j].out, mats[j].in, st), "transpose");
       // W^T [in][out]: M = in rows, K = out columns
@@ -1178,12 +1188,12 @@ int ensure_grad_maps(kvprm_ctx* ctx, int n_pad) {
 }
 
 template <typename T>
-int grow(kvprm_ctx* ctx, T** p, size_t* cap, size_t need, const char* what) {
+int grow(kvprm_ctx* ctx, T** p, size_t* cap, size_t need, const char* what, cudaStream_t st) {
   if (need <= *cap) return KVPRM_OK;
   cudaFree(*p);
   *p = nullptr;
   *cap = 0;
-  int rc = dalloc(ctx, p, need, what);
+  int rc = dalloc(ctx, p, need, what, st);
   if (rc) return rc;
   *cap = need;
   return KVPRM_OK;
@@ -1217,7 +1227,7 @@ int score_grad_device(kvprm_ctx* ctx, const void* kv_pages, int64_t n_pages, con
   kvprm::plan_attn_back(bt, sl, n, mb, n_pages, m.n_kv, g.ops != nullptr, ctx->num_sms, bp);
   const int n_shared = bp.n_atomic;
   auto send = [&](auto** dst, size_t* cap, const auto& src, const char* what) -> int {
-    if ((rc = grow(ctx, dst, cap, std::max<size_t>(src.size(), 1), what))) return rc;
+    if ((rc = grow(ctx, dst, cap, std::max<size_t>(src.size(), 1), what, st))) return rc;
     if (!src.empty())
       CK(cudaMemcpyAsync(*dst, src.data(), sizeof(src[0]) * src.size(), cudaMemcpyHostToDevice, st), what);
     return KVPRM_OK;
@@ -1621,7 +1631,7 @@ int kvprm_set_lora(kvprm_ctx* ctx, int32_t rank, float scale, const kvprm_lora* 
     }
   }
   CK(kvprm::gemm_configure((ctx->cfg.max_candidates + 15) / 16 * 16, true), "gemm_configure(adapter)");
-  if (!ctx->x_ready && (rc = dalloc(ctx, &ctx->x_ready, 4 * static_cast<size_t>(NL), "adapter marks"))) return rc;
+  if (!ctx->x_ready && (rc = dalloc_wait(ctx, &ctx->x_ready, 4 * static_cast<size_t>(NL), "adapter marks"))) return rc;
   const size_t need = static_cast<size_t>(ctx->npad_max) * rank;
   if (need > ctx->t_cap) {
     bf16 *th = nullptr, *tl = nullptr;
@@ -1638,8 +1648,11 @@ int kvprm_set_lora(kvprm_ctx* ctx, int32_t rank, float scale, const kvprm_lora* 
     ctx->t_cap = need;
   } else if (rank != ctx->lora_rank) {
     // padding rows of t (candidates >= n) are read as K-extension columns: keep them zero
+    // (after the calls in flight that use it, and before the next, whatever their streams)
+    CK(cudaDeviceSynchronize(), "cudaDeviceSynchronize(adapter buffers)");
     CK(cudaMemset(ctx->thi, 0, sizeof(bf16) * ctx->t_cap), "cudaMemset(t_hi)");
     CK(cudaMemset(ctx->tlo, 0, sizeof(bf16) * ctx->t_cap), "cudaMemset(t_lo)");
+    CK(cudaStreamSynchronize(nullptr), "cudaStreamSynchronize(adapter buffers)");
   }
   for (int j = 0; j < 4; ++j) {
     ctx->tm_la[j] = std::move(la[j]);
@@ -1828,22 +1841,22 @@ int kvprm_set_debug(kvprm_ctx* ctx, int flags) {
   if (!ctx) return KVPRM_EINVAL;
   if ((flags & 1) && !ctx->dbg) {
     const size_t count = static_cast<size_t>(ctx->cfg.n_layers) * ctx->cfg.max_candidates * ctx->md.n_q * ctx->md.hd;
-    int rc = dalloc(ctx, &ctx->dbg, count, "debug capture");
+    int rc = dalloc_wait(ctx, &ctx->dbg, count, "debug capture");
     if (rc) return rc;
   }
   const size_t NB = static_cast<size_t>(ctx->cfg.n_layers) * ctx->cfg.max_candidates;
   if ((flags & 2) && !ctx->dbg_q) {
-    int rc = dalloc(ctx, &ctx->dbg_q, NB * ctx->md.n_q * ctx->md.hd, "debug q");
-    if (!rc) rc = dalloc(ctx, &ctx->dbg_k, NB * ctx->md.n_kv * ctx->md.hd, "debug k");
-    if (!rc) rc = dalloc(ctx, &ctx->dbg_v, NB * ctx->md.n_kv * ctx->md.hd, "debug v");
+    int rc = dalloc_wait(ctx, &ctx->dbg_q, NB * ctx->md.n_q * ctx->md.hd, "debug q");
+    if (!rc) rc = dalloc_wait(ctx, &ctx->dbg_k, NB * ctx->md.n_kv * ctx->md.hd, "debug k");
+    if (!rc) rc = dalloc_wait(ctx, &ctx->dbg_v, NB * ctx->md.n_kv * ctx->md.hd, "debug v");
     if (rc) return rc;
   }
   if ((flags & 4) && !ctx->dbg_h) {
-    int rc = dalloc(ctx, &ctx->dbg_h, NB * ctx->md.d, "debug h");
+    int rc = dalloc_wait(ctx, &ctx->dbg_h, NB * ctx->md.d, "debug h");
     if (rc) return rc;
   }
   if ((flags & 32) && !ctx->tc_prof) {
-    int rc = dalloc(ctx, &ctx->tc_prof, kvprm::kTcEventLog + static_cast<size_t>(ctx->num_sms) * 16,
+    int rc = dalloc_wait(ctx, &ctx->tc_prof, kvprm::kTcEventLog + static_cast<size_t>(ctx->num_sms) * 16,
                     "tensor-core attention profile");
     if (rc) return rc;
   }
@@ -2016,7 +2029,7 @@ int kvprm_steer(kvprm_ctx* ctx, void* kv_pages, int64_t n_pages, const int32_t* 
   if (bytes > g.grad_own_bytes) {
     CK(cudaStreamSynchronize(st), "cudaStreamSynchronize(steering buffer)");
     size_t cap = g.grad_own_bytes / 4;
-    if ((rc = grow(ctx, &g.grad_own, &cap, bytes / 4, "steering gradient"))) {
+    if ((rc = grow(ctx, &g.grad_own, &cap, bytes / 4, "steering gradient", st))) {
       g.grad_own_bytes = 0;
       return rc;
     }
@@ -2078,7 +2091,7 @@ int kvprm_set_trace(kvprm_ctx* ctx, int enable) {
   if (!ctx) return KVPRM_EINVAL;
   if (enable && !ctx->trace_d) {
     ctx->trace_cap = 2 + 8 * ctx->cfg.n_layers + 8;
-    int rc = dalloc(ctx, &ctx->trace_d, static_cast<size_t>(kvprm::kTraceStride) * ctx->trace_cap, "trace");
+    int rc = dalloc_wait(ctx, &ctx->trace_d, static_cast<size_t>(kvprm::kTraceStride) * ctx->trace_cap, "trace");
     if (rc) return rc;
   }
   ctx->trace = enable != 0;
