@@ -289,7 +289,11 @@ int dalloc(kvprm_ctx* ctx, T** p, size_t count, const char* what, cudaStream_t s
     return fail(ctx, KVPRM_ENOMEM, "cudaMalloc(%s, %zu bytes): %s", what, count * sizeof(T), cudaGetErrorString(e));
   }
   e = cudaMemsetAsync(*p, 0, count * sizeof(T) > 0 ? count * sizeof(T) : 16, st);
-  if (e != cudaSuccess) return cuda_fail(ctx, e, "cudaMemsetAsync");
+  if (e != cudaSuccess) {
+    cudaFree(*p);
+    *p = nullptr;
+    return cuda_fail(ctx, e, "cudaMemsetAsync");
+  }
   return KVPRM_OK;
 }
 
@@ -299,6 +303,26 @@ int dalloc_wait(kvprm_ctx* ctx, T** p, size_t count, const char* what) {
   int rc = dalloc(ctx, p, count, what);
   if (rc == KVPRM_OK) CK(cudaStreamSynchronize(nullptr), what);
   return rc;
+}
+
+void free_grad(GradState& g) {
+  for (auto* p : g.wt) cudaFree(p);
+  cudaFree(g.sv.q);
+  cudaFree(g.dh);
+  cudaFree(g.ghi);
+  cudaFree(g.glo);
+  cudaFree(g.ops);
+  cudaFree(g.meta);
+  cudaFree(g.units);
+  cudaFree(g.items);
+  cudaFree(g.item_pages);
+  cudaFree(g.item_cands);
+  cudaFree(g.cta_item);
+  cudaFree(g.shared);
+  cudaFree(g.lists);
+  cudaFree(g.grad_own);
+  if (g.gexec) cudaGraphExecDestroy(g.gexec);
+  g = GradState();
 }
 
 void free_ctx(kvprm_ctx* c) {
@@ -336,25 +360,7 @@ void free_ctx(kvprm_ctx* c) {
   cudaFree(c->dummy_pool);
   cudaFree(c->dev_pool);
   cudaFree(c->probe_flag);
-  {
-    GradState& g = c->grad;
-    for (auto* p : g.wt) cudaFree(p);
-    cudaFree(g.sv.q);
-    cudaFree(g.dh);
-    cudaFree(g.ghi);
-    cudaFree(g.glo);
-    cudaFree(g.ops);
-    cudaFree(g.meta);
-    cudaFree(g.units);
-    cudaFree(g.items);
-    cudaFree(g.item_pages);
-    cudaFree(g.item_cands);
-    cudaFree(g.cta_item);
-    cudaFree(g.shared);
-    cudaFree(g.lists);
-    cudaFree(g.grad_own);
-    if (g.gexec) cudaGraphExecDestroy(g.gexec);
-  }
+  free_grad(c->grad);
   if (c->staging) cudaFreeHost(c->staging);
   if (c->h_rewards) cudaFreeHost(c->h_rewards);
   if (c->h_err) cudaFreeHost(c->h_err);
@@ -1100,11 +1106,9 @@ int finish_blocking(kvprm_ctx* ctx, int32_t n, float* rewards, cudaStream_t st) 
 }
 
 // ---------------------------------------------------------------- KV Steering: backward pass
-// First kvprm_score_grad call: transposed weight copies, forward saves and backward buffers, sized
-// for max_candidates.
-int ensure_grad(kvprm_ctx* ctx, cudaStream_t st) {
+// Transposed weight copies, forward saves and backward buffers, sized for max_candidates.
+int make_grad(kvprm_ctx* ctx, cudaStream_t st) {
   GradState& g = ctx->grad;
-  if (g.ready) return KVPRM_OK;
   const ModelDims& m = ctx->md;
   const int NL = ctx->cfg.n_layers;
   const size_t Bm = static_cast<size_t>(ctx->cfg.max_candidates);
@@ -1168,6 +1172,17 @@ int ensure_grad(kvprm_ctx* ctx, cudaStream_t st) {
   }
   g.ready = true;
   return KVPRM_OK;
+}
+
+// The first kvprm_score_grad call makes them; a failure leaves the context without any.
+int ensure_grad(kvprm_ctx* ctx, cudaStream_t st) {
+  if (ctx->grad.ready) return KVPRM_OK;
+  const int rc = make_grad(ctx, st);
+  if (rc) {
+    cudaStreamSynchronize(st);   // copies in flight to what is freed now
+    free_grad(ctx->grad);
+  }
+  return rc;
 }
 
 int ensure_grad_maps(kvprm_ctx* ctx, int n_pad) {

@@ -57,6 +57,41 @@ def test_allocation_budget(tiny):
         kp.kvprm_debug_set_alloc_limit(-1)
 
 
+def test_first_gradient_out_of_memory():
+    """The first gradient call allocates its buffers and a transposed copy of every weight.  Out of memory anywhere in
+    between, it leaves nothing behind: a later call gives the gradient, and destroying the context gives all back."""
+    import paper_2607_09153_gb300 as kp
+    torch = require_gpu()
+    w = ks.distinct("fail_grad", ks.Arch(2, 512, 8, 2, 64, 2048), 302, [40, 128, 77], gain_std=0.2)
+    dev = ks.DeviceInputs(w, ks.Tables.make(0.2))
+    want, got = (torch.zeros(dev.pool.shape, dtype=torch.float32, device="cuda") for _ in range(2))
+    st = torch.cuda.current_stream().cuda_stream
+
+    def cycle(limits, grad):
+        sc = make_scorer(dev, w.n_candidates, w.max_blocks)
+        args = (sc.ctx, dev.pool.data_ptr(), dev.n_pages, w.block_table, w.seq_lens, w.n_candidates, grad.data_ptr(), st)
+        try:
+            for limit in limits:   # the transposed weights alone are 14.5 MiB
+                kp.kvprm_debug_set_alloc_limit(limit)
+                with pytest.raises(kp.KvprmError) as e:
+                    kp.kvprm_score_grad(*args)
+                assert e.value.code == kp.KVPRM_ENOMEM
+        finally:
+            kp.kvprm_debug_set_alloc_limit(-1)
+        kp.kvprm_score_grad(*args)
+        torch.cuda.synchronize()
+        in_use = torch.cuda.mem_get_info()[0]
+        sc.close()
+        torch.cuda.synchronize()
+        return in_use, torch.cuda.mem_get_info()[0]
+
+    cycle([], want)   # loads the kernels
+    in_use, free = cycle([], want)
+    in_use2, free2 = cycle([0, 1 << 12] + [k << 20 for k in range(1, 15)] * 4, got)
+    assert ((got - want).norm() / want.norm()).item() < 1e-4   # sums in another order
+    assert in_use2 == in_use and free2 == free
+
+
 def test_injected_cuda_error(tiny):
     import paper_2607_09153_gb300 as kp
     w, t, dev = tiny
