@@ -1139,6 +1139,7 @@ bool build_attn_work(const int32_t* bt, const int32_t* sl, int n, int max_blocks
   w.n_tc_ctas = 0;
   w.packed = false;
   w.tc_concurrent = false;
+  w.fuse_cs = 0;
   w.tc_cta.clear();
   w.segs.clear();
   w.cta_seg.clear();
