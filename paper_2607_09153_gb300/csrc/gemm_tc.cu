@@ -143,7 +143,6 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   const int cend = min(cbeg + cols, ep.n_valid);
   const int nc = cend > cbeg ? cend - cbeg : 0;
   const bool hpreload = MODE == GemmEpilogue::RESID && nc <= kHPreCols;
-  constexpr int kEpiBatch = LARGE ? 8 : 1;
 
   if (threadIdx.x == 0) {
     for (int s = 0; s < stages; ++s) {
@@ -386,7 +385,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
   float* acc = reinterpret_cast<float*>(smem) - c_off * kBM;
   // 4 warps, or 8 (the large-batch image): warps w and w + 4 share TMEM lane quadrant w,
   // i.e. the tile's rows 32 w .. 32 w + 31, and take alternate 16-column groups (or columns)
-  const int nw = static_cast<int>(blockDim.x >> 5), nwh = nw >> 2, wh = warp >> 2;
+  const int nw = LARGE ? static_cast<int>(blockDim.x >> 5) : 4, nwh = LARGE ? nw >> 2 : 1, wh = LARGE ? warp >> 2 : 0;
   const int m = (warp & 3) * 32 + lane;
   const bool merged = has_lo && 2 * n_pad <= 256;
   const uint32_t tile_cols = tmem_cols / (PAIR ? 2u : 1u);
@@ -577,7 +576,7 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
       } else if (cs > 1) {   // two columns per round trip when the cluster has <= 8 ranks
         const int step = cs <= 8 ? 2 : 1;
 #pragma unroll 1
-        for (int c = cbeg + wh * step; c < cend; c += step * nwh) {
+        for (int c = cbeg; c < cend; c += step) {
           const bool two = step == 2 && c + 1 < cend;
           float v[16];
 #pragma unroll
@@ -798,31 +797,18 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
         }
       }
     } else if constexpr (MODE == GemmEpilogue::SILU) {
-      // 2 nhalf column groups of 64 threads (rows m and m + 64 of a column share a group)
-      const int r = m & 63, ng = 2 * nwh, grp = (m >> 6) + 2 * wh;
+      // two column groups of 64 threads (rows m and m + 64 of a column share a group)
+      const int r = m & 63;
       const int j = m_tile * 64 + r;
       if (j < ep.ff)
 #pragma unroll 1
-        for (int c0 = cbeg + grp; c0 < cend; c0 += ng * kEpiBatch) {
-          float g[kEpiBatch], u[kEpiBatch];   // a batch's operands, read before its first store
-#pragma unroll
-          for (int k = 0; k < kEpiBatch; ++k) {
-            const int c = c0 + ng * k;
-            const bool ok = c < cend;
-            const float rs = (ok && ep.rs_sumsq) ? rsc[c - cbeg] : 1.f;
-            g[k] = ok ? acc[c * kBM + r] * rs : 0.f;
-            u[k] = ok ? acc[c * kBM + 64 + r] * rs : 0.f;
-          }
-#pragma unroll
-          for (int k = 0; k < kEpiBatch; ++k) {
-            const int c = c0 + ng * k;
-            if (c < cend) {
-              store_hilo(ep.a_hi, ep.a_lo, static_cast<int64_t>(c) * ep.ff + j, g[k] / (1.0f + expf(-g[k])) * u[k]);
-              if (ep.gu_save) {   // gate and up pre-activations for a backward pass
-                ep.gu_save[static_cast<int64_t>(c) * 2 * ep.ff + j] = g[k];
-                ep.gu_save[static_cast<int64_t>(c) * 2 * ep.ff + ep.ff + j] = u[k];
-              }
-            }
+        for (int c = cbeg + (m >> 6); c < cend; c += 2) {
+          const float rs = ep.rs_sumsq ? rsc[c - cbeg] : 1.f;
+          const float g = acc[c * kBM + r] * rs, u = acc[c * kBM + 64 + r] * rs;
+          store_hilo(ep.a_hi, ep.a_lo, static_cast<int64_t>(c) * ep.ff + j, g / (1.0f + expf(-g)) * u);
+          if (ep.gu_save) {   // gate and up pre-activations for a backward pass
+            ep.gu_save[static_cast<int64_t>(c) * 2 * ep.ff + j] = g;
+            ep.gu_save[static_cast<int64_t>(c) * 2 * ep.ff + ep.ff + j] = u;
           }
         }
     } else if constexpr (LARGE) {   // QKV
@@ -905,8 +891,8 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
           }
         }
       }
-    } else {   // QKV: pair p = m & 63 of this tile, 2 nhalf column groups of 64 threads
-      const int p = m & 63, ng = 2 * nwh, grp = (m >> 6) + 2 * wh;
+    } else {   // QKV: pair p = m & 63 of this tile, two column groups of 64 threads
+      const int p = m & 63;
       const int lhd = ep.hd == 128 ? 7 : 6;               // head_dim is 64 or 128
       const int hd = 1 << lhd, half = hd >> 1;
       const int row_a = ((p >> (lhd - 1)) << lhd) + (p & (half - 1));   // first element of the pair, within the tile
@@ -923,43 +909,28 @@ __global__ void __launch_bounds__(256, 2) gemm_cluster_kernel(const __grid_const
       }
       const int hh_tile = row_a >> lhd;
 #pragma unroll 1
-      for (int c0 = cbeg + grp; c0 < cend; c0 += ng * kEpiBatch) {
-        // a batch's operands (accumulator pair and rotation), read before its first store
-        float av[kEpiBatch], bv[kEpiBatch];
-        float2 cs2[kEpiBatch];
-#pragma unroll
-        for (int k = 0; k < kEpiBatch; ++k) {
-          const int c = c0 + ng * k;
-          const bool ok = c < cend;
-          const float rs = !ok ? 1.f : (ep.qn_gain ? qkf[(c - cbeg) * 2 + hh_tile] : (ep.rs_sumsq ? rsc[c - cbeg] : 1.f));
-          av[k] = ok ? acc[c * kBM + row_a] * rs * gna : 0.f;
-          bv[k] = ok ? acc[c * kBM + row_b] * rs * gnb : 0.f;
-          cs2[k] = (ok && rot) ? ep.rope[c * half + i] : make_float2(1.f, 0.f);
+      for (int c = cbeg + (m >> 6); c < cend; c += 2) {
+        const float rs = ep.qn_gain ? qkf[(c - cbeg) * 2 + hh_tile] : (ep.rs_sumsq ? rsc[c - cbeg] : 1.f);
+        float a = acc[c * kBM + row_a] * rs * gna, b = acc[c * kBM + row_b] * rs * gnb;
+        if (rot) {
+          const float2 cs2 = ep.rope[c * half + i];
+          const float a2 = fmaf(a, cs2.x, -(b * cs2.y));
+          const float b2 = fmaf(a, cs2.y, b * cs2.x);
+          a = a2;
+          b = b2;
         }
-#pragma unroll
-        for (int k = 0; k < kEpiBatch; ++k) {
-          const int c = c0 + ng * k;
-          if (c >= cend) break;
-          float a = av[k], b = bv[k];
-          if (rot) {
-            const float a2 = a * cs2[k].x - b * cs2[k].y;
-            const float b2 = b * cs2[k].x + a * cs2[k].y;
-            a = a2;
-            b = b2;
-          }
-          if (head < ep.n_q) {
-            const int64_t o = (static_cast<int64_t>(c) * ep.n_q + head) * hd + i;
-            ep.q[o] = a;
-            ep.q[o + half] = b;
-            store_hilo(ep.q_hi, ep.q_lo, o, a);
-            store_hilo(ep.q_hi, ep.q_lo, o + half, b);
-          } else if (head < ep.n_q + 2 * ep.n_kv) {
-            const bool is_k = head < ep.n_q + ep.n_kv;
-            const int kvh = is_k ? head - ep.n_q : head - ep.n_q - ep.n_kv;
-            float* dst = (is_k ? ep.kself : ep.vself) + (static_cast<int64_t>(c) * ep.n_kv + kvh) * hd + i;
-            dst[0] = a;
-            dst[half] = b;
-          }
+        if (head < ep.n_q) {
+          const int64_t o = (static_cast<int64_t>(c) * ep.n_q + head) * hd + i;
+          ep.q[o] = a;
+          ep.q[o + half] = b;
+          store_hilo(ep.q_hi, ep.q_lo, o, a);
+          store_hilo(ep.q_hi, ep.q_lo, o + half, b);
+        } else if (head < ep.n_q + 2 * ep.n_kv) {
+          const bool is_k = head < ep.n_q + ep.n_kv;
+          const int kvh = is_k ? head - ep.n_q : head - ep.n_q - ep.n_kv;
+          float* dst = (is_k ? ep.kself : ep.vself) + (static_cast<int64_t>(c) * ep.n_kv + kvh) * hd + i;
+          dst[0] = a;
+          dst[half] = b;
         }
       }
     }
