@@ -378,7 +378,8 @@ def measure(w, args, world, local, steps: int, warmup: int, prof_steps: int, wit
     tp = time.perf_counter()
     for _ in range(5):
         kp.kvprm_plan_attention(w.block_table, w.seq_lens, a.n_kv_heads, a.n_q_heads // a.n_kv_heads,
-                                torch.cuda.get_device_properties(0).multi_processor_count, share | kp.KVPRM_PLAN_FUSE)
+                                torch.cuda.get_device_properties(0).multi_processor_count,
+                                share | kp.KVPRM_PLAN_FUSE | kp.KVPRM_PLAN_PACK)
     out["plan_us"] = round(1e6 * (time.perf_counter() - tp) / 5, 1)
 
     if with_e2e:   # end to end through the host-buffer call (cache copied H2D every step)

@@ -80,7 +80,8 @@ struct GemmEpilogue {
   __nv_bfloat16* t_hi = nullptr;
   __nv_bfloat16* t_lo = nullptr;
   // LOWRANK: *x_ready becomes the call's number *call once x may be read; the projection that takes t waits for
-  // that, instead of for its predecessor's end, before it reads x
+  // that, instead of for its predecessor's end, before it reads x.  (*call is a word of the call's tables, which are
+  // on the device before the call's first kernel starts.)
   int* x_ready = nullptr;
   const int* call = nullptr;
   // let the next kernel in the stream launch only once this one's partials are parked (after its
