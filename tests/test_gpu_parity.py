@@ -96,8 +96,8 @@ def test_layer_shapes(arch, lens):
 
 def test_two_tile_gate_up():
     """7B layer shapes at 200 candidates (padded to 208): the gate/up projection's one-tile CTAs
-    would not fit on the SMs at once, so each CTA takes two m-tiles (two accumulators of N = 208
-    side by side in TMEM, one activation stage for both); sampled candidates against the oracle."""
+    would not fit on the SMs at once, so pairs of CTAs take two m-tiles each (two accumulators of N = 208
+    side by side in TMEM, half of the activations in either CTA); sampled candidates against the oracle."""
     t = ks.Tables.make(0.2)
     lens = [(53 * b) % 257 for b in range(200)]
     w = ks.distinct("two_tile", ks.Arch(2, 3584, 28, 4, 128, 18944), 57, lens, gain_std=0.2)
@@ -281,7 +281,7 @@ def _lora_arch(arch, rank):
     (ks.Arch(2, 1536, 12, 2, 128, 8960), 256, [2048] * 16, None),                   # 1.5B layers, small image
     (ks.Arch(2, 3584, 28, 4, 128, 18944), 256, [(37 * b) % 300 for b in range(64)],  # 7B layers, B = 64
      [0, 1, 31, 63]),
-    (ks.Arch(2, 3584, 28, 4, 128, 18944), 128, [(53 * b) % 257 for b in range(200)],  # two m-tiles per gate/up CTA
+    (ks.Arch(2, 3584, 28, 4, 128, 18944), 128, [(53 * b) % 257 for b in range(200)],  # CTA pairs in every projection
      [0, 100, 199]),
 ])
 def test_lora(arch, rank, lens, sample):

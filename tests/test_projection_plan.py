@@ -1,7 +1,8 @@
 """The projection GEMM's launch plan (kvprm_plan_projection, host only) over the workloads' shapes,
 batch paddings and adapter ranks: the invariants the kernel relies on (shared memory within the
 configured limit, split-K ranks dividing the batch columns, the K tiles covered, tensor memory for
-every tile's accumulator, two-tile plans in one wave)."""
+every tile's accumulator, two-tile plans in one wave).  kt_per_split is ceil(k_tiles / cluster) by its definition;
+what a CTA streams is kt_per_rank."""
 import pytest
 
 import kvsynth as ks
