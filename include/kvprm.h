@@ -192,7 +192,8 @@ KVPRM_API const char* kvprm_last_error(const kvprm_ctx* ctx);
  *               siblings).  Entries j >= ceil(seq_lens[b] / 16) are ignored.
  *  seq_lens     host int32 [n_candidates]: cached length L_b in
  *               [0, 16 * max_blocks_per_seq].  L_b = 0 is legal (the verify
- *               token then attends to itself only).
+ *               token then attends to itself only).  The slots of a last page
+ *               past L_b have weight zero but are read: they must be finite.
  *  n_candidates 0 .. max_candidates (0 is a no-op).
  *  rewards      host float [n_candidates]: P(+) per candidate.
  *  stream       cudaStream_t or NULL.
@@ -465,7 +466,8 @@ KVPRM_API int kvprm_check_device(kvprm_ctx* ctx);
  * projection matrices of every layer (as much device memory as the weights)
  * and buffers for the intermediates (sized for max_candidates).
  * Scope: merged weights (no kvprm_set_lora adapter), readout depth 1, qk_norm
- * 0; otherwise KVPRM_EUNSUPPORTED.  Other errors as kvprm_score, KVPRM_ENOMEM.
+ * 0; otherwise KVPRM_EUNSUPPORTED, as for a first call on a stream that is being
+ * captured.  Other errors as kvprm_score, KVPRM_ENOMEM.
  * Blocking.  The caller's pages are only read.
  *
  * kvprm_steer runs `steps` steps of the algorithm on a caller-owned copy of the

@@ -1177,6 +1177,11 @@ int make_grad(kvprm_ctx* ctx, cudaStream_t st) {
 // The first kvprm_score_grad call makes them; a failure leaves the context without any.
 int ensure_grad(kvprm_ctx* ctx, cudaStream_t st) {
   if (ctx->grad.ready) return KVPRM_OK;
+  // what a capture records has not run: the copies would count as made
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  CK(cudaStreamIsCapturing(st, &cap), "cudaStreamIsCapturing");
+  if (cap != cudaStreamCaptureStatusNone)
+    return fail(ctx, KVPRM_EUNSUPPORTED, "the gradient call blocks: its stream cannot be captured");
   const int rc = make_grad(ctx, st);
   if (rc) {
     cudaStreamSynchronize(st);   // copies in flight to what is freed now

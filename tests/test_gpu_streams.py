@@ -42,6 +42,29 @@ def test_first_gradient_calls(group_of):
     sc.close()
 
 
+def test_first_gradient_call_on_a_captured_stream():
+    # refused before anything is made, so that the call after it makes its buffers
+    torch = require_gpu()
+    import paper_2607_09153_gb300 as kp
+    w = ks.shared_prefix("streams_c", ARCH, 942, 5, 70, 45, gain_std=0.2)
+    dev = ks.DeviceInputs(w, ks.Tables.make(0.2))
+    sc = make_scorer(dev, 5, w.max_blocks)
+    want = _grads(sc, dev, w, torch.cuda.default_stream(), 1)[0]
+    sc.close()
+    sc = make_scorer(dev, 5, w.max_blocks)
+    s, g = torch.cuda.Stream(), torch.zeros(dev.pool.shape, dtype=torch.float32, device="cuda")
+    x = torch.ones(4, device="cuda")
+    with torch.cuda.graph(torch.cuda.CUDAGraph(), stream=s, capture_error_mode="relaxed"):
+        x += 1
+        with pytest.raises(kp.KvprmError) as e:
+            kp.kvprm_score_grad(sc.ctx, dev.pool.data_ptr(), dev.n_pages, w.block_table, w.seq_lens, w.n_candidates,
+                                g.data_ptr(), s.cuda_stream)
+    assert e.value.code == kp.KVPRM_EUNSUPPORTED
+    got = _grads(sc, dev, w, torch.cuda.default_stream(), 1)[0]
+    assert ((got - want).norm() / want.norm()).item() < 1e-4
+    sc.close()
+
+
 def test_debug_capture_and_adapter():
     torch = require_gpu()
     import paper_2607_09153_gb300 as kp
