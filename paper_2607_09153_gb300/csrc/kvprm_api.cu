@@ -131,7 +131,7 @@ struct kvprm_ctx {
   bf16 *thi = nullptr, *tlo = nullptr;
   size_t t_cap = 0;
   int* x_ready = nullptr;   // [n_layers][4] the last call whose A x of that projection had its x
-  int32_t call = 0;         // number of the current call (in its tables)
+  uint32_t call = 0;        // number of the current call (in its tables)
   int tm_t_npad = -1;
   CUtensorMap tm_thi{}, tm_tlo{};
   // workspace
@@ -466,7 +466,7 @@ int upload_tables(kvprm_ctx* ctx, const int32_t* bt, const int32_t* sl, int32_t 
   if (++ctx->call == 0) ++ctx->call;   // x_ready's marks start at 0
   const struct {
     float* rewards;
-    int32_t call, pad;
+    uint32_t call, pad;
   } out{rewards_out, ctx->call, 0};
   std::memcpy(S, sl, sizeof(int32_t) * n);
   std::memcpy(S + Bmax, bt, sizeof(int32_t) * static_cast<size_t>(n) * mb);
